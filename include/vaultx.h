@@ -87,10 +87,11 @@ typedef struct vx_opts {
                                    Poisson count; 0 = default (12)                   */
     uint32_t hash_block;        /* threads per block of the hash kernels: 0 or 256
                                    (the one shape built; others are VX_EINVAL)      */
-    uint32_t nonces_per_thread; /* nonces each Table-1 hash thread handles: 0 (= 8),
-                                   4, 8 or 16 with the staged bucketing of a whole
-                                   plot; 8 with the direct bucketing or a window;
-                                   others VX_EINVAL.  Same tables for every value. */
+    uint32_t nonces_per_thread; /* nonces each Table-1 hash thread handles: 0 = automatic
+                                   (2 to 16 by the plot's size), or 4, 8 or 16 with
+                                   the staged bucketing of a whole plot; 8 with the
+                                   direct bucketing or a window; others VX_EINVAL.
+                                   Same tables for every value.                      */
     uint32_t scatter_mode;      /* bucketing of hashed records: 0 = automatic
                                    (staged), 1 = staged (shared-memory histogram per CTA, one
                                    claim per (CTA, bin), two levels), 2 = direct

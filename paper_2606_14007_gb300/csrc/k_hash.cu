@@ -58,59 +58,76 @@ cudaError_t launch_key_setup(Desc *descs, int nplots, cudaStream_t s)
 }
 
 // --------------------------------------------- hash + first-level scatter
-// Shared layout of one tile: staged key64[T], nonce[T], then per-bin
-// histogram, local offset and claimed global base (kMaxCoarseBits bins).
+// Shared layout of one tile of T nonces: key64[T] in nonce order, then per
+// record its bin (kNoBin: not kept), its rank inside the bin, and, once the
+// bins are scanned, the record order by bin; then per bin the histogram
+// (which becomes the bin's start in the tile) and the bin's place.  Bins,
+// ranks and starts are kept as the byte offsets they are used at (4 * bin,
+// 2 * rank, 2 * start), so that no use of them costs a shift.
 template <int NT, int NPT>
-struct HashSmem {
-    static constexpr int T = NT * NPT;
+struct HashTile {
+    static constexpr uint32_t T = NT * NPT;
     uint64_t keys[T];
-    uint32_t nonces[T];
-    uint32_t hist[1 << kMaxCoarseBits];
-    uint32_t loff[1 << kMaxCoarseBits];
-    uint32_t gbase[1 << kMaxCoarseBits];
+    uint16_t bin4[T], rank2[T], order[T];
+    uint32_t start2[1 << kMaxCoarseBits];
+    uint32_t place[1 << kMaxCoarseBits];
     uint32_t ws[NT / 32 + 1];
 };
+constexpr uint32_t kNoBin = 0xFFFFu;
+
+template <class X>
+__device__ __forceinline__ X &at_bytes(X *a, uint32_t off)
+{
+    return *reinterpret_cast<X *>(reinterpret_cast<unsigned char *>(a) + off);
+}
 
 // Rank of this lane's record within its bin's run of the tile.
 template <bool AGG>
-__device__ __forceinline__ uint32_t bin_rank(uint32_t *hist, uint32_t bin, bool valid)
+__device__ __forceinline__ uint32_t bin_rank(uint32_t *hist, uint32_t bin4, bool valid)
 {
     if (AGG) {
-        const uint32_t peers = __match_any_sync(0xffffffffu, valid ? bin : 0xffffffffu);
+        const uint32_t peers = __match_any_sync(0xffffffffu, valid ? bin4 : 0xffffffffu);
         const int leader = __ffs(peers) - 1;
         const int lane = threadIdx.x & 31;
         uint32_t base = 0;
-        if (lane == leader && valid) base = atomicAdd(&hist[bin], (uint32_t)__popc(peers));
+        if (lane == leader && valid) base = atomicAdd(&at_bytes(hist, bin4), (uint32_t)__popc(peers));
         base = __shfl_sync(0xffffffffu, base, leader);
         return base + (uint32_t)__popc(peers & ((1u << lane) - 1u));
     } else {
-        return valid ? atomicAdd(&hist[bin], 1u) : 0u;
+        return valid ? atomicAdd(&at_bytes(hist, bin4), 1u) : 0u;
     }
 }
 
-// Exclusive scan of hist[0..nbins) into loff, and one global claim per
-// non-empty bin: gbase[b] = atomicAdd(&cnt[bin_base + b], hist[b]).
-template <int NT>
-__device__ __forceinline__ void scan_and_claim(uint32_t *hist, uint32_t *loff, uint32_t *gbase,
-                                               uint32_t *ws, int nbins, uint32_t *cnt,
-                                               uint32_t bin_base)
+// Exclusive scan of the bin counts start2[0..nbins) in place, and one global
+// claim per non-empty bin; place[b] = b * cap + claim - start, so record i of
+// the bin-ordered tile goes to slot index place[bin] + i (32 bits, wrapping).
+// *total gets the records of the tile; true if a claim passes its slot's end.
+template <int NT, class S>
+__device__ __forceinline__ bool scan_and_claim(S &t, int nbins, uint32_t *cnt, uint32_t cap, uint32_t *total)
 {
-    const int per = (nbins + NT - 1) / NT;  // <= 4 for 1024 bins and 256 threads
+    constexpr int PB = ((1 << kMaxCoarseBits) + NT - 1) / NT;  // most bins a thread owns
+    const int per = (nbins + NT - 1) / NT;
     const int b0 = threadIdx.x * per;
-    uint32_t local = 0;
-    for (int k = 0; k < per; ++k)
-        if (b0 + k < nbins) local += hist[b0 + k];
-    uint32_t total;
-    uint32_t run = block_exclusive_scan_u32<NT>(local, ws, &total);
-    for (int k = 0; k < per; ++k) {
-        const int b = b0 + k;
-        if (b < nbins) {
-            const uint32_t h = hist[b];
-            loff[b] = run;
-            run += h;
-            gbase[b] = h ? atomicAdd(&cnt[bin_base + b], h) : 0u;
+    uint32_t h[PB], local = 0;
+#pragma unroll
+    for (int k = 0; k < PB; ++k) {
+        h[k] = k < per && b0 + k < nbins ? t.start2[b0 + k] : 0u;
+        local += h[k];
+    }
+    uint32_t run = block_exclusive_scan_u32<NT>(local, t.ws, total);
+    bool over = false;
+#pragma unroll
+    for (int k = 0; k < PB; ++k) {
+        if (k < per && b0 + k < nbins) {
+            const uint32_t b = b0 + k;
+            const uint32_t c = h[k] ? atomicAdd(&cnt[b], h[k]) : 0u;
+            over = over || (h[k] && (c > cap || h[k] > cap - c));
+            t.start2[b] = 2u * run;
+            t.place[b] = b * cap + c - run;
+            run += h[k];
         }
     }
+    return over;
 }
 
 // Windowed plots keep the keys whose top wbits equal win and bin them by the
@@ -133,17 +150,27 @@ template <bool WIN>
 __device__ __forceinline__ uint32_t key_bin(const Desc &d, uint64_t key, int bits)
 {
     const uint32_t hi = (uint32_t)(key >> 32);
-    return bits ? (WIN ? hi << d.wbits : hi) >> (32 - bits) : 0u;
+    // clamped funnel shift: bits 0 gives bin 0
+    return __funnelshift_rc(WIN ? hi << d.wbits : hi, 0u, 32 - bits);
 }
 
+// One CTA: a tile of NT * NPT nonces.  The hash is bound by the ALU pipe
+// (417 of its ~620 instructions are xors and rotations, which only that
+// half-rate pipe runs), so everything around it is laid out to spend few ALU
+// instructions: a rolled loop of two hashes per step (see b3_finish) that
+// leaves each record's key, bin and rank in shared memory; the tile's order
+// by bin as 16-bit record indices instead of moved records; slot places as
+// 32-bit indices whose addresses are multiply-adds on the FMA pipe.  The
+// extra shared-memory traffic is free: that path idles at 17% here.
 template <int NT, int NPT, bool AGG, bool HALO, int WM>
-__global__ void __launch_bounds__(NT) k_hash_scatter(const Desc *__restrict__ descs, int nplots,
+__global__ void __launch_bounds__(NT, NPT <= 12 ? 4 : 3) k_hash_scatter(const Desc *__restrict__ descs, int nplots,
                                                      const uint32_t *__restrict__ tile_start,
                                                      int chunk)
 {
-    using S = HashSmem<NT, NPT>;
-    constexpr int T = S::T;
+    using S = HashTile<NT, NPT>;
+    constexpr uint32_t T = S::T;
     constexpr bool WIN = WM != kWinNone;
+    static_assert(NPT % 2 == 0 && 2 * T <= 0x10000u && (4u << kMaxCoarseBits) < kNoBin, "16-bit offsets");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S &sm = *reinterpret_cast<S *>(smem_raw);
 
@@ -154,6 +181,7 @@ __global__ void __launch_bounds__(NT) k_hash_scatter(const Desc *__restrict__ de
     if (WM == kWinList) N = min(*d.wcount, d.listcap);
     const uint64_t base = lo + (uint64_t)(blockIdx.x - tile_start[plot]) * T;
     if (WM == kWinList && base >= N) return;  // the grid covers the list's capacity
+    const uint32_t left = (uint32_t)(N - base < T ? N - base : T);  // nonces of the tile
     const bool two_level = d.p2 > 0;
     const int bits = two_level ? d.p1 : d.p;
     const int nbins = 1 << bits;
@@ -163,96 +191,86 @@ __global__ void __launch_bounds__(NT) k_hash_scatter(const Desc *__restrict__ de
     uint64_t *__restrict__ okeys = two_level ? d.a_keys + slot0 * cap : d.b_keys;
     uint32_t *__restrict__ ononces = two_level ? d.a_nonces + slot0 * cap : d.b_nonces;
     uint32_t *cnt = two_level ? d.cnt1 + slot0 : d.cnt2;
+    const uint32_t *__restrict__ list = WM == kWinList ? d.wlist + base : nullptr;
+    const uint32_t nonce0 = (uint32_t)base;
 
-    uint32_t pre[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) pre[i] = d.pre1[i];
-
-    for (int b = threadIdx.x; b < nbins; b += NT) sm.hist[b] = 0u;
+    for (int b = threadIdx.x; b < nbins; b += NT) sm.start2[b] = 0u;
     __syncthreads();
-
-    uint64_t key[NPT];
-    uint32_t rank[NPT];
+    {
+        uint32_t pre[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) pre[i] = d.pre1[i];
+#pragma unroll 1
+        for (uint32_t i0 = threadIdx.x; i0 < T; i0 += 2 * NT) {
+            uint64_t key[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const uint32_t i = i0 + u * NT;
+                const uint32_t nonce = WM == kWinList ? (i < left ? list[i] : 0u) : nonce0 + i;
+                uint32_t h0, h1;
+                b3_finish<false>(pre, nonce, 0u, h0, h1);
+                key[u] = key64_of(h0, h1);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const uint32_t i = i0 + u * NT;
+                const bool valid = i < left && (WM != kWinFilter || in_window<true>(d, key[u]));
+                const uint32_t bin4 = 4u * key_bin<WIN>(d, key[u], bits);
+                sm.keys[i] = key[u];
+                sm.rank2[i] = (uint16_t)(2u * bin_rank<AGG>(sm.start2, bin4, valid));
+                sm.bin4[i] = (uint16_t)(WM != kWinFilter || valid ? bin4 : kNoBin);
+            }
+        }
+    }
+    __syncthreads();
     uint32_t count;  // records the tile keeps
-    if constexpr (!WIN) {
-#pragma unroll
-        for (int j = 0; j < NPT; ++j) {
-            const uint64_t nonce = base + (uint64_t)j * NT + threadIdx.x;
-            const bool valid = nonce < N;
-            uint32_t h0, h1;
-            b3_finish<false>(pre, (uint32_t)nonce, 0u, h0, h1);
-            key[j] = key64_of(h0, h1);
-            const uint32_t bin = bits ? (uint32_t)(key[j] >> (64 - bits)) : 0u;
-            rank[j] = bin_rank<AGG>(sm.hist, bin, valid);
+    const bool over = scan_and_claim<NT>(sm, nbins, cnt, cap, &count);
+    // Every place fits 32 bits unless all slots together hold 2^32 records
+    // or more (K = 32 in two levels).
+    const bool slow = __syncthreads_or(over) || ((uint64_t)cap << bits) > 0xFFFFFFFFull;
+#pragma unroll 4
+    for (uint32_t i = threadIdx.x; i < left; i += NT) {
+        const uint32_t bin4 = sm.bin4[i];
+        if (WM != kWinFilter || bin4 != kNoBin)
+            at_bytes(sm.order, at_bytes(sm.start2, bin4) + sm.rank2[i]) = (uint16_t)i;
+    }
+    __syncthreads();
+    if (!slow && (!HALO || two_level)) {
+#pragma unroll 4
+        for (uint32_t q = threadIdx.x; q < count; q += NT) {
+            const uint32_t i = sm.order[q];
+            const uint32_t at = at_bytes(sm.place, sm.bin4[i]) + q;
+            okeys[at] = sm.keys[i];
+            ononces[at] = WM == kWinList ? list[i] : nonce0 + i;
         }
-        __syncthreads();
-        scan_and_claim<NT>(sm.hist, sm.loff, sm.gbase, sm.ws, nbins, cnt, 0u);
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < NPT; ++j) {
-            const uint64_t nonce = base + (uint64_t)j * NT + threadIdx.x;
-            if (nonce < N) {
-                const uint32_t bin = bits ? (uint32_t)(key[j] >> (64 - bits)) : 0u;
-                const uint32_t pos = sm.loff[bin] + rank[j];
-                sm.keys[pos] = key[j];
-                sm.nonces[pos] = (uint32_t)nonce;
-            }
-        }
-        __syncthreads();
-        count = (uint32_t)((N - base) < (uint64_t)T ? (N - base) : (uint64_t)T);
-    } else {
-        uint32_t keep = 0;  // bit j: record j's nonce exists and its key is in the window
-#pragma unroll
-        for (int j = 0; j < NPT; ++j) {
-            const uint64_t idx = base + (uint64_t)j * NT + threadIdx.x;
-            uint32_t nonce;
-            if constexpr (WM == kWinList) nonce = idx < N ? d.wlist[idx] : 0u;
-            else nonce = (uint32_t)idx;
-            uint32_t h0, h1;
-            b3_finish<false>(pre, nonce, 0u, h0, h1);
-            key[j] = key64_of(h0, h1);
-            const bool valid = idx < N && (WM != kWinFilter || in_window<true>(d, key[j]));
-            keep |= (valid ? 1u : 0u) << j;
-            rank[j] = bin_rank<AGG>(sm.hist, key_bin<true>(d, key[j], bits), valid);
-        }
-        __syncthreads();
-        scan_and_claim<NT>(sm.hist, sm.loff, sm.gbase, sm.ws, nbins, cnt, 0u);
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < NPT; ++j) {
-            if (keep >> j & 1u) {
-                const uint64_t idx = base + (uint64_t)j * NT + threadIdx.x;
-                const uint32_t pos = sm.loff[key_bin<true>(d, key[j], bits)] + rank[j];
-                sm.keys[pos] = key[j];
-                sm.nonces[pos] = WM == kWinList ? d.wlist[idx] : (uint32_t)idx;
-            }
-        }
-        __syncthreads();
-        count = sm.loff[nbins - 1] + sm.hist[nbins - 1];  // the histogram's total
+        return;
     }
     bool overflow = false, hover = false;
-    for (uint32_t i = threadIdx.x; i < count; i += NT) {
+    for (uint32_t q = threadIdx.x; q < count; q += NT) {
+        const uint32_t i = sm.order[q];
         const uint64_t k = sm.keys[i];
-        const uint32_t bin = WIN ? key_bin<true>(d, k, bits) : (bits ? (uint32_t)(k >> (64 - bits)) : 0u);
-        const uint32_t g = sm.gbase[bin] + (i - sm.loff[bin]);
+        const uint32_t bin = sm.bin4[i] >> 2;
+        const uint32_t nonce = WM == kWinList ? list[i] : nonce0 + i;
+        const uint32_t g = sm.place[bin] + q - bin * cap;
         if (g < cap) {
             const uint64_t at = (uint64_t)bin * cap + g;
             okeys[at] = k;
-            ononces[at] = sm.nonces[i];
+            ononces[at] = nonce;
         } else {
             overflow = true;
         }
-        if (HALO && !two_level) halo_add(d, bin, k, sm.nonces[i], hover);  // final partitions
+        if (HALO && !two_level) halo_add(d, bin, k, nonce, hover);  // final partitions
     }
     if (overflow) atomicOr(d.status, two_level ? kStSlot1Overflow : kStSlot2Overflow);
     if (hover) atomicOr(d.status, kStHaloOverflow);
 }
 
-template <int NT, int NPT, bool AGG, bool HALO, int WM>
+template <int NPT, bool AGG, bool HALO, int WM>
 static cudaError_t launch_hs(const Desc *descs, int nplots, const uint32_t *tile_start,
                              uint32_t total_tiles, int chunk, cudaStream_t s)
 {
-    const size_t smem = sizeof(HashSmem<NT, NPT>);
+    constexpr int NT = kHashThreads;
+    const size_t smem = sizeof(HashTile<NT, NPT>);
     auto fn = k_hash_scatter<NT, NPT, AGG, HALO, WM>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -265,28 +283,30 @@ static cudaError_t launch_hs(const Desc *descs, int nplots, const uint32_t *tile
 // HALO instances carry the cross-bucket halo code and window instances the
 // window filter or the nonce list; plain launches carry neither.  A list
 // launch holds one windowed plot (never cross-bucket).
-// Whole plots may take 4 or 16 nonces per thread instead of 8 (a tuning
-// choice: more nonces per thread, more independent hashes in flight per
-// thread but fewer resident CTAs); windows always take 8.
-template <bool HALO, int WM, int P>
+template <bool HALO, int WM, int NPT>
 static cudaError_t launch_hs_npt(const Desc *descs, int nplots, const uint32_t *tile_start,
                                  uint32_t total_tiles, bool agg, int chunk, cudaStream_t s)
 {
-    constexpr int T = kHashThreads;
-    return agg ? launch_hs<T, P, true, HALO, WM>(descs, nplots, tile_start, total_tiles, chunk, s)
-               : launch_hs<T, P, false, HALO, WM>(descs, nplots, tile_start, total_tiles, chunk, s);
+    return agg ? launch_hs<NPT, true, HALO, WM>(descs, nplots, tile_start, total_tiles, chunk, s)
+               : launch_hs<NPT, false, HALO, WM>(descs, nplots, tile_start, total_tiles, chunk, s);
 }
 
 template <bool HALO, int WM>
 static cudaError_t launch_hs_agg(const Desc *descs, int nplots, const uint32_t *tile_start,
                                  uint32_t total_tiles, bool agg, int chunk, cudaStream_t s, int npt)
 {
-    if (WM == kWinNone && npt == 4)
-        return launch_hs_npt<HALO, kWinNone, 4>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
-    if (WM == kWinNone && npt == 16)
-        return launch_hs_npt<HALO, kWinNone, 16>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
-    if (npt != kHashNoncesPerThread) return cudaErrorInvalidValue;
-    return launch_hs_npt<HALO, WM, kHashNoncesPerThread>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
+    if (WM != kWinNone)
+        return npt == kHashNoncesPerThread
+                   ? launch_hs_npt<HALO, WM, kHashNoncesPerThread>(descs, nplots, tile_start, total_tiles, agg, chunk, s)
+                   : cudaErrorInvalidValue;
+    switch (npt) {
+    case 2: return launch_hs_npt<HALO, kWinNone, 2>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
+    case 4: return launch_hs_npt<HALO, kWinNone, 4>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
+    case 8: return launch_hs_npt<HALO, kWinNone, 8>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
+    case 12: return launch_hs_npt<HALO, kWinNone, 12>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
+    case 16: return launch_hs_npt<HALO, kWinNone, 16>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_hash_scatter(const Desc *descs, int nplots, const uint32_t *tile_start,
@@ -429,15 +449,21 @@ __global__ void __launch_bounds__(kT2HashThreads) k_t2_hash(const Desc *__restri
 #pragma unroll
     for (int i = 0; i < 16; ++i) g[i] = d.pre2[i];
     uint4 *__restrict__ t2 = reinterpret_cast<uint4 *>(d.t2);
-    // One record per iteration, loop kept rolled: the body is one
-    // compression, small enough for the instruction cache even when the
-    // warps (no barrier here) drift apart; unrolling several compressions
-    // made the warps stall on instruction fetch.
+    // Two records per step, loop kept rolled (see b3_finish).
+    const uint64_t stride = (uint64_t)ctas * NT;
 #pragma unroll 1
-    for (uint64_t q = lo + (uint64_t)me * NT + threadIdx.x; q < hi; q += (uint64_t)ctas * NT) {
+    for (uint64_t q = lo + (uint64_t)me * NT + threadIdx.x; q < hi; q += 2 * stride) {
         const uint4 v = t2[q];
         uint32_t h0, h1;
-        b3_finish<true>(g, v.x, v.y, h0, h1);
+        if (q + stride < hi) {
+            const uint4 u = t2[q + stride];
+            uint32_t h2, h3;
+            b3_finish<true>(g, v.x, v.y, h0, h1);
+            b3_finish<true>(g, u.x, u.y, h2, h3);
+            t2[q + stride] = make_uint4(u.x, u.y, h2, h3);
+        } else {
+            b3_finish<true>(g, v.x, v.y, h0, h1);
+        }
         t2[q] = make_uint4(v.x, v.y, h0, h1);
     }
 }
@@ -451,61 +477,65 @@ cudaError_t launch_t2_hash(const Desc *descs, int nplots, const uint32_t *tile_s
 }
 
 // Pair hash of the slot placement (Sec. III-A, Table 2): CTA b takes
-// partitions [8b, 8b + 8) of one plot, whose pairs the sort left in the
-// partitions' level-2 slots (pair k of partition f: key array of slot f
-// for k < cap2, nonce array for k >= cap2) and whose Table-2 offsets the
-// pair-count scan wrote; the CTA walks the group's pairs as one run, so
-// every warp reads consecutive pairs and writes consecutive records.
+// partitions [8b, 8b + 8) of one plot, a warp each, whose pairs the sort
+// left in the partitions' level-2 slots (pair k of partition f: key array of
+// slot f for k < cap2, nonce array for k >= cap2) and whose Table-2 offsets
+// the pair-count scan wrote.  Bound by the ALU pipe, so a pair costs little
+// but its hash: a warp reads consecutive pairs and writes consecutive
+// records at 32-bit indices, with no search for the pair's partition and no
+// barrier; two hashes per step (see b3_finish).
 __global__ void __launch_bounds__(kT2HashThreads) k_t2_hash_slots(const Desc *__restrict__ descs,
                                                                   int nplots,
                                                                   const uint32_t *__restrict__ tile_start)
 {
-    constexpr int NT = kT2HashThreads;
-    constexpr uint32_t G = kT2SlotGroup;
-    static_assert(G == 8, "the search below is written for groups of 8");
-    __shared__ uint32_t s_rel[G + 1];  // pair offsets relative to the group's first
-    __shared__ uint64_t s_base;
+    static_assert(kT2SlotGroup == kT2HashThreads / 32, "one partition per warp");
     const int plot = find_plot(tile_start, nplots, blockIdx.x);
     const Desc &d = descs[plot];
     if (*d.status & (kStT2Capacity | kStTimeout | kStBadTicket | kStPairSlot)) return;
     const uint64_t np = 1ull << d.p;
-    const uint64_t fa = (uint64_t)(blockIdx.x - tile_start[plot]) * G;
-    if (fa >= np) return;
+    const uint64_t f = (uint64_t)(blockIdx.x - tile_start[plot]) * kT2SlotGroup + (threadIdx.x >> 5);
+    if (f >= np) return;
     // The offsets exist only if the scan's chain reached its last chunk
     // (a broken chain has set a status bit, except for a withheld chunk 0
     // in a one-chunk scan).
     const uint64_t nchunks = (np + kScanChunk - 1) / kScanChunk;
     if ((ld_acquire_u64(d.lb + (nchunks - 1)) & ~kLbMask) != kLbIncl) return;
-    const uint32_t ng = (uint32_t)(np - fa < G ? np - fa : G);
-    if (threadIdx.x == 0) s_base = d.t2off[fa];
-    __syncthreads();
-    if (threadIdx.x <= G) {
-        // partitions past the plot's last read as "never reached"
-        s_rel[threadIdx.x] = threadIdx.x <= ng ? (uint32_t)(d.t2off[fa + threadIdx.x] - s_base)
-                                               : 0xFFFFFFFFu;
-    }
-    __syncthreads();
-    const uint32_t total = s_rel[ng];
+    const uint64_t off = d.t2off[f];
     const uint32_t cap = d.cap2;
-    if (s_base + total > d.t2cap) return;  // the scan flags this; never write past Table 2
+    // never past the pair slot (the sort flags this)
+    const uint32_t P = min((uint32_t)(d.t2off[f + 1] - off), cap + cap / 2u);
+    if (off + P > d.t2cap) return;  // the scan flags this; never write past Table 2
     uint32_t g[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) g[i] = d.pre2[i];
-    uint4 *__restrict__ t2 = reinterpret_cast<uint4 *>(d.t2) + s_base;
+    uint4 *__restrict__ t2 = reinterpret_cast<uint4 *>(d.t2) + off;
+    const uint2 *__restrict__ ab = reinterpret_cast<const uint2 *>(d.b_keys + f * cap);
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t seg = 0; seg < P; seg += cap) {  // key array, then nonce array
+        const uint32_t n = min(P - seg, cap);
+        // the next step's pairs are read before this step's hashes
+        uint2 x = lane < n ? ab[lane] : make_uint2(0u, 0u);
+        uint2 y = lane + 32 < n ? ab[lane + 32] : make_uint2(0u, 0u);
 #pragma unroll 1
-    for (uint32_t q = threadIdx.x; q < total; q += NT) {  // one compression per iteration
-        // partition of pair q: the last t with s_rel[t] <= q
-        uint32_t t = s_rel[4] <= q ? 4u : 0u;
-        t += s_rel[t + 2] <= q ? 2u : 0u;
-        t += s_rel[t + 1] <= q ? 1u : 0u;
-        const uint32_t k = q - s_rel[t];
-        const uint64_t f = fa + t;
-        if (k >= cap + cap / 2u) break;  // past the pair slot (the sort flags this)
-        const uint2 ab = k < cap ? reinterpret_cast<const uint2 *>(d.b_keys + f * cap)[k]
-                                 : reinterpret_cast<const uint2 *>(d.b_nonces + f * cap)[k - cap];
-        uint32_t h0, h1;
-        b3_finish<true>(g, ab.x, ab.y, h0, h1);
-        t2[q] = make_uint4(ab.x, ab.y, h0, h1);
+        for (uint32_t k0 = 0; k0 < n; k0 += 64) {
+            const uint32_t k = k0 + lane;
+            const uint2 nx = k + 64 < n ? ab[k + 64] : make_uint2(0u, 0u);
+            const uint2 ny = k + 96 < n ? ab[k + 96] : make_uint2(0u, 0u);
+            uint32_t h0, h1;
+            if (k0 + 32 < n) {  // the same for the whole warp
+                uint32_t h2, h3;
+                b3_finish<true>(g, x.x, x.y, h0, h1);
+                b3_finish<true>(g, y.x, y.y, h2, h3);
+                if (k + 32 < n) t2[k + 32] = make_uint4(y.x, y.y, h2, h3);
+            } else {
+                b3_finish<true>(g, x.x, x.y, h0, h1);
+            }
+            if (k < n) t2[k] = make_uint4(x.x, x.y, h0, h1);
+            x = nx;
+            y = ny;
+        }
+        t2 += cap;
+        ab = reinterpret_cast<const uint2 *>(d.b_nonces + f * cap);
     }
 }
 
@@ -532,7 +562,7 @@ __global__ void __launch_bounds__(256) k_window_ids(uint32_t k0, uint32_t k1, ui
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += stride) {
         uint32_t packed = 0;
-#pragma unroll
+#pragma unroll 2
         for (int j = 0; j < 4; ++j) {
             const uint64_t nonce = 4 * i + j;
             uint32_t h0, h1;
@@ -635,31 +665,27 @@ cudaError_t launch_hash_records(const uint32_t key[8], uint64_t nonce0, uint64_t
 }
 
 // Hash-only ceiling of the Table-1 hash: keyed BLAKE3 of nonces nonce0 ..
-// nonce0 + count - 1 in the Table-1 kernel's shape (256 threads, 8 nonces
-// per thread and step, key state from the per-key setup), with no record
-// stores: each thread folds its hash words into one word, stored once.  It
-// measures how fast the integer pipes run this instruction mix with no
-// memory work beside it.  Grid-stride over tiles of 2048 nonces.
+// nonce0 + count - 1 in the Table-1 kernel's shape (256 threads, a rolled
+// loop of two nonces per thread and step, key state from the per-key setup),
+// with no record stores: each thread folds its hash words into one word,
+// stored once.  It measures how fast the integer pipes run this instruction
+// mix with no memory work beside it.  Grid-stride over pairs of nonces.
 __global__ void __launch_bounds__(256) k_hash_peak(uint32_t k0, uint32_t k1, uint32_t k2,
                                                    uint32_t k3, uint32_t k4, uint32_t k5,
                                                    uint32_t k6, uint32_t k7, uint64_t nonce0,
                                                    uint64_t count, uint32_t *__restrict__ fold)
 {
-    constexpr int NPT = kHashNoncesPerThread;
-    constexpr uint64_t T = (uint64_t)kHashThreads * NPT;
     const uint32_t key[8] = {k0, k1, k2, k3, k4, k5, k6, k7};
     uint32_t pre[16];
     b3_key_setup(key, 4u, pre);
     uint32_t acc = 0;
-    const uint64_t tiles = (count + T - 1) / T;
-    for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-#pragma unroll
-        for (int j = 0; j < NPT; ++j) {
-            const uint64_t i = t * T + (uint64_t)j * kHashThreads + threadIdx.x;
-            uint32_t h0, h1;
-            b3_finish<false>(pre, (uint32_t)(nonce0 + i), 0u, h0, h1);
-            acc ^= i < count ? (h0 ^ h1) : 0u;
-        }
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+#pragma unroll 1
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += 2 * stride) {
+        uint32_t h0, h1, g0, g1;
+        b3_finish<false>(pre, (uint32_t)(nonce0 + i), 0u, h0, h1);
+        b3_finish<false>(pre, (uint32_t)(nonce0 + i + stride), 0u, g0, g1);
+        acc ^= h0 ^ h1 ^ (i + stride < count ? g0 ^ g1 : 0u);
     }
     fold[(uint64_t)blockIdx.x * blockDim.x + threadIdx.x] = acc;
 }

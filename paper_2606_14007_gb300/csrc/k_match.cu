@@ -162,11 +162,21 @@ __global__ void __launch_bounds__(kMatchThreads) k_match(const Desc *__restrict_
             }
         }
         __syncthreads();
-        for (uint32_t q = threadIdx.x; q < w1 - w0; q += NT) {
+#pragma unroll 1
+        for (uint32_t q = threadIdx.x; q < w1 - w0; q += 2 * NT) {  // two hashes per step (see b3_finish)
             const uint32_t e = list[q];
             const uint32_t a = nonces[e & 0xffffu], b = nonces[e >> 16];
             uint32_t h0, h1;
-            b3_finish<true>(g, a, b, h0, h1);
+            if (q + NT < w1 - w0) {
+                const uint32_t e2 = list[q + NT];
+                const uint32_t a2 = nonces[e2 & 0xffffu], b2 = nonces[e2 >> 16];
+                uint32_t h2, h3;
+                b3_finish<true>(g, a, b, h0, h1);
+                b3_finish<true>(g, a2, b2, h2, h3);
+                out[w0 + q + NT] = make_uint4(a2, b2, h2, h3);
+            } else {
+                b3_finish<true>(g, a, b, h0, h1);
+            }
             out[w0 + q] = make_uint4(a, b, h0, h1);
         }
         __syncthreads();

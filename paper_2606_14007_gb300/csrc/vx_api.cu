@@ -200,13 +200,16 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
     L->max_p2 = 0;
     int min_bits = 64;
     // One staged hash launch takes one shape: the plots' common nonces per
-    // thread, else the default (any shape gives the same records).
+    // thread, else the automatic one of their nonces together (any shape
+    // gives the same records).
     int npt = n > 0 && plots[0] ? plots[0]->plan.npt : kPlanNoncesPerThread;
-    for (int i = 0; i < n; ++i)
-        if (plots[i] && plots[i]->plan.npt != npt) npt = kPlanNoncesPerThread;
+    bool same_npt = true;
+    uint64_t nonces = 0;
     for (int i = 0; i < n; ++i) {
         if (!plots[i] || !plots[i]->d_t1) return VX_EINVAL;
         const Plan &pl = plots[i]->plan;
+        same_npt = same_npt && pl.npt == npt;
+        nonces += pl.N;
         fuse = fuse && pl.fuse_pair_hash;
         slots = slots && pl.pair_slots;
         halo = halo || pl.scope != 0;
@@ -223,6 +226,7 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
         L->max_p2 = std::max(L->max_p2, pl.p2);
         if (pl.mode == kScatterStaged) min_bits = std::min(min_bits, pl.p2 > 0 ? pl.p1 : pl.p);
     }
+    if (!same_npt) npt = win ? kPlanNoncesPerThread : vx::auto_nonces_per_thread(nonces);
     uint64_t acc[vx::kTileArrays] = {};
     for (int a = 0; a < vx::kTileArrays; ++a) h[a * W] = 0;
     for (int i = 0; i < n; ++i) {

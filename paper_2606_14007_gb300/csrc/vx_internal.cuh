@@ -87,8 +87,8 @@ struct Desc {
     uint8_t *t1;         // Table 1, 12-byte records
     uint8_t *t2;         // Table 2, 16-byte records
     uint32_t key[8];     // plot key, LE words
-    uint32_t pre1[16];   // Table-1 hash state after round-1 columns 1..3
-    uint32_t pre2[16];   // pair-hash state after round-1 columns 1..3
+    uint32_t pre1[16];   // Table-1 hash state of the key (b3_key_setup)
+    uint32_t pre2[16];   // pair-hash state of the key
 };
 
 // Table 2 sorted by hash2 (vx_sort_table2): one plot's second sorting pass
@@ -171,45 +171,77 @@ __device__ __forceinline__ uint32_t bswap32(uint32_t x) { return __byte_perm(x, 
     } while (0)
 
 // Per-key state of a one-block keyed hash whose message occupies words 0..1
-// only: v = {key, IV0..3, counter 0, 0, block_len, flags}, with the three
-// round-1 column G's that see only zero message words already applied.
+// only, from v = {key, IV0..3, counter 0, 0, block_len, flags}: the three
+// round-1 column G's that see only zero message words are applied, and with
+// them the first steps of later G's that see only per-key words.  pre[i] is
+// state word v_i except
+//   pre[0] = key0 + key4          (column 0's first sum, before m0)
+//   pre[1] = v1 + v6, pre[2] = v2 + v7   (diagonals 1 and 2's first sums)
+//   pre[13] = ror16(v13 ^ pre[2]) (diagonal 2's first rotation)
+// and pre[8], pre[12] are unused (IV0 and 0 in column 0, known constants).
+// Every hash saves 2 xors, 1 rotation and 3 sums of the ALU-bound hash this
+// way; loaded from memory as plain state words they cannot fold.
 __device__ __forceinline__ void b3_key_setup(const uint32_t key[8], uint32_t block_len,
                                              uint32_t pre[16])
 {
-    uint32_t v0 = key[0], v1 = key[1], v2 = key[2], v3 = key[3];
-    uint32_t v4 = key[4], v5 = key[5], v6 = key[6], v7 = key[7];
-    uint32_t v8 = kIV0, v9 = kIV1, v10 = kIV2, v11 = kIV3;
-    uint32_t v12 = 0, v13 = 0, v14 = block_len, v15 = kFlagsKeyedRootChunk;
+    uint32_t v1 = key[1], v2 = key[2], v3 = key[3];
+    uint32_t v5 = key[5], v6 = key[6], v7 = key[7];
+    uint32_t v9 = kIV1, v10 = kIV2, v11 = kIV3;
+    uint32_t v13 = 0, v14 = block_len, v15 = kFlagsKeyedRootChunk;
     VX_G(v1, v5, v9, v13, 0u, 0u);
     VX_G(v2, v6, v10, v14, 0u, 0u);
     VX_G(v3, v7, v11, v15, 0u, 0u);
-    pre[0] = v0; pre[1] = v1; pre[2] = v2; pre[3] = v3;
-    pre[4] = v4; pre[5] = v5; pre[6] = v6; pre[7] = v7;
-    pre[8] = v8; pre[9] = v9; pre[10] = v10; pre[11] = v11;
-    pre[12] = v12; pre[13] = v13; pre[14] = v14; pre[15] = v15;
+    pre[0] = key[0] + key[4];
+    pre[1] = v1 + v6; pre[2] = v2 + v7; pre[3] = v3;
+    pre[4] = key[4]; pre[5] = v5; pre[6] = v6; pre[7] = v7;
+    pre[8] = 0u; pre[9] = v9; pre[10] = v10; pre[11] = v11;
+    pre[12] = 0u; pre[13] = ror16(v13 ^ pre[2]); pre[14] = v14; pre[15] = v15;
 }
 
 // The rest of the compression for message words (m0, m1, 0, ..., 0):
 // round-1 column 0 and diagonals, rounds 2..7, and output words 0 and 1
 // (hash bytes 0..7).  TWO_WORDS = false fixes m1 = 0 (4-byte messages).
+// Bound by the ALU pipe (xors and rotations; the sums go to the FMA pipe):
+// callers run it two to an iteration of a rolled loop (2 x ~620
+// instructions stay in the instruction cache), which keeps that pipe 99%
+// busy; eight unrolled reach 88%, one 97%.
 template <bool TWO_WORDS>
 __device__ __forceinline__ void b3_finish(const uint32_t pre[16], uint32_t m0, uint32_t m1,
                                           uint32_t &h0, uint32_t &h1)
 {
-    uint32_t v0 = pre[0], v1 = pre[1], v2 = pre[2], v3 = pre[3];
+    uint32_t v1 = pre[1], v2 = pre[2], v3 = pre[3];
     uint32_t v4 = pre[4], v5 = pre[5], v6 = pre[6], v7 = pre[7];
-    uint32_t v8 = pre[8], v9 = pre[9], v10 = pre[10], v11 = pre[11];
-    uint32_t v12 = pre[12], v13 = pre[13], v14 = pre[14], v15 = pre[15];
+    uint32_t v9 = pre[9], v10 = pre[10], v11 = pre[11];
+    uint32_t v13 = pre[13], v14 = pre[14], v15 = pre[15];
     uint32_t m[16];
     m[0] = m0;
     m[1] = TWO_WORDS ? m1 : 0u;
 #pragma unroll
     for (int i = 2; i < 16; ++i) m[i] = 0u;
-    // Round 1 (columns 1..3 are in pre).
-    VX_G(v0, v4, v8, v12, m[0], m[1]);
+    // Round 1, column 0 (columns 1..3 are in pre): v12 = 0, v8 = IV0.
+    uint32_t v0 = pre[0] + m[0];
+    uint32_t v12 = ror16(v0);
+    uint32_t v8 = kIV0 + v12;
+    v4 = ror12(v4 ^ v8);
+    v0 = v0 + v4 + m[1];
+    v12 = ror8(v12 ^ v0);
+    v8 = v8 + v12;
+    v4 = ror7(v4 ^ v8);
+    // Diagonals; 1 and 2 start behind the steps pre already holds.
     VX_G(v0, v5, v10, v15, m[8], m[9]);
-    VX_G(v1, v6, v11, v12, m[10], m[11]);
-    VX_G(v2, v7, v8, v13, m[12], m[13]);
+    v12 = ror16(v12 ^ v1);
+    v11 = v11 + v12;
+    v6 = ror12(v6 ^ v11);
+    v1 = v1 + v6;
+    v12 = ror8(v12 ^ v1);
+    v11 = v11 + v12;
+    v6 = ror7(v6 ^ v11);
+    v8 = v8 + v13;
+    v7 = ror12(v7 ^ v8);
+    v2 = v2 + v7;
+    v13 = ror8(v13 ^ v2);
+    v8 = v8 + v13;
+    v7 = ror7(v7 ^ v8);
     VX_G(v3, v4, v9, v14, m[14], m[15]);
 #pragma unroll
     for (int r = 1; r < 7; ++r) {
@@ -524,7 +556,7 @@ struct HashCfg {
     bool halo;    // some plot of the launch matches across buckets (halo code)
     bool win;     // some plot of the launch is a window (window filter)
     bool list;    // the launch's one plot hashes its window's nonce list
-    int npt;      // nonces per thread of the staged Table-1 hash (4, 8, 16; 8 with a window)
+    int npt;      // nonces per thread of the staged Table-1 hash (2, 4, 8, 12, 16; 8 with a window)
 };
 cudaError_t launch_key_setup(Desc *descs, int nplots, cudaStream_t s);
 // Hash kernels and the second scatter level take one nonce chunk (of

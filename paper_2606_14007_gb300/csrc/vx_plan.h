@@ -29,7 +29,19 @@ constexpr uint64_t kWriteStageBytes = 256ull << 20;  // Sec. III-B: 256 MB pinne
 constexpr uint64_t kWriteChunkBytes = 4ull << 20;    // Sec. III-A: 4 MB sequential chunks
 constexpr uint64_t kPlanHashTile = 2048;   // nonces per hash CTA (threads x nonces/thread)
 constexpr int kPlanHashThreads = 256;      // threads per hash CTA
-constexpr int kPlanNoncesPerThread = 8;    // default nonces per hash thread
+constexpr int kPlanNoncesPerThread = 8;    // nonces per hash thread of windows and the direct bucketing
+
+// Nonces per thread of the staged Table-1 hash over n nonces.  A tile of 256
+// of them threads claims one run per bin, so large tiles claim less (16
+// against 8: 1.519 against 1.559 ms at 2^26 nonces); small plots need more
+// CTAs than large tiles give (2 against 8: 9.2 against 16.4 us at 2^14; at
+// 2^20, 2 pays 51 us in claims against 37 with 8), and between them 12 lets
+// four CTAs share an SM instead of three (398 us at 2^24; 404 with 8, 416
+// with 16).
+inline int auto_nonces_per_thread(uint64_t n)
+{
+    return n < (1ull << 18) ? 2 : n < (1ull << 22) ? 8 : n < (1ull << 25) ? 12 : 16;
+}
 
 // Table-1 hash CTAs over n nonces with npt nonces per thread.
 inline uint32_t hash_tiles(uint64_t n, int npt)
@@ -51,7 +63,7 @@ struct Plan {
     int pk;                                // partition bits in key space: p + wbits
     uint32_t wbits, win;                   // window: top wbits of key64 == win (wbits 0: whole plot)
     int mode;                              // kScatterStaged or kScatterDirect
-    int npt;                               // nonces per thread of the Table-1 hash (4, 8, 16)
+    int npt;                               // nonces per thread of the Table-1 hash (2, 4, 8, 12, 16)
     uint32_t test_flags, spin_limit;
     bool fuse_pair_hash;
     bool pair_slots;                       // pairs staged in the partition slots (t2_placement 2)
@@ -143,15 +155,15 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
             *why = "reserved vx_opts fields must be zero";
             return VX_EINVAL;
         }
-    // The hash kernels run 256 threads per CTA with 8 nonces per thread;
-    // the plain staged Table-1 hash is also compiled for 4 and 16.
+    // The hash kernels run 256 threads per CTA with 8 nonces per thread, the
+    // staged Table-1 hash of a whole plot with 2 to 16.
     if ((opts.hash_block != 0 && opts.hash_block != 256) ||
         (opts.nonces_per_thread != 0 && opts.nonces_per_thread != 4 && opts.nonces_per_thread != 8 &&
          opts.nonces_per_thread != 16)) {
         *why = "hash_block must be 0 or 256 and nonces_per_thread 0, 4, 8 or 16";
         return VX_EINVAL;
     }
-    P.npt = opts.nonces_per_thread ? (int)opts.nonces_per_thread : kPlanNoncesPerThread;
+    P.npt = (int)opts.nonces_per_thread;
     P.fuse_pair_hash = opts.fuse_pair_hash != 0;
     const uint32_t pc = opts.pipeline_chunks;
     if (pc != 0 && pc != 1 && pc != 2 && pc != 4 && pc != 8) {
@@ -189,7 +201,9 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
     // Automatic = staged: on GB300 the per-record slot claims of the direct
     // strategy cost more L2 atomic throughput than the second scatter pass.
     P.mode = opts.scatter_mode == kScatterDirect ? kScatterDirect : kScatterStaged;
-    if (P.npt != kPlanNoncesPerThread && (P.mode != kScatterStaged || P.wbits)) {
+    const bool fixed_npt = P.mode != kScatterStaged || P.wbits;
+    if (P.npt == 0) P.npt = fixed_npt ? kPlanNoncesPerThread : auto_nonces_per_thread(P.N);
+    if (P.npt != kPlanNoncesPerThread && fixed_npt) {
         *why = "nonces_per_thread 4 or 16 needs the staged bucketing and a whole plot (no window)";
         return VX_EINVAL;
     }

@@ -415,3 +415,28 @@ def test_split_and_fused_agree_mid_size(vx):
         p.close()
     for t1, t2 in outs[1:]:
         assert torch.equal(t1, outs[0][0]) and torch.equal(t2, outs[0][1])
+
+
+@pytest.mark.parametrize("npt", [4, 8, 16])
+@pytest.mark.parametrize("K", [1, 9, 13, 16])
+def test_hash_tile_shapes(vx, K, npt):
+    # tiles larger than the plot, ending in it, and several of them (K=13 in
+    # two levels); the automatic shapes 2, 8, 12 and 16 come with K
+    key = plot_key(500 + K)
+    kw = dict(nonces_per_thread=npt) if K != 13 else dict(nonces_per_thread=npt, partition_log2=6, coarse_bits=4)
+    t1, t2, n2, _ = run_plot(vx, K, key, vx.make_opts(**kw))
+    r1, r2 = oracle_plot(K, key)
+    assert np.array_equal(t1, r1)
+    assert n2 == r2.shape[0] and np.array_equal(t2, r2)
+
+
+@pytest.mark.parametrize("sixteenths", [1 / 128, 1 / 4, 1 / 2, 1, 16, 19, 22])
+def test_pair_hash_steps(vx, sixteenths):
+    # pairs per partition about 1, 32, 64, 128, 2048 (a warp's last step half
+    # or less full), about the slot's key array (2608 places) and beyond it
+    K, key = 14, plot_key(520)
+    D = int(orc.default_distance(K) * sixteenths / 16)
+    t1, t2, n2, _ = run_plot(vx, K, key, vx.make_opts(match_scope=1, match_distance=D, t2_placement=2))
+    r1, r2 = oracle_plot_global(K, key, D)
+    assert np.array_equal(t1, r1)
+    assert n2 == r2.shape[0] and np.array_equal(t2, r2)
