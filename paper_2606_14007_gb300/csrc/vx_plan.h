@@ -212,7 +212,12 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
     } else if (opts.coarse_bits >= 0) {
         P.p1 = opts.coarse_bits < P.p ? opts.coarse_bits : P.p;
     } else {
-        P.p1 = P.p <= 10 ? P.p : P.p / 2;
+        // Two levels: the first takes most bits.  It claims inside the
+        // ALU-bound hash, where more bins cost little, and the second then
+        // writes longer runs (K = 30: 9 + 10 bits 25.62 + 8.01 ms, 10 + 9
+        // bits 25.73 + 6.36); below 15 bits a few fewer (K = 25: 9 + 5 bits
+        // 2139 us per plot, 10 + 4 bits 2154, 7 + 7 bits 2142).
+        P.p1 = P.p <= 10 ? P.p : P.p < 14 ? 8 : P.p == 14 ? 9 : 10;
     }
     P.p2 = P.p - P.p1;
     if (P.mode == kScatterStaged && (P.p1 > 10 || P.p2 > 11)) {
