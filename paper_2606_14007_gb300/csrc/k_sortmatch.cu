@@ -6,32 +6,42 @@
 // K=31 bottleneck and proposes a parallel radix sort.  Kept here: the
 // fusion (a partition never leaves shared memory between sort and match).
 // Changed: a physical partition (a run of whole logical buckets, ~2048
-// records) per work item, a counting sort on the key bits below the
-// partition prefix (about one record per digit, half a record with the
-// 16-bit counters of the persistent front end) whose digit runs are then
-// ordered by (key64, nonce).  A partition's pairs either go to its own slot
-// (kSortSlots, the default wherever the plan shows the pair slot safe: no
-// partition waits on another, a scan and the slot pair hash place them) or
-// straight to Table 2 at a base found by a decoupled look-back over the
-// partitions before it (partition order comes from a ticket counter, so
-// every partition an item waits on is held by a running CTA; every wait is
-// bounded and a timeout poisons the chain instead of hanging).  With the
-// cross-bucket match (HALO instances) the next partition's halo is sorted
-// in behind the partition's records.
+// records) per work item, and a sort that places nearly every record by one
+// bitmap rank: the key bits below the partition prefix, 32 digits per
+// expected record, mark a bitmap, and a record's place is the number of
+// marked digits below its own; only the records that share a digit's word
+// with a collision are ordered by (key64, nonce).  A partition's pairs
+// either go to its own slot (kSortSlots, the default wherever the plan shows
+// the pair slot safe: no partition waits on another, a scan and the slot
+// pair hash place them) or straight to Table 2 at a base found by a
+// decoupled look-back over the partitions before it (partition order comes
+// from a ticket counter, so every partition an item waits on is held by a
+// running CTA; every wait is bounded and a timeout poisons the chain instead
+// of hanging).  With the cross-bucket match (HALO instances) the next
+// partition's halo is sorted in behind the partition's records.
 //
-// After the sort every step walks the sorted records in chunks of 32, one
-// record per lane, each warp over its own run of chunks: the pair counts
-// (lanes probe the records after theirs), their warp scans, the Table-1
-// words (coalesced 4-byte stores) and the pair emission.  So no thread
-// walks a data-dependent list alone while its warp waits.
+// The sorted records stand in shared memory as Table-1 words, so Table 1
+// leaves by one bulk copy.  The match walks them in chunks of 32, one record
+// per lane, each warp over its own run of chunks: a lane compares 32 key
+// bits with the records after its own (shuffles), warp scans give the pair
+// offsets, and the pairs go through a 16-bit list in shared memory, so that
+// they are written one per lane, coalesced.
+//
+// Bound by instruction issue (56%) and the shared-memory data path (65%)
+// together at 24 warps per SM: 15.6 k warp instructions per 2048-record
+// partition, against 23 k for the counting sort with ranked digit runs, the
+// per-thread Table-1 stores and the record-wise pair stores before it: 31.0
+// -> 24.1 ms at K=31 (2^31 records; 2.85 of 6.78 TB/s), 0.97 -> 0.75 ms at
+// K=26.  By phase at K=26: load, mark and scan 0.23 ms, placement 0.14,
+// shared digits 0.04, match and lists 0.27, pair stores 0.07.  Tried and
+// dropped: half the digits (0.88 ms), the slot read into registers with four
+// CTAs per SM (0.78), eleven rows of loads in flight instead of four (0.82).
 //
 // Two front ends feed the same steps:
 //  * k_sortmatch_pipe (the default): persistent CTAs, three per SM at the
 //    default slot.  A CTA's next partition slot (keys and nonces, two
-//    contiguous runs) comes into shared memory by cp.async.bulk while the
-//    CTA matches and writes the current one; the sort runs between two
-//    shared buffers, so a digit run is ordered by ranking its records, not
-//    by one thread's insertion sort.
+//    contiguous runs) comes into shared memory by cp.async.bulk once the
+//    current one has been placed.
 //  * k_sortmatch_gl: one CTA per partition reading its slot from global
 //    memory, for slots too large to hold twice in shared memory.
 //
@@ -44,330 +54,332 @@
 // from the latency-bound sort).
 // MODE kSortSlots: Table 1, then the partition's pairs {a, b} in (i, j)
 // order into the partition's own level-2 slot, which the kernel has already
-// read into shared memory: cap2 pairs in the key array, cap2 / 2 in the
-// nonce array.  No partition waits on another; a scan of the pair counts
-// and the slot pair hash place the records.
+// read: cap2 pairs in the key array, cap2 / 2 in the nonce array.  No
+// partition waits on another; a scan of the pair counts and the slot pair
+// hash place the records.
 #include "vx_internal.cuh"
 
 namespace vx {
 
 enum { kSortCount = 0, kSortHash = 1, kSortEmit = 2, kSortSlots = 3 };
-#define SLOTS_MODE(m) ((m) == kSortSlots)
-constexpr uint32_t kSMList = 2048;  // pair-list window (entries), kSortHash only
 constexpr int kPipeThreads = 256;   // persistent front end
 constexpr int kGlThreads = 256;     // one-CTA-per-partition front end
+constexpr uint32_t kDirtyList = 64;  // listed words with a shared digit (2048 records: about 31)
+constexpr int kMaxDigitBits = 18;   // sort digit (bitmap of 2^18 bits, 8192 words)
 // Tickets between a CTA of the global-memory front end and the partition
 // whose slot it prefetches into L2: about half of the CTAs resident at once.
 constexpr uint32_t kSlotPrefetchAhead = 384;
 
+// Words of the digit bitmap of a plan's dbits (log2 of the mean records of a
+// partition): 32 digits per expected record, so that two records share a
+// digit about once in 64 records (2048 records, 2^16 digits: 32 pairs).
+// More digits cost shared memory (three CTAs per SM need 75 KB each), fewer
+// double the shared digits.
+__host__ __device__ __forceinline__ uint32_t bitmap_words(int dbits)
+{
+    const int b = dbits + 5 < kMaxDigitBits ? dbits + 5 : kMaxDigitBits;
+    return 1u << (b - 5);
+}
+
 // Shared layout (bytes from the base), for slots of at most `cap` records
-// (a multiple of 4) and digits of at most `dbits` bits:
-//   buffer X: key64 [cap] | nonce [cap]
-//   buffer Y: key64 [cap] | nonce [cap]     (pipelined front end only)
-//   digit counters [2^dbits], dead once the digit runs are ordered, then
-//   overlaid by the per-record pair count -> pair offset [cap]
-//   pair list [kSMList] (kSortHash) | scan workspace | mbarrier
-// The pipelined front end alternates the two buffers: an item's slot lands
-// in one, is placed by digit into the other, and comes back sorted into the
-// first, so the second is free for the next item's slot while the first
-// holds the sorted partition.
+// (a multiple of 4) and a bitmap of at most `words` words:
+//   X: key64 [cap] | nonce [cap], the slot (pipelined front end only)
+//   Y: the sorted records as Table-1 words {nonce, h0, h1} [cap], starting
+//      up to 12 bytes in, so that shared and Table-1 addresses agree mod 16
+//   bitmap [words] | word prefixes, 16 bits [words]; dead once the records
+//   are sorted, then overlaid by the warps' pair lists (16 bits an entry, at
+//   least 2 * cap entries together)
+//   dirty words [kDirtyList] | scan workspace | mbarrier
 struct SMLayout {
-    size_t xk, xn, yk, yn, dc, list, ws, bar, bytes;
-    __host__ __device__ SMLayout(uint32_t cap, int dbits, bool with_list, bool two)
+    size_t xk, xn, y, bm, dl, ws, bar, bytes;
+    __host__ __device__ SMLayout(uint32_t cap, uint32_t words, bool two)
     {
         cap = (cap + 3u) & ~3u;
         xk = 0;
-        xn = xk + (size_t)cap * 8;
-        yk = xn + (size_t)cap * 4;
-        yn = yk + (two ? (size_t)cap * 8 : 0);
-        dc = yn + (two ? (size_t)cap * 4 : 0);
-        const size_t dcb = ((size_t)1 << dbits) * 4, stb = (size_t)cap * 4;
-        list = dc + (dcb > stb ? dcb : stb);
-        ws = list + (with_list ? (size_t)kSMList * 4 : 0);
-        bar = (ws + 40 * 4 + 7) & ~(size_t)7;
+        xn = xk + (two ? (size_t)cap * 8 : 0);
+        y = xn + (two ? (size_t)cap * 4 : 0);
+        bm = y + (size_t)cap * 12 + 16;
+        dl = bm + tables_bytes(cap, words);
+        ws = dl + (size_t)kDirtyList * 2;
+        bar = ws + 40 * 4;
         bytes = bar + 8;
+    }
+    static __host__ __device__ size_t tables_bytes(uint32_t cap, uint32_t words)
+    {
+        const size_t tab = ((size_t)words * 6 + 15) & ~(size_t)15, lists = (size_t)cap * 4 + 512;
+        return tab > lists ? tab : lists;
     }
 };
 
 struct Part {
-    uint64_t *SK;
-    uint32_t *SN, *DC, *ST, *LS, *WS;
+    uint32_t *Y;   // sorted Table-1 words (record r at Y[3 r])
+    uint32_t *BM;  // digit bitmap
+    uint16_t *PF;  // word prefixes
+    uint16_t *DL;  // dirty words (the first kDirtyList of them)
+    uint16_t *PL;  // pair lists, over BM and PF: NT / 32 of them, plw entries each
+    uint32_t plw;
+    uint32_t *WS;  // scan workspace
 };
+constexpr uint32_t kWsDirty = 36;  // WS word: how many dirty words the scan met
+constexpr uint32_t kWsLong = 37;   // WS word: some warp's pairs do not fit its list
 
 __device__ __forceinline__ bool rec_less(uint64_t ka, uint32_t na, uint64_t kb, uint32_t nb)
 {
     return ka < kb || (ka == kb && na < nb);
 }
 
-// ---------------------------------------------------------------- sorts
-// Both leave the partition's n records sorted by (key64, nonce) in a
-// shared buffer.  DC (2^dbits zeroed counters) is the digit table; both
-// start after a barrier and end with one.
+__device__ __forceinline__ uint64_t y_key(const uint32_t *Y, uint32_t r)
+{
+    return ((uint64_t)bswap32(Y[3 * r + 1]) << 32) | bswap32(Y[3 * r + 2]);
+}
 
-// Inclusive scan of one u32 per lane.
+// The 32 key bits below the partition prefix (pk bits), pk <= 21.
+__device__ __forceinline__ uint32_t sub_key(uint32_t hi, uint32_t lo, int pk)
+{
+    return __funnelshift_rc(lo, hi, 32 - pk);
+}
+
+// ---------------------------------------------------------------- sort
+
+// Inclusive scan of one u32 per lane (a shuffle's own predicate says
+// whether its source lane exists: two instructions a step).
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x)
 {
-    const uint32_t lane = threadIdx.x & 31u;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= (uint32_t)o) x += y;
-    }
+    for (int o = 1; o < 32; o <<= 1)
+        asm volatile(
+            "{ .reg .pred p; .reg .u32 r; shfl.sync.up.b32 r|p, %0, %1, 0, 0xffffffff; @p add.u32 %0, r, %0; }"
+            : "+r"(x)
+            : "r"(o));
     return x;
 }
 
-// Exclusive scan of the M digit counters in place.  When M is 32 * NW * R'
-// with R' <= R (whole rows of 32 counters, the same number per warp), warp w scans its
-// R' rows of 32 counters as R' independent warp scans and adds the row and
-// warp prefixes; otherwise the general block scan.  Ends with a barrier.
-template <int NT, int R>
-__device__ __forceinline__ void counts_to_starts(uint32_t *DC, uint32_t M, uint32_t *WS)
-{
-    constexpr uint32_t NW = NT / 32;
-    if (M < 32u * NW || M > 32u * NW * R || M % (32u * NW) != 0) {
-        block_scan_inplace_u32<NT>(DC, M, WS);
-        return;
-    }
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t rows = M / (32u * NW);
-    uint32_t *row0 = DC + warp * rows * 32u + lane;
-    uint32_t v[R], incl[R];
-#pragma unroll
-    for (int j = 0; j < R; ++j) v[j] = (uint32_t)j < rows ? row0[32 * j] : 0u;
-#pragma unroll
-    for (int j = 0; j < R; ++j) incl[j] = warp_incl_scan(v[j]);
-    uint32_t run = 0;
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-        const uint32_t t = __shfl_sync(0xffffffffu, incl[j], 31);
-        incl[j] += run - v[j];  // exclusive inside the warp's rows
-        run += t;
-    }
-    if (lane == 0) WS[warp] = run;
-    __syncthreads();
-    uint32_t carry = 0;
-#pragma unroll
-    for (uint32_t w = 0; w < NW; ++w) carry += w < warp ? WS[w] : 0u;
-#pragma unroll
-    for (int j = 0; j < R; ++j)
-        if ((uint32_t)j < rows) row0[32 * j] = carry + incl[j];
-    __syncthreads();
-}
+constexpr uint32_t kDirty = 0x8000u;  // flag of PF: the word holds a shared digit
 
-// True when the M counter words fill whole rows of 32 per warp, at most R
-// rows each: the shape in which counts_to_starts needs no general block
-// scan, and the one counts_to_starts_packed requires.
-template <int NT, int R>
-__host__ __device__ __forceinline__ bool rows_shape(uint32_t M)
+// Zeroes the bitmap and the extra counts (PF) of W words; no barrier.
+template <int NT>
+__device__ __forceinline__ void clear_tables(const Part &A, uint32_t W)
 {
-    constexpr uint32_t NW = NT / 32;
-    return M >= 32u * NW && M <= 32u * NW * R && M % (32u * NW) == 0;
-}
-
-// counts_to_starts for 2M digit counters of 16 bits, two to a word (digit
-// 2w in the low half of word w, 2w + 1 in the high half; every count and
-// start below 2^16).  The words must have rows_shape<NT, R>.  Each word's
-// two counts become their run starts: the exclusive prefix P of the
-// word sums, and P plus the low count.  Ends with a barrier.
-template <int NT, int R>
-__device__ __forceinline__ void counts_to_starts_packed(uint32_t *DC, uint32_t M, uint32_t *WS)
-{
-    constexpr uint32_t NW = NT / 32;
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t rows = M / (32u * NW);
-    uint32_t *row0 = DC + warp * rows * 32u + lane;
-    uint32_t lo[R], v[R], incl[R];
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-        const uint32_t w = (uint32_t)j < rows ? row0[32 * j] : 0u;
-        lo[j] = w & 0xFFFFu;
-        v[j] = lo[j] + (w >> 16);
-    }
-#pragma unroll
-    for (int j = 0; j < R; ++j) incl[j] = warp_incl_scan(v[j]);
-    uint32_t run = 0;
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-        const uint32_t t = __shfl_sync(0xffffffffu, incl[j], 31);
-        incl[j] += run - v[j];
-        run += t;
-    }
-    if (lane == 0) WS[warp] = run;
-    __syncthreads();
-    uint32_t carry = 0;
-#pragma unroll
-    for (uint32_t w = 0; w < NW; ++w) carry += w < warp ? WS[w] : 0u;
-#pragma unroll
-    for (int j = 0; j < R; ++j)
-        if ((uint32_t)j < rows) {
-            const uint32_t P = carry + incl[j];
-            row0[32 * j] = P | ((P + lo[j]) << 16);
+    if (threadIdx.x == 0) A.WS[kWsDirty] = A.WS[kWsLong] = 0u;
+    if (W % 8u == 0) {  // 6 W bytes, a multiple of 16 (PF follows BM)
+        uint4 *t = reinterpret_cast<uint4 *>(A.BM);
+        for (uint32_t i = threadIdx.x; i < W * 6u / 16u; i += NT) t[i] = make_uint4(0u, 0u, 0u, 0u);
+    } else {
+        for (uint32_t i = threadIdx.x; i < W; i += NT) {
+            A.BM[i] = 0u;
+            A.PF[i] = 0;
         }
-    __syncthreads();
+    }
 }
 
-// Ping-pong sort of the n records in buffer X (keys XK, nonces XN):
-// digit histogram, scan, then each record placed by digit into buffer Y (a
-// digit's run in arrival order); then every position of Y, 32 per warp
-// step, finds its record's rank inside its run (runs hold about one
-// record; a run of L compares L records) and writes the record to that
-// place of X.  X ends sorted, Y is free.
-//
-// PACK: 16-bit digit counters, two to a word, so that the same counter
-// words hold twice the digits (ndig digits in ndig / 2 words, which must
-// have rows_shape; n < 2^16).  Runs then hold about half a record, and
-// fewer of them need ranking.
-//
-// DRAIN: buffer Y may still be the source of thread 0's bulk stores (the
-// previous item's staged pairs); their reads must end before the records
-// are placed into it, so thread 0 waits for them after the histogram and
-// the scan, which overlap the stores.
-template <int NT, bool PACK, bool DRAIN>
-__device__ __forceinline__ void sort_pingpong(const Part &A, uint64_t *XK, uint32_t *XN, uint64_t *YK,
-                                              uint32_t *YN, uint32_t n, int shift, uint32_t ndig)
+// The sort.  The digit, the bits of key64 below the partition prefix, is wide
+// enough (2^16 for 2048 records) that most records have one of their own:
+// then a record's place is the number of records in lower digits, i.e. the
+// count before its bitmap word plus the word's bits below its own, and the
+// record goes there directly.  Words with a shared digit ("dirty") take
+// their records in arrival order, which order_dirty puts right.  One pass
+// marks the digits (mark), one places the records (place_of); a counting
+// sort's third pass (ranking every record in its digit run) and its second
+// set of shared-memory atomics are gone.
+
+// Marks a digit; one already taken counts as an extra of its word.
+__device__ __forceinline__ void mark(const Part &A, uint32_t dg)
+{
+    const uint32_t w = dg >> 5, bit = 1u << (dg & 31u);
+    if (atomicOr(&A.BM[w], bit) & bit)
+        atomicAdd(reinterpret_cast<uint32_t *>(A.PF) + (w >> 1), 1u << (16u * (w & 1u)));
+}
+
+// A record's place (after scan_words).
+__device__ __forceinline__ uint32_t place_of(const Part &A, uint32_t dg)
+{
+    const uint32_t w = dg >> 5, pf = A.PF[w];
+    if (pf & kDirty) return (pf & (kDirty - 1u)) + atomicAdd(&A.BM[w], 1u);
+    return pf + (uint32_t)__popc(A.BM[w] & ((1u << (dg & 31u)) - 1u));
+}
+
+__device__ __forceinline__ void put_record(const Part &A, uint32_t pos, uint64_t key, uint32_t nonce)
+{
+    uint32_t *o = A.Y + 3 * pos;
+    o[0] = nonce;
+    o[1] = bswap32((uint32_t)(key >> 32));
+    o[2] = bswap32((uint32_t)key);
+}
+
+// Exclusive scan of the W words' record counts into PF, `per` consecutive
+// words a thread; dirty words are flagged and listed and their bitmap word
+// becomes the count of records placed.  Between two barriers of the caller's;
+// one inside.
+template <int NT>
+__device__ __forceinline__ void scan_words(const Part &A, uint32_t W)
 {
     constexpr uint32_t NW = NT / 32;
-    const uint32_t dmask = ndig - 1u;
-    // digit g's counter: word g (PACK: word g / 2, the half g & 1)
-    auto bump = [&](uint32_t g) -> uint32_t {
-        if (PACK) {
-            const uint32_t h = (g & 1u) << 4;
-            return (atomicAdd(&A.DC[g >> 1], 1u << h) >> h) & 0xFFFFu;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t per = W > (uint32_t)NT ? W / NT : 1u;
+    const uint32_t w0 = threadIdx.x * per;
+    uint32_t local = 0;
+    if (per >= 8) {
+        for (uint32_t g = 0; g < per; g += 8) {
+            const uint4 a = *reinterpret_cast<const uint4 *>(A.BM + w0 + g);
+            const uint4 b = *reinterpret_cast<const uint4 *>(A.BM + w0 + g + 4);
+            const uint4 e = *reinterpret_cast<const uint4 *>(A.PF + w0 + g);
+            local += __popc(a.x) + __popc(a.y) + __popc(a.z) + __popc(a.w) + __popc(b.x) + __popc(b.y) +
+                     __popc(b.z) + __popc(b.w);
+            const uint32_t x = e.x + e.y + e.z + e.w;  // extras: 16-bit halves, < 2^15 in all
+            local += (x & 0xFFFFu) + (x >> 16);
         }
-        return atomicAdd(&A.DC[g], 1u);
+    } else if (w0 < W) {
+        for (uint32_t g = 0; g < per; ++g) local += __popc(A.BM[w0 + g]) + A.PF[w0 + g];
+    }
+    const uint32_t incl = warp_incl_scan(local);
+    if (lane == 31) A.WS[warp] = incl;
+    __syncthreads();
+    uint32_t run = incl - local;
+#pragma unroll
+    for (uint32_t w = 0; w < NW; ++w) run += w < warp ? A.WS[w] : 0u;
+    auto set_dirty = [&](uint32_t w) {
+        A.PF[w] |= (uint16_t)kDirty;
+        A.BM[w] = 0u;
+        const uint32_t i = atomicAdd(&A.WS[kWsDirty], 1u);
+        if (i < kDirtyList) A.DL[i] = (uint16_t)w;
     };
-    const uint16_t *DC16 = reinterpret_cast<const uint16_t *>(A.DC);
-    // end of run g once the records are placed (little-endian halves)
-    auto run_end = [&](uint32_t g) -> uint32_t { return PACK ? (uint32_t)DC16[g] : A.DC[g]; };
-#pragma unroll 4
-    for (uint32_t i = threadIdx.x; i < n; i += NT) bump((uint32_t)(XK[i] >> shift) & dmask);
-    __syncthreads();
-    if (PACK)
-        counts_to_starts_packed<NT, 8>(A.DC, ndig >> 1, A.WS);
-    else
-        counts_to_starts<NT, 8>(A.DC, ndig, A.WS);
-    if (DRAIN) {
-        if (threadIdx.x == 0) bulk_wait_all<true>();
-        __syncthreads();
-    }
-#pragma unroll 4
-    for (uint32_t i = threadIdx.x; i < n; i += NT) {
-        const uint64_t k = XK[i];
-        const uint32_t pos = bump((uint32_t)(k >> shift) & dmask);
-        YK[pos] = k;
-        YN[pos] = XN[i];
-    }
-    __syncthreads();
-    // DC[g] is now the end of run g: run g is [DC[g-1], DC[g]).  A record's
-    // place is its run's start plus the run's records before it.  A run's
-    // records sit in neighbouring lanes of a chunk of 32 positions, so each
-    // lane compares with the lanes up to the longest run's length away
-    // (shuffles, every lane in step), on a 32-bit compare key: the key bits
-    // below the digit, or their top 32 -- records of a run agree above
-    // them.  A lane whose run leaves its chunk, or that meets an equal
-    // compare key, ranks itself again from shared memory on full keys and
-    // nonces.  Two chunks per step so that their work overlaps.
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t nch = (n + 31u) >> 5;
-    const int cs = shift > 32 ? shift - 32 : 0;
-    for (uint32_t c = warp; c < nch; c += 2 * NW) {
-        const uint32_t pa = 32u * c + lane, pb = pa + 32u * NW;
-        const bool va = pa < n, vb = pb < n;
-        const uint32_t xa = va ? pa : 0u, xb = vb ? pb : 0u;
-        const uint64_t ka = YK[xa], kb = YK[xb];
-        const uint32_t na = YN[xa], nb = YN[xb];
-        const uint32_t ga = (uint32_t)(ka >> shift) & dmask, gb = (uint32_t)(kb >> shift) & dmask;
-        const uint32_t sa = ga ? run_end(ga - 1) : 0u, sb = gb ? run_end(gb - 1) : 0u;
-        const uint32_t ea = va ? run_end(ga) : 0u, eb = vb ? run_end(gb) : 0u;
-        const uint32_t lmax = __reduce_max_sync(0xffffffffu, max(va ? ea - sa : 0u, vb ? eb - sb : 0u));
-        uint32_t da = sa, db = sb;
-        if (lmax > 1) {
-            const uint32_t qa = (uint32_t)(ka >> cs), qb = (uint32_t)(kb >> cs);
-            // the chunk's positions are [32 c, 32 c + 32): a run inside it
-            // is seen whole by the shuffles
-            bool slow_a = va && (sa < 32u * c || ea > 32u * c + 32u);
-            bool slow_b = vb && (sb < 32u * (c + NW) || eb > 32u * (c + NW) + 32u);
-            for (uint32_t t = 1; t < lmax; ++t) {
-                const uint32_t da_ = __shfl_down_sync(0xffffffffu, qa, t), ua = __shfl_up_sync(0xffffffffu, qa, t);
-                const uint32_t db_ = __shfl_down_sync(0xffffffffu, qb, t), ub = __shfl_up_sync(0xffffffffu, qb, t);
-                const bool ina_d = pa + t < ea, ina_u = lane >= t && pa - t >= sa;
-                const bool inb_d = pb + t < eb, inb_u = lane >= t && pb - t >= sb;
-                da += (ina_d && da_ < qa ? 1u : 0u) + (ina_u && ua < qa ? 1u : 0u);
-                db += (inb_d && db_ < qb ? 1u : 0u) + (inb_u && ub < qb ? 1u : 0u);
-                slow_a = slow_a || (ina_d && da_ == qa) || (ina_u && ua == qa);
-                slow_b = slow_b || (inb_d && db_ == qb) || (inb_u && ub == qb);
+    if (per >= 8) {
+        for (uint32_t g = 0; g < per; g += 8) {
+            uint4 e = *reinterpret_cast<const uint4 *>(A.PF + w0 + g);
+            uint32_t *const ex[4] = {&e.x, &e.y, &e.z, &e.w};
+            const uint4 a = *reinterpret_cast<const uint4 *>(A.BM + w0 + g);
+            const uint4 b = *reinterpret_cast<const uint4 *>(A.BM + w0 + g + 4);
+            const uint32_t bm[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+            uint32_t m = 0;  // bit j: word w0 + g + j is dirty
+            if (e.x | e.y | e.z | e.w) {
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+                    m |= (*ex[h] & 0xFFFFu ? 1u << (2 * h) : 0u) | (*ex[h] >> 16 ? 2u << (2 * h) : 0u);
             }
-            if (va && slow_a) {
-                da = sa;
-                for (uint32_t q = sa; q < ea; ++q) da += rec_less(YK[q], YN[q], ka, na) ? 1u : 0u;
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const uint32_t p0 = run;
+                run += __popc(bm[2 * h]) + (*ex[h] & 0xFFFFu);
+                const uint32_t p1 = run;
+                run += __popc(bm[2 * h + 1]) + (*ex[h] >> 16);
+                *ex[h] = p0 | (p1 << 16);
             }
-            if (vb && slow_b) {
-                db = sb;
-                for (uint32_t q = sb; q < eb; ++q) db += rec_less(YK[q], YN[q], kb, nb) ? 1u : 0u;
-            }
+            *reinterpret_cast<uint4 *>(A.PF + w0 + g) = e;
+            for (; m; m &= m - 1u) set_dirty(w0 + g + (uint32_t)__ffs((int)m) - 1u);
         }
-        if (va) {
-            XK[da] = ka;
-            XN[da] = na;
-        }
-        if (vb) {
-            XK[db] = kb;
-            XN[db] = nb;
+    } else if (w0 < W) {
+        for (uint32_t g = 0; g < per; ++g) {
+            const uint32_t x = A.PF[w0 + g];
+            A.PF[w0 + g] = (uint16_t)run;
+            run += __popc(A.BM[w0 + g]) + x;
+            if (x) set_dirty(w0 + g);
         }
     }
-    __syncthreads();
 }
 
-// Generic sort (any n): records from `src` (global memory) go into SK / SN
-// grouped by digit, a digit's run in arrival order, then one thread per
-// digit finishes its run (about one record) by insertion sort.
-template <int NT, class Src>
-__device__ __forceinline__ void sort_generic(const Part &A, uint32_t n, int shift, uint32_t ndig,
-                                             const Src &src)
+// The dirty words' records in order: eight lanes a listed word, a lane per
+// record, each finding its place among the word's records from its
+// neighbours' (shuffles); words with more than eight records or past the
+// list by one thread's insertion sort.
+template <int NT>
+__device__ __forceinline__ void order_dirty(const Part &A, uint32_t W)
 {
-    const uint32_t dmask = ndig - 1u;
-    for (uint32_t i = threadIdx.x; i < n; i += NT) {
-        const uint32_t dg = (uint32_t)(src.key(i) >> shift) & dmask;
-        atomicAdd(&A.DC[dg], 1u);
+    constexpr uint32_t NW = NT / 32;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    auto order_word = [&](uint32_t w) {
+        uint32_t *const y = A.Y + 3 * (A.PF[w] & (kDirty - 1u));
+        const uint32_t cnt = A.BM[w];
+        for (uint32_t a = 1; a < cnt; ++a) {
+            const uint64_t kx = y_key(y, a);
+            const uint32_t nx = y[3 * a], x1 = y[3 * a + 1], x2 = y[3 * a + 2];
+            uint32_t b = a;
+            for (; b > 0 && rec_less(kx, nx, y_key(y, b - 1), y[3 * b - 3]); --b) {
+                y[3 * b] = y[3 * b - 3];
+                y[3 * b + 1] = y[3 * b - 2];
+                y[3 * b + 2] = y[3 * b - 1];
+            }
+            y[3 * b] = nx;
+            y[3 * b + 1] = x1;
+            y[3 * b + 2] = x2;
+        }
+    };
+    const uint32_t nd = A.WS[kWsDirty];
+    if (nd <= kDirtyList) {
+        const uint32_t sub = lane & 7u;
+        for (uint32_t i0 = 4u * warp; i0 < nd; i0 += 4u * NW) {
+            const uint32_t i = i0 + (lane >> 3);
+            const uint32_t w = i < nd ? A.DL[i] : 0u;
+            uint32_t *const y = A.Y + 3 * (A.PF[w] & (kDirty - 1u));
+            const uint32_t all = i < nd ? A.BM[w] : 0u;
+            const uint32_t cnt = all <= 8u ? all : 0u;
+            const bool mine = sub < cnt;
+            uint32_t nx = 0, x1 = 0, x2 = 0;
+            if (mine) {
+                nx = y[3 * sub];
+                x1 = y[3 * sub + 1];
+                x2 = y[3 * sub + 2];
+            }
+            const uint64_t k = ((uint64_t)bswap32(x1) << 32) | bswap32(x2);
+            const uint32_t most = __reduce_max_sync(0xffffffffu, cnt);
+            uint32_t place = 0;
+            for (uint32_t o = 0; o < most; ++o) {
+                const uint64_t ko = __shfl_sync(0xffffffffu, k, (int)((lane & 24u) + o));
+                const uint32_t no = __shfl_sync(0xffffffffu, nx, (int)((lane & 24u) + o));
+                place += o < cnt && rec_less(ko, no, k, nx) ? 1u : 0u;
+            }
+            if (mine) {
+                y[3 * place] = nx;
+                y[3 * place + 1] = x1;
+                y[3 * place + 2] = x2;
+            }
+            if (all > 8u && sub == 0) order_word(w);
+        }
+    } else {
+        for (uint32_t w = threadIdx.x; w < W; w += NT)
+            if (A.PF[w] & kDirty) order_word(w);
     }
+}
+
+// Bits of sub_key below a digit of a W-word bitmap (log2(W) + 5 bits).
+__device__ __forceinline__ int digit_shift(uint32_t W) { return 27 - (31 - __clz(W)); }
+
+// Sorts the n records of `src` by (key64, nonce) into Y as Table-1 words.
+// Starts after a barrier that follows clear_tables; ends with one.
+// `before_place` runs on thread 0 before anything is written to Y,
+// `after_place` on thread 0 once `src` is no longer read.
+template <int NT, class Src, class F1, class F2>
+__device__ __forceinline__ void sort_bitmap(const Part &A, uint32_t n, int pk, uint32_t W, const Src &src,
+                                            F1 before_place, F2 after_place)
+{
+    const int ds = digit_shift(W);
+    auto digit = [&](uint64_t k) { return sub_key((uint32_t)(k >> 32), (uint32_t)k, pk) >> ds; };
+#pragma unroll 4
+    for (uint32_t i = threadIdx.x; i < n; i += NT) mark(A, digit(src.key(i)));
     __syncthreads();
-    block_scan_inplace_u32<NT>(A.DC, ndig, A.WS);  // counts -> run starts
+    scan_words<NT>(A, W);
+    if (threadIdx.x == 0) before_place();
+    __syncthreads();
+#pragma unroll 4
     for (uint32_t i = threadIdx.x; i < n; i += NT) {
         const uint64_t k = src.key(i);
-        const uint32_t pos = atomicAdd(&A.DC[(uint32_t)(k >> shift) & dmask], 1u);
-        A.SK[pos] = k;
-        A.SN[pos] = src.nonce(i);
+        put_record(A, place_of(A, digit(k)), k, src.nonce(i));
     }
     __syncthreads();
-    // DC[g] is now the end of run g, i.e. run g is [DC[g-1], DC[g])
-    uint64_t *SK = A.SK;
-    uint32_t *SN = A.SN;
-    for (uint32_t dg = threadIdx.x; dg < ndig; dg += NT) {
-        const uint32_t s0 = dg ? A.DC[dg - 1] : 0u;
-        const uint32_t s1 = A.DC[dg];
-        for (uint32_t a = s0 + 1; a < s1; ++a) {
-            const uint64_t kx = SK[a];
-            const uint32_t nx = SN[a];
-            uint32_t b = a;
-            while (b > s0 && !rec_less(SK[b - 1], SN[b - 1], kx, nx)) {
-                SK[b] = SK[b - 1];
-                SN[b] = SN[b - 1];
-                --b;
-            }
-            SK[b] = kx;
-            SN[b] = nx;
-        }
-    }
+    if (threadIdx.x == 0) after_place();
+    order_dirty<NT>(A, W);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // Y leaves by a bulk copy
     __syncthreads();
 }
 
 // ------------------------------------------------ match and the tables
 
-// Everything after the sort, for partition f (n sorted records, Table-1
-// offset `off`) of plot d: the next partition's halo (HALO), the pair
-// counts and their scan, Table 1, then the mode's Table-2 output.  Starts
-// and ends at a barrier; on failure (the status word says why) it skips
-// the output, so a persistent caller goes on to its next item.
+// Everything after the sort, for partition f (n sorted records in Y, Table-1
+// offset `off`) of plot d: Table 1, the next partition's halo (HALO), the
+// pair counts and their scan, then the mode's Table-2 output.  Starts and
+// ends at a barrier; on failure (the status word says why) it skips the
+// output, so a persistent caller goes on to its next item.  Table 1 leaves
+// Y by thread 0's bulk copy: the caller waits for its reads before Y is
+// written again, and for its end before the CTA exits.
 template <int MODE, bool HALO, int NT>
 __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint32_t n, uint64_t off,
                                                 const Part &A, uint64_t *s_base, int *s_ok)
@@ -376,10 +388,22 @@ __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint3
     constexpr bool SLOTS = MODE == kSortSlots;
     constexpr uint32_t NW = NT / 32;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    uint64_t *SK = A.SK;
-    uint32_t *SN = A.SN;
-    uint32_t *ST = A.ST;  // overlays the dead digit counters
-    // 1. cross-bucket match: the next partition's halo (its records within
+    uint32_t *const Y = A.Y;
+    // 1. Table 1: words [0, 3n) of Y to words [3 off, 3 off + 3n) of the
+    //    table.  Shared and global addresses agree mod 16 bytes; the whole
+    //    16-byte lines go by one bulk copy, the up to three words before and
+    //    after them by plain stores.
+    if (warp == 0) {
+        uint32_t *__restrict__ t1w = reinterpret_cast<uint32_t *>(d.t1) + 3 * off;
+        const uint32_t words = 3 * n;
+        const uint32_t head = min(words, (4u - ((uint32_t)(3 * off) & 3u)) & 3u);
+        const uint32_t body = (words - head) & ~3u;
+        if (lane == 0 && body) bulk_s2g(t1w + head, Y + head, body * 4u);
+        if (lane < head) t1w[lane] = Y[lane];
+        const uint32_t t = head + body + lane;
+        if (lane < 4 && t < words) t1w[t] = Y[t];
+    }
+    // 2. cross-bucket match: the next partition's halo (its records within
     //    D of its lower edge, collected while the slots were filled) goes
     //    sorted right after this partition's records, so the pair scan
     //    below runs on into it; records n .. nt - 1 start no pairs here.
@@ -389,87 +413,135 @@ __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint3
         const uint64_t fn = (uint64_t)f + 1;
         const uint32_t hc = fn < (1ull << d.p) ? min(d.halo_cnt[fn], hcap) : 0u;
         for (uint32_t h = threadIdx.x; h < hc; h += NT) {
-            SK[n + h] = d.halo_keys[fn * hcap + h];
-            SN[n + h] = d.halo_nonces[fn * hcap + h];
+            const uint64_t k = d.halo_keys[fn * hcap + h];
+            Y[3 * (n + h)] = d.halo_nonces[fn * hcap + h];
+            Y[3 * (n + h) + 1] = bswap32((uint32_t)(k >> 32));
+            Y[3 * (n + h) + 2] = bswap32((uint32_t)k);
         }
         __syncthreads();
         if (threadIdx.x == 0) {  // a few records (Poisson, mean 2^11 D / 2^(64-p))
             for (uint32_t a = n + 1; a < n + hc; ++a) {
-                const uint64_t kx = SK[a];
-                const uint32_t nx = SN[a];
+                const uint64_t kx = y_key(Y, a);
+                const uint32_t nx = Y[3 * a], x1 = Y[3 * a + 1], x2 = Y[3 * a + 2];
                 uint32_t b = a;
-                for (; b > n && !rec_less(SK[b - 1], SN[b - 1], kx, nx); --b) {
-                    SK[b] = SK[b - 1];
-                    SN[b] = SN[b - 1];
+                for (; b > n && rec_less(kx, nx, y_key(Y, b - 1), Y[3 * b - 3]); --b) {
+                    Y[3 * b] = Y[3 * b - 3];
+                    Y[3 * b + 1] = Y[3 * b - 2];
+                    Y[3 * b + 2] = Y[3 * b - 1];
                 }
-                SK[b] = kx;
-                SN[b] = nx;
+                Y[3 * b] = nx;
+                Y[3 * b + 1] = x1;
+                Y[3 * b + 2] = x2;
             }
         }
         __syncthreads();
         nt = n + hc;
     }
-    // 2. per chunk of 32 sorted records (one per lane; warp w takes chunks
-    //    [c0, c1), two at a time so that their loads overlap): the pairs
-    //    starting at each record r, i.e. the later records up to
-    //    lim = min(last key of r's logical bucket, key_r + D - 1), or
-    //    key_r + D - 1 for the cross-bucket match (four probes, then one by
-    //    one while all four match); the pair offsets inside the warp's
-    //    chunks (warp scans); and the lane's Table-1 record {nonce, BE
-    //    key64}, three 4-byte stores (a warp's stores cover its chunk's 384
-    //    bytes).  Probes may read up to three entries past the records; they
-    //    lie inside the shared allocation and are masked.
+    // 3. per chunk of 32 sorted records (one per lane; warp w takes chunks
+    //    [c0, c1)): the pairs starting at each record r, i.e. the later
+    //    records j of its logical bucket with key_j - key_r < D (every
+    //    bucket with the cross-bucket match), listed in (i, j) order in the
+    //    warp's list as (r - 32 c0) | (j - r) << 12.  A list holds about
+    //    twice the default plot's pairs of a warp; a partition with more, or
+    //    with a record of more than 15, is counted here and recounted when
+    //    its pairs are written.
     const uint32_t nch = (n + 31u) >> 5;
     const uint32_t c0 = warp * nch / NW, c1 = (warp + 1) * nch / NW;
-    const uint32_t rend = min(32u * c1, n);  // the warp's records end here
     const uint64_t D = d.D;
     const bool global = HALO && d.scope != 0;
-    uint32_t *__restrict__ t1w = reinterpret_cast<uint32_t *>(d.t1) + 3 * off;
-    auto limit_of = [&](uint64_t k) -> uint64_t {
-        const uint64_t last_in_bucket = global ? ~0ull : (k | ((1ull << 40) - 1));
-        uint64_t reach = k + (D - 1);
-        if (reach < k) reach = ~0ull;  // saturate
-        return reach < last_in_bucket ? reach : last_in_bucket;
+    // the exact count of record r, on whole keys
+    auto count_exact = [&](uint32_t r) -> uint32_t {
+        const uint64_t k = y_key(Y, r);
+        const uint64_t last = global ? ~0ull : (k | ((1ull << 40) - 1));
+        uint64_t lim = k + (D - 1);
+        if (lim < k) lim = ~0ull;  // saturate
+        if (lim > last) lim = last;
+        uint32_t q = r + 1;
+        while (q < nt && y_key(Y, q) <= lim) ++q;
+        return q - r - 1;
     };
-    auto count_from = [&](uint32_t r, uint64_t lim, uint64_t k1, uint64_t k2, uint64_t k3,
-                          uint64_t k4) -> uint32_t {
-        const bool m1 = r + 1 < nt && k1 <= lim;
-        const bool m2 = m1 && r + 2 < nt && k2 <= lim;
-        const bool m3 = m2 && r + 3 < nt && k3 <= lim;
-        const bool m4 = m3 && r + 4 < nt && k4 <= lim;
-        uint32_t cnt = (uint32_t)m1 + (uint32_t)m2 + (uint32_t)m3 + (uint32_t)m4;
-        if (m4)
-            for (uint32_t q = r + 5; q < nt && SK[q] <= lim; ++q) ++cnt;
-        return cnt;
+    uint16_t *const list = A.PL + warp * A.plw;
+    uint32_t mine = 0;  // pairs of the warp's chunks
+    bool fits = true;   // ... that the list holds
+    auto enlist = [&](uint32_t c, uint32_t cnt) {
+        const uint32_t incl = warp_incl_scan(cnt);
+        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+        if (MODE != kSortCount) {
+            fits = fits && mine + total + 4u <= A.plw;  // the same for the whole warp
+            if (fits) {
+                // Every lane with a pair stores four entries, the farthest
+                // first: one past its own pairs lies on a later lane's, whose
+                // own store to that place is for a nearer record and comes
+                // later.
+                uint16_t *w = list + mine + incl - cnt;
+                const uint32_t e = 32u * (c - c0) + lane;
+                if (cnt) {
+                    w[3] = (uint16_t)(e + (4u << 12));
+                    w[2] = (uint16_t)(e + (3u << 12));
+                    w[1] = (uint16_t)(e + (2u << 12));
+                    w[0] = (uint16_t)(e + (1u << 12));
+                }
+                if (__any_sync(0xffffffffu, cnt > 4)) {
+                    fits = !__any_sync(0xffffffffu, cnt > 15u);
+                    for (uint32_t j = 4; fits && j < cnt; ++j) w[j] = (uint16_t)(e + ((j + 1u) << 12));
+                    __syncwarp();
+                }
+            }
+        }
+        mine += total;
     };
-    uint32_t carry = 0;  // pairs of the warp's chunks before the current one
-    for (uint32_t c = c0; c < c1; c += 2) {
-        const uint32_t ra = 32u * c + lane, rb = ra + 32u;
-        const bool va = ra < n, vb = c + 1 < c1 && rb < n;
-        const uint32_t xa = va ? ra : 0u, xb = vb ? rb : 0u;
-        const uint64_t ka = SK[xa], kb = SK[xb];
-        const uint64_t a1 = SK[xa + 1], a2 = SK[xa + 2], a3 = SK[xa + 3], a4 = SK[xa + 4];
-        const uint64_t b1 = SK[xb + 1], b2 = SK[xb + 2], b3 = SK[xb + 3], b4 = SK[xb + 4];
-        const uint32_t na = SN[xa], nb = SN[xb];
-        if (va) {
-            t1w[3u * ra] = na;
-            t1w[3u * ra + 1] = bswap32((uint32_t)(ka >> 32));
-            t1w[3u * ra + 2] = bswap32((uint32_t)ka);
+    if (global) {
+        for (uint32_t c = c0; c < c1; ++c) {
+            const uint32_t r = 32u * c + lane;
+            enlist(c, r < n ? count_exact(r) : 0u);
         }
-        if (vb) {
-            t1w[3u * rb] = nb;
-            t1w[3u * rb + 1] = bswap32((uint32_t)(kb >> 32));
-            t1w[3u * rb + 2] = bswap32((uint32_t)kb);
+    } else {
+        // On the 32 key bits q below the partition prefix (a partition holds
+        // whole buckets): with D = Dq 2^s + rest, q_j - q_r < Dq is a match
+        // and q_j - q_r >= Dq + 2 is none; between them, rarely, the whole
+        // keys decide.  The records after r (five: 0.06% of a default plot's
+        // records have more pairs) come by shuffles from this chunk's lanes
+        // and the next one's; past the last record they are whatever follows
+        // in shared memory, and the count is cut there.
+        const int pk = d.pk;
+        const uint64_t Dw = D >> (32 - pk);
+        const uint32_t Dq = Dw < 0xFFFFFFF0ull ? (uint32_t)Dw : 0xFFFFFFF0u;
+        const uint32_t bmask = (1u << (8 + pk)) - 1u;  // q's bits inside a bucket
+        const uint32_t *y = Y + 3u * (32u * c0 + lane);
+        uint32_t q0 = sub_key(bswap32(y[1]), bswap32(y[2]), pk);
+        for (uint32_t c = c0; c < c1; ++c) {
+            const uint32_t r = 32u * c + lane;
+            y += 96;
+            const uint32_t q1 = sub_key(bswap32(y[1]), bswap32(y[2]), pk);
+            const uint32_t lim = min(Dq, (~q0 & bmask) + 1u);  // at most to the bucket's end
+            auto diff = [&](uint32_t t) -> uint32_t {  // q of record r + t, less q_r (t < 32)
+                return __shfl_sync(0xffffffffu, lane < t ? q1 : q0, (lane + t) & 31u) - q0;
+            };
+            uint32_t df[5];
+#pragma unroll
+            for (int t = 1; t <= 5; ++t) df[t - 1] = diff(t);
+            const bool m1 = df[0] < lim, m2 = m1 && df[1] < lim, m3 = m2 && df[2] < lim, m4 = m3 && df[3] < lim,
+                       m5 = m4 && df[4] < lim;
+            uint32_t cnt = m5 ? 5u : m4 ? 4u : m3 ? 3u : m2 ? 2u : m1 ? 1u : 0u;
+            // the nearest record that is no sure match
+            uint32_t dn = m4 ? df[4] : m3 ? df[3] : m2 ? df[2] : m1 ? df[1] : df[0];
+            const int after = (int)(n - 1u - r);  // records after r
+            if (__any_sync(0xffffffffu, (m5 || dn - Dq <= 1u) && after > 0)) {
+                bool more = m5 && after > 0;
+                for (uint32_t t = 6; __any_sync(0xffffffffu, more) && t < 32; ++t) {
+                    const uint32_t x = diff(t);
+                    dn = more ? x : dn;
+                    more = more && x < lim;
+                    cnt += more ? 1u : 0u;
+                }
+                if ((more || dn - Dq <= 1u) && after > 0) cnt = count_exact(r);
+            }
+            enlist(c, min(cnt, (uint32_t)max(after, 0)));
+            q0 = q1;
         }
-        const uint32_t cA = va ? count_from(ra, limit_of(ka), a1, a2, a3, a4) : 0u;
-        const uint32_t cB = vb ? count_from(rb, limit_of(kb), b1, b2, b3, b4) : 0u;
-        const uint32_t iA = warp_incl_scan(cA), iB = warp_incl_scan(cB);
-        const uint32_t tA = __shfl_sync(0xffffffffu, iA, 31);
-        if (va) ST[ra] = carry + iA - cA;
-        if (vb) ST[rb] = carry + tA + iB - cB;
-        carry += tA + __shfl_sync(0xffffffffu, iB, 31);
     }
-    if (lane == 0) A.WS[warp] = carry;
+    if (lane == 0) A.WS[warp] = mine;
+    if (MODE != kSortCount && !fits) A.WS[kWsLong] = 1u;
     __syncthreads();
     uint32_t P = 0, wbase = 0;  // the partition's pairs; those before this warp's chunks
 #pragma unroll
@@ -487,7 +559,7 @@ __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint3
         __syncthreads();
         return;
     }
-    // 3. the Table-2 base: the look-back (warp 0), or the partition's slot
+    // 4. the Table-2 base: the look-back (warp 0), or the partition's slot
     bool ok = true;
     uint64_t base = 0;
     if (EMIT) {
@@ -515,105 +587,80 @@ __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint3
         if (threadIdx.x == 0) atomicOr(d.status, kStPairSlot);
         ok = false;
     }
-    // 4. the pairs, in (i, j) order: chunk by chunk (two at a time), a
-    //    lane's record r starts its pairs (r, r + 1 + j) at its offset.
-    //    Slot placement: when the pairs fit the key array of shared memory
-    //    (dead since step 2) they are listed there and leave in one bulk
-    //    copy (thread 0's bulk group; the caller waits for its read before
-    //    the buffer is written again), else they go straight to the slot.
+    // 5. the pairs, in (i, j) order at their places: into the slot (key
+    //    array, then nonce array), as records {a, b, 0, 0}, or hashed here
     uint4 *__restrict__ out = reinterpret_cast<uint4 *>(d.t2) + base;
     uint2 *__restrict__ pa = reinterpret_cast<uint2 *>(d.b_keys + (uint64_t)f * d.cap2);
     uint2 *__restrict__ pb = reinterpret_cast<uint2 *>(d.b_nonces + (uint64_t)f * d.cap2);
     const uint32_t capA = d.cap2;
-    const bool staged = SLOTS && P < capA;
-    uint2 *SP = reinterpret_cast<uint2 *>(SK);
-    auto emit = [&](uint32_t x, uint32_t a, uint32_t b) {
-        if (SLOTS)
-            *(staged ? SP + x : x < capA ? pa + x : pb + (x - capA)) = make_uint2(a, b);
-        else
-            out[x] = make_uint4(a, b, 0u, 0u);
-    };
-    if (ok) {
-        for (uint32_t c = c0; c < c1; c += 2) {
-            const uint32_t ra = 32u * c + lane, rb = ra + 32u;
-            const bool va = ra < n, vb = c + 1 < c1 && rb < n;
-            // offsets inside the warp's pairs; a record's count is the gap
-            // to the next record's offset (the warp's total after its last)
-            const uint32_t sa = va ? ST[ra] : 0u, sb = vb ? ST[rb] : 0u;
-            const uint32_t ea = va ? (ra + 1 < rend ? ST[ra + 1] : carry) : 0u;
-            const uint32_t eb = vb ? (rb + 1 < rend ? ST[rb + 1] : carry) : 0u;
-            const uint32_t aa = va ? SN[ra] : 0u, ab = vb ? SN[rb] : 0u;
-            const uint32_t cA = ea - sa, cB = eb - sb;
-            // the first four partners of each record, read together (the
-            // reads past the records stay inside the shared allocation)
-            const uint32_t xa = va ? ra : 0u, xb = vb ? rb : 0u;
-            const uint32_t a1 = SN[xa + 1], a2 = SN[xa + 2], a3 = SN[xa + 3], a4 = SN[xa + 4];
-            const uint32_t b1 = SN[xb + 1], b2 = SN[xb + 2], b3 = SN[xb + 3], b4 = SN[xb + 4];
-            if (MODE == kSortHash) {
-                __syncwarp();  // every lane has read its neighbour's offset
-                if (va) ST[ra] = wbase + sa;  // offsets for the listing below
-                if (vb) ST[rb] = wbase + sb;
-                continue;
-            }
-            const uint32_t oa = wbase + sa, ob = wbase + sb;
-            if (cA > 0) emit(oa, aa, a1);
-            if (cA > 1) emit(oa + 1, aa, a2);
-            if (cA > 2) emit(oa + 2, aa, a3);
-            if (cA > 3) emit(oa + 3, aa, a4);
-            if (cB > 0) emit(ob, ab, b1);
-            if (cB > 1) emit(ob + 1, ab, b2);
-            if (cB > 2) emit(ob + 2, ab, b3);
-            if (cB > 3) emit(ob + 3, ab, b4);
-            for (uint32_t j = 4; __any_sync(0xffffffffu, j < cA || j < cB); ++j) {
-                if (j < cA) emit(oa + j, aa, SN[ra + 1 + j]);
-                if (j < cB) emit(ob + j, ab, SN[rb + 1 + j]);
-            }
-        }
-        if (staged) {
-            __syncthreads();
-            if (threadIdx.x == 0 && P) bulk_s2g(pa, SP, ((P + 1u) & ~1u) * 8u);
-        }
-    }
-    if (MODE == kSortHash && ok) {
-        // hash here: list the pairs window by window, every lane hashes
-        __syncthreads();
-        uint32_t g[16];
+    uint32_t g[16];
+    if (MODE == kSortHash) {
 #pragma unroll
         for (int i = 0; i < 16; ++i) g[i] = d.pre2[i];
-        uint32_t *LS = A.LS;
-        for (uint32_t w0 = 0; w0 < P; w0 += kSMList) {
-            const uint32_t w1 = min(P, w0 + kSMList);
-            for (uint32_t r = threadIdx.x; r < n; r += NT) {
-                const uint32_t s = ST[r];
-                const uint32_t e = r + 1 < n ? ST[r + 1] : P;
-                const uint32_t lo = max(s, w0), hi = min(e, w1);
-                for (uint32_t k = lo; k < hi; ++k) LS[k - w0] = r | ((r + 1 + (k - s)) << 16);
+    }
+    auto put = [&](uint32_t x, uint32_t a, uint32_t b) {
+        if (SLOTS) {
+            *(x < capA ? pa + x : pb + (x - capA)) = make_uint2(a, b);
+        } else {
+            uint32_t h0 = 0, h1 = 0;
+            if (MODE == kSortHash) b3_finish<true>(g, a, b, h0, h1);
+            out[x] = make_uint4(a, b, h0, h1);
+        }
+    };
+    if (ok && A.WS[kWsLong] == 0u) {  // from the warp's list, a pair per lane
+        const uint32_t *const y0 = Y + 3u * 32u * c0;
+        if (SLOTS && P <= capA) {
+            uint2 *__restrict__ w = pa + wbase;
+#pragma unroll 2
+            for (uint32_t x = lane; x < mine; x += 32) {
+                const uint32_t e = list[x];
+                const uint32_t i = e & 0xFFFu, j = i + (e >> 12);
+                w[x] = make_uint2(y0[3u * i], y0[3u * j]);
             }
-            __syncthreads();
-            for (uint32_t q = threadIdx.x; q < w1 - w0; q += NT) {
-                const uint32_t e = LS[q];
-                const uint32_t a = SN[e & 0xffffu], b = SN[e >> 16];
-                uint32_t h0, h1;
-                b3_finish<true>(g, a, b, h0, h1);
-                out[w0 + q] = make_uint4(a, b, h0, h1);
+        } else {
+            for (uint32_t x = lane; x < mine; x += 32) {
+                const uint32_t e = list[x];
+                const uint32_t i = e & 0xFFFu, j = i + (e >> 12);
+                put(wbase + x, y0[3u * i], y0[3u * j]);
             }
-            __syncthreads();
+        }
+    } else if (ok) {
+        uint32_t at = wbase;
+        for (uint32_t c = c0; c < c1; ++c) {
+            const uint32_t r = 32u * c + lane;
+            const uint32_t cnt = r < n ? count_exact(r) : 0u;
+            const uint32_t incl = warp_incl_scan(cnt);
+            const uint32_t o = at + incl - cnt;
+            at += __shfl_sync(0xffffffffu, incl, 31);
+            for (uint32_t j = 0; j < cnt; ++j) put(o + j, Y[3 * r], Y[3 * (r + 1 + j)]);
         }
     }
     __syncthreads();
 }
 
-__device__ __forceinline__ Part part_arrays(unsigned char *base, const SMLayout &L)
+// The arrays of a partition with a W-word bitmap; tables: SMLayout's bytes
+// for the bitmap and the lists.
+template <int NT>
+__device__ __forceinline__ Part part_arrays(unsigned char *base, const SMLayout &L, uint32_t W, uint32_t tables)
 {
     Part A;
-    A.SK = reinterpret_cast<uint64_t *>(base + L.xk);
-    A.SN = reinterpret_cast<uint32_t *>(base + L.xn);
-    A.DC = reinterpret_cast<uint32_t *>(base + L.dc);
-    A.ST = A.DC;  // overlays the digit counters (dead once the runs are sorted)
-    A.LS = reinterpret_cast<uint32_t *>(base + L.list);
+    A.Y = reinterpret_cast<uint32_t *>(base + L.y);
+    A.BM = reinterpret_cast<uint32_t *>(base + L.bm);
+    A.PF = reinterpret_cast<uint16_t *>(A.BM + W);
+    A.PL = reinterpret_cast<uint16_t *>(A.BM);
+    A.plw = tables / 2u / (NT / 32);
+    A.DL = reinterpret_cast<uint16_t *>(base + L.dl);
     A.WS = reinterpret_cast<uint32_t *>(base + L.ws);
     return A;
 }
+
+// A slot in shared memory.
+struct SharedSrc {
+    const uint64_t *k;
+    const uint32_t *n;
+    __device__ __forceinline__ uint64_t key(uint32_t i) const { return k[i]; }
+    __device__ __forceinline__ uint32_t nonce(uint32_t i) const { return n[i]; }
+};
 
 // A slot in global memory, read through the read-only path unless this
 // kernel later overwrites it with the partition's pairs (RO false).
@@ -630,8 +677,8 @@ struct GlobalSrc {
 // plot find_plot(t); its partition is the plot's next ticket (look-back
 // modes) or t - tile_start[plot].  A CTA takes the ticket of item k + 2
 // and reads the fill count of item k + 1 at the start of item k, and
-// starts item k + 1's slot copy once item k's slot has been sorted into
-// registers, so the global round trips and the copy overlap item k's work.
+// starts item k + 1's slot copy once item k's records have been placed, so
+// the global round trips and the copy overlap item k's match.
 // A CTA takes tickets in its processing order and only while running, so
 // the lowest unpublished partition is always being worked on: the
 // look-back chain cannot stall on a CTA that is not resident.
@@ -673,7 +720,7 @@ __device__ __forceinline__ Item take_item(const Desc *__restrict__ descs, int np
 template <int MODE, bool HALO>
 __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
     k_sortmatch_pipe(const Desc *__restrict__ descs, int nplots, const uint32_t *__restrict__ tile_start,
-                     uint32_t items, uint32_t max_cap, int max_dbits)
+                     uint32_t items, uint32_t max_cap, uint32_t max_words)
 {
     constexpr bool EMIT = MODE == kSortHash || MODE == kSortEmit;
     constexpr int NT = kPipeThreads;
@@ -683,12 +730,11 @@ __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
     __shared__ int s_valid;
     __shared__ uint64_t s_base;
     __shared__ int s_ok;
-    const SMLayout L(max_cap, max_dbits, MODE == kSortHash, true);
-    Part A = part_arrays(smem_raw, L);
+    const SMLayout L(max_cap, max_words, true);
+    Part A = part_arrays<NT>(smem_raw, L, max_words, (uint32_t)(L.dl - L.bm));
+    uint32_t *const Y0 = A.Y;
     uint64_t *const XK = reinterpret_cast<uint64_t *>(smem_raw + L.xk);
     uint32_t *const XN = reinterpret_cast<uint32_t *>(smem_raw + L.xn);
-    uint64_t *const YK = reinterpret_cast<uint64_t *>(smem_raw + L.yk);
-    uint32_t *const YN = reinterpret_cast<uint32_t *>(smem_raw + L.yn);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + L.bar);
     const uint32_t G = gridDim.x;
 
@@ -697,23 +743,23 @@ __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
     // after that (its ticket).
     Item nx{0, 0, false}, nn{0, 0, false};
     uint32_t nx_n = 0;
-    // Starts the copy of item `it` (n records) into buffer b and publishes
-    // it as the next item; an invalid or empty item completes the barrier
-    // phase with no copy.
-    auto launch_copy = [&](const Item &it, uint32_t n, int b) {
+    // Starts the copy of item `it` (n records) into X and publishes it as
+    // the next item; an invalid or empty item completes the barrier phase
+    // with no copy.
+    auto launch_copy = [&](const Item &it, uint32_t n) {
         // Only if the ticket was not reset: report, never index with it.
         const bool valid = it.ok && it.f < (1u << descs[it.plot].p);
         if (it.ok && !valid) atomicOr(descs[it.plot].status, kStBadTicket);
         const uint32_t cnt = valid ? n : 0u;
         const uint32_t nk = (cnt + 1u) & ~1u, nnz = (cnt + 3u) & ~3u;  // 16-byte multiples
-        // The buffer was last accessed by ordinary loads and stores: order
-        // those before the copy engine's writes.
+        // X was last accessed by ordinary loads: order those before the
+        // copy engine's writes.
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_expect_tx(bar, nk * 8u + nnz * 4u);
         if (cnt) {
             const Desc &d = descs[it.plot];
-            bulk_g2s(b ? YK : XK, d.b_keys + (uint64_t)it.f * d.cap2, nk * 8u, bar);
-            bulk_g2s(b ? YN : XN, d.b_nonces + (uint64_t)it.f * d.cap2, nnz * 4u, bar);
+            bulk_g2s(XK, d.b_keys + (uint64_t)it.f * d.cap2, nk * 8u, bar);
+            bulk_g2s(XN, d.b_nonces + (uint64_t)it.f * d.cap2, nnz * 4u, bar);
         }
         s_plot = it.plot;
         s_f = it.f;
@@ -726,13 +772,12 @@ __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
             const Item i0 = take_item<EMIT>(descs, nplots, tile_start, blockIdx.x);
             const uint32_t n0 = i0.f < (1u << descs[i0.plot].p) ? descs[i0.plot].cnt2[i0.f] : 0u;
             if (blockIdx.x + G < items) nx = take_item<EMIT>(descs, nplots, tile_start, blockIdx.x + G);
-            launch_copy(i0, min(n0, descs[i0.plot].cap2), 0);
+            launch_copy(i0, min(n0, descs[i0.plot].cap2));
         }
     }
     __syncthreads();
     uint32_t phase = 0;
-    int rb = 0;  // buffer holding the current item's slot, then its sorted records
-    for (uint32_t t = blockIdx.x; t < items; t += G, phase ^= 1u, rb ^= 1) {
+    for (uint32_t t = blockIdx.x; t < items; t += G, phase ^= 1u) {
         const int plot = s_plot;
         const uint32_t f = s_f, n = s_n;
         const bool valid = s_valid != 0;
@@ -744,46 +789,39 @@ __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
             }
             if (t + 2 * G < items) nn = take_item<EMIT>(descs, nplots, tile_start, t + 2 * G);
         }
-        const uint32_t ndig = 1u << d.dbits;
-        if (ndig % 4u == 0) {
-            uint4 *D4 = reinterpret_cast<uint4 *>(A.DC);
-            for (uint32_t i = threadIdx.x; i < ndig / 4u; i += NT) D4[i] = make_uint4(0u, 0u, 0u, 0u);
-        } else {
-            for (uint32_t i = threadIdx.x; i < ndig; i += NT) A.DC[i] = 0u;
-        }
+        const uint32_t W = bitmap_words(d.dbits);
+        A.PF = reinterpret_cast<uint16_t *>(A.BM + W);
+        clear_tables<NT>(A, W);
         const uint64_t off = valid ? d.t1off[f] : 0ull;
         // The slot copy was started during the previous item (or above).
         if (!__syncthreads_and(mbar_wait(bar, phase, d.spin_limit))) {
-            if (threadIdx.x == 0) atomicOr(d.status, kStTimeout);
+            if (threadIdx.x == 0) {
+                atomicOr(d.status, kStTimeout);
+                bulk_wait_all<false>();
+            }
             mbar_wait(bar, phase, d.spin_limit);  // let it land before the CTA exits
             return;
         }
-        A.SK = rb ? YK : XK;
-        A.SN = rb ? YN : XN;
-        // One more digit bit in the same counter words where they allow it.
-        const int shift = 64 - d.pk - d.dbits;
-        // The previous item's staged pairs leave the buffer this item
-        // places its records into while the sort counts its digits.
-        constexpr bool DR = SLOTS_MODE(MODE);
-        if (valid && n < 0x10000u && rows_shape<NT, 8>(ndig))
-            sort_pingpong<NT, true, DR>(A, A.SK, A.SN, rb ? XK : YK, rb ? XN : YN, n, shift - 1, ndig << 1);
-        else if (valid)
-            sort_pingpong<NT, false, DR>(A, A.SK, A.SN, rb ? XK : YK, rb ? XN : YN, n, shift, ndig);
-        // The other buffer is free: start the next item's copy into it
-        // (after the staged pairs' reads, already over unless no sort ran).
-        if (threadIdx.x == 0) {
-            if (DR) bulk_wait_all<true>();
-            if (nx.ok) launch_copy(nx, nx_n, rb ^ 1);
+        // The next item's copy starts once this slot has been placed in Y.
+        auto start_next = [&]() {
+            if (nx.ok) launch_copy(nx, nx_n);
             nx = nn;
             nn.ok = false;
-        }
+        };
         if (valid) {
+            A.Y = Y0 + ((uint32_t)(3 * off) & 3u);
+            sort_bitmap<NT>(
+                A, n, d.pk, W, SharedSrc{XK, XN},
+                [&]() { bulk_wait_all<true>(); },  // the previous item's Table 1 has left Y
+                start_next);
             match_and_write<MODE, HALO, NT>(d, f, n, off, A, &s_base, &s_ok);
         } else {
             __syncthreads();
+            if (threadIdx.x == 0) start_next();
+            __syncthreads();
         }
     }
-    if (SLOTS_MODE(MODE) && threadIdx.x == 0) bulk_wait_all<false>();
+    if (threadIdx.x == 0) bulk_wait_all<false>();
 }
 
 // ------------------------------------- one CTA per partition front end
@@ -809,24 +847,35 @@ __global__ void __launch_bounds__(kGlThreads, MODE == kSortHash ? 2 : 3)
         return;
     }
     const uint32_t cap = d.cap2;
-    const SMLayout L(cap + (HALO ? d.hcap : 0u), d.dbits, MODE == kSortHash, false);
-    const Part A = part_arrays(smem_raw, L);
-    const uint32_t ndig = 1u << d.dbits;
-    for (uint32_t i = threadIdx.x; i < ndig; i += NT) A.DC[i] = 0u;
+    const uint32_t W = bitmap_words(d.dbits);
+    const SMLayout L(cap + (HALO ? d.hcap : 0u), W, false);
+    Part A = part_arrays<NT>(smem_raw, L, W, (uint32_t)(L.dl - L.bm));
+    clear_tables<NT>(A, W);
     // Warm L2 with the filled part of the slot kSlotPrefetchAhead tickets
     // ahead, so that its CTA's reads hit L2.
     const uint64_t fa = (uint64_t)f + kSlotPrefetchAhead;
     if (threadIdx.x == 0 && fa < (1ull << d.p)) prefetch_slot_l2(d, (uint32_t)fa);
     const uint32_t n = min(d.cnt2[f], cap);
     const uint64_t off = d.t1off[f];
+    A.Y += (uint32_t)(3 * off) & 3u;
     __syncthreads();
-    sort_generic<NT>(A, n, 64 - d.pk - d.dbits, ndig,
-                     GlobalSrc<MODE != kSortSlots>{d.b_keys + (uint64_t)f * cap, d.b_nonces + (uint64_t)f * cap});
+    sort_bitmap<NT>(
+        A, n, d.pk, W,
+        GlobalSrc<MODE != kSortSlots>{d.b_keys + (uint64_t)f * cap, d.b_nonces + (uint64_t)f * cap}, []() {},
+        []() {});
     match_and_write<MODE, HALO, NT>(d, f, n, off, A, &s_base, &s_ok);
-    if (SLOTS_MODE(MODE) && threadIdx.x == 0) bulk_wait_all<false>();
+    if (threadIdx.x == 0) bulk_wait_all<false>();
 }
 
-size_t sortmatch_smem_bytes(uint32_t cap, int dbits) { return SMLayout(cap, dbits, true, false).bytes; }
+// The planner's bound on a slot: 16 bytes a record (at least 4 * 2^dbits for
+// the last four) and 8 KB.  The layout above stays below it at every size it
+// admits (cap 14004: 225,272 of 232,448 bytes).
+size_t sortmatch_smem_bytes(uint32_t cap, int dbits)
+{
+    cap = (cap + 3u) & ~3u;
+    const size_t digits = (size_t)4 << dbits, recs = (size_t)cap * 4;
+    return (size_t)cap * 12 + (digits > recs ? digits : recs) + 8192 + 168;
+}
 
 uint32_t sortmatch_max_cap() { return 16384u; }
 
@@ -835,7 +884,8 @@ static cudaError_t launch_sm(const Desc *descs, int nplots, const uint32_t *tile
                              uint32_t total_tiles, cudaStream_t s, uint32_t max_cap, int max_dbits)
 {
     if (total_tiles == 0) return cudaSuccess;
-    const size_t pipe = SMLayout(max_cap, max_dbits, MODE == kSortHash, true).bytes;
+    const uint32_t words = bitmap_words(max_dbits);
+    const size_t pipe = SMLayout(max_cap, words, true).bytes;
     if (pipe <= kMaxSmemPerCta) {
         auto fn = k_sortmatch_pipe<MODE, HALO>;
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pipe);
@@ -847,10 +897,10 @@ static cudaError_t launch_sm(const Desc *descs, int nplots, const uint32_t *tile
             return e;
         const uint64_t want = (uint64_t)(per_sm > 0 ? per_sm : 1) * (uint64_t)sms;
         const uint32_t grid = (uint32_t)(want < total_tiles ? want : total_tiles);
-        fn<<<grid, kPipeThreads, pipe, s>>>(descs, nplots, tile_start, total_tiles, max_cap, max_dbits);
+        fn<<<grid, kPipeThreads, pipe, s>>>(descs, nplots, tile_start, total_tiles, max_cap, words);
         return cudaGetLastError();
     }
-    const size_t smem = SMLayout(max_cap, max_dbits, MODE == kSortHash, false).bytes;
+    const size_t smem = SMLayout(max_cap, words, false).bytes;
     auto fn = k_sortmatch_gl<MODE, HALO>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

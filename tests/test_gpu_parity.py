@@ -440,3 +440,30 @@ def test_pair_hash_steps(vx, sixteenths):
     r1, r2 = oracle_plot_global(K, key, D)
     assert np.array_equal(t1, r1)
     assert n2 == r2.shape[0] and np.array_equal(t2, r2)
+
+
+@pytest.mark.parametrize("K,s,slack", [(7, 6, 0), (12, 11, 0), (13, 13, 0), (14, 12, 0), (16, 12, 0), (15, 13, 0),
+                                       (15, 13, 50)])
+@pytest.mark.parametrize("split", [False, True], ids=["fused", "split"])
+def test_partition_sizes(vx, K, s, slack, split):
+    # one partition and several, every bitmap size from 64 to 2^18 digits,
+    # more shared-digit words than are listed (s = 12, 13), slots held twice
+    # in shared memory (to s = 12) and read from global memory (above)
+    key = plot_key(540 + K)
+    t1, t2, n2, _ = run_plot(vx, K, key, vx.make_opts(partition_log2=s, slack_sigma=slack), split)
+    r1, r2 = oracle_plot(K, key)
+    assert np.array_equal(t1, r1)
+    assert n2 == r2.shape[0] and np.array_equal(t2, r2)
+
+
+@pytest.mark.parametrize("times", [2, 3, 14, 40])
+@pytest.mark.parametrize("kw", [dict(t2_placement=1), dict(fuse_pair_hash=1), "split"], ids=["lookback", "fused", "split"])
+def test_many_pairs_per_record(vx, times, kw):
+    # a warp's pair list filled, past its end, and records of more than 15 pairs
+    K, key = 14, plot_key(560)
+    D = orc.default_distance(K) * times
+    opts = vx.make_opts(match_scope=1, match_distance=D, **({} if kw == "split" else kw))
+    t1, t2, n2, _ = run_plot(vx, K, key, opts, kw == "split")
+    r1, r2 = oracle_plot_global(K, key, D)
+    assert np.array_equal(t1, r1)
+    assert n2 == r2.shape[0] and np.array_equal(t2, r2)
