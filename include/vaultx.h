@@ -217,9 +217,10 @@ int vx_match(vx_plot *plot, void *stream);
  * hashes them in place) or into the partition's own slot (t2_placement 2,
  * the automatic choice when they fit; a scan of the pair counts and the
  * slot pair hash then write Table 2).  fuse_pair_hash hashes inside the
- * sort kernel instead.  Same tables as vx_table1 + vx_match.  Ends with a
- * 12-byte copy of the status and the Table-2 count to pinned host memory
- * and an event that vx_sync waits on.  Allocates if nothing is bound.
+ * sort kernel instead.  Same tables as vx_table1 + vx_match.  Ends with the
+ * status and the record counts in the handle's pinned host memory (left
+ * there by the slot pair hash, copied otherwise) and an event that vx_sync
+ * waits on.  Allocates if nothing is bound.
  * Asynchronous.  One plot's runs must not overlap on the GPU (two runs of
  * the same plot on different streams race on its buffers): different plots
  * may run concurrently. */
@@ -228,8 +229,8 @@ int vx_plot_run(vx_plot *plot, void *stream);
 /* Waits for the plot's work, reads its status word and Table-2 count, and
  * maps the status to VX_OK / VX_EOVERFLOW / VX_ENOMEM / VX_ETIMEDOUT.
  * Synchronous.  After vx_plot_run it waits on an event recorded behind that
- * run (vx_plot_run ends with a 12-byte device-to-host copy of the status and
- * count into the handle's pinned block), so work queued later on the same
+ * run (vx_plot_run ends with the status and counts in the handle's pinned
+ * block), so work queued later on the same
  * stream is not waited for, and the values are this run's even when a later
  * plot on the stream reuses the same Table-1 and scratch buffers.  After
  * vx_table1, vx_match or vx_plot_batch it synchronises the whole stream and

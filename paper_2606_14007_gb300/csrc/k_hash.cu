@@ -16,19 +16,17 @@
 
 namespace vx {
 
-// ------------------------------------------------------------ key setup
-// One CTA row per plot: thread 0 of block x == 0 derives the per-key hash
-// states; every CTA zeroes a share of the plot's fill counters and the
-// status word.
+// --------------------------------------------------------------- setup
+// One CTA row per plot: every CTA zeroes a share of the plot's fill counters
+// and look-back words, one thread the tickets and the status word.  (The
+// per-key hash states come with the descriptor, so the hash may start beside
+// this kernel and waits for it before its first claim.)
 __global__ void k_key_setup(Desc *descs)
 {
+    pdl_wait();
+    pdl_go();
     Desc &d = descs[blockIdx.y];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        uint32_t pre[16];
-        b3_key_setup(d.key, 4u, pre);
-        for (int i = 0; i < 16; ++i) d.pre1[i] = pre[i];
-        b3_key_setup(d.key, 8u, pre);
-        for (int i = 0; i < 16; ++i) d.pre2[i] = pre[i];
         *d.status = 0u;
         *d.ticket = 0u;
         *d.ticket_s = 0u;
@@ -50,10 +48,10 @@ __global__ void k_key_setup(Desc *descs)
     }
 }
 
-cudaError_t launch_key_setup(Desc *descs, int nplots, cudaStream_t s)
+cudaError_t launch_key_setup(Desc *descs, int nplots, On on)
 {
     dim3 grid(64, nplots);
-    k_key_setup<<<grid, 256, 0, s>>>(descs);
+    k_key_setup<<<grid, 256, 0, on.s>>>(descs);
     return cudaGetLastError();
 }
 
@@ -174,6 +172,8 @@ __global__ void __launch_bounds__(NT, NPT <= 12 ? 4 : 3) k_hash_scatter(const De
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S &sm = *reinterpret_cast<S *>(smem_raw);
 
+    pdl_go();
+    if (WM == kWinList) pdl_wait();
     const int plot = find_plot(tile_start, nplots, blockIdx.x);
     const Desc &d = descs[plot];
     uint64_t lo, N;  // this chunk's nonces: [lo, N), or (list) list entries [0, N)
@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(NT, NPT <= 12 ? 4 : 3) k_hash_scatter(const De
             }
         }
     }
+    if (WM != kWinList) pdl_wait();  // up to here only the descriptor was read
     __syncthreads();
     uint32_t count;  // records the tile keeps
     const bool over = scan_and_claim<NT>(sm, nbins, cnt, cap, &count);
@@ -267,15 +268,15 @@ __global__ void __launch_bounds__(NT, NPT <= 12 ? 4 : 3) k_hash_scatter(const De
 
 template <int NPT, bool AGG, bool HALO, int WM>
 static cudaError_t launch_hs(const Desc *descs, int nplots, const uint32_t *tile_start,
-                             uint32_t total_tiles, int chunk, cudaStream_t s)
+                             uint32_t total_tiles, int chunk, On on)
 {
     constexpr int NT = kHashThreads;
+    static SmemSeen seen;
     const size_t smem = sizeof(HashTile<NT, NPT>);
     auto fn = k_hash_scatter<NT, NPT, AGG, HALO, WM>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(fn, smem, seen);
     if (e != cudaSuccess) return e;
-    fn<<<total_tiles, NT, smem, s>>>(descs, nplots, tile_start, chunk);
-    return cudaGetLastError();
+    return launch_on(on, fn, total_tiles, NT, smem, descs, nplots, tile_start, chunk);
 }
 
 // AGG (warp-aggregated ranks) pays off when a warp's 32 records fall into
@@ -285,43 +286,43 @@ static cudaError_t launch_hs(const Desc *descs, int nplots, const uint32_t *tile
 // launch holds one windowed plot (never cross-bucket).
 template <bool HALO, int WM, int NPT>
 static cudaError_t launch_hs_npt(const Desc *descs, int nplots, const uint32_t *tile_start,
-                                 uint32_t total_tiles, bool agg, int chunk, cudaStream_t s)
+                                 uint32_t total_tiles, bool agg, int chunk, On on)
 {
-    return agg ? launch_hs<NPT, true, HALO, WM>(descs, nplots, tile_start, total_tiles, chunk, s)
-               : launch_hs<NPT, false, HALO, WM>(descs, nplots, tile_start, total_tiles, chunk, s);
+    return agg ? launch_hs<NPT, true, HALO, WM>(descs, nplots, tile_start, total_tiles, chunk, on)
+               : launch_hs<NPT, false, HALO, WM>(descs, nplots, tile_start, total_tiles, chunk, on);
 }
 
 template <bool HALO, int WM>
 static cudaError_t launch_hs_agg(const Desc *descs, int nplots, const uint32_t *tile_start,
-                                 uint32_t total_tiles, bool agg, int chunk, cudaStream_t s, int npt)
+                                 uint32_t total_tiles, bool agg, int chunk, On on, int npt)
 {
     if (WM != kWinNone)
         return npt == kHashNoncesPerThread
-                   ? launch_hs_npt<HALO, WM, kHashNoncesPerThread>(descs, nplots, tile_start, total_tiles, agg, chunk, s)
+                   ? launch_hs_npt<HALO, WM, kHashNoncesPerThread>(descs, nplots, tile_start, total_tiles, agg, chunk, on)
                    : cudaErrorInvalidValue;
     switch (npt) {
-    case 2: return launch_hs_npt<HALO, kWinNone, 2>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
-    case 4: return launch_hs_npt<HALO, kWinNone, 4>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
-    case 8: return launch_hs_npt<HALO, kWinNone, 8>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
-    case 12: return launch_hs_npt<HALO, kWinNone, 12>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
-    case 16: return launch_hs_npt<HALO, kWinNone, 16>(descs, nplots, tile_start, total_tiles, agg, chunk, s);
+    case 2: return launch_hs_npt<HALO, kWinNone, 2>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
+    case 4: return launch_hs_npt<HALO, kWinNone, 4>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
+    case 8: return launch_hs_npt<HALO, kWinNone, 8>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
+    case 12: return launch_hs_npt<HALO, kWinNone, 12>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
+    case 16: return launch_hs_npt<HALO, kWinNone, 16>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
     default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t launch_hash_scatter(const Desc *descs, int nplots, const uint32_t *tile_start,
-                                uint32_t total_tiles, HashCfg cfg, int chunk, cudaStream_t s)
+                                uint32_t total_tiles, HashCfg cfg, int chunk, On on)
 {
     if (total_tiles == 0) return cudaSuccess;
     const int npt = cfg.npt;
     if (cfg.list)
         return cfg.halo ? cudaErrorInvalidValue
-                        : launch_hs_agg<false, kWinList>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, s, npt);
+                        : launch_hs_agg<false, kWinList>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt);
     if (cfg.win)
-        return cfg.halo ? launch_hs_agg<true, kWinFilter>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, s, npt)
-                        : launch_hs_agg<false, kWinFilter>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, s, npt);
-    return cfg.halo ? launch_hs_agg<true, kWinNone>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, s, npt)
-                    : launch_hs_agg<false, kWinNone>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, s, npt);
+        return cfg.halo ? launch_hs_agg<true, kWinFilter>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt)
+                        : launch_hs_agg<false, kWinFilter>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt);
+    return cfg.halo ? launch_hs_agg<true, kWinNone>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt)
+                    : launch_hs_agg<false, kWinNone>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt);
 }
 
 // ------------------------------------------------- hash + direct scatter
@@ -337,6 +338,8 @@ __global__ void __launch_bounds__(NT) k_hash_direct(const Desc *__restrict__ des
                                                     int chunk)
 {
     constexpr bool WIN = WM != kWinNone;
+    pdl_go();
+    pdl_wait();
     const int plot = find_plot(tile_start, nplots, blockIdx.x);
     const Desc &d = descs[plot];
     uint64_t lo, N;  // this chunk's nonces: [lo, N), or (list) list entries [0, N)
@@ -391,25 +394,24 @@ __global__ void __launch_bounds__(NT) k_hash_direct(const Desc *__restrict__ des
 
 template <bool HALO, int WM>
 static cudaError_t launch_hd(const Desc *descs, int nplots, const uint32_t *tile_start,
-                             uint32_t total_tiles, int chunk, cudaStream_t s)
+                             uint32_t total_tiles, int chunk, On on)
 {
-    k_hash_direct<kHashThreads, kHashNoncesPerThread, HALO, WM><<<total_tiles, kHashThreads, 0, s>>>(
-        descs, nplots, tile_start, chunk);
-    return cudaGetLastError();
+    return launch_on(on, k_hash_direct<kHashThreads, kHashNoncesPerThread, HALO, WM>, total_tiles, kHashThreads, 0,
+                     descs, nplots, tile_start, chunk);
 }
 
 cudaError_t launch_hash_direct(const Desc *descs, int nplots, const uint32_t *tile_start,
-                               uint32_t total_tiles, int chunk, cudaStream_t s, HashCfg cfg)
+                               uint32_t total_tiles, int chunk, On on, HashCfg cfg)
 {
     if (total_tiles == 0) return cudaSuccess;
     if (cfg.list)
         return cfg.halo ? cudaErrorInvalidValue
-                        : launch_hd<false, kWinList>(descs, nplots, tile_start, total_tiles, chunk, s);
+                        : launch_hd<false, kWinList>(descs, nplots, tile_start, total_tiles, chunk, on);
     if (cfg.win)
-        return cfg.halo ? launch_hd<true, kWinFilter>(descs, nplots, tile_start, total_tiles, chunk, s)
-                        : launch_hd<false, kWinFilter>(descs, nplots, tile_start, total_tiles, chunk, s);
-    return cfg.halo ? launch_hd<true, kWinNone>(descs, nplots, tile_start, total_tiles, chunk, s)
-                    : launch_hd<false, kWinNone>(descs, nplots, tile_start, total_tiles, chunk, s);
+        return cfg.halo ? launch_hd<true, kWinFilter>(descs, nplots, tile_start, total_tiles, chunk, on)
+                        : launch_hd<false, kWinFilter>(descs, nplots, tile_start, total_tiles, chunk, on);
+    return cfg.halo ? launch_hd<true, kWinNone>(descs, nplots, tile_start, total_tiles, chunk, on)
+                    : launch_hd<false, kWinNone>(descs, nplots, tile_start, total_tiles, chunk, on);
 }
 
 // ------------------------------------------------ Table-2 pair hashing
@@ -429,6 +431,8 @@ __global__ void __launch_bounds__(kT2HashThreads) k_t2_hash(const Desc *__restri
                                                             int chunk)
 {
     constexpr int NT = kT2HashThreads;
+    pdl_go();
+    pdl_wait();
     const int plot = find_plot(tile_start, nplots, blockIdx.x);
     const Desc &d = descs[plot];
     if (*d.status & (kStT2Capacity | kStTimeout | kStBadTicket)) return;
@@ -469,11 +473,10 @@ __global__ void __launch_bounds__(kT2HashThreads) k_t2_hash(const Desc *__restri
 }
 
 cudaError_t launch_t2_hash(const Desc *descs, int nplots, const uint32_t *tile_start,
-                           uint32_t total_tiles, int chunk, cudaStream_t s)
+                           uint32_t total_tiles, int chunk, On on)
 {
     if (total_tiles == 0) return cudaSuccess;
-    k_t2_hash<<<total_tiles, kT2HashThreads, 0, s>>>(descs, nplots, tile_start, chunk);
-    return cudaGetLastError();
+    return launch_on(on, k_t2_hash, total_tiles, kT2HashThreads, 0, descs, nplots, tile_start, chunk);
 }
 
 // Pair hash of the slot placement (Sec. III-A, Table 2): CTA b takes
@@ -489,8 +492,17 @@ __global__ void __launch_bounds__(kT2HashThreads) k_t2_hash_slots(const Desc *__
                                                                   const uint32_t *__restrict__ tile_start)
 {
     static_assert(kT2SlotGroup == kT2HashThreads / 32, "one partition per warp");
+    pdl_go();
+    pdl_wait();
     const int plot = find_plot(tile_start, nplots, blockIdx.x);
     const Desc &d = descs[plot];
+    // The run's result, final since the scan before this kernel, goes
+    // straight to the caller's pinned words (three copies less per run).
+    if (d.result && blockIdx.x == tile_start[plot] && threadIdx.x == 0) {
+        d.result[0] = *d.status;
+        d.result[1] = d.t2off[1ull << d.p];
+        d.result[2] = d.t1off[1ull << d.p];
+    }
     if (*d.status & (kStT2Capacity | kStTimeout | kStBadTicket | kStPairSlot)) return;
     const uint64_t np = 1ull << d.p;
     const uint64_t f = (uint64_t)(blockIdx.x - tile_start[plot]) * kT2SlotGroup + (threadIdx.x >> 5);
@@ -540,11 +552,10 @@ __global__ void __launch_bounds__(kT2HashThreads) k_t2_hash_slots(const Desc *__
 }
 
 cudaError_t launch_t2_hash_slots(const Desc *descs, int nplots, const uint32_t *tile_start,
-                                 uint32_t total_tiles, cudaStream_t s)
+                                 uint32_t total_tiles, On on)
 {
     if (total_tiles == 0) return cudaSuccess;
-    k_t2_hash_slots<<<total_tiles, kT2HashThreads, 0, s>>>(descs, nplots, tile_start);
-    return cudaGetLastError();
+    return launch_on(on, k_t2_hash_slots, total_tiles, kT2HashThreads, 0, descs, nplots, tile_start);
 }
 
 // ------------------------------------------------ tiled plots: windows
@@ -597,6 +608,8 @@ __global__ void __launch_bounds__(kListThreads) k_window_list(const Desc *__rest
 {
     __shared__ uint32_t ws[kListThreads / 32 + 1];
     __shared__ uint32_t s_base;
+    pdl_go();
+    pdl_wait();
     const Desc &d = *dp;
     const uint64_t n0 = ((uint64_t)blockIdx.x * kListThreads + threadIdx.x) * kListPerThread;
     uint4 v = make_uint4(0u, 0u, 0u, 0u);

@@ -35,6 +35,8 @@ __global__ void __launch_bounds__(kMatchThreads) k_match(const Desc *__restrict_
 {
     constexpr int NT = kMatchThreads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_go();
+    pdl_wait();
     const int plot = find_plot(tile_start, nplots, blockIdx.x);
     const Desc &d = descs[plot];
     const uint32_t f = blockIdx.x - tile_start[plot];
@@ -186,14 +188,13 @@ __global__ void __launch_bounds__(kMatchThreads) k_match(const Desc *__restrict_
 size_t match_smem_bytes(uint32_t cap) { return MatchLayout(cap).bytes; }
 
 cudaError_t launch_match(const Desc *descs, int nplots, const uint32_t *tile_start,
-                         uint32_t total_tiles, cudaStream_t s, uint32_t max_cap)
+                         uint32_t total_tiles, On on, uint32_t max_cap)
 {
+    static SmemSeen seen;
     const size_t smem = match_smem_bytes(max_cap);
-    cudaError_t e = cudaFuncSetAttribute(k_match, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    const cudaError_t e = allow_smem(k_match, smem, seen);
     if (e != cudaSuccess) return e;
-    k_match<<<total_tiles, kMatchThreads, smem, s>>>(descs, nplots, tile_start);
-    return cudaGetLastError();
+    return launch_on(on, k_match, total_tiles, kMatchThreads, smem, descs, nplots, tile_start);
 }
 
 }  // namespace vx

@@ -39,6 +39,8 @@ __global__ void __launch_bounds__(kScatterThreads) k_scatter2(const Desc *__rest
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Scatter2Smem<FB> &sm = *reinterpret_cast<Scatter2Smem<FB> *>(smem_raw);
 
+    pdl_go();
+    pdl_wait();
     const int plot = find_plot(tile_start, nplots, blockIdx.x);
     const Desc &d = descs[plot];
     const uint32_t local = blockIdx.x - tile_start[plot];
@@ -147,18 +149,17 @@ __global__ void __launch_bounds__(kScatterThreads) k_scatter2(const Desc *__rest
 }
 
 cudaError_t launch_scatter2(const Desc *descs, int nplots, const uint32_t *tile_start,
-                            uint32_t total_tiles, int chunk, cudaStream_t s, bool halo,
-                            int fine_bits)
+                            uint32_t total_tiles, int chunk, On on, bool halo, int fine_bits)
 {
     if (total_tiles == 0) return cudaSuccess;
     const bool wide = fine_bits > kMaxFineBits;
     const size_t smem = wide ? sizeof(Scatter2Smem<kMaxFineBitsWide>) : sizeof(Scatter2Smem<kMaxFineBits>);
     auto fn = wide ? (halo ? k_scatter2<true, kMaxFineBitsWide> : k_scatter2<false, kMaxFineBitsWide>)
                    : (halo ? k_scatter2<true, kMaxFineBits> : k_scatter2<false, kMaxFineBits>);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemSeen seen[4];
+    const cudaError_t e = allow_smem(fn, smem, seen[(wide ? 2 : 0) + (halo ? 1 : 0)]);
     if (e != cudaSuccess) return e;
-    fn<<<total_tiles, kScatterThreads, smem, s>>>(descs, nplots, tile_start, chunk);
-    return cudaGetLastError();
+    return launch_on(on, fn, total_tiles, kScatterThreads, smem, descs, nplots, tile_start, chunk);
 }
 
 // ------------------------------- Table-1 / Table-2 offsets (counts scan)
@@ -186,6 +187,8 @@ __global__ void __launch_bounds__(kScanCtaThreads) k_scan_counts(const Desc *__r
     __shared__ uint32_t s_c;
     __shared__ uint64_t s_base;
     __shared__ int s_ok;
+    pdl_go();
+    pdl_wait();
     const int plot = find_plot(tile_start, nplots, blockIdx.x);
     const Desc &d = descs[plot];
     uint32_t *ticket = SRC == 0 ? d.ticket_s : d.ticket;
@@ -253,17 +256,15 @@ __global__ void __launch_bounds__(kScanCtaThreads) k_scan_counts(const Desc *__r
 }
 
 cudaError_t launch_scan_counts(const Desc *descs, int nplots, const uint32_t *tile_start,
-                               uint32_t total_tiles, cudaStream_t s)
+                               uint32_t total_tiles, On on)
 {
-    k_scan_counts<0><<<total_tiles, kScanCtaThreads, 0, s>>>(descs, nplots, tile_start);
-    return cudaGetLastError();
+    return launch_on(on, k_scan_counts<0>, total_tiles, kScanCtaThreads, 0, descs, nplots, tile_start);
 }
 
 cudaError_t launch_scan_pair_counts(const Desc *descs, int nplots, const uint32_t *tile_start,
-                                    uint32_t total_tiles, cudaStream_t s)
+                                    uint32_t total_tiles, On on)
 {
-    k_scan_counts<1><<<total_tiles, kScanCtaThreads, 0, s>>>(descs, nplots, tile_start);
-    return cudaGetLastError();
+    return launch_on(on, k_scan_counts<1>, total_tiles, kScanCtaThreads, 0, descs, nplots, tile_start);
 }
 
 // ------------------------------------------------------ pair-offset scan
@@ -277,6 +278,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_pairs(const Desc *__restr
     constexpr int NT = kScanThreads, NW = NT / 32, PER = 4;
     __shared__ uint64_t ws[NW];
     __shared__ uint64_t s_tile;
+    pdl_go();
+    pdl_wait();
     const Desc &d = descs[blockIdx.x];
     const uint64_t n = 1ull << d.p;
     uint64_t *out = d.t2off;
@@ -330,10 +333,9 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_pairs(const Desc *__restr
     }
 }
 
-cudaError_t launch_scan_pairs(const Desc *descs, int nplots, cudaStream_t s)
+cudaError_t launch_scan_pairs(const Desc *descs, int nplots, On on)
 {
-    k_scan_pairs<<<nplots, kScanThreads, 0, s>>>(descs);
-    return cudaGetLastError();
+    return launch_on(on, k_scan_pairs, (uint32_t)nplots, kScanThreads, 0, descs);
 }
 
 // ----------------------------------------------- logical bucket offsets

@@ -737,6 +737,8 @@ __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
     uint32_t *const XN = reinterpret_cast<uint32_t *>(smem_raw + L.xn);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + L.bar);
     const uint32_t G = gridDim.x;
+    pdl_go();
+    pdl_wait();
 
     // Thread 0's pipeline: the item after the current one (its ticket and,
     // from the start of the current item on, its fill count) and the one
@@ -835,6 +837,8 @@ __global__ void __launch_bounds__(kGlThreads, MODE == kSortHash ? 2 : 3)
     __shared__ uint32_t s_f;
     __shared__ uint64_t s_base;
     __shared__ int s_ok;
+    pdl_go();
+    pdl_wait();
     const int plot = find_plot(tile_start, nplots, blockIdx.x);
     const Desc &d = descs[plot];
     if (EMIT) {
@@ -881,59 +885,68 @@ uint32_t sortmatch_max_cap() { return 16384u; }
 
 template <int MODE, bool HALO>
 static cudaError_t launch_sm(const Desc *descs, int nplots, const uint32_t *tile_start,
-                             uint32_t total_tiles, cudaStream_t s, uint32_t max_cap, int max_dbits)
+                             uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits)
 {
     if (total_tiles == 0) return cudaSuccess;
     const uint32_t words = bitmap_words(max_dbits);
     const size_t pipe = SMLayout(max_cap, words, true).bytes;
     if (pipe <= kMaxSmemPerCta) {
         auto fn = k_sortmatch_pipe<MODE, HALO>;
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pipe);
+        static SmemSeen seen;
+        // (shared memory, CTAs that fit the device at once) of the last
+        // launch on each device: asking again costs as much as a launch
+        static std::atomic<uint64_t> fits[kMaxDevices];
+        cudaError_t e = allow_smem(fn, pipe, seen);
         if (e != cudaSuccess) return e;
         int dev = 0, sms = 0, per_sm = 0;
         if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kPipeThreads, pipe)) != cudaSuccess)
-            return e;
-        const uint64_t want = (uint64_t)(per_sm > 0 ? per_sm : 1) * (uint64_t)sms;
-        const uint32_t grid = (uint32_t)(want < total_tiles ? want : total_tiles);
-        fn<<<grid, kPipeThreads, pipe, s>>>(descs, nplots, tile_start, total_tiles, max_cap, words);
-        return cudaGetLastError();
+        const bool known = dev >= 0 && dev < kMaxDevices;
+        uint64_t fit = known ? fits[dev].load(std::memory_order_acquire) : 0ull;
+        if (fit >> 32 != pipe) {
+            if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kPipeThreads, pipe)) != cudaSuccess)
+                return e;
+            fit = (uint64_t)pipe << 32 | (uint64_t)((per_sm > 0 ? per_sm : 1) * sms);
+            if (known) fits[dev].store(fit, std::memory_order_release);
+        }
+        const uint32_t want = (uint32_t)fit;
+        return launch_on(on, fn, want < total_tiles ? want : total_tiles, kPipeThreads, pipe, descs, nplots,
+                         tile_start, total_tiles, max_cap, words);
     }
     const size_t smem = SMLayout(max_cap, words, false).bytes;
     auto fn = k_sortmatch_gl<MODE, HALO>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemSeen seen_gl;
+    const cudaError_t e = allow_smem(fn, smem, seen_gl);
     if (e != cudaSuccess) return e;
-    fn<<<total_tiles, kGlThreads, smem, s>>>(descs, nplots, tile_start);
-    return cudaGetLastError();
+    return launch_on(on, fn, total_tiles, kGlThreads, smem, descs, nplots, tile_start);
 }
 
 template <int MODE>
 static cudaError_t launch_sm2(const Desc *descs, int nplots, const uint32_t *tile_start,
-                              uint32_t total_tiles, cudaStream_t s, uint32_t max_cap, int max_dbits,
+                              uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
                               bool halo)
 {
     // HALO instances carry the cross-bucket code; plain launches do not.
-    return halo ? launch_sm<MODE, true>(descs, nplots, tile_start, total_tiles, s, max_cap, max_dbits)
-                : launch_sm<MODE, false>(descs, nplots, tile_start, total_tiles, s, max_cap, max_dbits);
+    return halo ? launch_sm<MODE, true>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits)
+                : launch_sm<MODE, false>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits);
 }
 
 cudaError_t launch_sortmatch(const Desc *descs, int nplots, const uint32_t *tile_start,
-                             uint32_t total_tiles, cudaStream_t s, uint32_t max_cap, int max_dbits,
+                             uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
                              SortMatchOut out, bool halo)
 {
     if (out == kOutLookbackHashed)
-        return launch_sm2<kSortHash>(descs, nplots, tile_start, total_tiles, s, max_cap, max_dbits, halo);
+        return launch_sm2<kSortHash>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo);
     if (out == kOutSlots)
-        return launch_sm2<kSortSlots>(descs, nplots, tile_start, total_tiles, s, max_cap, max_dbits, halo);
-    return launch_sm2<kSortEmit>(descs, nplots, tile_start, total_tiles, s, max_cap, max_dbits, halo);
+        return launch_sm2<kSortSlots>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo);
+    return launch_sm2<kSortEmit>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo);
 }
 
 cudaError_t launch_sort(const Desc *descs, int nplots, const uint32_t *tile_start,
-                        uint32_t total_tiles, cudaStream_t s, uint32_t max_cap, int max_dbits,
+                        uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
                         bool halo)
 {
-    return launch_sm2<kSortCount>(descs, nplots, tile_start, total_tiles, s, max_cap, max_dbits, halo);
+    return launch_sm2<kSortCount>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo);
 }
 
 }  // namespace vx

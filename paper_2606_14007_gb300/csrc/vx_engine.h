@@ -63,6 +63,8 @@ struct Trace {
 struct Lanes {
     cudaStream_t main, aux, aux_lo;
     cudaEvent_t *sync;  // kSyncEvents
+    bool pdl = false;   // one stream, no events between the kernels: each may start
+                        // while the one before runs its last CTAs
 };
 
 }  // namespace vx

@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace vx {
 
 // ---------------------------------------------------------------- limits
@@ -38,8 +40,7 @@ constexpr uint32_t kStSort2 = 1u << 9;        // sorted Table 2: slot overflow o
 constexpr uint32_t kStWinList = 1u << 10;     // a window's nonce list exceeds its capacity
 
 // ------------------------------------------------------ plot descriptor
-// One plot's plan and buffers.  The host fills everything but pre1/pre2,
-// which the key-setup kernel derives from the key on the device.
+// One plot's plan and buffers, filled by the host.
 struct Desc {
     uint64_t N;          // 2^K nonces
     uint64_t D;          // match distance
@@ -84,6 +85,8 @@ struct Desc {
     uint64_t *lbs;       // [chunks] look-back words of the Table-1 offset scan
     uint32_t *ticket_s;  // chunk ticket of the Table-1 offset scan
     uint32_t *status;    // status word
+    uint64_t *result;    // pinned host words {status, Table-2 count, Table-1 count}
+                         //   the slot pair hash leaves the run's result in, or null
     uint8_t *t1;         // Table 1, 12-byte records
     uint8_t *t2;         // Table 2, 16-byte records
     uint32_t key[8];     // plot key, LE words
@@ -140,10 +143,18 @@ constexpr uint32_t kFlagsKeyedRootChunk = 1u /*CHUNK_START*/ | 2u /*CHUNK_END*/ 
                                           8u /*ROOT*/ | 16u /*KEYED_HASH*/;
 
 // Rotations by 16 and 8 are byte moves (PRMT); by 12 and 7 funnel shifts.
+// (The host derives the per-key state with the same functions.)
+#ifdef __CUDA_ARCH__
 __device__ __forceinline__ uint32_t ror16(uint32_t x) { return __byte_perm(x, 0, 0x1032); }
 __device__ __forceinline__ uint32_t ror8(uint32_t x) { return __byte_perm(x, 0, 0x0321); }
 __device__ __forceinline__ uint32_t ror12(uint32_t x) { return __funnelshift_r(x, x, 12); }
 __device__ __forceinline__ uint32_t ror7(uint32_t x) { return __funnelshift_r(x, x, 7); }
+#else
+inline uint32_t ror16(uint32_t x) { return x >> 16 | x << 16; }
+inline uint32_t ror8(uint32_t x) { return x >> 8 | x << 24; }
+inline uint32_t ror12(uint32_t x) { return x >> 12 | x << 20; }
+inline uint32_t ror7(uint32_t x) { return x >> 7 | x << 25; }
+#endif
 __device__ __forceinline__ uint32_t bswap32(uint32_t x) { return __byte_perm(x, 0, 0x0123); }
 
 #define VX_G(a, b, c, d, mx, my)       \
@@ -181,8 +192,8 @@ __device__ __forceinline__ uint32_t bswap32(uint32_t x) { return __byte_perm(x, 
 // and pre[8], pre[12] are unused (IV0 and 0 in column 0, known constants).
 // Every hash saves 2 xors, 1 rotation and 3 sums of the ALU-bound hash this
 // way; loaded from memory as plain state words they cannot fold.
-__device__ __forceinline__ void b3_key_setup(const uint32_t key[8], uint32_t block_len,
-                                             uint32_t pre[16])
+__host__ __device__ __forceinline__ void b3_key_setup(const uint32_t key[8], uint32_t block_len,
+                                                      uint32_t pre[16])
 {
     uint32_t v1 = key[1], v2 = key[2], v3 = key[3];
     uint32_t v5 = key[5], v6 = key[6], v7 = key[7];
@@ -474,6 +485,16 @@ __device__ __forceinline__ void halo_add(const Desc &d, uint64_t part, uint64_t 
     }
 }
 
+// ------------------------------------------ programmatic dependent launch
+// A kernel launched so may start while its predecessor in the stream still
+// runs its last CTAs; pdl_wait waits until the predecessor has finished and
+// its writes are visible (no wait at all when launched the ordinary way).
+// Every CTA of every kernel of a chain calls it, so that a kernel's end
+// implies the end of all before it.  pdl_go lets the successor start once
+// every CTA of this grid has called it or left.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // -------------------------------------------------- TMA bulk copy helpers
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
@@ -551,6 +572,50 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32
 // arrays (exclusive prefixes of per-plot CTA counts, nplots + 1 entries)
 // live in device memory; nplots >= 1.
 namespace vx {
+// Where a launch goes: the stream, and whether it may start before its
+// predecessor there has ended (its kernel then calls pdl_wait).
+struct On {
+    cudaStream_t s;
+    bool pdl;
+    On(cudaStream_t stream, bool p = false) : s(stream), pdl(p) {}
+};
+
+template <class... P, class... A>
+cudaError_t launch_on(On on, void (*fn)(P...), uint32_t grid, uint32_t block, size_t smem, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = on.s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = on.pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
+
+// Allows a kernel `bytes` of dynamic shared memory on the current device.
+// The call is made when a device first needs that much (it costs as much
+// as a launch); `seen` is the kernel's own table, one entry per device.
+constexpr int kMaxDevices = 64;
+struct SmemSeen {
+    std::atomic<size_t> allowed[kMaxDevices] = {};
+};
+template <class Fn>
+cudaError_t allow_smem(Fn fn, size_t bytes, SmemSeen &seen)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool known = dev >= 0 && dev < kMaxDevices;
+    if (known && seen.allowed[dev].load(std::memory_order_acquire) >= bytes) return cudaSuccess;
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && known) seen.allowed[dev].store(bytes, std::memory_order_release);
+    return e;
+}
+
 struct HashCfg {
     bool agg;     // warp-aggregated histogram (few first-level bins)
     bool halo;    // some plot of the launch matches across buckets (halo code)
@@ -558,46 +623,46 @@ struct HashCfg {
     bool list;    // the launch's one plot hashes its window's nonce list
     int npt;      // nonces per thread of the staged Table-1 hash (2, 4, 8, 12, 16; 8 with a window)
 };
-cudaError_t launch_key_setup(Desc *descs, int nplots, cudaStream_t s);
+cudaError_t launch_key_setup(Desc *descs, int nplots, On on);
 // Hash kernels and the second scatter level take one nonce chunk (of
 // Desc::hchunks); the pair hash takes one partition chunk (of Desc::pchunks).
 cudaError_t launch_hash_scatter(const Desc *descs, int nplots, const uint32_t *tile_start,
-                                uint32_t total_tiles, HashCfg cfg, int chunk, cudaStream_t s);
+                                uint32_t total_tiles, HashCfg cfg, int chunk, On on);
 cudaError_t launch_hash_direct(const Desc *descs, int nplots, const uint32_t *tile_start,
-                               uint32_t total_tiles, int chunk, cudaStream_t s, HashCfg cfg);
+                               uint32_t total_tiles, int chunk, On on, HashCfg cfg);
 // Sort + match variants: Table-2 records at final offsets found by a
 // look-back ({a, b, 0, 0}, hashed later by launch_t2_hash; or hashed in the
 // kernel), or pairs {a, b} written into each partition's own slot.
 enum SortMatchOut { kOutLookback = 0, kOutLookbackHashed = 1, kOutSlots = 2 };
 cudaError_t launch_sortmatch(const Desc *descs, int nplots, const uint32_t *tile_start,
-                             uint32_t total_tiles, cudaStream_t s, uint32_t max_cap, int max_dbits,
+                             uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
                              SortMatchOut out, bool halo);
 cudaError_t launch_t2_hash(const Desc *descs, int nplots, const uint32_t *tile_start,
-                           uint32_t total_tiles, int chunk, cudaStream_t s);
+                           uint32_t total_tiles, int chunk, On on);
 // Pair hash of the slot placement: kT2SlotGroup partitions per CTA, pairs
 // read from the partition slots, records written at the scanned offsets.
 constexpr uint32_t kT2SlotGroup = 8;
 cudaError_t launch_t2_hash_slots(const Desc *descs, int nplots, const uint32_t *tile_start,
-                                 uint32_t total_tiles, cudaStream_t s);
+                                 uint32_t total_tiles, On on);
 constexpr uint64_t kT2HashTile = 256 * 8;  // Table-2 records per pair-hash CTA
 size_t sortmatch_smem_bytes(uint32_t cap, int dbits);
 uint32_t sortmatch_max_cap();  // largest slot the sort keeps in registers
 cudaError_t launch_scatter2(const Desc *descs, int nplots, const uint32_t *tile_start,
-                            uint32_t total_tiles, int chunk, cudaStream_t s, bool halo,
+                            uint32_t total_tiles, int chunk, On on, bool halo,
                             int fine_bits);  // the launch's widest second level
 cudaError_t launch_scan_counts(const Desc *descs, int nplots, const uint32_t *tile_start,
-                               uint32_t total_tiles, cudaStream_t s);
+                               uint32_t total_tiles, On on);
 // Same chunked look-back scan over the per-partition pair counts (slot
 // placement) -> Table-2 offsets, with the Table-2 capacity check.
 cudaError_t launch_scan_pair_counts(const Desc *descs, int nplots, const uint32_t *tile_start,
-                                    uint32_t total_tiles, cudaStream_t s);
+                                    uint32_t total_tiles, On on);
 constexpr uint32_t kScanChunk = 4096;      // counters per CTA of the Table-1 offset scan
 cudaError_t launch_sort(const Desc *descs, int nplots, const uint32_t *tile_start,
-                        uint32_t total_tiles, cudaStream_t s, uint32_t max_cap, int max_dbits,
+                        uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
                         bool halo);
-cudaError_t launch_scan_pairs(const Desc *descs, int nplots, cudaStream_t s);
+cudaError_t launch_scan_pairs(const Desc *descs, int nplots, On on);
 cudaError_t launch_match(const Desc *descs, int nplots, const uint32_t *tile_start,
-                         uint32_t total_tiles, cudaStream_t s, uint32_t max_cap);
+                         uint32_t total_tiles, On on, uint32_t max_cap);
 cudaError_t launch_bucket_offsets(const Desc *desc, uint64_t *out, cudaStream_t s);
 // Table 2 sorted by hash2: grids of the five kernels of one sort.
 struct Sort2Launch {

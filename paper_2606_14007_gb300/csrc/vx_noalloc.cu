@@ -86,7 +86,7 @@ extern "C" int vx_plot_run_noalloc(int K, const uint8_t key[32], const vx_opts *
     if (e == cudaSuccess)
         e = cudaMemcpyAsync((void *)d_tiles, tiles, sizeof(tiles), cudaMemcpyHostToDevice, s);
     // One stream, one kernel after the other (no second stream, no events).
-    if (e == cudaSuccess) e = vx::launch_plot_seq(L, vx::Lanes{s, nullptr, nullptr, nullptr});
+    if (e == cudaSuccess) e = vx::launch_plot_seq(L, vx::Lanes{s, nullptr, nullptr, nullptr, p.plan.hchunks == 1 && p.plan.pchunks == 1});
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     uint32_t st = 0;
     uint64_t total = 0;
