@@ -490,22 +490,25 @@ __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint3
         }
         mine += total;
     };
-    if (global) {
+    // On the 32 key bits q below the partition prefix (a partition holds whole
+    // buckets): with D = Dq 2^s + rest, q_j - q_r < Dq is a match and
+    // q_j - q_r >= Dq + 2 is none; between them, rarely, the whole keys
+    // decide.  The records after r (five: 0.06% of a default plot's records
+    // have more pairs) come by shuffles from this chunk's lanes and the next
+    // one's; past the last record they are whatever follows in shared memory,
+    // and the count is cut there.  Halo records lie past the partition's end,
+    // so their q has wrapped: q_j - q_r is still their distance unless that
+    // is a partition's width or more, which takes an r within D of the lower
+    // edge that sees the halo; such an r is counted on whole keys.
+    const int pk = d.pk;
+    const uint64_t Dw = D >> (32 - pk);
+    const uint32_t Dq = Dw < 0xFFFFFFF0ull ? (uint32_t)Dw : 0xFFFFFFF0u;
+    if (global && Dw >= 0xFFFFFFF0ull) {  // D about a partition's width
         for (uint32_t c = c0; c < c1; ++c) {
             const uint32_t r = 32u * c + lane;
             enlist(c, r < n ? count_exact(r) : 0u);
         }
     } else {
-        // On the 32 key bits q below the partition prefix (a partition holds
-        // whole buckets): with D = Dq 2^s + rest, q_j - q_r < Dq is a match
-        // and q_j - q_r >= Dq + 2 is none; between them, rarely, the whole
-        // keys decide.  The records after r (five: 0.06% of a default plot's
-        // records have more pairs) come by shuffles from this chunk's lanes
-        // and the next one's; past the last record they are whatever follows
-        // in shared memory, and the count is cut there.
-        const int pk = d.pk;
-        const uint64_t Dw = D >> (32 - pk);
-        const uint32_t Dq = Dw < 0xFFFFFFF0ull ? (uint32_t)Dw : 0xFFFFFFF0u;
         const uint32_t bmask = (1u << (8 + pk)) - 1u;  // q's bits inside a bucket
         const uint32_t *y = Y + 3u * (32u * c0 + lane);
         uint32_t q0 = sub_key(bswap32(y[1]), bswap32(y[2]), pk);
@@ -513,7 +516,7 @@ __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint3
             const uint32_t r = 32u * c + lane;
             y += 96;
             const uint32_t q1 = sub_key(bswap32(y[1]), bswap32(y[2]), pk);
-            const uint32_t lim = min(Dq, (~q0 & bmask) + 1u);  // at most to the bucket's end
+            const uint32_t lim = global ? Dq : min(Dq, (~q0 & bmask) + 1u);  // at most to the bucket's end
             auto diff = [&](uint32_t t) -> uint32_t {  // q of record r + t, less q_r (t < 32)
                 return __shfl_sync(0xffffffffu, lane < t ? q1 : q0, (lane + t) & 31u) - q0;
             };
@@ -525,8 +528,10 @@ __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint3
             uint32_t cnt = m5 ? 5u : m4 ? 4u : m3 ? 3u : m2 ? 2u : m1 ? 1u : 0u;
             // the nearest record that is no sure match
             uint32_t dn = m4 ? df[4] : m3 ? df[3] : m2 ? df[2] : m1 ? df[1] : df[0];
-            const int after = (int)(n - 1u - r);  // records after r
-            if (__any_sync(0xffffffffu, (m5 || dn - Dq <= 1u) && after > 0)) {
+            // records after r (none to count for r past the partition)
+            const int after = HALO ? (r < n ? (int)(nt - 1u - r) : 0) : (int)(n - 1u - r);
+            const bool edge = global && nt > n && q0 <= Dq + 1u && r + 32u >= n;
+            if (__any_sync(0xffffffffu, (m5 || edge || dn - Dq <= 1u) && after > 0)) {
                 bool more = m5 && after > 0;
                 for (uint32_t t = 6; __any_sync(0xffffffffu, more) && t < 32; ++t) {
                     const uint32_t x = diff(t);
@@ -534,7 +539,7 @@ __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint3
                     more = more && x < lim;
                     cnt += more ? 1u : 0u;
                 }
-                if ((more || dn - Dq <= 1u) && after > 0) cnt = count_exact(r);
+                if ((more || edge || dn - Dq <= 1u) && after > 0) cnt = count_exact(r);
             }
             enlist(c, min(cnt, (uint32_t)max(after, 0)));
             q0 = q1;

@@ -467,3 +467,19 @@ def test_many_pairs_per_record(vx, times, kw):
     r1, r2 = oracle_plot_global(K, key, D)
     assert np.array_equal(t1, r1)
     assert n2 == r2.shape[0] and np.array_equal(t2, r2)
+
+
+@pytest.mark.parametrize("frac", [0.02, 0.3, 0.9, 1.0])
+@pytest.mark.parametrize("K", [7, 9])
+@pytest.mark.parametrize("split", [False, True], ids=["fused", "split"])
+def test_cross_bucket_wide_distance(vx, K, frac, split):
+    # partitions of 64 records and a distance up to their width: records near
+    # the lower edge that see the halo, and distances of 2^32 and more in the
+    # 32 key bits the match compares
+    key = plot_key(600 + K)
+    D = int((1 << (64 - (K - 6))) * frac)
+    opts = vx.make_opts(match_scope=1, match_distance=D, partition_log2=6, t2_placement=1)
+    t1, t2, n2, _ = run_plot(vx, K, key, opts, split)
+    r1, r2 = oracle_plot_global(K, key, D)
+    assert np.array_equal(t1, r1)
+    assert n2 == r2.shape[0] and np.array_equal(t2, r2)
