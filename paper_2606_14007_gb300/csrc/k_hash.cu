@@ -30,6 +30,7 @@ __global__ void k_key_setup(Desc *descs)
         *d.status = 0u;
         *d.ticket = 0u;
         *d.ticket_s = 0u;
+        d.totals[0] = d.totals[1] = 0ull;
         if (d.wcount) *d.wcount = 0u;
     }
     const uint64_t n1 = d.p2 > 0 ? ((uint64_t)d.hchunks << d.p1) : 0ull;
@@ -489,7 +490,8 @@ cudaError_t launch_t2_hash(const Desc *descs, int nplots, const uint32_t *tile_s
 // barrier; two hashes per step (see b3_finish).
 __global__ void __launch_bounds__(kT2HashThreads) k_t2_hash_slots(const Desc *__restrict__ descs,
                                                                   int nplots,
-                                                                  const uint32_t *__restrict__ tile_start)
+                                                                  const uint32_t *__restrict__ tile_start,
+                                                                  bool split)
 {
     static_assert(kT2SlotGroup == kT2HashThreads / 32, "one partition per warp");
     pdl_go();
@@ -498,7 +500,7 @@ __global__ void __launch_bounds__(kT2HashThreads) k_t2_hash_slots(const Desc *__
     const Desc &d = descs[plot];
     // The run's result, final since the scan before this kernel, goes
     // straight to the caller's pinned words (three copies less per run).
-    if (d.result && blockIdx.x == tile_start[plot] && threadIdx.x == 0) {
+    if (d.result && !split && blockIdx.x == tile_start[plot] && threadIdx.x == 0) {
         d.result[0] = *d.status;
         d.result[1] = d.t2off[1ull << d.p];
         d.result[2] = d.t1off[1ull << d.p];
@@ -511,11 +513,12 @@ __global__ void __launch_bounds__(kT2HashThreads) k_t2_hash_slots(const Desc *__
     // (a broken chain has set a status bit, except for a withheld chunk 0
     // in a one-chunk scan).
     const uint64_t nchunks = (np + kScanChunk - 1) / kScanChunk;
-    if ((ld_acquire_u64(d.lb + (nchunks - 1)) & ~kLbMask) != kLbIncl) return;
+    if (!split && (ld_acquire_u64(d.lb + (nchunks - 1)) & ~kLbMask) != kLbIncl) return;
     const uint64_t off = d.t2off[f];
     const uint32_t cap = d.cap2;
-    // never past the pair slot (the sort flags this)
-    const uint32_t P = min((uint32_t)(d.t2off[f + 1] - off), cap + cap / 2u);
+    const uint64_t P64 = d.t2off[f + 1] - off;
+    if (P64 > cap + cap / 2u) return;  // past the pair slot: the sort left none
+    const uint32_t P = (uint32_t)P64;
     if (off + P > d.t2cap) return;  // the scan flags this; never write past Table 2
     uint32_t g[16];
 #pragma unroll
@@ -552,10 +555,10 @@ __global__ void __launch_bounds__(kT2HashThreads) k_t2_hash_slots(const Desc *__
 }
 
 cudaError_t launch_t2_hash_slots(const Desc *descs, int nplots, const uint32_t *tile_start,
-                                 uint32_t total_tiles, On on)
+                                 uint32_t total_tiles, On on, bool split)
 {
     if (total_tiles == 0) return cudaSuccess;
-    return launch_on(on, k_t2_hash_slots, total_tiles, kT2HashThreads, 0, descs, nplots, tile_start);
+    return launch_on(on, k_t2_hash_slots, total_tiles, kT2HashThreads, 0, descs, nplots, tile_start, split);
 }
 
 // ------------------------------------------------ tiled plots: windows

@@ -30,21 +30,12 @@ struct MatchLayout {
     }
 };
 
-__global__ void __launch_bounds__(kMatchThreads) k_match(const Desc *__restrict__ descs, int nplots,
-                                                         const uint32_t *__restrict__ tile_start)
+// Partition f of plot d: P pairs, Table-2 records from pbase on.  Ends with a
+// barrier.
+__device__ __forceinline__ void match_partition(const Desc &d, uint32_t f, uint64_t np, uint64_t pbase, uint32_t P,
+                                                unsigned char *smem_raw)
 {
     constexpr int NT = kMatchThreads;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_go();
-    pdl_wait();
-    const int plot = find_plot(tile_start, nplots, blockIdx.x);
-    const Desc &d = descs[plot];
-    const uint32_t f = blockIdx.x - tile_start[plot];
-    const uint64_t np = 1ull << d.p;
-    if (d.t2off[np] > d.t2cap) return;  // capacity exceeded: the scan flagged it
-    const uint64_t pbase = d.t2off[f];
-    const uint32_t P = (uint32_t)(d.t2off[f + 1] - pbase);
-    if (P == 0) return;
     const uint64_t off = d.t1off[f];
     const uint32_t n = (uint32_t)(d.t1off[f + 1] - off);
     const MatchLayout L(d.cap2 + d.hcap);  // + the next partition's halo
@@ -185,6 +176,43 @@ __global__ void __launch_bounds__(kMatchThreads) k_match(const Desc *__restrict_
     }
 }
 
+__global__ void __launch_bounds__(kMatchThreads) k_match(const Desc *__restrict__ descs, int nplots,
+                                                         const uint32_t *__restrict__ tile_start)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_go();
+    pdl_wait();
+    const int plot = find_plot(tile_start, nplots, blockIdx.x);
+    const Desc &d = descs[plot];
+    const uint32_t f = blockIdx.x - tile_start[plot];
+    const uint64_t np = 1ull << d.p;
+    if (d.t2off[np] > d.t2cap) return;  // capacity exceeded: the scan flagged it
+    const uint64_t pbase = d.t2off[f];
+    const uint32_t P = (uint32_t)(d.t2off[f + 1] - pbase);
+    if (P) match_partition(d, f, np, pbase, P, smem_raw);
+}
+
+// The partitions whose pairs did not fit their slot (next to never), found
+// 256 at a time; CTA row y takes plot y.
+__global__ void __launch_bounds__(kMatchThreads) k_match_over(const Desc *__restrict__ descs)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_go();
+    pdl_wait();
+    const Desc &d = descs[blockIdx.y];
+    const uint64_t np = 1ull << d.p;
+    if (d.t2off[np] > d.t2cap) return;
+    const uint64_t slot = d.cap2 + d.cap2 / 2u;
+    for (uint64_t f0 = (uint64_t)blockIdx.x * kMatchThreads; f0 < np; f0 += (uint64_t)gridDim.x * kMatchThreads) {
+        const uint64_t mine = f0 + threadIdx.x;
+        if (!__syncthreads_or(mine < np && d.t2off[mine + 1] - d.t2off[mine] > slot)) continue;
+        for (uint64_t f = f0; f < np && f < f0 + kMatchThreads; ++f) {
+            const uint64_t pbase = d.t2off[f], P = d.t2off[f + 1] - pbase;
+            if (P > slot) match_partition(d, (uint32_t)f, np, pbase, (uint32_t)P, smem_raw);
+        }
+    }
+}
+
 size_t match_smem_bytes(uint32_t cap) { return MatchLayout(cap).bytes; }
 
 cudaError_t launch_match(const Desc *descs, int nplots, const uint32_t *tile_start,
@@ -195,6 +223,25 @@ cudaError_t launch_match(const Desc *descs, int nplots, const uint32_t *tile_sta
     const cudaError_t e = allow_smem(k_match, smem, seen);
     if (e != cudaSuccess) return e;
     return launch_on(on, k_match, total_tiles, kMatchThreads, smem, descs, nplots, tile_start);
+}
+
+cudaError_t launch_match_over(const Desc *descs, int nplots, On on, uint32_t max_cap)
+{
+    static SmemSeen seen;
+    const size_t smem = match_smem_bytes(max_cap);
+    const cudaError_t e = allow_smem(k_match_over, smem, seen);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(152, (unsigned)nplots);
+    cfg.blockDim = dim3(kMatchThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = on.s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = on.pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_match_over, descs);
 }
 
 }  // namespace vx

@@ -245,6 +245,7 @@ __global__ void __launch_bounds__(kScanCtaThreads) k_scan_counts(const Desc *__r
     if (c + 1 == nchunks && threadIdx.x == 0) {
         const uint64_t all = s_base + total;
         out[n] = all;
+        d.totals[SRC == 0 ? 1 : 0] = all;
         if (SRC == 0) {
             // Every nonce exactly once; a window's share is random (the
             // windows of one plot add up to 2^K, checked by their caller).
@@ -326,6 +327,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_pairs(const Desc *__restr
     }
     if (threadIdx.x == 0) {
         out[n] = carry;
+        d.totals[0] = carry;
         // A re-run of the match (e.g. after a larger Table-2 buffer was
         // bound) re-decides the capacity bit.
         if (carry > d.t2cap) atomicOr(d.status, kStT2Capacity);

@@ -382,7 +382,7 @@ __device__ __forceinline__ void sort_bitmap(const Part &A, uint32_t n, int pk, u
 // written again, and for its end before the CTA exits.
 template <int MODE, bool HALO, int NT>
 __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint32_t n, uint64_t off,
-                                                const Part &A, uint64_t *s_base, int *s_ok)
+                                                const Part &A, uint64_t *s_base, int *s_ok, bool quiet)
 {
     constexpr bool EMIT = MODE == kSortHash || MODE == kSortEmit;  // look-back placement
     constexpr bool SLOTS = MODE == kSortSlots;
@@ -575,7 +575,7 @@ __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint3
                 if (got) {
                     const uint64_t np = 1ull << d.p;
                     d.t2off[f] = excl;
-                    if (f + 1 == np) d.t2off[np] = excl + P;
+                    if (f + 1 == np) d.t2off[np] = d.totals[0] = excl + P;
                     if (excl + P > d.t2cap) {
                         atomicOr(d.status, kStT2Capacity);
                         got = 0;
@@ -589,7 +589,7 @@ __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint3
         ok = *s_ok != 0;
         base = *s_base;
     } else if (P > d.cap2 + d.cap2 / 2u) {
-        if (threadIdx.x == 0) atomicOr(d.status, kStPairSlot);
+        if (threadIdx.x == 0 && !quiet) atomicOr(d.status, kStPairSlot);
         ok = false;
     }
     // 5. the pairs, in (i, j) order at their places: into the slot (key
@@ -725,7 +725,7 @@ __device__ __forceinline__ Item take_item(const Desc *__restrict__ descs, int np
 template <int MODE, bool HALO>
 __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
     k_sortmatch_pipe(const Desc *__restrict__ descs, int nplots, const uint32_t *__restrict__ tile_start,
-                     uint32_t items, uint32_t max_cap, uint32_t max_words)
+                     uint32_t items, uint32_t max_cap, uint32_t max_words, bool quiet)
 {
     constexpr bool EMIT = MODE == kSortHash || MODE == kSortEmit;
     constexpr int NT = kPipeThreads;
@@ -821,7 +821,7 @@ __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
                 A, n, d.pk, W, SharedSrc{XK, XN},
                 [&]() { bulk_wait_all<true>(); },  // the previous item's Table 1 has left Y
                 start_next);
-            match_and_write<MODE, HALO, NT>(d, f, n, off, A, &s_base, &s_ok);
+            match_and_write<MODE, HALO, NT>(d, f, n, off, A, &s_base, &s_ok, quiet);
         } else {
             __syncthreads();
             if (threadIdx.x == 0) start_next();
@@ -834,7 +834,7 @@ __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
 // ------------------------------------- one CTA per partition front end
 template <int MODE, bool HALO>
 __global__ void __launch_bounds__(kGlThreads, MODE == kSortHash ? 2 : 3)
-    k_sortmatch_gl(const Desc *__restrict__ descs, int nplots, const uint32_t *__restrict__ tile_start)
+    k_sortmatch_gl(const Desc *__restrict__ descs, int nplots, const uint32_t *__restrict__ tile_start, bool quiet)
 {
     constexpr bool EMIT = MODE == kSortHash || MODE == kSortEmit;
     constexpr int NT = kGlThreads;
@@ -872,7 +872,7 @@ __global__ void __launch_bounds__(kGlThreads, MODE == kSortHash ? 2 : 3)
         A, n, d.pk, W,
         GlobalSrc<MODE != kSortSlots>{d.b_keys + (uint64_t)f * cap, d.b_nonces + (uint64_t)f * cap}, []() {},
         []() {});
-    match_and_write<MODE, HALO, NT>(d, f, n, off, A, &s_base, &s_ok);
+    match_and_write<MODE, HALO, NT>(d, f, n, off, A, &s_base, &s_ok, quiet);
     if (threadIdx.x == 0) bulk_wait_all<false>();
 }
 
@@ -890,7 +890,7 @@ uint32_t sortmatch_max_cap() { return 16384u; }
 
 template <int MODE, bool HALO>
 static cudaError_t launch_sm(const Desc *descs, int nplots, const uint32_t *tile_start,
-                             uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits)
+                             uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits, bool quiet)
 {
     if (total_tiles == 0) return cudaSuccess;
     const uint32_t words = bitmap_words(max_dbits);
@@ -916,42 +916,42 @@ static cudaError_t launch_sm(const Desc *descs, int nplots, const uint32_t *tile
         }
         const uint32_t want = (uint32_t)fit;
         return launch_on(on, fn, want < total_tiles ? want : total_tiles, kPipeThreads, pipe, descs, nplots,
-                         tile_start, total_tiles, max_cap, words);
+                         tile_start, total_tiles, max_cap, words, quiet);
     }
     const size_t smem = SMLayout(max_cap, words, false).bytes;
     auto fn = k_sortmatch_gl<MODE, HALO>;
     static SmemSeen seen_gl;
     const cudaError_t e = allow_smem(fn, smem, seen_gl);
     if (e != cudaSuccess) return e;
-    return launch_on(on, fn, total_tiles, kGlThreads, smem, descs, nplots, tile_start);
+    return launch_on(on, fn, total_tiles, kGlThreads, smem, descs, nplots, tile_start, quiet);
 }
 
 template <int MODE>
 static cudaError_t launch_sm2(const Desc *descs, int nplots, const uint32_t *tile_start,
                               uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
-                              bool halo)
+                              bool halo, bool quiet)
 {
     // HALO instances carry the cross-bucket code; plain launches do not.
-    return halo ? launch_sm<MODE, true>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits)
-                : launch_sm<MODE, false>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits);
+    return halo ? launch_sm<MODE, true>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, quiet)
+                : launch_sm<MODE, false>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, quiet);
 }
 
 cudaError_t launch_sortmatch(const Desc *descs, int nplots, const uint32_t *tile_start,
                              uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
-                             SortMatchOut out, bool halo)
+                             SortMatchOut out, bool halo, bool quiet)
 {
     if (out == kOutLookbackHashed)
-        return launch_sm2<kSortHash>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo);
+        return launch_sm2<kSortHash>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo, false);
     if (out == kOutSlots)
-        return launch_sm2<kSortSlots>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo);
-    return launch_sm2<kSortEmit>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo);
+        return launch_sm2<kSortSlots>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo, quiet);
+    return launch_sm2<kSortEmit>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo, false);
 }
 
 cudaError_t launch_sort(const Desc *descs, int nplots, const uint32_t *tile_start,
                         uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
                         bool halo)
 {
-    return launch_sm2<kSortCount>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo);
+    return launch_sm2<kSortCount>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo, false);
 }
 
 }  // namespace vx

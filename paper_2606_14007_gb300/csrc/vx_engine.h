@@ -86,6 +86,7 @@ struct vx_plot {
     bool have_last = false;
     cudaEvent_t ev_done = nullptr;  // behind vx_plot_run's kernels and result copy
     bool res_pending = false;       // vx_sync reads the pinned result block after ev_done
+    bool slot_pairs = false;       // the last Table 1 left its pairs in the partition slots
     int stage = 0;                 // 0 created, 1 Table 1 issued, 2 match issued
     bool t2_known = false;
     uint64_t t2_count = 0;

@@ -85,6 +85,7 @@ struct Desc {
     uint64_t *lbs;       // [chunks] look-back words of the Table-1 offset scan
     uint32_t *ticket_s;  // chunk ticket of the Table-1 offset scan
     uint32_t *status;    // status word
+    uint64_t *totals;    // {Table-2 count, Table-1 count}, 8 bytes past the status word
     uint64_t *result;    // pinned host words {status, Table-2 count, Table-1 count}
                          //   the slot pair hash leaves the run's result in, or null
     uint8_t *t1;         // Table 1, 12-byte records
@@ -632,18 +633,22 @@ cudaError_t launch_hash_direct(const Desc *descs, int nplots, const uint32_t *ti
                                uint32_t total_tiles, int chunk, On on, HashCfg cfg);
 // Sort + match variants: Table-2 records at final offsets found by a
 // look-back ({a, b, 0, 0}, hashed later by launch_t2_hash; or hashed in the
-// kernel), or pairs {a, b} written into each partition's own slot.
+// kernel), or pairs {a, b} written into each partition's own slot (quiet: a
+// partition with more pairs than its slot holds leaves none and sets no
+// status bit; launch_match_over sees to it).
 enum SortMatchOut { kOutLookback = 0, kOutLookbackHashed = 1, kOutSlots = 2 };
 cudaError_t launch_sortmatch(const Desc *descs, int nplots, const uint32_t *tile_start,
                              uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
-                             SortMatchOut out, bool halo);
+                             SortMatchOut out, bool halo, bool quiet = false);
 cudaError_t launch_t2_hash(const Desc *descs, int nplots, const uint32_t *tile_start,
                            uint32_t total_tiles, int chunk, On on);
 // Pair hash of the slot placement: kT2SlotGroup partitions per CTA, pairs
-// read from the partition slots, records written at the scanned offsets.
+// read from the partition slots, records written at the scanned offsets
+// (split: offsets from launch_scan_pairs, partitions past their slot left to
+// launch_match_over).
 constexpr uint32_t kT2SlotGroup = 8;
 cudaError_t launch_t2_hash_slots(const Desc *descs, int nplots, const uint32_t *tile_start,
-                                 uint32_t total_tiles, On on);
+                                 uint32_t total_tiles, On on, bool split = false);
 constexpr uint64_t kT2HashTile = 256 * 8;  // Table-2 records per pair-hash CTA
 size_t sortmatch_smem_bytes(uint32_t cap, int dbits);
 uint32_t sortmatch_max_cap();  // largest slot the sort keeps in registers
@@ -663,6 +668,8 @@ cudaError_t launch_sort(const Desc *descs, int nplots, const uint32_t *tile_star
 cudaError_t launch_scan_pairs(const Desc *descs, int nplots, On on);
 cudaError_t launch_match(const Desc *descs, int nplots, const uint32_t *tile_start,
                          uint32_t total_tiles, On on, uint32_t max_cap);
+// The same for the partitions with more pairs than their slot holds.
+cudaError_t launch_match_over(const Desc *descs, int nplots, On on, uint32_t max_cap);
 cudaError_t launch_bucket_offsets(const Desc *desc, uint64_t *out, cudaStream_t s);
 // Table 2 sorted by hash2: grids of the five kernels of one sort.
 struct Sort2Launch {

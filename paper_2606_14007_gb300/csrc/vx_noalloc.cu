@@ -88,14 +88,10 @@ extern "C" int vx_plot_run_noalloc(int K, const uint8_t key[32], const vx_opts *
     // One stream, one kernel after the other (no second stream, no events).
     if (e == cudaSuccess) e = vx::launch_plot_seq(L, vx::Lanes{s, nullptr, nullptr, nullptr, p.plan.hchunks == 1 && p.plan.pchunks == 1});
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    uint32_t st = 0;
-    uint64_t total = 0;
+    uint64_t words[3] = {};  // {status, Table-2 count, Table-1 count}
     if (e == cudaSuccess)
-        e = cudaMemcpy(&st, p.d_scratch + p.plan.o_status, sizeof(st), cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(&total, p.d_scratch + p.plan.o_t2off + 8 * (1ull << p.plan.p), sizeof(total),
-                       cudaMemcpyDeviceToHost);
+        e = cudaMemcpy(words, p.d_scratch + p.plan.o_status, sizeof(words), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return VX_ECUDA;
-    if (t2_count) *t2_count = total;
-    return vx::map_status_ext(st);
+    if (t2_count) *t2_count = words[1];
+    return vx::map_status_ext((uint32_t)words[0]);
 }

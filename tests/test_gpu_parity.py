@@ -483,3 +483,29 @@ def test_cross_bucket_wide_distance(vx, K, frac, split):
     r1, r2 = oracle_plot_global(K, key, D)
     assert np.array_equal(t1, r1)
     assert n2 == r2.shape[0] and np.array_equal(t2, r2)
+
+
+@pytest.mark.parametrize("times", [1, 2, 3])
+def test_split_match_past_the_pair_slots(vx, times):
+    # split path, slots forced: at 2 and 3 times the default distance every
+    # partition (2048 records, 3912 places) has about 4096 and 6144 pairs, so
+    # some or all are matched again from Table 1; a second vx_match and one
+    # after a fused run give the same table
+    K, key = 15, plot_key(620)
+    D = orc.default_distance(K) * times
+    p = vx.Plot(K, key, vx.make_opts(match_scope=1, match_distance=D, t2_placement=2))
+    r1, r2 = oracle_plot_global(K, key, D)
+    p.run_split()
+    assert p.sync() == r2.shape[0]
+    assert np.array_equal(p.t1.cpu().numpy(), r1) and np.array_equal(p.t2.cpu().numpy(), r2)
+    p._t2.zero_()
+    p.match()
+    assert p.sync() == r2.shape[0] and np.array_equal(p.t2.cpu().numpy(), r2)
+    if times == 1:
+        p.run()
+        p.match()
+        assert p.sync() == r2.shape[0] and np.array_equal(p.t2.cpu().numpy(), r2)
+        vx.vx_plot_batch([p.handle])
+        p.match()
+        assert p.sync() == r2.shape[0] and np.array_equal(p.t2.cpu().numpy(), r2)
+    p.close()
