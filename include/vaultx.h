@@ -315,8 +315,8 @@ int vx_plot_tiled_bytes(int K, const vx_opts *opts, int window_bits, uint64_t *d
                         uint64_t *host_t1_bytes, uint64_t *host_t2_bytes);
 
 /* How many times vx_plot_tiled hashes every nonce at window_bits c, into
- * *passes: 1 for c = 0 (the whole plot), 2 for 1 <= c <= 8 without nonce
- * chunks (a first pass stores one window-id byte per nonce, then each window
+ * *passes, rounded up: 1 for c = 0 (the whole plot), 2 for 1 <= c <= 8 without
+ * nonce chunks (one pass stores a window-id byte per nonce, then a window
  * hashes only its own nonces), else 2^c (each window hashes every nonce and
  * keeps its share: at K=31 a hash pass takes ~51 ms, so c = 9 costs ~26 s).
  * The cost to weigh against vx_plot_tiled_bytes' footprint: above 8 bits
@@ -353,9 +353,10 @@ int vx_plot_tiled_window_bits(int K, const vx_opts *opts, uint64_t budget_bytes,
  * host_t2_bytes long.  The host tables equal the whole plot's (vx_plot_run
  * without windows) byte for byte.  Pinned host memory (cudaHostAlloc) makes
  * the copies asynchronous; pageable memory works but serialises them.
- * With 1..8 window bits a first pass hashes every nonce and stores its
- * window (one byte), and each window hashes only the nonces listed for it:
- * two hashes of every nonce in all.  With more window bits, or the hash
+ * With 1..8 window bits one pass hashes every nonce and stores its window
+ * (one byte; the first window's own hash does with the staged bucketing),
+ * and the windows after it hash only the nonces listed for them: at most two
+ * hashes of every nonce in all.  With more window bits, or the hash
  * split into nonce chunks (vx_opts.pipeline_chunks), each window hashes
  * every nonce and keeps its share.  *t1_count / *t2_count (may be
  * NULL) get the record counts.  Returns VX_OK; VX_ENOMEM if Table 2 did not

@@ -133,8 +133,10 @@ __device__ __forceinline__ bool scan_and_claim(S &t, int nbins, uint32_t *cnt, u
 // bits after those.  kWinFilter instances hash every nonce and test its key
 // (a plot without a window, wbits 0, keeps every key, so one such launch may
 // also carry whole plots); kWinList instances hash only the nonces listed
-// for the window (Desc::wlist, from a pass that stored every nonce's window).
-enum { kWinNone = 0, kWinFilter = 1, kWinList = 2 };
+// for the window (Desc::wlist, from a pass that stored every nonce's window);
+// kWinIds instances are kWinFilter ones that store the windows beside their
+// own records.
+enum { kWinNone = 0, kWinFilter = 1, kWinList = 2, kWinIds = 3 };
 
 // Window bits plus bin bits are at most the 21 partition bits, so both tests
 // read only the key's high word.
@@ -168,7 +170,7 @@ __global__ void __launch_bounds__(NT, NPT <= 12 ? 4 : 3) k_hash_scatter(const De
 {
     using S = HashTile<NT, NPT>;
     constexpr uint32_t T = S::T;
-    constexpr bool WIN = WM != kWinNone;
+    constexpr bool WIN = WM != kWinNone, FILTER = WM == kWinFilter || WM == kWinIds;
     static_assert(NPT % 2 == 0 && 2 * T <= 0x10000u && (4u << kMaxCoarseBits) < kNoBin, "16-bit offsets");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S &sm = *reinterpret_cast<S *>(smem_raw);
@@ -215,11 +217,12 @@ __global__ void __launch_bounds__(NT, NPT <= 12 ? 4 : 3) k_hash_scatter(const De
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const uint32_t i = i0 + u * NT;
-                const bool valid = i < left && (WM != kWinFilter || in_window<true>(d, key[u]));
+                const bool valid = i < left && (!FILTER || in_window<true>(d, key[u]));
                 const uint32_t bin4 = 4u * key_bin<WIN>(d, key[u], bits);
                 sm.keys[i] = key[u];
+                if (WM == kWinIds && i < left) d.wids[base + i] = (uint8_t)(key[u] >> (64 - d.wbits));
                 sm.rank2[i] = (uint16_t)(2u * bin_rank<AGG>(sm.start2, bin4, valid));
-                sm.bin4[i] = (uint16_t)(WM != kWinFilter || valid ? bin4 : kNoBin);
+                sm.bin4[i] = (uint16_t)(!FILTER || valid ? bin4 : kNoBin);
             }
         }
     }
@@ -233,7 +236,7 @@ __global__ void __launch_bounds__(NT, NPT <= 12 ? 4 : 3) k_hash_scatter(const De
 #pragma unroll 4
     for (uint32_t i = threadIdx.x; i < left; i += NT) {
         const uint32_t bin4 = sm.bin4[i];
-        if (WM != kWinFilter || bin4 != kNoBin)
+        if (!FILTER || bin4 != kNoBin)
             at_bytes(sm.order, at_bytes(sm.start2, bin4) + sm.rank2[i]) = (uint16_t)i;
     }
     __syncthreads();
@@ -297,16 +300,13 @@ template <bool HALO, int WM>
 static cudaError_t launch_hs_agg(const Desc *descs, int nplots, const uint32_t *tile_start,
                                  uint32_t total_tiles, bool agg, int chunk, On on, int npt)
 {
-    if (WM != kWinNone)
-        return npt == kHashNoncesPerThread
-                   ? launch_hs_npt<HALO, WM, kHashNoncesPerThread>(descs, nplots, tile_start, total_tiles, agg, chunk, on)
-                   : cudaErrorInvalidValue;
+    if (WM != kWinNone && npt != kHashNoncesPerThread && npt != 16) return cudaErrorInvalidValue;
     switch (npt) {
     case 2: return launch_hs_npt<HALO, kWinNone, 2>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
     case 4: return launch_hs_npt<HALO, kWinNone, 4>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
-    case 8: return launch_hs_npt<HALO, kWinNone, 8>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
+    case 8: return launch_hs_npt<HALO, WM, 8>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
     case 12: return launch_hs_npt<HALO, kWinNone, 12>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
-    case 16: return launch_hs_npt<HALO, kWinNone, 16>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
+    case 16: return launch_hs_npt<HALO, WM, 16>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -319,6 +319,9 @@ cudaError_t launch_hash_scatter(const Desc *descs, int nplots, const uint32_t *t
     if (cfg.list)
         return cfg.halo ? cudaErrorInvalidValue
                         : launch_hs_agg<false, kWinList>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt);
+    if (cfg.ids)
+        return cfg.halo ? cudaErrorInvalidValue
+                        : launch_hs_agg<false, kWinIds>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt);
     if (cfg.win)
         return cfg.halo ? launch_hs_agg<true, kWinFilter>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt)
                         : launch_hs_agg<false, kWinFilter>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt);
@@ -405,6 +408,7 @@ cudaError_t launch_hash_direct(const Desc *descs, int nplots, const uint32_t *ti
                                uint32_t total_tiles, int chunk, On on, HashCfg cfg)
 {
     if (total_tiles == 0) return cudaSuccess;
+    if (cfg.ids) return cudaErrorInvalidValue;
     if (cfg.list)
         return cfg.halo ? cudaErrorInvalidValue
                         : launch_hd<false, kWinList>(descs, nplots, tile_start, total_tiles, chunk, on);

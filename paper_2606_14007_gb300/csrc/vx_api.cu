@@ -33,7 +33,6 @@ using vx::Desc;
 using vx::LaunchSet;
 
 namespace vx {
-static_assert(kPlanHashTile == (uint64_t)kHashTile, "planner and hash kernel tiles differ");
 static_assert(kPlanScanChunk == (uint64_t)kScanChunk, "planner and scan kernel chunks differ");
 static_assert(kPlanScatterTile == (uint64_t)kScatterTile, "planner and scatter kernel tiles differ");
 static_assert(kPlanT2HashTile == kT2HashTile, "planner and pair-hash kernel tiles differ");
@@ -197,7 +196,7 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
     const int W = n + 1;
     enum { A_STG = 0, A_DIR = 8, A_S2 = 16, A_PC = 24, A_T2H = 32, A_SCAN = 40, A_PART = 41 };
     static_assert(A_PART + 1 == vx::kTileArrays, "tile arrays");
-    bool fuse = true, slots = true, halo = false, win = false, list = false;
+    bool fuse = true, slots = true, halo = false, win = false, list = false, ids = false;
     L->G = L->C = 1;
     L->max_cap2 = 0;
     L->max_dbits = 1;
@@ -221,7 +220,8 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
         if (plots[i]->wids && pl.wbits) {
             // a listed window runs alone, its hash in one nonce chunk
             if (n != 1 || pl.hchunks != 1) return VX_EINVAL;
-            list = true;
+            ids = plots[i]->store_ids;
+            list = !ids;
         }
         L->G = std::max(L->G, pl.hchunks);
         L->C = std::max(L->C, pl.pchunks);
@@ -268,6 +268,7 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
     L->halo = halo;
     L->win = win;
     L->list = list;
+    L->ids = ids;
     L->list_N = list ? plots[0]->plan.N : 0;
     for (int g = 0; g < vx::kMaxChunks; ++g) {
         L->t_staged[g] = d + (A_STG + g) * W;
@@ -408,10 +409,10 @@ cudaError_t launch_front(const LaunchSet &L, const vx::Lanes &ln, const vx::Trac
     for (int g = 0; g < L.G; ++g) {
         if (L.n_staged[g])
             VX_LAUNCH(KID_STAGED, A, vx::launch_hash_scatter(L.descs, L.n, L.t_staged[g], L.n_staged[g],
-                                                             vx::HashCfg{L.agg, L.halo, L.win, L.list, L.npt}, g, on));
+                                                             vx::HashCfg{L.agg, L.halo, L.win, L.list, L.ids, L.npt}, g, on));
         if (L.n_direct[g])
             VX_LAUNCH(KID_DIRECT, A, vx::launch_hash_direct(L.descs, L.n, L.t_direct[g], L.n_direct[g], g, on,
-                                                            vx::HashCfg{L.agg, L.halo, L.win, L.list, L.npt}));
+                                                            vx::HashCfg{L.agg, L.halo, L.win, L.list, L.ids, L.npt}));
         if (L.n_s2[g]) {
             if (ov) {
                 cudaEventRecord(ln.sync[g], A);

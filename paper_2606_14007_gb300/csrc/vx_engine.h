@@ -42,6 +42,7 @@ struct LaunchSet {
     bool halo;         // some plot matches across buckets: kernels with the halo code
     bool win;          // some plot is a window: hash kernels with the window filter
     bool list;         // the one plot hashes its window's nonce list (tiled plots)
+    bool ids;          // the one plot stores every nonce's window id (tiled plots, first window)
     uint64_t list_N;   // its nonce count (the list kernel's input)
     uint32_t max_cap2;
     int max_dbits;
@@ -92,8 +93,10 @@ struct vx_plot {
     uint64_t t2_count = 0;
     bool t1_known = false;          // a window's Table-1 count, read by vx_sync
     uint64_t t1_count = 0;
-    const uint8_t *wids = nullptr;  // window id of every nonce (tiled plots): the
+    uint8_t *wids = nullptr;        // window id of every nonce (tiled plots): the
                                     // window hashes its listed nonces only
+    bool store_ids = false;         // ... or, the first window, hashes every nonce and
+                                    // stores the ids beside its own records
     uint32_t status = 0;
     std::string err;
     // Second streams and fork/join events of the pipelined run.

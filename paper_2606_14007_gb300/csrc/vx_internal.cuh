@@ -64,7 +64,7 @@ struct Desc {
     uint32_t wbits;      // window: the plot keeps the records whose top wbits
     uint32_t win;        //   key bits equal win (wbits 0: every record)
     uint32_t listcap;    // window nonce list capacity (entries), if wids
-    const uint8_t *wids; // window id of every nonce (top wbits of key64), or null:
+    uint8_t *wids;       // window id of every nonce (top wbits of key64), or null:
                          //   the hash kernels then hash every nonce and filter
     uint32_t *wlist;     // [listcap] the window's nonces, listed from wids
     uint32_t *wcount;    // entries in wlist (zeroed by the key setup)
@@ -622,7 +622,8 @@ struct HashCfg {
     bool halo;    // some plot of the launch matches across buckets (halo code)
     bool win;     // some plot of the launch is a window (window filter)
     bool list;    // the launch's one plot hashes its window's nonce list
-    int npt;      // nonces per thread of the staged Table-1 hash (2, 4, 8, 12, 16; 8 with a window)
+    bool ids;     // the launch's one plot, a window, stores every nonce's window id
+    int npt;      // nonces per thread of the staged Table-1 hash (2, 4, 8, 12, 16; 8 or 16 with a window)
 };
 cudaError_t launch_key_setup(Desc *descs, int nplots, On on);
 // Hash kernels and the second scatter level take one nonce chunk (of
@@ -696,5 +697,4 @@ size_t sort_smem_bytes(uint32_t cap, int dbits);
 size_t match_smem_bytes(uint32_t cap);
 constexpr int kHashThreads = 256;
 constexpr int kHashNoncesPerThread = 8;
-constexpr int kHashTile = kHashThreads * kHashNoncesPerThread;
 }  // namespace vx

@@ -11,9 +11,12 @@
 // moving the 26 GB of unsorted records across the host link once, so
 // recomputing beats spilling the records and reading them back.
 //
-// A first pass hashes every nonce once and stores its window (one byte);
-// each window then lists its own nonces from those bytes and hashes only
-// them, so a plot of 2^c windows costs two hashes of every nonce, not 2^c.
+// The first window hashes every nonce, keeps its own records and stores each
+// nonce's window (one byte); every other window lists its own nonces from
+// those bytes and hashes only them, so a plot of 2^c windows costs less than
+// two hashes of every nonce, not 2^c.  (The copies of the tables bound a
+// tiled plot: with the ids from a pass of their own the first copy of a K=26
+// plot in four windows started 0.5 ms later.)
 // (Without the byte array -- more than 8 window bits, or the hash split
 // into nonce chunks -- each window hashes every nonce and keeps its share.)
 //
@@ -120,7 +123,9 @@ int tiled_run(int K, const uint8_t key[32], const vx_opts *opts, int window_bits
             for (int i = 0; i < 8; ++i)
                 kw[i] = (uint32_t)key[4 * i] | ((uint32_t)key[4 * i + 1] << 8) |
                         ((uint32_t)key[4 * i + 2] << 16) | ((uint32_t)key[4 * i + 3] << 24);
-            if (vx::launch_window_ids(kw, N, window_bits, ids, s) != cudaSuccess) rc = VX_ECUDA;
+            // The staged hash of the first window stores the ids itself.
+            if (pl.mode != vx::kScatterStaged && vx::launch_window_ids(kw, N, window_bits, ids, s) != cudaSuccess)
+                rc = VX_ECUDA;
             for (int i = 0; i < nbuf; ++i) P[i]->wids = ids;
         }
     }
@@ -164,6 +169,7 @@ int tiled_run(int K, const uint8_t key[32], const vx_opts *opts, int window_bits
         X->plan.win = w;
         X->opts.window = w;
         X->desc_dirty = true;
+        X->store_ids = w == 0 && ids && pl.mode == vx::kScatterStaged;
         rc = vx_plot_run(X, s);
         if (rc == VX_OK && w >= 1) rc = drain(slot ^ 1);
     }
