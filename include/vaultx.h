@@ -79,7 +79,8 @@ typedef struct vx_opts {
                                    counterpart                                       */
     uint64_t match_distance;    /* D of the match predicate; 0 = 2^(64-K)            */
     int32_t partition_log2;     /* log2 of the mean records per physical partition
-                                   (6..13); 0 = default (11).  Partitions are runs
+                                   (6..13); 0 = automatic (11; 9 or 10 for small
+                                   whole plots, K <= 18).  Partitions are runs
                                    of whole logical buckets; at most 2^24 of them.  */
     int32_t coarse_bits;        /* bits of the first scatter level (0..10);
                                    -1 = automatic                                     */

@@ -139,6 +139,14 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
     P.N = 1ull << K;
     P.D = opts.match_distance ? opts.match_distance : (1ull << (64 - K));
     P.s = opts.partition_log2 ? opts.partition_log2 : kDefaultPartLog2;
+    // Small whole plots leave most SMs idle with 2048-record partitions: one
+    // partition's sort is then the time (run, back to back, with 2^9 / 2^10 /
+    // 2^11 records: K=12 22.1 / 22.8 / 26.2 us, K=16 24.4 / 25.6 / 28.0,
+    // K=18 39.5 / 34.6 / 37.0, K=19 55.7 / 49.6 / 46.5).  Options that the
+    // partition count bears on keep the fixed size.
+    if (!opts.partition_log2 && K <= 18 && opts.coarse_bits < 0 && !opts.window_bits && !opts.match_scope &&
+        !opts.t2_placement)
+        P.s = K <= 16 ? 9 : 10;
     if (P.s < 6 || P.s > 13) {
         *why = "partition_log2 must be in 6..13";
         return VX_EINVAL;
