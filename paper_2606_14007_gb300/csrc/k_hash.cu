@@ -63,13 +63,14 @@ cudaError_t launch_key_setup(Desc *descs, int nplots, On on)
 // (which becomes the bin's start in the tile) and the bin's place.  Bins,
 // ranks and starts are kept as the byte offsets they are used at (4 * bin,
 // 2 * rank, 2 * start), so that no use of them costs a shift.
-template <int NT, int NPT>
+// CB: the most first-level bits the instance handles.
+template <int NT, int NPT, int CB>
 struct HashTile {
     static constexpr uint32_t T = NT * NPT;
     uint64_t keys[T];
     uint16_t bin4[T], rank2[T], order[T];
-    uint32_t start2[1 << kMaxCoarseBits];
-    uint32_t place[1 << kMaxCoarseBits];
+    uint32_t start2[1 << CB];
+    uint32_t place[1 << CB];
     uint32_t ws[NT / 32 + 1];
 };
 constexpr uint32_t kNoBin = 0xFFFFu;
@@ -101,10 +102,10 @@ __device__ __forceinline__ uint32_t bin_rank(uint32_t *hist, uint32_t bin4, bool
 // claim per non-empty bin; place[b] = b * cap + claim - start, so record i of
 // the bin-ordered tile goes to slot index place[bin] + i (32 bits, wrapping).
 // *total gets the records of the tile; true if a claim passes its slot's end.
-template <int NT, class S>
+template <int NT, int CB, class S>
 __device__ __forceinline__ bool scan_and_claim(S &t, int nbins, uint32_t *cnt, uint32_t cap, uint32_t *total)
 {
-    constexpr int PB = ((1 << kMaxCoarseBits) + NT - 1) / NT;  // most bins a thread owns
+    constexpr int PB = ((1 << CB) + NT - 1) / NT;  // most bins a thread owns
     const int per = (nbins + NT - 1) / NT;
     const int b0 = threadIdx.x * per;
     uint32_t h[PB], local = 0;
@@ -163,15 +164,15 @@ __device__ __forceinline__ uint32_t key_bin(const Desc &d, uint64_t key, int bit
 // by bin as 16-bit record indices instead of moved records; slot places as
 // 32-bit indices whose addresses are multiply-adds on the FMA pipe.  The
 // extra shared-memory traffic is free: that path idles at 17% here.
-template <int NT, int NPT, bool AGG, bool HALO, int WM>
+template <int NT, int NPT, bool AGG, bool HALO, int WM, int CB>
 __global__ void __launch_bounds__(NT, NPT <= 12 ? 4 : 3) k_hash_scatter(const Desc *__restrict__ descs, int nplots,
                                                      const uint32_t *__restrict__ tile_start,
                                                      int chunk)
 {
-    using S = HashTile<NT, NPT>;
+    using S = HashTile<NT, NPT, CB>;
     constexpr uint32_t T = S::T;
     constexpr bool WIN = WM != kWinNone, FILTER = WM == kWinFilter || WM == kWinIds;
-    static_assert(NPT % 2 == 0 && 2 * T <= 0x10000u && (4u << kMaxCoarseBits) < kNoBin, "16-bit offsets");
+    static_assert(NPT % 2 == 0 && 2 * T <= 0x10000u && (4u << CB) < kNoBin, "16-bit offsets");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S &sm = *reinterpret_cast<S *>(smem_raw);
 
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(NT, NPT <= 12 ? 4 : 3) k_hash_scatter(const De
     if (WM != kWinList) pdl_wait();  // up to here only the descriptor was read
     __syncthreads();
     uint32_t count;  // records the tile keeps
-    const bool over = scan_and_claim<NT>(sm, nbins, cnt, cap, &count);
+    const bool over = scan_and_claim<NT, CB>(sm, nbins, cnt, cap, &count);
     // Every place fits 32 bits unless all slots together hold 2^32 records
     // or more (K = 32 in two levels).
     const bool slow = __syncthreads_or(over) || ((uint64_t)cap << bits) > 0xFFFFFFFFull;
@@ -270,14 +271,14 @@ __global__ void __launch_bounds__(NT, NPT <= 12 ? 4 : 3) k_hash_scatter(const De
     if (hover) atomicOr(d.status, kStHaloOverflow);
 }
 
-template <int NPT, bool AGG, bool HALO, int WM>
+template <int NPT, bool AGG, bool HALO, int WM, int CB = kMaxCoarseBits>
 static cudaError_t launch_hs(const Desc *descs, int nplots, const uint32_t *tile_start,
                              uint32_t total_tiles, int chunk, On on)
 {
     constexpr int NT = kHashThreads;
     static SmemSeen seen;
-    const size_t smem = sizeof(HashTile<NT, NPT>);
-    auto fn = k_hash_scatter<NT, NPT, AGG, HALO, WM>;
+    const size_t smem = sizeof(HashTile<NT, NPT, CB>);
+    auto fn = k_hash_scatter<NT, NPT, AGG, HALO, WM, CB>;
     const cudaError_t e = allow_smem(fn, smem, seen);
     if (e != cudaSuccess) return e;
     return launch_on(on, fn, total_tiles, NT, smem, descs, nplots, tile_start, chunk);
@@ -298,9 +299,16 @@ static cudaError_t launch_hs_npt(const Desc *descs, int nplots, const uint32_t *
 
 template <bool HALO, int WM>
 static cudaError_t launch_hs_agg(const Desc *descs, int nplots, const uint32_t *tile_start,
-                                 uint32_t total_tiles, bool agg, int chunk, On on, int npt)
+                                 uint32_t total_tiles, bool agg, int chunk, On on, int npt, int bits)
 {
     if (WM != kWinNone && npt != kHashNoncesPerThread && npt != 16) return cudaErrorInvalidValue;
+    if (bits > kMaxCoarseBits) {  // 2^20 partitions and more: tiles of 4096 only
+        if constexpr (WM == kWinNone || WM == kWinFilter)
+            return npt == 16 ? launch_hs<16, false, HALO, WM, kMaxCoarseBitsWide>(descs, nplots, tile_start, total_tiles,
+                                                                                 chunk, on)
+                             : cudaErrorInvalidValue;
+        return cudaErrorInvalidValue;
+    }
     switch (npt) {
     case 2: return launch_hs_npt<HALO, kWinNone, 2>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
     case 4: return launch_hs_npt<HALO, kWinNone, 4>(descs, nplots, tile_start, total_tiles, agg, chunk, on);
@@ -318,15 +326,15 @@ cudaError_t launch_hash_scatter(const Desc *descs, int nplots, const uint32_t *t
     const int npt = cfg.npt;
     if (cfg.list)
         return cfg.halo ? cudaErrorInvalidValue
-                        : launch_hs_agg<false, kWinList>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt);
+                        : launch_hs_agg<false, kWinList>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt, cfg.bits);
     if (cfg.ids)
         return cfg.halo ? cudaErrorInvalidValue
-                        : launch_hs_agg<false, kWinIds>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt);
+                        : launch_hs_agg<false, kWinIds>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt, cfg.bits);
     if (cfg.win)
-        return cfg.halo ? launch_hs_agg<true, kWinFilter>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt)
-                        : launch_hs_agg<false, kWinFilter>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt);
-    return cfg.halo ? launch_hs_agg<true, kWinNone>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt)
-                    : launch_hs_agg<false, kWinNone>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt);
+        return cfg.halo ? launch_hs_agg<true, kWinFilter>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt, cfg.bits)
+                        : launch_hs_agg<false, kWinFilter>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt, cfg.bits);
+    return cfg.halo ? launch_hs_agg<true, kWinNone>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt, cfg.bits)
+                    : launch_hs_agg<false, kWinNone>(descs, nplots, tile_start, total_tiles, cfg.agg, chunk, on, npt, cfg.bits);
 }
 
 // ------------------------------------------------- hash + direct scatter

@@ -201,7 +201,7 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
     L->max_cap2 = 0;
     L->max_dbits = 1;
     L->max_p2 = 0;
-    int min_bits = 64;
+    int min_bits = 64, max_bits = 0;
     // One staged hash launch takes one shape: the plots' common nonces per
     // thread, else the automatic one of their nonces together (any shape
     // gives the same records).
@@ -228,9 +228,13 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
         L->max_cap2 = std::max(L->max_cap2, pl.cap2 + pl.hcap);
         L->max_dbits = std::max(L->max_dbits, pl.dbits);
         L->max_p2 = std::max(L->max_p2, pl.p2);
-        if (pl.mode == kScatterStaged) min_bits = std::min(min_bits, pl.p2 > 0 ? pl.p1 : pl.p);
+        if (pl.mode == kScatterStaged) {
+            min_bits = std::min(min_bits, pl.p2 > 0 ? pl.p1 : pl.p);
+            max_bits = std::max(max_bits, pl.p2 > 0 ? pl.p1 : pl.p);
+        }
     }
-    if (!same_npt) npt = win ? kPlanNoncesPerThread : vx::auto_nonces_per_thread(nonces);
+    if (max_bits > vx::kMaxCoarseBits) npt = 16;  // the one tile with more bins
+    else if (!same_npt) npt = win ? kPlanNoncesPerThread : vx::auto_nonces_per_thread(nonces);
     uint64_t acc[vx::kTileArrays] = {};
     for (int a = 0; a < vx::kTileArrays; ++a) h[a * W] = 0;
     for (int i = 0; i < n; ++i) {
@@ -262,6 +266,7 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
     }
     L->n = n;
     L->agg = min_bits <= kAggMaxBits;
+    L->hash_bits = max_bits;
     L->npt = npt;
     L->fuse_pair_hash = fuse;
     L->pair_slots = slots;
@@ -409,10 +414,10 @@ cudaError_t launch_front(const LaunchSet &L, const vx::Lanes &ln, const vx::Trac
     for (int g = 0; g < L.G; ++g) {
         if (L.n_staged[g])
             VX_LAUNCH(KID_STAGED, A, vx::launch_hash_scatter(L.descs, L.n, L.t_staged[g], L.n_staged[g],
-                                                             vx::HashCfg{L.agg, L.halo, L.win, L.list, L.ids, L.npt}, g, on));
+                                                             vx::HashCfg{L.agg, L.halo, L.win, L.list, L.ids, L.hash_bits, L.npt}, g, on));
         if (L.n_direct[g])
             VX_LAUNCH(KID_DIRECT, A, vx::launch_hash_direct(L.descs, L.n, L.t_direct[g], L.n_direct[g], g, on,
-                                                            vx::HashCfg{L.agg, L.halo, L.win, L.list, L.ids, L.npt}));
+                                                            vx::HashCfg{L.agg, L.halo, L.win, L.list, L.ids, L.hash_bits, L.npt}));
         if (L.n_s2[g]) {
             if (ov) {
                 cudaEventRecord(ln.sync[g], A);

@@ -16,6 +16,7 @@ namespace vx {
 constexpr int kBucketBits = 24;          // 2^24 logical buckets (Sec. I-A, III-B)
 constexpr int kMaxK = 32;                // u32 nonces
 constexpr int kMaxCoarseBits = 10;       // first scatter level, <= 1024 bins
+constexpr int kMaxCoarseBitsWide = 11;   // ... up to 2048 (2^20 partitions and more)
 constexpr int kMaxFineBits = 10;         // second scatter level, <= 1024 bins
 constexpr int kMaxFineBitsWide = 11;     // ... up to 2048 (2^21 partitions, K = 32)
 constexpr int kScatterTile = 4096;       // records per CTA in the second scatter level
@@ -623,6 +624,7 @@ struct HashCfg {
     bool win;     // some plot of the launch is a window (window filter)
     bool list;    // the launch's one plot hashes its window's nonce list
     bool ids;     // the launch's one plot, a window, stores every nonce's window id
+    int bits;     // most first-level bits of the launch's plots (staged hash)
     int npt;      // nonces per thread of the staged Table-1 hash (2, 4, 8, 12, 16; 8 or 16 with a window)
 };
 cudaError_t launch_key_setup(Desc *descs, int nplots, On on);

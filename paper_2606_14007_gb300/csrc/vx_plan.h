@@ -230,10 +230,14 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
         // writes longer runs (K = 30: 9 + 10 bits 25.62 + 8.01 ms, 10 + 9
         // bits 25.73 + 6.36); below 15 bits a few fewer (K = 25: 9 + 5 bits
         // 2139 us per plot, 10 + 4 bits 2154, 7 + 7 bits 2142).
-        P.p1 = P.p <= 10 ? P.p : P.p < 14 ? 8 : P.p == 14 ? 9 : 10;
+        // At 2^20 partitions and more 11 bits, which the largest tile's
+        // kernel also takes (K = 31: 10 + 10 bits 48.5 + 15.6 ms, 11 + 9
+        // bits 49.1 + 13.0; K = 32: 10 + 11 bits 99.6 + 55.0, 11 + 10 bits
+        // 100.7 + 31.1).
+        P.p1 = P.p <= 10 ? P.p : P.p < 14 ? 8 : P.p == 14 ? 9 : P.p < 20 || P.wbits || P.npt != 16 ? 10 : 11;
     }
     P.p2 = P.p - P.p1;
-    if (P.mode == kScatterStaged && (P.p1 > 10 || P.p2 > 11)) {
+    if (P.mode == kScatterStaged && (P.p1 > (opts.coarse_bits < 0 ? 11 : 10) || P.p2 > 11)) {
         *why = "coarse_bits leaves a scatter level wider than 10 (first) or 11 (second) bits";
         return VX_EINVAL;
     }

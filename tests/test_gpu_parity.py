@@ -509,3 +509,32 @@ def test_split_match_past_the_pair_slots(vx, times):
         p.match()
         assert p.sync() == r2.shape[0] and np.array_equal(p.t2.cpu().numpy(), r2)
     p.close()
+
+
+@pytest.mark.parametrize("scope", [0, 1], ids=["bucket", "cross"])
+def test_two_to_the_20_partitions(vx, scope):
+    # first scatter level of 11 bits (2^20 partitions of 64 records), alone
+    # and in a batch with a window, against the plan of 2^15 partitions
+    K, key = 26, plot_key(640)
+    D = 1 << 34
+    a = vx.Plot(K, key, vx.make_opts(match_scope=scope, match_distance=D))
+    a.run()
+    n = a.sync()
+    b = vx.Plot(K, key, vx.make_opts(match_scope=scope, match_distance=D, partition_log2=6))
+    b.run()
+    assert b.sync() == n and torch.equal(a.t1, b.t1) and torch.equal(a.t2, b.t2)
+    w = vx.Plot(16, key, vx.make_opts(window_bits=2, window=1))
+    b._t1.zero_()
+    b._t2.zero_()
+    vx.vx_plot_batch([b.handle, w.handle])
+    w.sync()
+    assert b.sync() == n and torch.equal(a.t1, b.t1) and torch.equal(a.t2, b.t2)
+    for p in (a, b, w):
+        p.close()
+
+
+def test_coarse_bits_past_ten_stay_refused(vx):
+    for K in (24, 31):
+        with pytest.raises(vx.VxError) as e:
+            vx.vx_plot_required_bytes(K, vx.make_opts(coarse_bits=11))
+        assert e.value.code == vx.VX_EINVAL
