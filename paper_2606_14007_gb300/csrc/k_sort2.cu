@@ -16,12 +16,9 @@
 
 namespace vx {
 
-constexpr int kS2Threads = 512;              // first level: 512 threads x 8 records
-constexpr int kS2PerThread = 8;
-constexpr uint32_t kS2Tile1 = kS2Threads * kS2PerThread;
-static_assert(kS2Tile1 == kPlanS2Tile1, "planner and first-level sort tiles differ");
-constexpr int kS2BThreads = 512;             // second level: 512 threads x 8 records
-constexpr uint32_t kS2Tile2 = 4096;
+constexpr int kS2Threads = 512;              // both levels: 512 threads x 8 records
+constexpr uint32_t kS2Tile = 4096;
+static_assert(kS2Tile == kPlanS2Tile1, "planner and scatter tiles differ");
 constexpr int kS2SortThreads = 256;
 
 __device__ __forceinline__ uint64_t sort2_key(uint4 r)
@@ -45,186 +42,109 @@ __global__ void k_s2_setup(Sort2Desc *dp)
     }
 }
 
-// ---------------------------------------------------- first scatter level
-// A CTA takes kS2Tile1 consecutive Table-2 records, ranks them in shared memory
-// by their level bin, claims one run per (CTA, bin) with a global atomic,
-// and writes them bin by bin (key2 and the packed pair (a << 32 | b)).
-struct S2Smem1 {
-    uint64_t keys[kS2Tile1];
-    uint64_t vals[kS2Tile1];
-    uint32_t hist[1 << kMaxCoarseBits];
-    uint32_t loff[1 << kMaxCoarseBits];
-    uint32_t gbase[1 << kMaxCoarseBits];
-    uint32_t ws[kS2Threads / 32 + 1];
+// ------------------------------------------------------- scatter levels
+// A CTA takes a tile of up to kS2Tile records (level 1: of Table 2, level 2:
+// of a first-level slot) by one bulk copy, ranks them by their bin, claims
+// one run per (CTA, bin) with a global atomic (its result first needed after
+// the order is known), and writes the records bin by bin.  Bound by shared
+// memory (90% of its wavefronts, most of them the random 16-byte reads on
+// the way out), close to HBM: 58.7 M records take 299 and 307 us, 6.3 TB/s
+// (543 and 380 with keys and pairs in arrays of their own, held in registers
+// over an in-place restage: two CTAs per SM, the first level's loads one
+// after the other).  The records stay where the copy left them: a 16-bit
+// order says which one goes next, so no registers hold them and three CTAs
+// fit an SM up to 9 bits, with the bin counters sized to the level.
+struct S2ScatterLayout {
+    size_t order, hist, ws, bar, bytes;
+    __host__ __device__ explicit S2ScatterLayout(int bits)
+    {
+        order = (size_t)kS2Tile * 16;
+        hist = order + (size_t)kS2Tile * 2;
+        ws = hist + ((size_t)4 << bits);
+        bar = (ws + (kS2Threads / 32 + 1) * 4 + 7) & ~(size_t)7;
+        bytes = bar + 8;
+    }
 };
 
-__global__ void __launch_bounds__(kS2Threads) k_s2_scatter1(const Sort2Desc *__restrict__ dp)
+template <int LEVEL>
+__global__ void __launch_bounds__(kS2Threads, 3) k_s2_scatter(const Sort2Desc *__restrict__ dp)
 {
-    constexpr int NT = kS2Threads, PER = kS2PerThread;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    S2Smem1 &sm = *reinterpret_cast<S2Smem1 *>(smem_raw);
+    constexpr int NT = kS2Threads, PER = kS2Tile / NT;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
     const Sort2Desc &d = *dp;
-    const uint64_t n = *d.count;
-    const uint64_t base = (uint64_t)blockIdx.x * kS2Tile1;
-    if (base >= n) return;
-    const bool two_level = d.p2 > 0;
-    const int bits = two_level ? d.p1 : d.p;
+    const bool last = LEVEL == 2 || d.p2 == 0;  // the level that fills the partitions
+    const int bits = LEVEL == 2 ? d.p2 : last ? d.p : d.p1;
+    const uint4 *src;
+    uint64_t left, bin0 = 0;  // records from the tile on; first bin of the CTA
+    if (LEVEL == 1) {
+        const uint64_t n = *d.count, base = (uint64_t)blockIdx.x * kS2Tile;
+        if (base >= n) return;
+        src = d.t2 + base;
+        left = n - base;
+    } else {
+        const uint32_t c = blockIdx.x / d.chunks1, start = (blockIdx.x - c * d.chunks1) * kS2Tile;
+        const uint32_t filled = min(d.cnt1[c], d.cap1);
+        if (start >= filled) return;
+        src = d.a_recs + (uint64_t)c * d.cap1 + start;
+        left = filled - start;
+        bin0 = (uint64_t)c << bits;
+    }
+    const uint32_t count = (uint32_t)(left < kS2Tile ? left : kS2Tile);
+    const S2ScatterLayout L(bits);
+    const uint4 *X = reinterpret_cast<const uint4 *>(smem_raw);
+    uint16_t *order = reinterpret_cast<uint16_t *>(smem_raw + L.order);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + L.hist);
+    uint32_t *ws = reinterpret_cast<uint32_t *>(smem_raw + L.ws);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + L.bar);
+    if (threadIdx.x == 0) {
+        mbar_init(bar, 1);
+        mbar_expect_tx(bar, count * 16u);
+        bulk_g2s(smem_raw, src, count * 16u, bar);
+    }
     const int nbins = 1 << bits;
-    const uint32_t cap = two_level ? d.cap1 : d.cap2;
-    uint64_t *okeys = two_level ? d.a_keys : d.b_keys;
-    uint64_t *ovals = two_level ? d.a_vals : d.b_vals;
-    uint32_t *cnt = two_level ? d.cnt1 : d.cnt2;
-    for (int b = threadIdx.x; b < nbins; b += NT) sm.hist[b] = 0u;
+    // the bin: bits of the key's top 32 (d.p <= 20), below the first level's
+    const int shift = 32 - (last ? d.p : d.p1);
+    const uint32_t bin_mask = (uint32_t)nbins - 1u;
+    auto bin_of = [&](uint32_t z) { return bits ? (bswap32(z) >> shift) & bin_mask : 0u; };
+    for (int b = threadIdx.x; b < nbins; b += NT) hist[b] = 0u;
     __syncthreads();
-    uint64_t key[PER], val[PER];
-    uint32_t rank[PER];
+    if (!__syncthreads_and(mbar_wait(bar, 0, d.spin_limit))) {  // one answer for all threads
+        if (threadIdx.x == 0) atomicOr(d.status, kStTimeout);
+        mbar_wait(bar, 0, d.spin_limit);  // let the copy land before leaving
+        return;
+    }
+    uint32_t where[PER];  // bin << 16 | rank in the bin
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-        const uint64_t i = base + (uint64_t)j * NT + threadIdx.x;
-        const bool valid = i < n;
-        const uint4 r = valid ? d.t2[i] : make_uint4(0u, 0u, 0u, 0u);
-        key[j] = sort2_key(r);
-        val[j] = ((uint64_t)r.x << 32) | r.y;
-        const uint32_t bin = bits ? (uint32_t)(key[j] >> (64 - bits)) : 0u;
-        rank[j] = valid ? atomicAdd(&sm.hist[bin], 1u) : 0u;
+        const uint32_t i = (uint32_t)j * NT + threadIdx.x;
+        where[j] = 0u;
+        if (i < count) {
+            const uint32_t bin = bin_of(X[i].z);
+            where[j] = bin << 16 | atomicAdd(&hist[bin], 1u);
+        }
     }
     __syncthreads();
     constexpr int PB = ((1 << kMaxCoarseBits) + NT - 1) / NT;  // most bins a thread owns
     const int per = (nbins + NT - 1) / NT;
     const int b0 = threadIdx.x * per;
+    const uint32_t cap = last ? d.cap2 : d.cap1;
     uint32_t claim[PB];
     {
+        uint32_t *cnt = (last ? d.cnt2 : d.cnt1) + bin0;
         uint32_t loc = 0;
         for (int k = 0; k < per; ++k)
-            if (b0 + k < nbins) loc += sm.hist[b0 + k];
+            if (b0 + k < nbins) loc += hist[b0 + k];
         uint32_t total;
-        uint32_t run = block_exclusive_scan_u32<NT>(loc, sm.ws, &total);
+        uint32_t run = block_exclusive_scan_u32<NT>(loc, ws, &total);
 #pragma unroll
         for (int k = 0; k < PB; ++k) {
             const int b = b0 + k;
             claim[k] = 0u;
             if (k < per && b < nbins) {
-                const uint32_t h = sm.hist[b];
-                sm.loff[b] = run;
+                const uint32_t h = hist[b];
+                if (h) claim[k] = atomicAdd(&cnt[b], h);
+                hist[b] = run;
                 run += h;
-                if (h) claim[k] = atomicAdd(&cnt[b], h);  // result first needed after the restage
-            }
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        const uint64_t i = base + (uint64_t)j * NT + threadIdx.x;
-        if (i < n) {
-            const uint32_t bin = bits ? (uint32_t)(key[j] >> (64 - bits)) : 0u;
-            const uint32_t pos = sm.loff[bin] + rank[j];
-            sm.keys[pos] = key[j];
-            sm.vals[pos] = val[j];
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < PB; ++k)
-        if (k < per && b0 + k < nbins) sm.gbase[b0 + k] = claim[k];
-    __syncthreads();
-    const uint32_t count = (uint32_t)(n - base < kS2Tile1 ? n - base : kS2Tile1);
-    bool overflow = false;
-    // unrolled over the thread's PER records so that their dependent
-    // shared-memory reads (key, then its bin's bases) overlap
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        const uint32_t i = (uint32_t)j * NT + threadIdx.x;
-        if (i >= count) break;
-        const uint64_t k = sm.keys[i];
-        const uint32_t bin = bits ? (uint32_t)(k >> (64 - bits)) : 0u;
-        const uint32_t g = sm.gbase[bin] + (i - sm.loff[bin]);
-        if (g < cap) {
-            const uint64_t at = (uint64_t)bin * cap + g;
-            okeys[at] = k;
-            ovals[at] = sm.vals[i];
-        } else {
-            overflow = true;
-        }
-    }
-    if (overflow) atomicOr(d.status, kStSort2);
-}
-
-// --------------------------------------------------- second scatter level
-// One CTA per tile of up to 4096 records of a first-level slot: two TMA bulk
-// copies (keys, packed pairs) into shared memory, ranks by the fine bin,
-// claims issued before the in-place restage and read after it, coalesced
-// runs out.
-struct S2Smem2 {
-    uint64_t keys[kS2Tile2];
-    uint64_t vals[kS2Tile2];
-    uint32_t hist[1 << kMaxFineBits];
-    uint32_t loff[1 << kMaxFineBits];
-    uint32_t gbase[1 << kMaxFineBits];
-    uint32_t ws[kS2BThreads / 32 + 1];
-    uint64_t bar;
-};
-
-__global__ void __launch_bounds__(kS2BThreads) k_s2_scatter2(const Sort2Desc *__restrict__ dp)
-{
-    constexpr int NT = kS2BThreads;
-    constexpr int PER = kS2Tile2 / NT;
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    S2Smem2 &sm = *reinterpret_cast<S2Smem2 *>(smem_raw);
-    const Sort2Desc &d = *dp;
-    const uint32_t c = blockIdx.x / d.chunks1;
-    const uint32_t part = blockIdx.x - c * d.chunks1;
-    const uint32_t filled = min(d.cnt1[c], d.cap1);
-    const uint32_t start = part * kS2Tile2;
-    if (start >= filled) return;
-    const uint32_t count = min(kS2Tile2, filled - start);
-    const int p2 = d.p2;
-    const int nbins = 1 << p2;
-    const int shift = 64 - d.p;
-    const uint32_t bin_mask = (uint32_t)nbins - 1u;
-    const uint32_t ncopy = (count + 1u) & ~1u;  // 16-byte multiples; cap1 is even
-    if (threadIdx.x == 0) {
-        mbar_init(&sm.bar, 1);
-        mbar_expect_tx(&sm.bar, ncopy * 16u);
-        bulk_g2s(sm.keys, d.a_keys + (uint64_t)c * d.cap1 + start, ncopy * 8u, &sm.bar);
-        bulk_g2s(sm.vals, d.a_vals + (uint64_t)c * d.cap1 + start, ncopy * 8u, &sm.bar);
-    }
-    for (int b = threadIdx.x; b < nbins; b += NT) sm.hist[b] = 0u;
-    __syncthreads();
-    if (!__syncthreads_and(mbar_wait(&sm.bar, 0, d.spin_limit))) {  // one answer for all threads
-        if (threadIdx.x == 0) atomicOr(d.status, kStTimeout);
-        mbar_wait(&sm.bar, 0, d.spin_limit);  // let the copy land before leaving
-        return;
-    }
-    uint64_t key[PER], val[PER];
-    uint32_t rank[PER];
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        const uint32_t i = (uint32_t)j * NT + threadIdx.x;
-        const bool valid = i < count;
-        key[j] = valid ? sm.keys[i] : 0ull;
-        val[j] = valid ? sm.vals[i] : 0ull;
-        const uint32_t bin = (uint32_t)(key[j] >> shift) & bin_mask;
-        rank[j] = valid ? atomicAdd(&sm.hist[bin], 1u) : 0u;
-    }
-    __syncthreads();
-    constexpr int PB = ((1 << kMaxFineBits) + NT - 1) / NT;
-    const int per = (nbins + NT - 1) / NT;
-    const int b0 = threadIdx.x * per;
-    uint32_t claim[PB];
-    {
-        uint32_t loc = 0;
-        for (int k = 0; k < per; ++k)
-            if (b0 + k < nbins) loc += sm.hist[b0 + k];
-        uint32_t total;
-        uint32_t run = block_exclusive_scan_u32<NT>(loc, sm.ws, &total);
-#pragma unroll
-        for (int k = 0; k < PB; ++k) {
-            const int b = b0 + k;
-            claim[k] = 0u;
-            if (k < per && b < nbins) {
-                const uint32_t h = sm.hist[b];
-                sm.loff[b] = run;
-                run += h;
-                if (h) claim[k] = atomicAdd(&d.cnt2[((uint64_t)c << p2) + b], h);
             }
         }
     }
@@ -232,33 +152,26 @@ __global__ void __launch_bounds__(kS2BThreads) k_s2_scatter2(const Sort2Desc *__
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
         const uint32_t i = (uint32_t)j * NT + threadIdx.x;
-        if (i < count) {
-            const uint32_t bin = (uint32_t)(key[j] >> shift) & bin_mask;
-            const uint32_t pos = sm.loff[bin] + rank[j];
-            sm.keys[pos] = key[j];
-            sm.vals[pos] = val[j];
-        }
+        if (i < count) order[hist[where[j] >> 16] + (where[j] & 0xFFFFu)] = (uint16_t)i;
     }
+    __syncthreads();
 #pragma unroll
     for (int k = 0; k < PB; ++k)
-        if (k < per && b0 + k < nbins) sm.gbase[b0 + k] = claim[k];
+        if (k < per && b0 + k < nbins) hist[b0 + k] = claim[k] - hist[b0 + k];  // run's start less its order index
     __syncthreads();
-    const uint32_t cap = d.cap2;
+    uint4 *__restrict__ out = (last ? d.b_recs : d.a_recs) + bin0 * cap;
     bool overflow = false;
 #pragma unroll
-    for (int j = 0; j < (int)(kS2Tile2 / kS2BThreads); ++j) {
-        const uint32_t i = (uint32_t)j * NT + threadIdx.x;
-        if (i >= count) break;
-        const uint64_t k = sm.keys[i];
-        const uint32_t bin = (uint32_t)(k >> shift) & bin_mask;
-        const uint32_t g = sm.gbase[bin] + (i - sm.loff[bin]);
-        if (g < cap) {
-            const uint64_t at = (((uint64_t)c << p2) + bin) * cap + g;
-            d.b_keys[at] = k;
-            d.b_vals[at] = sm.vals[i];
-        } else {
+    for (int j = 0; j < PER; ++j) {
+        const uint32_t q = (uint32_t)j * NT + threadIdx.x;
+        if (q >= count) break;
+        const uint4 r = X[order[q]];
+        const uint32_t bin = bin_of(r.z);
+        const uint32_t g = hist[bin] + q;
+        if (g < cap)
+            out[(uint64_t)bin * cap + g] = r;
+        else
             overflow = true;
-        }
     }
     if (overflow) atomicOr(d.status, kStSort2);
 }
@@ -356,28 +269,27 @@ __device__ __forceinline__ void block_scan_packed16(uint32_t *A, uint32_t M, uin
 }
 
 // ------------------------------------------------------- partition sort
-// One CTA per partition: counting sort on the dbits key bits below the
+// One CTA per partition, its slot brought into shared memory by one bulk
+// copy: counting sort of the record indices on the dbits key bits below the
 // partition prefix, then each record ranked inside its digit run by
 // (key2, a, b) with warp shuffles and written straight to its place at the
-// partition's offset as {a, b, hash2}.  Shared memory holds each record's
-// key and its index in the slot (12 B with the digit rank); the packed pair
-// is read from the slot (L2) when the record is written out, or when two
-// keys tie.
+// partition's offset.
 constexpr uint32_t kS2PrefetchAhead = 384;  // partitions ahead: ~half the resident CTAs
 
 struct S2SortLayout {
-    size_t idx, rank, dcnt, ws, bytes;
+    size_t idx, rank, dcnt, ws, bar, bytes;
     __host__ __device__ S2SortLayout(uint32_t cap, int dbits)
     {
-        idx = (size_t)cap * 8;
+        idx = (size_t)cap * 16;
         rank = idx + (size_t)((cap + 1) & ~1u) * 2;
         dcnt = rank + (size_t)((cap + 1) & ~1u) * 2;
         ws = dcnt + ((size_t)1 << dbits) * 4;
-        bytes = ws + 40 * 4;
+        bar = (ws + 40 * 4 + 7) & ~(size_t)7;
+        bytes = bar + 8;
     }
 };
 
-__global__ void __launch_bounds__(kS2SortThreads, 5) k_s2_sort(const Sort2Desc *__restrict__ dp)
+__global__ void __launch_bounds__(kS2SortThreads, 4) k_s2_sort(const Sort2Desc *__restrict__ dp)
 {
     constexpr int NT = kS2SortThreads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -388,15 +300,19 @@ __global__ void __launch_bounds__(kS2SortThreads, 5) k_s2_sort(const Sort2Desc *
     const int dbits = d.dbits;
     const uint32_t ndig = 1u << dbits;
     const S2SortLayout L(cap, dbits);
-    uint64_t *SK = reinterpret_cast<uint64_t *>(smem_raw);
+    const uint4 *X = reinterpret_cast<const uint4 *>(smem_raw);
     uint16_t *SI = reinterpret_cast<uint16_t *>(smem_raw + L.idx);
     uint16_t *RK = reinterpret_cast<uint16_t *>(smem_raw + L.rank);
     uint32_t *DC = reinterpret_cast<uint32_t *>(smem_raw + L.dcnt);
     uint32_t *WS = reinterpret_cast<uint32_t *>(smem_raw + L.ws);
     const uint32_t n = min(d.cnt2[f], cap);
     const uint64_t o = d.off[f];
-    const uint64_t *__restrict__ ik = d.b_keys + (uint64_t)f * cap;
-    const uint64_t *__restrict__ iv = d.b_vals + (uint64_t)f * cap;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + L.bar);
+    if (n && threadIdx.x == 0) {
+        mbar_init(bar, 1);
+        mbar_expect_tx(bar, n * 16u);
+        bulk_g2s(smem_raw, d.b_recs + (uint64_t)f * cap, n * 16u, bar);
+    }
     // one more digit bit than the plan's in the same counter words: 16-bit
     // counters, two to a word (n < 2^16), runs of about half the records
     const int shift = 64 - d.p - dbits - 1;
@@ -407,26 +323,30 @@ __global__ void __launch_bounds__(kS2SortThreads, 5) k_s2_sort(const Sort2Desc *
     const uint64_t fa = (uint64_t)f + kS2PrefetchAhead;
     const uint32_t nfa = (threadIdx.x == 0 && fa < (1ull << d.p)) ? min(d.cnt2[fa], cap) : 0u;
     for (uint32_t i = threadIdx.x; i < ndig; i += NT) DC[i] = 0u;
+    if (n == 0) return;
     __syncthreads();
+    if (!__syncthreads_and(mbar_wait(bar, 0, d.spin_limit))) {  // one answer for all threads
+        if (threadIdx.x == 0) atomicOr(d.status, kStTimeout);
+        mbar_wait(bar, 0, d.spin_limit);  // let the copy land before leaving
+        return;
+    }
+    auto key_at = [&](uint32_t i) {
+        const uint2 h = *reinterpret_cast<const uint2 *>(&X[i].z);
+        return ((uint64_t)bswap32(h.x) << 32) | bswap32(h.y);
+    };
+#pragma unroll 4
     for (uint32_t i = threadIdx.x; i < n; i += NT) {
-        const uint32_t g = (uint32_t)(__ldg(ik + i) >> shift) & dmask, h = (g & 1u) << 4;
+        const uint32_t g = (uint32_t)(key_at(i) >> shift) & dmask, h = (g & 1u) << 4;
         RK[i] = (uint16_t)(atomicAdd(&DC[g >> 1], 1u << h) >> h);
     }
-    if (nfa) {
-        const uint32_t nb = ((nfa + 1u) & ~1u) * 8u;  // 16-byte multiple (cap is even)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(d.b_keys + fa * cap), "r"(nb)
+    if (nfa)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(d.b_recs + fa * cap), "r"(nfa * 16u)
                      : "memory");
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(d.b_vals + fa * cap), "r"(nb)
-                     : "memory");
-    }
     __syncthreads();
     block_scan_packed16<NT>(DC, ndig, WS);
-    for (uint32_t i = threadIdx.x; i < n; i += NT) {
-        const uint64_t k = __ldg(ik + i);
-        const uint32_t pos = DC16[(uint32_t)(k >> shift) & dmask] + RK[i];
-        SK[pos] = k;
-        SI[pos] = (uint16_t)i;
-    }
+#pragma unroll 4
+    for (uint32_t i = threadIdx.x; i < n; i += NT)
+        SI[DC16[(uint32_t)(key_at(i) >> shift) & dmask] + RK[i]] = (uint16_t)i;
     __syncthreads();
     // DC16[g] is the start of run g (records of digit g in arrival order);
     // the run ends at DC16[g + 1] (n for the last digit).  Every position, 32
@@ -437,8 +357,7 @@ __global__ void __launch_bounds__(kS2SortThreads, 5) k_s2_sort(const Sort2Desc *
     // in step) on a 32-bit compare key: the key bits below the digit, or
     // their top 32 (records of a run agree above them).  A lane whose run
     // leaves its chunk, or that meets an equal compare key, ranks itself
-    // from shared memory on full keys, then on the packed pairs (a << 32 |
-    // b) for equal keys.  Two chunks per step so that their work overlaps.
+    // from shared memory on the whole record (key2, a, b).  Two chunks per step so that their work overlaps.
     uint4 *__restrict__ out = d.t2 + o;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     constexpr uint32_t NW = NT / 32;
@@ -449,31 +368,23 @@ __global__ void __launch_bounds__(kS2SortThreads, 5) k_s2_sort(const Sort2Desc *
         s0 = DC16[g];
         s1 = g + 1 < pdig ? DC16[g + 1] : n;
     };
-    // place of the record (k, slot index ix) among the run [s0, s1)
-    auto rank_slow = [&](uint64_t k, uint16_t ix, uint32_t s0, uint32_t s1) -> uint32_t {
-        uint32_t r = s0;
-        uint64_t v = 0;
-        bool have_v = false;
+    // place of record r among the run [s0, s1)
+    auto rank_slow = [&](uint4 r, uint32_t s0, uint32_t s1) -> uint32_t {
+        const uint64_t k = sort2_key(r), v = (uint64_t)r.x << 32 | r.y;
+        uint32_t at = s0;
         for (uint32_t q = s0; q < s1; ++q) {
-            const uint64_t kq = SK[q];
-            if (kq < k) {
-                ++r;
-            } else if (kq == k && SI[q] != ix) {
-                if (!have_v) {
-                    v = __ldg(iv + ix);
-                    have_v = true;
-                }
-                r += __ldg(iv + SI[q]) < v ? 1u : 0u;
-            }
+            const uint4 x = X[SI[q]];
+            const uint64_t kq = sort2_key(x);
+            at += kq < k || (kq == k && ((uint64_t)x.x << 32 | x.y) < v) ? 1u : 0u;
         }
-        return r;
+        return at;
     };
     for (uint32_t c = warp; c < nch; c += 2 * NW) {
         const uint32_t pa = 32u * c + lane, pb = pa + 32u * NW;
         const bool va = pa < n, vb = pb < n;
         const uint32_t xa = va ? pa : 0u, xb = vb ? pb : 0u;
-        const uint64_t ka = SK[xa], kb = SK[xb];
-        const uint16_t ia = SI[xa], ib = SI[xb];
+        const uint4 ra = X[SI[xa]], rb = X[SI[xb]];
+        const uint64_t ka = sort2_key(ra), kb = sort2_key(rb);
         uint32_t sa, ea, sb, eb;
         run_bounds(ka, sa, ea);
         run_bounds(kb, sb, eb);
@@ -495,19 +406,11 @@ __global__ void __launch_bounds__(kS2SortThreads, 5) k_s2_sort(const Sort2Desc *
                 slow_a = slow_a || (ina_d && da_ == qa) || (ina_u && ua == qa);
                 slow_b = slow_b || (inb_d && db_ == qb) || (inb_u && ub == qb);
             }
-            if (va && slow_a) da = rank_slow(ka, ia, sa, ea);
-            if (vb && slow_b) db = rank_slow(kb, ib, sb, eb);
+            if (va && slow_a) da = rank_slow(ra, sa, ea);
+            if (vb && slow_b) db = rank_slow(rb, sb, eb);
         }
-        if (va) {
-            const uint64_t v = __ldg(iv + ia);
-            out[da] = make_uint4((uint32_t)(v >> 32), (uint32_t)v, bswap32((uint32_t)(ka >> 32)),
-                                 bswap32((uint32_t)ka));
-        }
-        if (vb) {
-            const uint64_t v = __ldg(iv + ib);
-            out[db] = make_uint4((uint32_t)(v >> 32), (uint32_t)v, bswap32((uint32_t)(kb >> 32)),
-                                 bswap32((uint32_t)kb));
-        }
+        if (va) out[da] = ra;
+        if (vb) out[db] = rb;
     }
 }
 
@@ -515,32 +418,27 @@ size_t sort2_smem_bytes(uint32_t cap, int dbits) { return S2SortLayout(cap, dbit
 
 cudaError_t launch_sort2(const Sort2Desc *d_desc, const Sort2Launch &g, cudaStream_t s)
 {
+    static SmemSeen seen1, seen2, seen3;
     cudaError_t e;
     k_s2_setup<<<64, 256, 0, s>>>(const_cast<Sort2Desc *>(d_desc));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (g.tiles1) {
-        const size_t sm1 = sizeof(S2Smem1);
-        if ((e = cudaFuncSetAttribute(k_s2_scatter1, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sm1)) != cudaSuccess)
-            return e;
-        k_s2_scatter1<<<g.tiles1, kS2Threads, sm1, s>>>(d_desc);
+        const size_t sm = S2ScatterLayout(g.p - g.p2).bytes;
+        if ((e = allow_smem(k_s2_scatter<1>, sm, seen1)) != cudaSuccess) return e;
+        k_s2_scatter<1><<<g.tiles1, kS2Threads, sm, s>>>(d_desc);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (g.tiles2) {
-        const size_t sm2 = sizeof(S2Smem2);
-        if ((e = cudaFuncSetAttribute(k_s2_scatter2, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sm2)) != cudaSuccess)
-            return e;
-        k_s2_scatter2<<<g.tiles2, kS2BThreads, sm2, s>>>(d_desc);
+        const size_t sm = S2ScatterLayout(g.p2).bytes;
+        if ((e = allow_smem(k_s2_scatter<2>, sm, seen2)) != cudaSuccess) return e;
+        k_s2_scatter<2><<<g.tiles2, kS2Threads, sm, s>>>(d_desc);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     k_s2_scan<<<g.tiles_scan, 256, 0, s>>>(d_desc);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const size_t sm3 = sort2_smem_bytes(g.cap2, g.dbits);
-    if ((e = cudaFuncSetAttribute(k_s2_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3)) !=
-        cudaSuccess)
-        return e;
-    k_s2_sort<<<g.parts, kS2SortThreads, sm3, s>>>(d_desc);
+    const size_t sm = sort2_smem_bytes(g.cap2, g.dbits);
+    if ((e = allow_smem(k_s2_sort, sm, seen3)) != cudaSuccess) return e;
+    k_s2_sort<<<g.parts, kS2SortThreads, sm, s>>>(d_desc);
     return cudaGetLastError();
 }
 

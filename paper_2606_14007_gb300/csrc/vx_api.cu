@@ -838,10 +838,8 @@ int vx_sort_table2(vx_plot *p, void *d_work, uint64_t work_bytes, void *stream)
     d.chunks1 = sp.chunks1;
     d.spin_limit = pl.spin_limit;
     d.t2 = reinterpret_cast<uint4 *>(p->d_t2);
-    d.a_keys = reinterpret_cast<uint64_t *>(w + sp.o_akeys);
-    d.a_vals = reinterpret_cast<uint64_t *>(w + sp.o_avals);
-    d.b_keys = reinterpret_cast<uint64_t *>(w + sp.o_bkeys);
-    d.b_vals = reinterpret_cast<uint64_t *>(w + sp.o_bvals);
+    d.a_recs = reinterpret_cast<uint4 *>(w + sp.o_arecs);
+    d.b_recs = reinterpret_cast<uint4 *>(w + sp.o_brecs);
     d.cnt1 = reinterpret_cast<uint32_t *>(w + sp.o_cnt1);
     d.cnt2 = reinterpret_cast<uint32_t *>(w + sp.o_cnt2);
     d.off = reinterpret_cast<uint64_t *>(w + sp.o_off);
@@ -850,7 +848,8 @@ int vx_sort_table2(vx_plot *p, void *d_work, uint64_t work_bytes, void *stream)
     d.status = reinterpret_cast<uint32_t *>(p->d_scratch + pl.o_status);
     vx::Sort2Desc *dd = reinterpret_cast<vx::Sort2Desc *>(w + sp.o_desc);
     VX_TRY(p, cudaMemcpyAsync(dd, &d, sizeof(d), cudaMemcpyHostToDevice, s));
-    const vx::Sort2Launch g{sp.tiles1, sp.tiles2, sp.tiles_scan, sp.parts, sp.cap2, sp.dbits};
+    const vx::Sort2Launch g{sp.tiles1, sp.tiles2, sp.tiles_scan, sp.parts, sp.cap2,
+                            sp.p, sp.p2, sp.dbits};
     cudaError_t e = vx::launch_sort2(dd, g, s);
     if (e != cudaSuccess) return cuda_fail(p, "sort Table 2", e);
     p->last = s;

@@ -107,8 +107,8 @@ struct Sort2Desc {
     uint32_t chunks1;      // second-level CTAs per first-level slot
     uint32_t spin_limit;   // polls before a bounded wait gives up
     uint4 *t2;             // Table 2: read by the first level, rewritten sorted
-    uint64_t *a_keys, *a_vals; // first-level slots [2^p1][cap1]: key2, a << 32 | b
-    uint64_t *b_keys, *b_vals; // partitions [2^p][cap2]
+    uint4 *a_recs;         // first-level slots [2^p1][cap1]
+    uint4 *b_recs;         // partitions [2^p][cap2]
     uint32_t *cnt1, *cnt2; // fill counters
     uint64_t *off;         // [2^p + 1] partition offsets in the sorted table
     uint64_t *lbs;         // look-back words of the offset scan
@@ -677,7 +677,7 @@ cudaError_t launch_bucket_offsets(const Desc *desc, uint64_t *out, cudaStream_t 
 // Table 2 sorted by hash2: grids of the five kernels of one sort.
 struct Sort2Launch {
     uint32_t tiles1, tiles2, tiles_scan, parts, cap2;
-    int dbits;
+    int p, p2, dbits;
 };
 cudaError_t launch_sort2(const Sort2Desc *d_desc, const Sort2Launch &g, cudaStream_t s);
 size_t sort2_smem_bytes(uint32_t cap, int dbits);

@@ -406,7 +406,7 @@ struct Sort2Plan {
     int p, p1, p2, dbits;
     uint32_t cap1, cap2, chunks1;
     uint32_t tiles1, tiles2, tiles_scan, parts;
-    uint64_t o_desc, o_ticket, o_cnt1, o_cnt2, o_off, o_lbs, o_akeys, o_avals, o_bkeys, o_bvals;
+    uint64_t o_desc, o_ticket, o_cnt1, o_cnt2, o_off, o_lbs, o_arecs, o_brecs;
     uint64_t bytes;
 };
 
@@ -448,10 +448,8 @@ inline int make_sort2_plan(uint64_t n, Sort2Plan *out, size_t desc_bytes)
     S.o_cnt2 = at; at = round_up(at + 4 * np, 256);
     S.o_off = at; at = round_up(at + 8 * (np + 1), 256);
     S.o_lbs = at; at = round_up(at + 8 * (uint64_t)S.tiles_scan, 256);
-    S.o_akeys = at; at = round_up(at + 8 * n1 * S.cap1, 256);
-    S.o_avals = at; at = round_up(at + 8 * n1 * S.cap1, 256);
-    S.o_bkeys = at; at = round_up(at + 8 * np * S.cap2, 256);
-    S.o_bvals = at; at = round_up(at + 8 * np * S.cap2, 256);
+    S.o_arecs = at; at = round_up(at + 16 * n1 * S.cap1, 256);
+    S.o_brecs = at; at = round_up(at + 16 * np * S.cap2, 256);
     S.bytes = at;
     *out = S;
     return VX_OK;
