@@ -6,11 +6,11 @@
 // with the Table-1 machinery applied to 16-byte records: a first scatter
 // level by the top p1 bits of key2, a second level by the next p2 bits into
 // 2^p Poisson-sized partitions, a scan of the partition counts, and a
-// shared-memory sort of every partition (counting sort on the next
-// dbits + 1 key bits, each record ranked inside its digit run by warp
-// shuffles) that writes its records straight back into the Table-2 buffer
-// at their places.  Table 2 is read completely by
-// the first level before anything writes it.
+// shared-memory sort of every partition (ranks by a digit bitmap of the next
+// key bits) that writes its records straight back into the Table-2 buffer at
+// their places.  Table 2 is read completely by the first level before
+// anything writes it.
+#include "bitmap_sort.cuh"
 #include "vx_internal.cuh"
 #include "vx_plan.h"
 
@@ -231,190 +231,159 @@ __global__ void __launch_bounds__(256) k_s2_scan(const Sort2Desc *__restrict__ d
     }
 }
 
-// In-place exclusive scan of 2M digit counters of 16 bits, two to a word
-// (digit 2w in the low half of word w, 2w + 1 in the high half; every
-// count and start below 2^16), by a CTA of NT threads: each word's two
-// counts become their starts.  Warp w takes a contiguous run of the words,
-// 32 at a time; `ws` holds NT/32 words.  Ends with a __syncthreads.
-template <int NT>
-__device__ __forceinline__ void block_scan_packed16(uint32_t *A, uint32_t M, uint32_t *ws)
-{
-    constexpr int NW = NT / 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t chunk = (M + NW - 1) / NW;
-    const uint32_t lo = min(M, (uint32_t)warp * chunk), hi = min(M, lo + chunk);
-    uint32_t sum = 0;
-    for (uint32_t i = lo + lane; i < hi; i += 32) sum += (A[i] & 0xFFFFu) + (A[i] >> 16);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) ws[warp] = sum;
-    __syncthreads();
-    uint32_t carry = 0;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) carry += w < warp ? ws[w] : 0u;
-    for (uint32_t base = lo; base < hi; base += 32) {
-        const uint32_t i = base + lane;
-        const uint32_t a = i < hi ? A[i] : 0u, l = a & 0xFFFFu, v = l + (a >> 16);
-        uint32_t incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        const uint32_t P = carry + incl - v;
-        if (i < hi) A[i] = P | ((P + l) << 16);
-        carry += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    __syncthreads();
-}
-
 // ------------------------------------------------------- partition sort
 // One CTA per partition, its slot brought into shared memory by one bulk
-// copy: counting sort of the record indices on the dbits key bits below the
-// partition prefix, then each record ranked inside its digit run by
-// (key2, a, b) with warp shuffles and written straight to its place at the
-// partition's offset.
+// copy.  The records stay there: a digit bitmap ranks them as in Table 1's
+// sort, a 16-bit order takes their indices, the few words with a shared digit
+// are put in order by (key2, a, b), and the records leave in that order as
+// whole 16-byte words at the partition's offset.  Bound by shared memory (73%
+// of its wavefronts) and the wait for the slot: 58.7 M records take 449 us
+// (502 with a counting sort and every record ranked in its digit run by
+// shuffles, 7.3 instructions a record).  512 threads a CTA, or five CTAs of
+// half the digits, measured 5 to 10% slower.
 constexpr uint32_t kS2PrefetchAhead = 384;  // partitions ahead: ~half the resident CTAs
 
+// Twice the digits of Table 1's sort for the same dbits: a partition holds
+// 2^dbits to 2^(dbits + 1) records.
+__host__ __device__ __forceinline__ uint32_t sort2_words(int dbits) { return bitmap_words(dbits + 1); }
+
 struct S2SortLayout {
-    size_t idx, rank, dcnt, ws, bar, bytes;
-    __host__ __device__ S2SortLayout(uint32_t cap, int dbits)
+    size_t bm, order, dl, ws, bar, bytes;
+    __host__ __device__ S2SortLayout(uint32_t cap, uint32_t words)
     {
-        idx = (size_t)cap * 16;
-        rank = idx + (size_t)((cap + 1) & ~1u) * 2;
-        dcnt = rank + (size_t)((cap + 1) & ~1u) * 2;
-        ws = dcnt + ((size_t)1 << dbits) * 4;
+        bm = (size_t)cap * 16;
+        order = bm + (size_t)words * 6;
+        dl = (order + (size_t)cap * 2 + 3) & ~(size_t)3;
+        ws = dl + (size_t)kDirtyList * 2;
         bar = (ws + 40 * 4 + 7) & ~(size_t)7;
         bytes = bar + 8;
     }
 };
 
+// Puts the dirty words' indices in the order of their records: eight lanes a
+// listed word, a lane per record; words with more than eight records or past
+// the list by one thread's insertion sort.
+template <int NT>
+__device__ __forceinline__ void order_dirty_indices(const Bitmap &A, uint32_t W, const uint4 *X, uint16_t *order)
+{
+    constexpr uint32_t NW = NT / 32;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    auto less = [](const uint4 &p, const uint4 &q) {
+        const uint64_t kp = sort2_key(p), kq = sort2_key(q);
+        return kp < kq || (kp == kq && (p.x < q.x || (p.x == q.x && p.y < q.y)));
+    };
+    auto order_word = [&](uint32_t w) {
+        uint16_t *const o = order + (A.PF[w] & (kDirty - 1u));
+        const uint32_t cnt = A.BM[w];
+        for (uint32_t a = 1; a < cnt; ++a) {
+            const uint16_t ix = o[a];
+            const uint4 r = X[ix];
+            uint32_t b = a;
+            for (; b > 0 && less(r, X[o[b - 1]]); --b) o[b] = o[b - 1];
+            o[b] = ix;
+        }
+    };
+    const uint32_t nd = A.WS[kWsDirty];
+    if (nd > kDirtyList) {
+        for (uint32_t w = threadIdx.x; w < W; w += NT)
+            if (A.PF[w] & kDirty) order_word(w);
+        return;
+    }
+    const uint32_t sub = lane & 7u;
+    for (uint32_t i0 = 4u * warp; i0 < nd; i0 += 4u * NW) {
+        const uint32_t i = i0 + (lane >> 3);
+        const uint32_t w = i < nd ? A.DL[i] : 0u;
+        uint16_t *const o = order + (A.PF[w] & (kDirty - 1u));
+        const uint32_t all = i < nd ? A.BM[w] : 0u;
+        const uint32_t cnt = all <= 8u ? all : 0u;
+        const bool mine = sub < cnt;
+        const uint32_t ix = mine ? o[sub] : 0u;
+        const uint4 r = X[ix];
+        const uint32_t most = __reduce_max_sync(0xffffffffu, cnt);
+        uint32_t place = 0;
+        for (uint32_t t = 0; t < most; ++t) {
+            const uint32_t other = __shfl_sync(0xffffffffu, ix, (int)((lane & 24u) + t));
+            place += t < cnt && less(X[other], r) ? 1u : 0u;
+        }
+        if (mine) o[place] = (uint16_t)ix;
+        if (all > 8u && sub == 0) order_word(w);
+    }
+}
+
 __global__ void __launch_bounds__(kS2SortThreads, 4) k_s2_sort(const Sort2Desc *__restrict__ dp)
 {
     constexpr int NT = kS2SortThreads;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(128) unsigned char smem_raw[];
     const Sort2Desc &d = *dp;
     if (*d.status & (kStSort2 | kStTimeout | kStBadTicket)) return;  // offsets not trusted
     const uint32_t f = blockIdx.x;
     const uint32_t cap = d.cap2;
-    const int dbits = d.dbits;
-    const uint32_t ndig = 1u << dbits;
-    const S2SortLayout L(cap, dbits);
-    const uint4 *X = reinterpret_cast<const uint4 *>(smem_raw);
-    uint16_t *SI = reinterpret_cast<uint16_t *>(smem_raw + L.idx);
-    uint16_t *RK = reinterpret_cast<uint16_t *>(smem_raw + L.rank);
-    uint32_t *DC = reinterpret_cast<uint32_t *>(smem_raw + L.dcnt);
-    uint32_t *WS = reinterpret_cast<uint32_t *>(smem_raw + L.ws);
     const uint32_t n = min(d.cnt2[f], cap);
-    const uint64_t o = d.off[f];
+    if (n == 0) return;
+    const uint32_t W = sort2_words(d.dbits);
+    const S2SortLayout L(cap, W);
+    const uint4 *X = reinterpret_cast<const uint4 *>(smem_raw);
+    uint16_t *order = reinterpret_cast<uint16_t *>(smem_raw + L.order);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + L.bar);
-    if (n && threadIdx.x == 0) {
+    Bitmap A;
+    A.BM = reinterpret_cast<uint32_t *>(smem_raw + L.bm);
+    A.PF = reinterpret_cast<uint16_t *>(A.BM + W);
+    A.DL = reinterpret_cast<uint16_t *>(smem_raw + L.dl);
+    A.WS = reinterpret_cast<uint32_t *>(smem_raw + L.ws);
+    if (threadIdx.x == 0) {
         mbar_init(bar, 1);
         mbar_expect_tx(bar, n * 16u);
         bulk_g2s(smem_raw, d.b_recs + (uint64_t)f * cap, n * 16u, bar);
     }
-    // one more digit bit than the plan's in the same counter words: 16-bit
-    // counters, two to a word (n < 2^16), runs of about half the records
-    const int shift = 64 - d.p - dbits - 1;
-    const uint32_t pdig = ndig << 1, dmask = pdig - 1u;
-    const uint16_t *DC16 = reinterpret_cast<const uint16_t *>(DC);
-    // the filled part of the slot kS2PrefetchAhead partitions ahead goes to
-    // L2 after step 1 (its fill count is read now)
+    // the filled part of the slot kS2PrefetchAhead partitions ahead goes to L2
     const uint64_t fa = (uint64_t)f + kS2PrefetchAhead;
-    const uint32_t nfa = (threadIdx.x == 0 && fa < (1ull << d.p)) ? min(d.cnt2[fa], cap) : 0u;
-    for (uint32_t i = threadIdx.x; i < ndig; i += NT) DC[i] = 0u;
-    if (n == 0) return;
+    if (threadIdx.x == 0 && fa < (1ull << d.p)) {
+        const uint32_t nfa = min(d.cnt2[fa], cap);
+        if (nfa)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(d.b_recs + fa * cap), "r"(nfa * 16u)
+                         : "memory");
+    }
+    const uint64_t o = d.off[f];
+    clear_tables<NT>(A, W);
     __syncthreads();
     if (!__syncthreads_and(mbar_wait(bar, 0, d.spin_limit))) {  // one answer for all threads
         if (threadIdx.x == 0) atomicOr(d.status, kStTimeout);
         mbar_wait(bar, 0, d.spin_limit);  // let the copy land before leaving
         return;
     }
-    auto key_at = [&](uint32_t i) {
+    // log2(W) + 5 bits below the partition prefix
+    const int shift = 64 - d.p - (36 - __clz(W));
+    const uint32_t dmask = 32u * W - 1u;
+    auto digit = [&](uint32_t i) {
         const uint2 h = *reinterpret_cast<const uint2 *>(&X[i].z);
-        return ((uint64_t)bswap32(h.x) << 32) | bswap32(h.y);
+        return (uint32_t)((((uint64_t)bswap32(h.x) << 32) | bswap32(h.y)) >> shift) & dmask;
     };
-#pragma unroll 4
-    for (uint32_t i = threadIdx.x; i < n; i += NT) {
-        const uint32_t g = (uint32_t)(key_at(i) >> shift) & dmask, h = (g & 1u) << 4;
-        RK[i] = (uint16_t)(atomicAdd(&DC[g >> 1], 1u << h) >> h);
+    constexpr int KEEP = 8;  // digits a thread keeps from the marking to the placing (2048 records)
+    uint32_t dg[KEEP];
+#pragma unroll
+    for (int j = 0; j < KEEP; ++j) {
+        const uint32_t i = threadIdx.x + (uint32_t)j * NT;
+        if (i < n) mark(A, dg[j] = digit(i));
     }
-    if (nfa)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(d.b_recs + fa * cap), "r"(nfa * 16u)
-                     : "memory");
+    for (uint32_t i = threadIdx.x + KEEP * NT; i < n; i += NT) mark(A, digit(i));
     __syncthreads();
-    block_scan_packed16<NT>(DC, ndig, WS);
-#pragma unroll 4
-    for (uint32_t i = threadIdx.x; i < n; i += NT)
-        SI[DC16[(uint32_t)(key_at(i) >> shift) & dmask] + RK[i]] = (uint16_t)i;
+    scan_words<NT>(A, W);
     __syncthreads();
-    // DC16[g] is the start of run g (records of digit g in arrival order);
-    // the run ends at DC16[g + 1] (n for the last digit).  Every position, 32
-    // per warp step and one per lane, finds its record's rank inside its run
-    // and the record goes straight to its place in the sorted table.  A
-    // run's records sit in neighbouring lanes, so each lane compares with
-    // the lanes up to the longest run's length away (shuffles, every lane
-    // in step) on a 32-bit compare key: the key bits below the digit, or
-    // their top 32 (records of a run agree above them).  A lane whose run
-    // leaves its chunk, or that meets an equal compare key, ranks itself
-    // from shared memory on the whole record (key2, a, b).  Two chunks per step so that their work overlaps.
+#pragma unroll
+    for (int j = 0; j < KEEP; ++j) {
+        const uint32_t i = threadIdx.x + (uint32_t)j * NT;
+        if (i < n) order[place_of(A, dg[j])] = (uint16_t)i;
+    }
+    for (uint32_t i = threadIdx.x + KEEP * NT; i < n; i += NT) order[place_of(A, digit(i))] = (uint16_t)i;
+    __syncthreads();
+    order_dirty_indices<NT>(A, W, X, order);
+    __syncthreads();
     uint4 *__restrict__ out = d.t2 + o;
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    constexpr uint32_t NW = NT / 32;
-    const uint32_t nch = (n + 31u) >> 5;
-    const int cs = shift > 32 ? shift - 32 : 0;
-    auto run_bounds = [&](uint64_t k, uint32_t &s0, uint32_t &s1) {
-        const uint32_t g = (uint32_t)(k >> shift) & dmask;
-        s0 = DC16[g];
-        s1 = g + 1 < pdig ? DC16[g + 1] : n;
-    };
-    // place of record r among the run [s0, s1)
-    auto rank_slow = [&](uint4 r, uint32_t s0, uint32_t s1) -> uint32_t {
-        const uint64_t k = sort2_key(r), v = (uint64_t)r.x << 32 | r.y;
-        uint32_t at = s0;
-        for (uint32_t q = s0; q < s1; ++q) {
-            const uint4 x = X[SI[q]];
-            const uint64_t kq = sort2_key(x);
-            at += kq < k || (kq == k && ((uint64_t)x.x << 32 | x.y) < v) ? 1u : 0u;
-        }
-        return at;
-    };
-    for (uint32_t c = warp; c < nch; c += 2 * NW) {
-        const uint32_t pa = 32u * c + lane, pb = pa + 32u * NW;
-        const bool va = pa < n, vb = pb < n;
-        const uint32_t xa = va ? pa : 0u, xb = vb ? pb : 0u;
-        const uint4 ra = X[SI[xa]], rb = X[SI[xb]];
-        const uint64_t ka = sort2_key(ra), kb = sort2_key(rb);
-        uint32_t sa, ea, sb, eb;
-        run_bounds(ka, sa, ea);
-        run_bounds(kb, sb, eb);
-        if (!va) sa = ea = 0u;
-        if (!vb) sb = eb = 0u;
-        const uint32_t lmax = __reduce_max_sync(0xffffffffu, max(ea - sa, eb - sb));
-        uint32_t da = sa, db = sb;
-        if (lmax > 1) {
-            const uint32_t qa = (uint32_t)(ka >> cs), qb = (uint32_t)(kb >> cs);
-            bool slow_a = va && (sa < 32u * c || ea > 32u * c + 32u);
-            bool slow_b = vb && (sb < 32u * (c + NW) || eb > 32u * (c + NW) + 32u);
-            for (uint32_t t = 1; t < lmax; ++t) {
-                const uint32_t da_ = __shfl_down_sync(0xffffffffu, qa, t), ua = __shfl_up_sync(0xffffffffu, qa, t);
-                const uint32_t db_ = __shfl_down_sync(0xffffffffu, qb, t), ub = __shfl_up_sync(0xffffffffu, qb, t);
-                const bool ina_d = pa + t < ea, ina_u = lane >= t && pa - t >= sa;
-                const bool inb_d = pb + t < eb, inb_u = lane >= t && pb - t >= sb;
-                da += (ina_d && da_ < qa ? 1u : 0u) + (ina_u && ua < qa ? 1u : 0u);
-                db += (inb_d && db_ < qb ? 1u : 0u) + (inb_u && ub < qb ? 1u : 0u);
-                slow_a = slow_a || (ina_d && da_ == qa) || (ina_u && ua == qa);
-                slow_b = slow_b || (inb_d && db_ == qb) || (inb_u && ub == qb);
-            }
-            if (va && slow_a) da = rank_slow(ra, sa, ea);
-            if (vb && slow_b) db = rank_slow(rb, sb, eb);
-        }
-        if (va) out[da] = ra;
-        if (vb) out[db] = rb;
-    }
+#pragma unroll 4
+    for (uint32_t i = threadIdx.x; i < n; i += NT) out[i] = X[order[i]];
 }
 
-size_t sort2_smem_bytes(uint32_t cap, int dbits) { return S2SortLayout(cap, dbits).bytes; }
+size_t sort2_smem_bytes(uint32_t cap, int dbits) { return S2SortLayout(cap, sort2_words(dbits)).bytes; }
 
 cudaError_t launch_sort2(const Sort2Desc *d_desc, const Sort2Launch &g, cudaStream_t s)
 {

@@ -57,6 +57,7 @@
 // read: cap2 pairs in the key array, cap2 / 2 in the nonce array.  No
 // partition waits on another; a scan of the pair counts and the slot pair
 // hash place the records.
+#include "bitmap_sort.cuh"
 #include "vx_internal.cuh"
 
 namespace vx {
@@ -64,22 +65,9 @@ namespace vx {
 enum { kSortCount = 0, kSortHash = 1, kSortEmit = 2, kSortSlots = 3 };
 constexpr int kPipeThreads = 256;   // persistent front end
 constexpr int kGlThreads = 256;     // one-CTA-per-partition front end
-constexpr uint32_t kDirtyList = 64;  // listed words with a shared digit (2048 records: about 31)
-constexpr int kMaxDigitBits = 18;   // sort digit (bitmap of 2^18 bits, 8192 words)
 // Tickets between a CTA of the global-memory front end and the partition
 // whose slot it prefetches into L2: about half of the CTAs resident at once.
 constexpr uint32_t kSlotPrefetchAhead = 384;
-
-// Words of the digit bitmap of a plan's dbits (log2 of the mean records of a
-// partition): 32 digits per expected record, so that two records share a
-// digit about once in 64 records (2048 records, 2^16 digits: 32 pairs).
-// More digits cost shared memory (three CTAs per SM need 75 KB each), fewer
-// double the shared digits.
-__host__ __device__ __forceinline__ uint32_t bitmap_words(int dbits)
-{
-    const int b = dbits + 5 < kMaxDigitBits ? dbits + 5 : kMaxDigitBits;
-    return 1u << (b - 5);
-}
 
 // Shared layout (bytes from the base), for slots of at most `cap` records
 // (a multiple of 4) and a bitmap of at most `words` words:
@@ -111,18 +99,11 @@ struct SMLayout {
     }
 };
 
-struct Part {
+struct Part : Bitmap {
     uint32_t *Y;   // sorted Table-1 words (record r at Y[3 r])
-    uint32_t *BM;  // digit bitmap
-    uint16_t *PF;  // word prefixes
-    uint16_t *DL;  // dirty words (the first kDirtyList of them)
     uint16_t *PL;  // pair lists, over BM and PF: NT / 32 of them, plw entries each
     uint32_t plw;
-    uint32_t *WS;  // scan workspace
 };
-constexpr uint32_t kWsDirty = 36;  // WS word: how many dirty words the scan met
-constexpr uint32_t kWsLong = 37;   // WS word: some warp's pairs do not fit its list
-
 __device__ __forceinline__ bool rec_less(uint64_t ka, uint32_t na, uint64_t kb, uint32_t nb)
 {
     return ka < kb || (ka == kb && na < nb);
@@ -141,140 +122,12 @@ __device__ __forceinline__ uint32_t sub_key(uint32_t hi, uint32_t lo, int pk)
 
 // ---------------------------------------------------------------- sort
 
-// Inclusive scan of one u32 per lane (a shuffle's own predicate says
-// whether its source lane exists: two instructions a step).
-__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x)
-{
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1)
-        asm volatile(
-            "{ .reg .pred p; .reg .u32 r; shfl.sync.up.b32 r|p, %0, %1, 0, 0xffffffff; @p add.u32 %0, r, %0; }"
-            : "+r"(x)
-            : "r"(o));
-    return x;
-}
-
-constexpr uint32_t kDirty = 0x8000u;  // flag of PF: the word holds a shared digit
-
-// Zeroes the bitmap and the extra counts (PF) of W words; no barrier.
-template <int NT>
-__device__ __forceinline__ void clear_tables(const Part &A, uint32_t W)
-{
-    if (threadIdx.x == 0) A.WS[kWsDirty] = A.WS[kWsLong] = 0u;
-    if (W % 8u == 0) {  // 6 W bytes, a multiple of 16 (PF follows BM)
-        uint4 *t = reinterpret_cast<uint4 *>(A.BM);
-        for (uint32_t i = threadIdx.x; i < W * 6u / 16u; i += NT) t[i] = make_uint4(0u, 0u, 0u, 0u);
-    } else {
-        for (uint32_t i = threadIdx.x; i < W; i += NT) {
-            A.BM[i] = 0u;
-            A.PF[i] = 0;
-        }
-    }
-}
-
-// The sort.  The digit, the bits of key64 below the partition prefix, is wide
-// enough (2^16 for 2048 records) that most records have one of their own:
-// then a record's place is the number of records in lower digits, i.e. the
-// count before its bitmap word plus the word's bits below its own, and the
-// record goes there directly.  Words with a shared digit ("dirty") take
-// their records in arrival order, which order_dirty puts right.  One pass
-// marks the digits (mark), one places the records (place_of); a counting
-// sort's third pass (ranking every record in its digit run) and its second
-// set of shared-memory atomics are gone.
-
-// Marks a digit; one already taken counts as an extra of its word.
-__device__ __forceinline__ void mark(const Part &A, uint32_t dg)
-{
-    const uint32_t w = dg >> 5, bit = 1u << (dg & 31u);
-    if (atomicOr(&A.BM[w], bit) & bit)
-        atomicAdd(reinterpret_cast<uint32_t *>(A.PF) + (w >> 1), 1u << (16u * (w & 1u)));
-}
-
-// A record's place (after scan_words).
-__device__ __forceinline__ uint32_t place_of(const Part &A, uint32_t dg)
-{
-    const uint32_t w = dg >> 5, pf = A.PF[w];
-    if (pf & kDirty) return (pf & (kDirty - 1u)) + atomicAdd(&A.BM[w], 1u);
-    return pf + (uint32_t)__popc(A.BM[w] & ((1u << (dg & 31u)) - 1u));
-}
-
 __device__ __forceinline__ void put_record(const Part &A, uint32_t pos, uint64_t key, uint32_t nonce)
 {
     uint32_t *o = A.Y + 3 * pos;
     o[0] = nonce;
     o[1] = bswap32((uint32_t)(key >> 32));
     o[2] = bswap32((uint32_t)key);
-}
-
-// Exclusive scan of the W words' record counts into PF, `per` consecutive
-// words a thread; dirty words are flagged and listed and their bitmap word
-// becomes the count of records placed.  Between two barriers of the caller's;
-// one inside.
-template <int NT>
-__device__ __forceinline__ void scan_words(const Part &A, uint32_t W)
-{
-    constexpr uint32_t NW = NT / 32;
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t per = W > (uint32_t)NT ? W / NT : 1u;
-    const uint32_t w0 = threadIdx.x * per;
-    uint32_t local = 0;
-    if (per >= 8) {
-        for (uint32_t g = 0; g < per; g += 8) {
-            const uint4 a = *reinterpret_cast<const uint4 *>(A.BM + w0 + g);
-            const uint4 b = *reinterpret_cast<const uint4 *>(A.BM + w0 + g + 4);
-            const uint4 e = *reinterpret_cast<const uint4 *>(A.PF + w0 + g);
-            local += __popc(a.x) + __popc(a.y) + __popc(a.z) + __popc(a.w) + __popc(b.x) + __popc(b.y) +
-                     __popc(b.z) + __popc(b.w);
-            const uint32_t x = e.x + e.y + e.z + e.w;  // extras: 16-bit halves, < 2^15 in all
-            local += (x & 0xFFFFu) + (x >> 16);
-        }
-    } else if (w0 < W) {
-        for (uint32_t g = 0; g < per; ++g) local += __popc(A.BM[w0 + g]) + A.PF[w0 + g];
-    }
-    const uint32_t incl = warp_incl_scan(local);
-    if (lane == 31) A.WS[warp] = incl;
-    __syncthreads();
-    uint32_t run = incl - local;
-#pragma unroll
-    for (uint32_t w = 0; w < NW; ++w) run += w < warp ? A.WS[w] : 0u;
-    auto set_dirty = [&](uint32_t w) {
-        A.PF[w] |= (uint16_t)kDirty;
-        A.BM[w] = 0u;
-        const uint32_t i = atomicAdd(&A.WS[kWsDirty], 1u);
-        if (i < kDirtyList) A.DL[i] = (uint16_t)w;
-    };
-    if (per >= 8) {
-        for (uint32_t g = 0; g < per; g += 8) {
-            uint4 e = *reinterpret_cast<const uint4 *>(A.PF + w0 + g);
-            uint32_t *const ex[4] = {&e.x, &e.y, &e.z, &e.w};
-            const uint4 a = *reinterpret_cast<const uint4 *>(A.BM + w0 + g);
-            const uint4 b = *reinterpret_cast<const uint4 *>(A.BM + w0 + g + 4);
-            const uint32_t bm[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-            uint32_t m = 0;  // bit j: word w0 + g + j is dirty
-            if (e.x | e.y | e.z | e.w) {
-#pragma unroll
-                for (int h = 0; h < 4; ++h)
-                    m |= (*ex[h] & 0xFFFFu ? 1u << (2 * h) : 0u) | (*ex[h] >> 16 ? 2u << (2 * h) : 0u);
-            }
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                const uint32_t p0 = run;
-                run += __popc(bm[2 * h]) + (*ex[h] & 0xFFFFu);
-                const uint32_t p1 = run;
-                run += __popc(bm[2 * h + 1]) + (*ex[h] >> 16);
-                *ex[h] = p0 | (p1 << 16);
-            }
-            *reinterpret_cast<uint4 *>(A.PF + w0 + g) = e;
-            for (; m; m &= m - 1u) set_dirty(w0 + g + (uint32_t)__ffs((int)m) - 1u);
-        }
-    } else if (w0 < W) {
-        for (uint32_t g = 0; g < per; ++g) {
-            const uint32_t x = A.PF[w0 + g];
-            A.PF[w0 + g] = (uint16_t)run;
-            run += __popc(A.BM[w0 + g]) + x;
-            if (x) set_dirty(w0 + g);
-        }
-    }
 }
 
 // The dirty words' records in order: eight lanes a listed word, a lane per

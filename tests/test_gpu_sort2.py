@@ -49,6 +49,20 @@ def test_sort_table2_matches_oracle(vx, K, seed, kw):
     p.close()
 
 
+@pytest.mark.parametrize("K,mult", [(4, 2), (10, 1), (10, 2), (12, 3), (16, 4), (21, 1), (21, 2)])
+def test_sort_table2_levels_and_fills(vx, K, mult):
+    # One partition of few records and of more than its digits' words like
+    # (several pairs per record), one scatter level with a partial last tile,
+    # 10 partition bits in one level and, from 2^21 records on, 11 in two.
+    key = plot_key(60 + K)
+    D = mult * orc.default_distance(K)
+    p, got, _ = sorted_plot(vx, K, key, dict(match_scope=1, match_distance=D, t2_capacity=(mult + 1) << K))
+    ref = orc.sort_table2(orc.match_global(key, orc.table1(K, key), D))
+    assert K < 21 or (got.shape[0] >= 1 << 21) == (mult == 2)
+    assert np.array_equal(got, ref)
+    p.close()
+
+
 def test_sort_table2_after_split_path_and_twice(vx):
     K, key = 20, plot_key(44)
     p, got, work = sorted_plot(vx, K, key, {}, split=True)
