@@ -30,6 +30,7 @@ __global__ void k_key_setup(Desc *descs)
         *d.status = 0u;
         *d.ticket = 0u;
         *d.ticket_s = 0u;
+        for (int c = 0; c < kMaxPartChunks; ++c) d.ticket_i[c] = 0u;
         d.totals[0] = d.totals[1] = 0ull;
         if (d.wcount) *d.wcount = 0u;
     }

@@ -531,10 +531,17 @@ struct GlobalSrc {
 };
 
 // ------------------------------------------------- persistent front end
-// Work item t of the launch (CTA b takes b, b + G, b + 2G, ...) belongs to
-// plot find_plot(t); its partition is the plot's next ticket (look-back
-// modes) or t - tile_start[plot].  A CTA takes the ticket of item k + 2
-// and reads the fill count of item k + 1 at the start of item k, and
+// CTA b starts with work item b of the launch and takes the next ones from a
+// counter (the first plot's ticket_i of the launch's chunk), so that all end
+// together, also when a CTA starts late: CTAs of a dependent launch come onto
+// an SM as the kernel before leaves it, in whatever shared memory is free, so
+// that a few SMs host two instead of three and the CTAs left over start when
+// the others end (K=28, taking b, b + G, b + 2G, ...: two of 456, a sort of
+// 5.0 ms instead of 3.0).  Where all start together it evens out the end:
+// K=26 0.75 -> 0.72 ms, K=31 24.2 -> 22.8 ms.  Item t belongs to plot find_plot(t); its partition
+// is the plot's next ticket (look-back modes) or t - tile_start[plot].  A CTA
+// takes its items two ahead (look-back modes: three, with the ticket of the
+// second and the fill count of the first read at the start of an item) and
 // starts item k + 1's slot copy once item k's records have been placed, so
 // the global round trips and the copy overlap item k's match.
 // A CTA takes tickets in its processing order and only while running, so
@@ -578,14 +585,14 @@ __device__ __forceinline__ Item take_item(const Desc *__restrict__ descs, int np
 template <int MODE, bool HALO>
 __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
     k_sortmatch_pipe(const Desc *__restrict__ descs, int nplots, const uint32_t *__restrict__ tile_start,
-                     uint32_t items, uint32_t max_cap, uint32_t max_words, bool quiet)
+                     uint32_t items, uint32_t max_cap, uint32_t max_words, bool quiet, int chunk)
 {
     constexpr bool EMIT = MODE == kSortHash || MODE == kSortEmit;
     constexpr int NT = kPipeThreads;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_plot;
     __shared__ uint32_t s_f, s_n;
-    __shared__ int s_valid;
+    __shared__ int s_valid, s_more;
     __shared__ uint64_t s_base;
     __shared__ int s_ok;
     const SMLayout L(max_cap, max_words, true);
@@ -598,11 +605,20 @@ __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
     pdl_go();
     pdl_wait();
 
-    // Thread 0's pipeline: the item after the current one (its ticket and,
-    // from the start of the current item on, its fill count) and the one
-    // after that (its ticket).
+    // Thread 0's pipeline: the item after the current one (from the start of
+    // the current item on with its fill count), in the look-back modes the one
+    // after that, and the number of the next.
     Item nx{0, 0, false}, nn{0, 0, false};
-    uint32_t nx_n = 0;
+    uint32_t nx_n = 0, nt = items;
+    auto next_number = [&]() {
+        if (nt < items) nt = G + atomicAdd(descs->ticket_i + chunk, 1u);
+    };
+    auto take = [&]() {  // item nt; its successor's number is on its way
+        Item it{0, 0, false};
+        if (nt < items) it = take_item<EMIT>(descs, nplots, tile_start, nt);
+        next_number();
+        return it;
+    };
     // Starts the copy of item `it` (n records) into X and publishes it as
     // the next item; an invalid or empty item completes the barrier phase
     // with no copy.
@@ -628,31 +644,35 @@ __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
     };
     if (threadIdx.x == 0) {
         mbar_init(bar, 1);
+        s_more = blockIdx.x < items ? 1 : 0;
         if (blockIdx.x < items) {
             const Item i0 = take_item<EMIT>(descs, nplots, tile_start, blockIdx.x);
             const uint32_t n0 = i0.f < (1u << descs[i0.plot].p) ? descs[i0.plot].cnt2[i0.f] : 0u;
-            if (blockIdx.x + G < items) nx = take_item<EMIT>(descs, nplots, tile_start, blockIdx.x + G);
+            nt = 0;
+            next_number();
+            if (EMIT) nx = take();
             launch_copy(i0, min(n0, descs[i0.plot].cap2));
         }
     }
     __syncthreads();
     uint32_t phase = 0;
-    for (uint32_t t = blockIdx.x; t < items; t += G, phase ^= 1u) {
+    for (; s_more; phase ^= 1u) {
         const int plot = s_plot;
         const uint32_t f = s_f, n = s_n;
         const bool valid = s_valid != 0;
         const Desc &d = descs[plot];
-        if (threadIdx.x == 0) {
-            if (nx.ok) {
-                const Desc &dn = descs[nx.plot];
-                nx_n = nx.f < (1u << dn.p) ? min(dn.cnt2[nx.f], dn.cap2) : 0u;
-            }
-            if (t + 2 * G < items) nn = take_item<EMIT>(descs, nplots, tile_start, t + 2 * G);
-        }
         const uint32_t W = bitmap_words(d.dbits);
         A.PF = reinterpret_cast<uint16_t *>(A.BM + W);
         clear_tables<NT>(A, W);
         const uint64_t off = valid ? d.t1off[f] : 0ull;
+        if (threadIdx.x == 0) {
+            if (!EMIT) nx = take();
+            if (nx.ok) {
+                const Desc &dn = descs[nx.plot];
+                nx_n = nx.f < (1u << dn.p) ? min(dn.cnt2[nx.f], dn.cap2) : 0u;
+            }
+            if (EMIT) nn = take();
+        }
         // The slot copy was started during the previous item (or above).
         if (!__syncthreads_and(mbar_wait(bar, phase, d.spin_limit))) {
             if (threadIdx.x == 0) {
@@ -664,9 +684,11 @@ __global__ void __launch_bounds__(kPipeThreads, MODE == kSortHash ? 2 : 3)
         }
         // The next item's copy starts once this slot has been placed in Y.
         auto start_next = [&]() {
-            if (nx.ok) launch_copy(nx, nx_n);
+            if (nx.ok)
+                launch_copy(nx, nx_n);
+            else
+                s_more = 0;
             nx = nn;
-            nn.ok = false;
         };
         if (valid) {
             A.Y = Y0 + ((uint32_t)(3 * off) & 3u);
@@ -743,7 +765,8 @@ uint32_t sortmatch_max_cap() { return 16384u; }
 
 template <int MODE, bool HALO>
 static cudaError_t launch_sm(const Desc *descs, int nplots, const uint32_t *tile_start,
-                             uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits, bool quiet)
+                             uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits, bool quiet,
+                             int chunk)
 {
     if (total_tiles == 0) return cudaSuccess;
     const uint32_t words = bitmap_words(max_dbits);
@@ -769,7 +792,7 @@ static cudaError_t launch_sm(const Desc *descs, int nplots, const uint32_t *tile
         }
         const uint32_t want = (uint32_t)fit;
         return launch_on(on, fn, want < total_tiles ? want : total_tiles, kPipeThreads, pipe, descs, nplots,
-                         tile_start, total_tiles, max_cap, words, quiet);
+                         tile_start, total_tiles, max_cap, words, quiet, chunk);
     }
     const size_t smem = SMLayout(max_cap, words, false).bytes;
     auto fn = k_sortmatch_gl<MODE, HALO>;
@@ -782,29 +805,33 @@ static cudaError_t launch_sm(const Desc *descs, int nplots, const uint32_t *tile
 template <int MODE>
 static cudaError_t launch_sm2(const Desc *descs, int nplots, const uint32_t *tile_start,
                               uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
-                              bool halo, bool quiet)
+                              bool halo, bool quiet, int chunk)
 {
     // HALO instances carry the cross-bucket code; plain launches do not.
-    return halo ? launch_sm<MODE, true>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, quiet)
-                : launch_sm<MODE, false>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, quiet);
+    return halo ? launch_sm<MODE, true>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, quiet,
+                                         chunk)
+                : launch_sm<MODE, false>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, quiet,
+                                          chunk);
 }
 
 cudaError_t launch_sortmatch(const Desc *descs, int nplots, const uint32_t *tile_start,
                              uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
-                             SortMatchOut out, bool halo, bool quiet)
+                             SortMatchOut out, bool halo, bool quiet, int chunk)
 {
     if (out == kOutLookbackHashed)
-        return launch_sm2<kSortHash>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo, false);
+        return launch_sm2<kSortHash>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo, false,
+                                      chunk);
     if (out == kOutSlots)
-        return launch_sm2<kSortSlots>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo, quiet);
-    return launch_sm2<kSortEmit>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo, false);
+        return launch_sm2<kSortSlots>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo, quiet,
+                                       chunk);
+    return launch_sm2<kSortEmit>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo, false, chunk);
 }
 
 cudaError_t launch_sort(const Desc *descs, int nplots, const uint32_t *tile_start,
                         uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
                         bool halo)
 {
-    return launch_sm2<kSortCount>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo, false);
+    return launch_sm2<kSortCount>(descs, nplots, tile_start, total_tiles, on, max_cap, max_dbits, halo, false, 0);
 }
 
 }  // namespace vx

@@ -39,6 +39,7 @@ static_assert(kPlanT2HashTile == kT2HashTile, "planner and pair-hash kernel tile
 static_assert(kPlanT2SlotGroup == (uint64_t)kT2SlotGroup, "planner and slot pair-hash groups differ");
 static_assert(kHashThreads == kPlanHashThreads && kHashNoncesPerThread == kPlanNoncesPerThread,
               "hash shape the planner accepts");
+static_assert(kMaxPartChunks >= kMaxChunks, "a counter per chunk of the sort");
 static_assert(kMatchThreads >= 256, "k_match loads a halo (<= 256 records) one per thread");
 static_assert(sizeof(Desc) + 64 <= kStageTilesOffset, "descriptor overlaps staged tiles");
 static_assert(kStageTilesOffset + kTileArrays * 2 * sizeof(uint32_t) <= kStageResultOffset &&
@@ -168,6 +169,7 @@ void fill_desc(const vx_plot *p, Desc *d)
     d->ticket = reinterpret_cast<uint32_t *>(s + pl.o_ticket);
     d->lbs = reinterpret_cast<uint64_t *>(s + pl.o_lbs);
     d->ticket_s = reinterpret_cast<uint32_t *>(s + pl.o_ticket_s);
+    d->ticket_i = reinterpret_cast<uint32_t *>(s + pl.o_ticket_i);
     if (pl.hcap) {
         d->halo_cnt = reinterpret_cast<uint32_t *>(s + pl.o_halo_cnt);
         d->halo_keys = reinterpret_cast<uint64_t *>(s + pl.o_halo_keys);
@@ -496,7 +498,7 @@ cudaError_t launch_fused(const LaunchSet &L, const vx::Lanes &ln, const vx::Trac
                                                              L.max_cap2, L.max_dbits,
                                                              L.fuse_pair_hash ? vx::kOutLookbackHashed
                                                                               : vx::kOutLookback,
-                                                             L.halo));
+                                                             L.halo, false, c));
         if (ph && L.n_t2h[c]) {
             if (ov) {
                 cudaEventRecord(ln.sync[vx::kMaxChunks + 1 + c], A);

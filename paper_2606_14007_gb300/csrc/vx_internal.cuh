@@ -24,6 +24,7 @@ constexpr int kScatterThreads = 512;
 constexpr int kSortThreads = 256;
 constexpr int kMatchThreads = 256;
 constexpr int kMaxSortDigitBits = 13;    // counting-sort digit of the partition sort
+constexpr int kMaxPartChunks = 8;         // partition chunks of a plot
 constexpr uint32_t kMaxPartition = 16384;  // records one partition may hold (smem)
 constexpr size_t kMaxSmemPerCta = 227 * 1024;  // opt-in dynamic shared memory per CTA
 
@@ -85,6 +86,7 @@ struct Desc {
     uint32_t *ticket;    // partition ticket of the fused sort+match
     uint64_t *lbs;       // [chunks] look-back words of the Table-1 offset scan
     uint32_t *ticket_s;  // chunk ticket of the Table-1 offset scan
+    uint32_t *ticket_i;  // [kMaxPartChunks] items handed out by a persistent sort launch (its first plot's)
     uint32_t *status;    // status word
     uint64_t *totals;    // {Table-2 count, Table-1 count}, 8 bytes past the status word
     uint64_t *result;    // pinned host words {status, Table-2 count, Table-1 count}
@@ -642,7 +644,7 @@ cudaError_t launch_hash_direct(const Desc *descs, int nplots, const uint32_t *ti
 enum SortMatchOut { kOutLookback = 0, kOutLookbackHashed = 1, kOutSlots = 2 };
 cudaError_t launch_sortmatch(const Desc *descs, int nplots, const uint32_t *tile_start,
                              uint32_t total_tiles, On on, uint32_t max_cap, int max_dbits,
-                             SortMatchOut out, bool halo, bool quiet = false);
+                             SortMatchOut out, bool halo, bool quiet = false, int chunk = 0);
 cudaError_t launch_t2_hash(const Desc *descs, int nplots, const uint32_t *tile_start,
                            uint32_t total_tiles, int chunk, On on);
 // Pair hash of the slot placement: kT2SlotGroup partitions per CTA, pairs

@@ -81,7 +81,7 @@ struct Plan {
     uint64_t regionA_keys, regionB_keys;   // byte offset of the nonce array in each slot region
     uint64_t regionA_bytes, regionB_bytes;
     uint64_t t1_bytes, t2_bytes, scratch_bytes;
-    uint64_t o_status, o_ticket, o_ticket_s, o_cnt1, o_cnt2, o_t1off, o_pairs, o_t2off, o_lb, o_lbs,
+    uint64_t o_status, o_ticket, o_ticket_s, o_ticket_i, o_cnt1, o_cnt2, o_t1off, o_pairs, o_t2off, o_lb, o_lbs,
         o_desc, o_tiles;
     uint64_t o_regionB;                    // final-partition slots (scratch buffer)
     uint64_t o_halo_cnt, o_halo_keys, o_halo_nonces;  // scope 1 halos (scratch buffer)
@@ -377,6 +377,7 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
     P.o_status = at;
     P.o_ticket = at + 64;
     P.o_ticket_s = at + 128;
+    P.o_ticket_i = at + 192;  // one word per pipeline chunk
     at += 256;
     P.o_cnt1 = at; at = round_up(at + 4 * ((uint64_t)P.hchunks << P.p1), 256);
     P.o_cnt2 = at; at = round_up(at + 4 * np, 256);
