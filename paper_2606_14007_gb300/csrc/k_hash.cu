@@ -303,7 +303,7 @@ static cudaError_t launch_hs_agg(const Desc *descs, int nplots, const uint32_t *
                                  uint32_t total_tiles, bool agg, int chunk, On on, int npt, int bits)
 {
     if (WM != kWinNone && npt != kHashNoncesPerThread && npt != 16) return cudaErrorInvalidValue;
-    if (bits > kMaxCoarseBits) {  // 2^20 partitions and more: tiles of 4096 only
+    if (bits > kMaxCoarseBits) {  // 2^19 partitions and more: tiles of 4096 only
         if constexpr (WM == kWinNone || WM == kWinFilter)
             return npt == 16 ? launch_hs<16, false, HALO, WM, kMaxCoarseBitsWide>(descs, nplots, tile_start, total_tiles,
                                                                                  chunk, on)

@@ -16,7 +16,7 @@ namespace vx {
 constexpr int kBucketBits = 24;          // 2^24 logical buckets (Sec. I-A, III-B)
 constexpr int kMaxK = 32;                // u32 nonces
 constexpr int kMaxCoarseBits = 10;       // first scatter level, <= 1024 bins
-constexpr int kMaxCoarseBitsWide = 11;   // ... up to 2048 (2^20 partitions and more)
+constexpr int kMaxCoarseBitsWide = 11;   // ... up to 2048 (2^19 partitions and more)
 constexpr int kMaxFineBits = 10;         // second scatter level, <= 1024 bins
 constexpr int kMaxFineBitsWide = 11;     // ... up to 2048 (2^21 partitions, K = 32)
 constexpr int kScatterTile = 4096;       // records per CTA in the second scatter level

@@ -227,14 +227,14 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
     } else {
         // Two levels: the first takes most bits.  It claims inside the
         // ALU-bound hash, where more bins cost little, and the second then
-        // writes longer runs (K = 30: 9 + 10 bits 25.62 + 8.01 ms, 10 + 9
-        // bits 25.73 + 6.36); below 15 bits a few fewer (K = 25: 9 + 5 bits
-        // 2139 us per plot, 10 + 4 bits 2154, 7 + 7 bits 2142).
-        // At 2^20 partitions and more 11 bits, which the largest tile's
-        // kernel also takes (K = 31: 10 + 10 bits 48.5 + 15.6 ms, 11 + 9
-        // bits 49.1 + 13.0; K = 32: 10 + 11 bits 99.6 + 55.0, 11 + 10 bits
-        // 100.7 + 31.1).
-        P.p1 = P.p <= 10 ? P.p : P.p < 14 ? 8 : P.p == 14 ? 9 : P.p < 20 || P.wbits || P.npt != 16 ? 10 : 11;
+        // writes longer runs (K = 28: 8 + 9 bits 6.04 + 1.34 ms, 9 + 8 bits
+        // 6.06 + 1.17, 10 + 7 bits 6.09 + 1.13); below 15 bits a few fewer
+        // (K = 25: 9 + 5 bits 2139 us per plot, 10 + 4 bits 2154, 7 + 7 bits
+        // 2142).  At 2^19 partitions and more 11 bits, which the largest
+        // tile's kernel also takes (K = 31: 10 + 10 bits 48.5 + 15.4 ms, 11 +
+        // 9 bits 49.0 + 10.6; K = 30: 10 + 9 bits 24.27 + 5.38, 11 + 8 bits
+        // 24.52 + 4.68; K = 29 not yet: 12.15 + 2.35 against 12.26 + 2.25).
+        P.p1 = P.p <= 10 ? P.p : P.p < 14 ? 8 : P.p == 14 ? 9 : P.p < 19 || P.wbits || P.npt != 16 ? 10 : 11;
     }
     P.p2 = P.p - P.p1;
     if (P.mode == kScatterStaged && (P.p1 > (opts.coarse_bits < 0 ? 11 : 10) || P.p2 > 11)) {

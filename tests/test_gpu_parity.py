@@ -511,11 +511,11 @@ def test_split_match_past_the_pair_slots(vx, times):
     p.close()
 
 
-@pytest.mark.parametrize("scope", [0, 1], ids=["bucket", "cross"])
-def test_two_to_the_20_partitions(vx, scope):
-    # first scatter level of 11 bits (2^20 partitions of 64 records), alone
-    # and in a batch with a window, against the plan of 2^15 partitions
-    K, key = 26, plot_key(640)
+@pytest.mark.parametrize("K,scope", [(25, 0), (26, 0), (26, 1)], ids=["19-bucket", "bucket", "cross"])
+def test_two_to_the_20_partitions(vx, K, scope):
+    # first scatter level of 11 bits (2^19 and 2^20 partitions of 64 records),
+    # alone and in a batch with a window, against partitions of 2048 records
+    key = plot_key(640)
     D = 1 << 34
     a = vx.Plot(K, key, vx.make_opts(match_scope=scope, match_distance=D))
     a.run()
