@@ -185,8 +185,8 @@ KERNEL_SOURCES = {
     "hash_staged": ["paper_2606_14007_gb300/csrc/k_hash.cu", _H],
     "hash_direct": ["paper_2606_14007_gb300/csrc/k_hash.cu", _H],
     "scatter2": ["paper_2606_14007_gb300/csrc/k_sort.cu", _H],
-    "sort": ["paper_2606_14007_gb300/csrc/k_sortmatch.cu", _H],
-    "sortmatch": ["paper_2606_14007_gb300/csrc/k_sortmatch.cu", _H],
+    "sort": ["paper_2606_14007_gb300/csrc/k_sortmatch.cu", "paper_2606_14007_gb300/csrc/bitmap_sort.cuh", _H],
+    "sortmatch": ["paper_2606_14007_gb300/csrc/k_sortmatch.cu", "paper_2606_14007_gb300/csrc/bitmap_sort.cuh", _H],
     "pairhash": ["paper_2606_14007_gb300/csrc/k_hash.cu", _H],
     "match": ["paper_2606_14007_gb300/csrc/k_match.cu", _H],
 }

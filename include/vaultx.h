@@ -319,7 +319,7 @@ int vx_plot_tiled_bytes(int K, const vx_opts *opts, int window_bits, uint64_t *d
  * *passes, rounded up: 1 for c = 0 (the whole plot), 2 for 1 <= c <= 8 without
  * nonce chunks (one pass stores a window-id byte per nonce, then a window
  * hashes only its own nonces), else 2^c (each window hashes every nonce and
- * keeps its share: at K=31 a hash pass takes ~51 ms, so c = 9 costs ~26 s).
+ * keeps its share: at K=31 a hash pass takes ~49 ms, so c = 9 costs ~25 s).
  * The cost to weigh against vx_plot_tiled_bytes' footprint: above 8 bits
  * the id bytes are gone (K=31: 2.93 GB at c = 8, 0.39 GB at c = 9) but the
  * hashing grows 256-fold.  VX_EINVAL as vx_plot_tiled_bytes.  Host only.

@@ -27,15 +27,17 @@
 // offsets, and the pairs go through a 16-bit list in shared memory, so that
 // they are written one per lane, coalesced.
 //
-// Bound by instruction issue (56%) and the shared-memory data path (65%)
-// together at 24 warps per SM: 15.6 k warp instructions per 2048-record
+// Bound by instruction issue (59%) and the shared-memory data path (66%)
+// together at 24 warps per SM: 15.9 k warp instructions per 2048-record
 // partition, against 23 k for the counting sort with ranked digit runs, the
 // per-thread Table-1 stores and the record-wise pair stores before it: 31.0
-// -> 24.1 ms at K=31 (2^31 records; 2.85 of 6.78 TB/s), 0.97 -> 0.75 ms at
-// K=26.  By phase at K=26: load, mark and scan 0.23 ms, placement 0.14,
+// -> 24.1 ms at K=31, 0.97 -> 0.75 ms at K=26, and with the items handed out
+// by a counter 22.8 ms (2^31 records; 3.0 of 6.78 TB/s) and 0.72 ms.  By
+// phase at K=26, of 0.75 ms: load, mark and scan 0.23 ms, placement 0.14,
 // shared digits 0.04, match and lists 0.27, pair stores 0.07.  Tried and
-// dropped: half the digits (0.88 ms), the slot read into registers with four
-// CTAs per SM (0.78), eleven rows of loads in flight instead of four (0.82).
+// dropped, against 0.75: half the digits (0.88 ms), the slot read into
+// registers with four CTAs per SM (0.78), eleven rows of loads in flight
+// instead of four (0.82).
 //
 // Two front ends feed the same steps:
 //  * k_sortmatch_pipe (the default): persistent CTAs, three per SM at the
