@@ -29,6 +29,7 @@ __device__ __forceinline__ uint64_t sort2_key(uint4 r)
 // ------------------------------------------------------------------ setup
 __global__ void k_s2_setup(Sort2Desc *dp)
 {
+    pdl_go();
     Sort2Desc &d = *dp;
     const uint64_t n1 = d.p2 > 0 ? (1ull << d.p1) : 0ull;
     const uint64_t n2 = 1ull << d.p;
@@ -71,6 +72,8 @@ __global__ void __launch_bounds__(kS2Threads, 3) k_s2_scatter(const Sort2Desc *_
 {
     constexpr int NT = kS2Threads, PER = kS2Tile / NT;
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    pdl_go();
+    pdl_wait();
     const Sort2Desc &d = *dp;
     const bool last = LEVEL == 2 || d.p2 == 0;  // the level that fills the partitions
     const int bits = LEVEL == 2 ? d.p2 : last ? d.p : d.p1;
@@ -188,6 +191,8 @@ __global__ void __launch_bounds__(256) k_s2_scan(const Sort2Desc *__restrict__ d
     __shared__ uint32_t s_c;
     __shared__ uint64_t s_base;
     __shared__ int s_ok;
+    pdl_go();
+    pdl_wait();
     const Sort2Desc &d = *dp;
     if (threadIdx.x == 0) s_c = atomicAdd(d.ticket, 1u);
     __syncthreads();
@@ -314,6 +319,8 @@ __global__ void __launch_bounds__(kS2SortThreads, 4) k_s2_sort(const Sort2Desc *
 {
     constexpr int NT = kS2SortThreads;
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    pdl_go();
+    pdl_wait();
     const Sort2Desc &d = *dp;
     if (*d.status & (kStSort2 | kStTimeout | kStBadTicket)) return;  // offsets not trusted
     const uint32_t f = blockIdx.x;
@@ -388,27 +395,29 @@ size_t sort2_smem_bytes(uint32_t cap, int dbits) { return S2SortLayout(cap, sort
 cudaError_t launch_sort2(const Sort2Desc *d_desc, const Sort2Launch &g, cudaStream_t s)
 {
     static SmemSeen seen1, seen2, seen3;
+    // One level (under 2^21 records), bound by the chain of launches: each
+    // kernel a programmatic dependent of the one before (K=16 35.9 -> 33.0 us,
+    // K=20 47.5 -> 42.0).  Two levels gain as much or lose (K=26 1092 -> 1087
+    // us, K=28 4.80 -> 4.94 ms: CTAs of the next kernel take the places of the
+    // last ones of this), so those launch plainly.
+    const On on(s, g.tiles2 == 0);
     cudaError_t e;
     k_s2_setup<<<64, 256, 0, s>>>(const_cast<Sort2Desc *>(d_desc));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (g.tiles1) {
         const size_t sm = S2ScatterLayout(g.p - g.p2).bytes;
         if ((e = allow_smem(k_s2_scatter<1>, sm, seen1)) != cudaSuccess) return e;
-        k_s2_scatter<1><<<g.tiles1, kS2Threads, sm, s>>>(d_desc);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_on(on, k_s2_scatter<1>, g.tiles1, kS2Threads, sm, d_desc)) != cudaSuccess) return e;
     }
     if (g.tiles2) {
         const size_t sm = S2ScatterLayout(g.p2).bytes;
         if ((e = allow_smem(k_s2_scatter<2>, sm, seen2)) != cudaSuccess) return e;
-        k_s2_scatter<2><<<g.tiles2, kS2Threads, sm, s>>>(d_desc);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_on(on, k_s2_scatter<2>, g.tiles2, kS2Threads, sm, d_desc)) != cudaSuccess) return e;
     }
-    k_s2_scan<<<g.tiles_scan, 256, 0, s>>>(d_desc);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_on(on, k_s2_scan, g.tiles_scan, 256, 0, d_desc)) != cudaSuccess) return e;
     const size_t sm = sort2_smem_bytes(g.cap2, g.dbits);
     if ((e = allow_smem(k_s2_sort, sm, seen3)) != cudaSuccess) return e;
-    k_s2_sort<<<g.parts, kS2SortThreads, sm, s>>>(d_desc);
-    return cudaGetLastError();
+    return launch_on(on, k_s2_sort, g.parts, kS2SortThreads, sm, d_desc);
 }
 
 }  // namespace vx
