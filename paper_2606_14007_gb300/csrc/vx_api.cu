@@ -204,16 +204,17 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
     L->max_dbits = 1;
     L->max_p2 = 0;
     int min_bits = 64, max_bits = 0;
-    // One staged hash launch takes one shape: the plots' common nonces per
-    // thread, else the automatic one of their nonces together (any shape
-    // gives the same records).
+    // One staged hash launch takes one shape (any gives the same records): the
+    // plots' common nonces per thread, else, or where the planner chose for
+    // every plot, the automatic one of their nonces together.
     int npt = n > 0 && plots[0] ? plots[0]->plan.npt : kPlanNoncesPerThread;
-    bool same_npt = true;
+    bool same_npt = true, auto_npt = n > 1;
     uint64_t nonces = 0;
     for (int i = 0; i < n; ++i) {
         if (!plots[i] || !plots[i]->d_t1) return VX_EINVAL;
         const Plan &pl = plots[i]->plan;
         same_npt = same_npt && pl.npt == npt;
+        auto_npt = auto_npt && pl.npt_auto;
         nonces += pl.N;
         fuse = fuse && pl.fuse_pair_hash;
         slots = slots && pl.pair_slots;
@@ -236,7 +237,7 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
         }
     }
     if (max_bits > vx::kMaxCoarseBits) npt = 16;  // the one tile with more bins
-    else if (!same_npt) npt = win ? kPlanNoncesPerThread : vx::auto_nonces_per_thread(nonces);
+    else if (!same_npt || (auto_npt && !win)) npt = win ? kPlanNoncesPerThread : vx::auto_nonces_per_thread(nonces);
     uint64_t acc[vx::kTileArrays] = {};
     for (int a = 0; a < vx::kTileArrays; ++a) h[a * W] = 0;
     for (int i = 0; i < n; ++i) {

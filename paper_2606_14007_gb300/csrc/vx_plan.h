@@ -34,12 +34,14 @@ constexpr int kPlanNoncesPerThread = 8;    // nonces per hash thread of the dire
 // of them threads claims one run per bin, so large tiles claim less (16
 // against 8: 1.519 against 1.559 ms at 2^26 nonces); small plots need more
 // CTAs than large tiles give (2 against 8: 9.2 against 16.4 us at 2^14; at
-// 2^20, 2 pays 51 us in claims against 37 with 8), and between them 12 lets
-// four CTAs share an SM instead of three (398 us at 2^24; 404 with 8, 416
-// with 16).
+// 2^20, where 2 pays 51 us in claims, 4 leaves enough tiles for a second one
+// to hash while the first claims and stores: a plot takes 71.6 us against
+// 73.7 with 8, at 2^19 45.6 against 47, at 2^21 137 against 113), and above
+// them 12 lets four CTAs share an SM instead of three (398 us at 2^24; 404
+// with 8, 416 with 16).
 inline int auto_nonces_per_thread(uint64_t n)
 {
-    return n < (1ull << 18) ? 2 : n < (1ull << 22) ? 8 : n < (1ull << 25) ? 12 : 16;
+    return n < (1ull << 18) ? 2 : n <= (1ull << 20) ? 4 : n < (1ull << 22) ? 8 : n < (1ull << 25) ? 12 : 16;
 }
 
 // Table-1 hash CTAs over n nonces with npt nonces per thread.
@@ -63,6 +65,7 @@ struct Plan {
     uint32_t wbits, win;                   // window: top wbits of key64 == win (wbits 0: whole plot)
     int mode;                              // kScatterStaged or kScatterDirect
     int npt;                               // nonces per thread of the Table-1 hash (2, 4, 8, 12, 16)
+    bool npt_auto;                         // chosen by the planner
     uint32_t test_flags, spin_limit;
     bool fuse_pair_hash;
     bool pair_slots;                       // pairs staged in the partition slots (t2_placement 2)
@@ -171,6 +174,7 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
         return VX_EINVAL;
     }
     P.npt = (int)opts.nonces_per_thread;
+    P.npt_auto = P.npt == 0;
     P.fuse_pair_hash = opts.fuse_pair_hash != 0;
     const uint32_t pc = opts.pipeline_chunks;
     if (pc != 0 && pc != 1 && pc != 2 && pc != 4 && pc != 8) {
