@@ -16,6 +16,7 @@
 #include <cstddef>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -299,15 +300,26 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
 
 // Uploads the descriptor and the single-plot tile prefixes if they changed
 // and caches the single-plot launch set.
+// The plot's pinned block; *result is where the device writes a run's result.
+cudaError_t ensure_stage(vx_plot *p, uint64_t **result)
+{
+    cudaError_t e = cudaSuccess;
+    void *h = p->h_stage, *r = nullptr;
+    if (!h) {
+        if ((e = cudaMallocHost(&h, vx::kStageBytes)) != cudaSuccess) return e;
+        p->h_stage = reinterpret_cast<Desc *>(h);
+    }
+    if (!p->ev_stage && (e = cudaEventCreateWithFlags(&p->ev_stage, cudaEventDisableTiming)) != cudaSuccess) return e;
+    e = cudaHostGetDevicePointer(&r, static_cast<uint8_t *>(h) + vx::kStageResultOffset, 0);
+    *result = static_cast<uint64_t *>(r);
+    return e;
+}
+
 int upload_desc(vx_plot *p, cudaStream_t s)
 {
     if (!p->desc_dirty) return VX_OK;
-    if (!p->h_stage) {
-        void *h = nullptr;
-        VX_TRY(p, cudaMallocHost(&h, vx::kStageBytes));
-        p->h_stage = reinterpret_cast<Desc *>(h);
-        VX_TRY(p, cudaEventCreateWithFlags(&p->ev_stage, cudaEventDisableTiming));
-    }
+    uint64_t *result = nullptr;
+    VX_TRY(p, ensure_stage(p, &result));
     if (p->ev_pending) VX_TRY(p, cudaEventSynchronize(p->ev_stage));
     fill_desc(p, p->h_stage);
     uint32_t *t = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(p->h_stage) +
@@ -319,12 +331,7 @@ int upload_desc(vx_plot *p, cudaStream_t s)
     }
     p->single.descs = dev_desc(p);
     // The slot pair hash leaves the run's result in the pinned block itself.
-    p->h_stage->result = nullptr;
-    if (p->single.pair_slots) {
-        void *r = nullptr;
-        VX_TRY(p, cudaHostGetDevicePointer(&r, reinterpret_cast<uint8_t *>(p->h_stage) + vx::kStageResultOffset, 0));
-        p->h_stage->result = reinterpret_cast<uint64_t *>(r);
-    }
+    p->h_stage->result = p->single.pair_slots ? result : nullptr;
     VX_TRY(p, cudaMemcpyAsync(dev_desc(p), p->h_stage, sizeof(Desc), cudaMemcpyHostToDevice, s));
     VX_TRY(p, cudaMemcpyAsync(dev_tiles(p), t, vx::kTileArrays * 2 * sizeof(uint32_t),
                               cudaMemcpyHostToDevice, s));
@@ -680,7 +687,7 @@ int vx_table1(vx_plot *p, void *stream)
     p->t1_known = false;
     p->last = s;
     p->have_last = true;
-    p->res_pending = false;
+    p->res_pending = p->res_batch = false;
     return VX_OK;
 }
 
@@ -708,7 +715,7 @@ int vx_match(vx_plot *p, void *stream)
     p->t1_known = false;
     p->last = s;
     p->have_last = true;
-    p->res_pending = false;
+    p->res_pending = p->res_batch = false;
     return VX_OK;
 }
 
@@ -752,7 +759,7 @@ int vx_plot_run(vx_plot *p, void *stream)
     p->t1_known = false;
     p->last = s;
     p->have_last = true;
-    p->res_pending = false;
+    p->res_pending = p->res_batch = false;
     return record_result(p, s, p->single.pair_slots);
 }
 
@@ -779,7 +786,10 @@ int vx_sync(vx_plot *p)
     }
     if (p->have_last) VX_TRY(p, cudaStreamSynchronize(p->last));
     uint64_t words[3];  // {status, Table-2 count, Table-1 count}
-    VX_TRY(p, cudaMemcpy(words, p->d_scratch + p->plan.o_status, sizeof(words), cudaMemcpyDeviceToHost));
+    if (p->res_batch)
+        memcpy(words, reinterpret_cast<const uint8_t *>(p->h_stage) + vx::kStageResultOffset, sizeof(words));
+    else
+        VX_TRY(p, cudaMemcpy(words, p->d_scratch + p->plan.o_status, sizeof(words), cudaMemcpyDeviceToHost));
     const uint32_t st = (uint32_t)words[0];
     p->status = st;
     if (p->stage >= 1) {
@@ -857,7 +867,7 @@ int vx_sort_table2(vx_plot *p, void *d_work, uint64_t work_bytes, void *stream)
     if (e != cudaSuccess) return cuda_fail(p, "sort Table 2", e);
     p->last = s;
     p->have_last = true;
-    p->res_pending = false;
+    p->res_pending = p->res_batch = false;
     return record_result(p, s, false);  // vx_sync now waits for the sort and reads its status
 }
 
@@ -1146,6 +1156,7 @@ namespace {
 // sequence of plot handles (and their buffers) it was built for.
 struct BatchEntry {
     std::vector<vx_plot *> plots;
+    std::vector<vx_plot *> pinned;  // those whose pinned blocks take the results
     std::vector<uint8_t *> bufs;
     uint8_t *d_ws = nullptr;
     uint8_t *h_ws = nullptr;
@@ -1208,7 +1219,7 @@ size_t batch_ws_bytes(int n)
     return o_tiles + (size_t)kTileArrays * (size_t)(n + 1) * 4;
 }
 
-int batch_prepare(vx_plot *const *plots, int n, uint8_t *h_ws, uint8_t *d_ws, LaunchSet *L)
+int batch_prepare(vx_plot *const *plots, int n, uint8_t *h_ws, uint8_t *d_ws, LaunchSet *L, bool *results)
 {
     const size_t o_tiles = ((size_t)n * sizeof(Desc) + 255) & ~(size_t)255;
     Desc *hd = reinterpret_cast<Desc *>(h_ws);
@@ -1219,6 +1230,12 @@ int batch_prepare(vx_plot *const *plots, int n, uint8_t *h_ws, uint8_t *d_ws, La
     const int rc = build_tiles(plots, n, reinterpret_cast<uint32_t *>(h_ws + o_tiles),
                                reinterpret_cast<const uint32_t *>(d_ws + o_tiles), L);
     L->descs = reinterpret_cast<Desc *>(d_ws);
+    for (int i = 0; results && i < n; ++i) {
+        uint64_t *r = nullptr;
+        results[i] = rc == VX_OK && L->pair_slots && ensure_stage(plots[i], &r) == cudaSuccess;
+        if (results[i]) hd[i].result = r;
+        else cudaGetLastError();
+    }
     return rc;
 }
 
@@ -1258,7 +1275,7 @@ void mark_issued(vx_plot *const *plots, int n, cudaStream_t s)
         p->t1_known = false;
         p->last = s;
         p->have_last = true;
-        p->res_pending = false;
+        p->res_pending = p->res_batch = false;
     }
 }
 
@@ -1307,11 +1324,14 @@ extern "C" int vx_plot_batch(vx_plot *const *plots, int n, void *stream)
         LaunchSet L[2];
         for (int l = 0; l < nl; ++l) {
             const size_t at = l ? ws0 : 0;
-            if (vx::batch_prepare(lane[l].data(), (int)lane[l].size(), b->h_ws + at, b->d_ws + at, &L[l]) !=
-                VX_OK) {
+            std::unique_ptr<bool[]> pinned(new bool[lane[l].size()]());
+            if (vx::batch_prepare(lane[l].data(), (int)lane[l].size(), b->h_ws + at, b->d_ws + at, &L[l],
+                                  pinned.get()) != VX_OK) {
                 drop_batch(b);
                 return VX_EINVAL;
             }
+            for (size_t i = 0; i < lane[l].size(); ++i)
+                if (pinned[i]) b->pinned.push_back(lane[l][i]);
         }
         // The workspace is uploaded once; replays of the graph reuse it.
         cudaError_t e = cudaMemcpy(b->d_ws, b->h_ws, b->ws_bytes, cudaMemcpyHostToDevice);
@@ -1361,6 +1381,7 @@ extern "C" int vx_plot_batch(vx_plot *const *plots, int n, void *stream)
         return VX_ECUDA;
     }
     vx::mark_issued(plots, n, s);
+    for (vx_plot *p : b->pinned) p->res_batch = true;
     return VX_OK;
 }
 

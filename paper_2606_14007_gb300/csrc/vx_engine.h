@@ -88,6 +88,7 @@ struct vx_plot {
     bool have_last = false;
     cudaEvent_t ev_done = nullptr;  // behind vx_plot_run's kernels and result copy
     bool res_pending = false;       // vx_sync reads the pinned result block after ev_done
+    bool res_batch = false;         // ... after everything on `last` (a batch left it there)
     bool slot_pairs = false;       // the last Table 1 left its pairs in the partition slots
     int stage = 0;                 // 0 created, 1 Table 1 issued, 2 match issued
     bool t2_known = false;
@@ -120,8 +121,10 @@ namespace vx {
 // Batch workspace: descs[n] | kTileArrays tile prefixes of n + 1 entries.
 size_t batch_ws_bytes(int n);
 // Fills the host workspace for plots[0..n) (each bound) and the launch set
-// that reads it from d_ws.  Returns VX_OK or VX_EINVAL.
-int batch_prepare(vx_plot *const *plots, int n, uint8_t *h_ws, uint8_t *d_ws, LaunchSet *L);
+// that reads it from d_ws.  Returns VX_OK or VX_EINVAL.  With `results` the
+// plots of the slot placement leave their results in their pinned blocks
+// (allocated here if need be), results[i] says which do.
+int batch_prepare(vx_plot *const *plots, int n, uint8_t *h_ws, uint8_t *d_ws, LaunchSet *L, bool *results = nullptr);
 // Whole-plot kernel sequence (sort + match path, pipelined when lanes.aux).
 cudaError_t launch_plot_seq(const LaunchSet &L, const Lanes &lanes);
 // Creates the two aux streams (highest / lowest priority, non-blocking) and

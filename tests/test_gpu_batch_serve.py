@@ -124,3 +124,36 @@ def test_batch_mixed_scope_and_placement(vx):
             assert np.array_equal(p.t2.cpu().numpy(), r2), (rep, K)
     for p in plots:
         p.close()
+
+
+@pytest.mark.parametrize("placement", [0, 1], ids=["slots", "lookback"])
+def test_batch_results_of_good_and_failed_plots(vx, placement):
+    # each plot's status and counts after a batch, for the plots whose results
+    # the last kernel leaves in pinned memory and for the others: a Table 2
+    # that is too small, one that fits, a slot overflow; then the match alone
+    # on a larger buffer, a run of its own between two batches
+    opts = [dict(t2_capacity=16), dict(), dict(partition_log2=6, slack_sigma=1)]
+    mix = [(16, 201), (14, 202), (18, 203)]
+    plots = [vx.Plot(K, plot_key(s), vx.make_opts(t2_placement=placement, **o)) for (K, s), o in zip(mix, opts)]
+    handles = [p.handle for p in plots]
+    want = [oracle_tables(K, s)[1] for K, s in mix]
+    for rep in range(2):
+        vx.vx_plot_batch(handles)
+        codes = [vx.vx_sync(h, check=False) for h in handles]
+        assert codes == [vx.VX_ENOMEM, vx.VX_OK, vx.VX_EOVERFLOW], (rep, codes)
+        assert vx.vx_table_info(handles[0], vx.VX_TABLE2, check=False)[1] == want[0].shape[0]
+        assert vx.vx_table_info(handles[1], vx.VX_TABLE2)[1] == want[1].shape[0]
+        plots[1].run()
+        assert plots[1].sync() == want[1].shape[0]
+        assert np.array_equal(plots[1].t2.cpu().numpy(), want[1])
+    vx.vx_plot_batch(handles)
+    need = want[0].shape[0]
+    big = torch.empty(16 * need + 256, dtype=torch.uint8, device="cuda")
+    p = plots[0]
+    vx.vx_plot_bind(p.handle, p._t1.data_ptr(), big.data_ptr(), p._scratch.data_ptr(), need)
+    vx.vx_match(p.handle)
+    assert vx.vx_sync(p.handle) == vx.VX_OK
+    assert np.array_equal(big[: 16 * need].view(need, 16).cpu().numpy(), want[0])
+    torch.cuda.synchronize()
+    for p in plots:
+        p.close()
