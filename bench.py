@@ -181,12 +181,14 @@ def source_digest(files) -> str:
 
 
 _H = "paper_2606_14007_gb300/csrc/vx_internal.cuh"
+_SORT = ["paper_2606_14007_gb300/csrc/k_sortmatch.cu", "paper_2606_14007_gb300/csrc/bitmap_sort.cuh",
+         "paper_2606_14007_gb300/csrc/pair_list.h", _H]
 KERNEL_SOURCES = {
     "hash_staged": ["paper_2606_14007_gb300/csrc/k_hash.cu", _H],
     "hash_direct": ["paper_2606_14007_gb300/csrc/k_hash.cu", _H],
     "scatter2": ["paper_2606_14007_gb300/csrc/k_sort.cu", _H],
-    "sort": ["paper_2606_14007_gb300/csrc/k_sortmatch.cu", "paper_2606_14007_gb300/csrc/bitmap_sort.cuh", _H],
-    "sortmatch": ["paper_2606_14007_gb300/csrc/k_sortmatch.cu", "paper_2606_14007_gb300/csrc/bitmap_sort.cuh", _H],
+    "sort": _SORT,
+    "sortmatch": _SORT,
     "pairhash": ["paper_2606_14007_gb300/csrc/k_hash.cu", _H],
     "match": ["paper_2606_14007_gb300/csrc/k_match.cu", _H],
 }

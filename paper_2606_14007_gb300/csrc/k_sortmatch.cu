@@ -60,6 +60,7 @@
 // partition waits on another; a scan of the pair counts and the slot pair
 // hash place the records.
 #include "bitmap_sort.cuh"
+#include "pair_list.h"
 #include "vx_internal.cuh"
 
 namespace vx {
@@ -322,24 +323,14 @@ __device__ __forceinline__ void match_and_write(const Desc &d, uint32_t f, uint3
         const uint32_t incl = warp_incl_scan(cnt);
         const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
         if (MODE != kSortCount) {
-            fits = fits && mine + total + 4u <= A.plw;  // the same for the whole warp
+            fits = fits && mine + total <= A.plw;  // the same for the whole warp
             if (fits) {
-                // Every lane with a pair stores four entries, the farthest
-                // first: one past its own pairs lies on a later lane's, whose
-                // own store to that place is for a nearer record and comes
-                // later.
                 uint16_t *w = list + mine + incl - cnt;
                 const uint32_t e = 32u * (c - c0) + lane;
-                if (cnt) {
-                    w[3] = (uint16_t)(e + (4u << 12));
-                    w[2] = (uint16_t)(e + (3u << 12));
-                    w[1] = (uint16_t)(e + (2u << 12));
-                    w[0] = (uint16_t)(e + (1u << 12));
-                }
+                put_nearest_pairs(w, e, cnt);
                 if (__any_sync(0xffffffffu, cnt > 4)) {
                     fits = !__any_sync(0xffffffffu, cnt > 15u);
-                    for (uint32_t j = 4; fits && j < cnt; ++j) w[j] = (uint16_t)(e + ((j + 1u) << 12));
-                    __syncwarp();
+                    for (uint32_t j = 4; fits && j < cnt; ++j) w[j] = pair_entry(e, j + 1u);
                 }
             }
         }

@@ -1,0 +1,46 @@
+"""Host-compilable pieces of the library, compiled with g++ and driven here:
+what needs no GPU to be shown right."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2606_14007_gb300", "csrc")
+
+
+def run_cpp(tmp_path, source):
+    """Compiles a C++ program against csrc/ and runs it; its output."""
+    gxx = shutil.which("g++") or pytest.skip("no g++")
+    src, exe = tmp_path / "driver.cpp", tmp_path / "driver"
+    src.write_text(source)
+    subprocess.run([gxx, "-std=c++17", "-O1", "-Wall", "-pthread", "-I", CSRC, "-o", str(exe), str(src)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return r.stdout
+
+
+def test_pair_list_records_store_their_own_entries_only(tmp_path):
+    # The records of a chunk are 32 lanes whose stores come in no fixed order:
+    # a store outside a record's own places could undo another record's.
+    out = run_cpp(tmp_path, r"""
+#include <cstdio>
+#include "pair_list.h"
+int main()
+{
+    for (uint32_t cnt = 0; cnt <= 15; ++cnt) {
+        uint16_t list[32];
+        for (uint16_t &x : list) x = 0xABCDu;
+        vx::put_nearest_pairs(list + 8, 77u, cnt);
+        const uint32_t own = cnt < 4u ? cnt : 4u;
+        for (uint32_t i = 0; i < 32; ++i) {
+            const bool mine = i >= 8 && i < 8 + own;
+            const uint16_t want = mine ? (uint16_t)(77u + ((i - 7u) << 12)) : (uint16_t)0xABCDu;
+            if (list[i] != want) return printf("count %u: place %d holds %#x\n", cnt, (int)i - 8, list[i]), 1;
+        }
+    }
+    puts("ok");
+}
+""")
+    assert out.strip() == "ok"
