@@ -171,9 +171,8 @@ int vx_version(void);
  *   t1_bytes:      Table-1 buffer (>= 12 * 2^K; a staged two-level scatter
  *                  also uses it for its first level, so it may be larger)
  *   t2_bytes:      Table-2 buffer (16 * Table-2 capacity, + 256)
- *   scratch_bytes: counters, offsets, the plot descriptor, and the partition
- *                  slots the hashed records are bucketed into (about
- *                  12 * 2^K * 1.3 bytes)
+ *   scratch_bytes: counters, offsets, and the partition slots the hashed
+ *                  records are bucketed into (about 12 * 2^K * 1.3 bytes)
  * Any output pointer may be NULL.  1 <= K <= 32.  No allocation. */
 int vx_plot_required_bytes(int K, const vx_opts *opts, uint64_t *t1_bytes,
                            uint64_t *t2_bytes, uint64_t *scratch_bytes);
@@ -221,10 +220,14 @@ int vx_match(vx_plot *plot, void *stream);
  * sort kernel instead.  Same tables as vx_table1 + vx_match.  Ends with the
  * status and the record counts in the handle's pinned host memory (left
  * there by the slot pair hash, copied otherwise) and an event that vx_sync
- * waits on.  Allocates if nothing is bound.
+ * waits on.  Allocates if nothing is bound; a handle's first run also takes
+ * 4 KB of device and 4 KB of pinned host memory, its own until
+ * vx_plot_destroy.
  * Asynchronous.  One plot's runs must not overlap on the GPU (two runs of
  * the same plot on different streams race on its buffers): different plots
- * may run concurrently. */
+ * may run concurrently.  Plots that share Table-1 and scratch buffers may
+ * run one after the other on a stream, in any order and any number of
+ * times. */
 int vx_plot_run(vx_plot *plot, void *stream);
 
 /* Waits for the plot's work, reads its status word and Table-2 count, and

@@ -183,8 +183,8 @@ void fill_desc(const vx_plot *p, Desc *d)
     vx::b3_key_setup(d->key, 8u, d->pre2);
 }
 
-Desc *dev_desc(vx_plot *p) { return reinterpret_cast<Desc *>(p->d_scratch + p->plan.o_desc); }
-uint32_t *dev_tiles(vx_plot *p) { return reinterpret_cast<uint32_t *>(p->d_scratch + p->plan.o_tiles); }
+Desc *dev_desc(vx_plot *p) { return reinterpret_cast<Desc *>(p->d_stage); }
+uint32_t *dev_tiles(vx_plot *p) { return reinterpret_cast<uint32_t *>(p->d_stage + vx::kStageTilesOffset); }
 
 // Tile prefixes (exclusive prefix of per-plot CTA counts) of every launch of
 // a run over plots[0..n), written to h (host) for upload to d (device), and
@@ -298,8 +298,6 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
     return VX_OK;
 }
 
-// Uploads the descriptor and the single-plot tile prefixes if they changed
-// and caches the single-plot launch set.
 // The plot's pinned block; *result is where the device writes a run's result.
 cudaError_t ensure_stage(vx_plot *p, uint64_t **result)
 {
@@ -315,11 +313,25 @@ cudaError_t ensure_stage(vx_plot *p, uint64_t **result)
     return e;
 }
 
+// Uploads the descriptor and the single-plot tile prefixes if they changed
+// and caches the single-plot launch set.  The device copy is the handle's
+// own: the scratch buffer may be shared with other plots, whose runs may
+// have overwritten anything in it by this plot's next run.
 int upload_desc(vx_plot *p, cudaStream_t s)
 {
     if (!p->desc_dirty) return VX_OK;
     uint64_t *result = nullptr;
     VX_TRY(p, ensure_stage(p, &result));
+    if (!p->d_stage) {
+        void *d = nullptr;
+        const cudaError_t e = dev_alloc(&d, vx::kStageResultOffset);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            set_err(p, std::string("descriptor allocation failed: ") + cudaGetErrorName(e));
+            return e == cudaErrorMemoryAllocation ? VX_ENOMEM : VX_ECUDA;
+        }
+        p->d_stage = static_cast<uint8_t *>(d);
+    }
     if (p->ev_pending) VX_TRY(p, cudaEventSynchronize(p->ev_stage));
     fill_desc(p, p->h_stage);
     uint32_t *t = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(p->h_stage) +
@@ -332,8 +344,7 @@ int upload_desc(vx_plot *p, cudaStream_t s)
     p->single.descs = dev_desc(p);
     // The slot pair hash leaves the run's result in the pinned block itself.
     p->h_stage->result = p->single.pair_slots ? result : nullptr;
-    VX_TRY(p, cudaMemcpyAsync(dev_desc(p), p->h_stage, sizeof(Desc), cudaMemcpyHostToDevice, s));
-    VX_TRY(p, cudaMemcpyAsync(dev_tiles(p), t, vx::kTileArrays * 2 * sizeof(uint32_t),
+    VX_TRY(p, cudaMemcpyAsync(p->d_stage, p->h_stage, vx::kStageTilesOffset + vx::kTileArrays * 2 * sizeof(uint32_t),
                               cudaMemcpyHostToDevice, s));
     VX_TRY(p, cudaEventRecord(p->ev_stage, s));
     p->ev_pending = true;
@@ -1005,6 +1016,7 @@ void vx_plot_destroy(vx_plot *p)
     if (p->release) p->release(p->release_ctx, p);
     free_owned(p);
     if (p->h_stage) cudaFreeHost(p->h_stage);
+    if (p->d_stage) cudaFree(p->d_stage);
     if (p->ev_stage) cudaEventDestroy(p->ev_stage);
     if (p->ev_done) cudaEventDestroy(p->ev_done);
     vx_plot_profile(p, 0);

@@ -81,7 +81,8 @@ struct vx_plot {
     bool owned = false;
     uint64_t t2cap = 0;            // records the bound Table-2 buffer holds
     bool desc_dirty = true;        // descriptor needs an upload
-    vx::Desc *h_stage = nullptr;   // pinned staging: Desc + tile prefixes
+    vx::Desc *h_stage = nullptr;   // pinned block: Desc, tile prefixes, a run's result
+    uint8_t *d_stage = nullptr;    // the first two on the device, at the same offsets
     cudaEvent_t ev_stage = nullptr;
     bool ev_pending = false;
     cudaStream_t last = nullptr;

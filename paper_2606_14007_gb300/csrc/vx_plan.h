@@ -22,7 +22,7 @@ constexpr int kSort2PartLog2 = 10;         // the same for the sort of Table 2 b
 constexpr uint32_t kDefaultSlackSigma = 12;
 constexpr int kMaxPartBits = 21;           // scatter levels of <= 10 and <= 11 bits
 constexpr int kAggMaxBits = 6;             // warp-aggregate ranks up to 64 bins
-constexpr size_t kStageBytes = 4096;       // pinned staging: Desc + tile prefixes
+constexpr size_t kStageBytes = 4096;       // a handle's pinned block: Desc, tile prefixes, result
 constexpr size_t kStageTilesOffset = 3584;
 constexpr size_t kStageResultOffset = 4064;  // status u32 at +0, Table-2 count u64 at +8
 constexpr uint64_t kWriteStageBytes = 256ull << 20;  // Sec. III-B: 256 MB pinned staging
@@ -85,7 +85,7 @@ struct Plan {
     uint64_t regionA_bytes, regionB_bytes;
     uint64_t t1_bytes, t2_bytes, scratch_bytes;
     uint64_t o_status, o_ticket, o_ticket_s, o_ticket_i, o_cnt1, o_cnt2, o_t1off, o_pairs, o_t2off, o_lb, o_lbs,
-        o_desc, o_tiles;
+        o_desc, o_tiles;                   // the descriptor and tile prefixes of vx_plot_run_noalloc
     uint64_t o_regionB;                    // final-partition slots (scratch buffer)
     uint64_t o_halo_cnt, o_halo_keys, o_halo_nonces;  // scope 1 halos (scratch buffer)
     uint64_t o_wcount;                     // window nonce list entry counter (scratch buffer)

@@ -319,6 +319,44 @@ def test_sync_reads_its_own_plot_when_buffers_are_reused(vx):
         vx.vx_plot_destroy(h)
 
 
+@pytest.mark.parametrize("K,other,keep", [(18, 18, True), (18, 18, False), (16, 20, True), (20, 14, False)],
+                         ids=["same-K", "same-K-other-destroyed", "larger-between", "smaller-between-destroyed"])
+def test_runs_again_after_another_plot_on_the_same_buffers(vx, K, other, keep):
+    # Plots A and B share Table 1 and scratch on one stream, each with its own
+    # Table 2.  A, B, then A again: A's second run is A's plot in A's Table 2,
+    # whatever B left in the scratch and whether B still exists, and vx_sync
+    # reads that run.
+    sizes = [vx.vx_plot_required_bytes(k) for k in (K, other)]
+    t1, sc = (torch.empty(max(b[i] for b in sizes), dtype=torch.uint8, device="cuda") for i in (0, 2))
+    keys = [plot_key(65), plot_key(66)]
+    t2, hs = [], []
+    for k, key, (_, t2b, _) in zip((K, other), keys, sizes):
+        t2.append(torch.zeros(t2b, dtype=torch.uint8, device="cuda"))
+        hs.append(vx.vx_plot_create(k, key))
+        vx.vx_plot_bind(hs[-1], t1.data_ptr(), t2[-1].data_ptr(), sc.data_ptr(), (t2b - 256) // 16)
+    ra, rb = oracle_plot(K, keys[0]), oracle_plot(other, keys[1])[1]
+
+    def holds(i, ref):
+        assert vx.vx_table_info(hs[i], vx.VX_TABLE2)[1] == ref.shape[0]
+        return np.array_equal(t2[i][: ref.size].view(-1, 16).cpu().numpy(), ref)
+
+    for i in (0, 1):
+        vx.vx_plot_run(hs[i])
+        vx.vx_sync(hs[i])
+    assert holds(0, ra[1]) and holds(1, rb)
+    b_before = t2[1].clone()
+    if not keep:
+        vx.vx_plot_destroy(hs.pop())
+    t2[0].zero_()
+    vx.vx_plot_run(hs[0])
+    assert vx.vx_sync(hs[0]) == vx.VX_OK
+    assert holds(0, ra[1])
+    assert np.array_equal(t1[: ra[0].size].view(-1, 12).cpu().numpy(), ra[0])
+    assert torch.equal(t2[1], b_before)
+    for h in hs:
+        vx.vx_plot_destroy(h)
+
+
 @pytest.mark.parametrize("K,s,placement", [(16, 8, 1), (20, 6, 2)], ids=["lookback", "slots"])
 def test_lookback_wait_times_out(vx, K, s, placement):
     # Partition 0 (look-back placement) or chunk 0 of the pair-count scan
