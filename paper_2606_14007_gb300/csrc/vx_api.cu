@@ -1164,12 +1164,24 @@ int vx_test_fail_next_allocs(int count)
 // ------------------------------------------------------------- batch
 namespace {
 
+// What a recorded batch knows of a plot besides its handle's fixed plan and
+// key: everything vx_plot_bind may change.
+struct Binding {
+    const uint8_t *t1, *t2, *scratch;
+    uint64_t t2cap;
+    explicit Binding(const vx_plot *p) : t1(p->d_t1), t2(p->d_t2), scratch(p->d_scratch), t2cap(p->t2cap) {}
+    bool operator==(const Binding &o) const
+    {
+        return t1 == o.t1 && t2 == o.t2 && scratch == o.scratch && t2cap == o.t2cap;
+    }
+};
+
 // A batch's device workspace and its recorded graph, cached by the exact
-// sequence of plot handles (and their buffers) it was built for.
+// sequence of plot handles (and their bindings) it was built for.
 struct BatchEntry {
     std::vector<vx_plot *> plots;
     std::vector<vx_plot *> pinned;  // those whose pinned blocks take the results
-    std::vector<uint8_t *> bufs;
+    std::vector<Binding> bound;
     uint8_t *d_ws = nullptr;
     uint8_t *h_ws = nullptr;
     size_t ws_bytes = 0;
@@ -1192,7 +1204,7 @@ BatchEntry *find_batch(vx_plot *const *plots, int n)
         if ((int)b->plots.size() != n) continue;
         bool same = true;
         for (int i = 0; i < n && same; ++i)
-            same = b->plots[i] == plots[i] && b->bufs[i] == plots[i]->d_scratch;
+            same = b->plots[i] == plots[i] && b->bound[i] == Binding(plots[i]);
         if (same) return b;
     }
     return nullptr;
@@ -1309,7 +1321,7 @@ extern "C" int vx_plot_batch(vx_plot *const *plots, int n, void *stream)
     if (!b) {
         b = new BatchEntry();
         b->plots.assign(plots, plots + n);
-        for (int i = 0; i < n; ++i) b->bufs.push_back(plots[i]->d_scratch);
+        for (int i = 0; i < n; ++i) b->bound.emplace_back(plots[i]);
         // Two lanes of grouped launches, balanced by nonces (largest plots
         // first, each to the lighter lane), recorded on two branches of the
         // graph so that one lane's kernels can run beside the other's.

@@ -157,3 +157,33 @@ def test_batch_results_of_good_and_failed_plots(vx, placement):
     torch.cuda.synchronize()
     for p in plots:
         p.close()
+
+
+@pytest.mark.parametrize("placement", [0, 1], ids=["slots", "lookback"])
+def test_batch_follows_rebound_tables(vx, placement):
+    # The same handles batched again after a plot's Table 2, then its Table 1,
+    # was bound elsewhere with the scratch kept: the batch fills the new
+    # buffers, up to the new capacity, and leaves the old ones alone.
+    opts = [dict(t2_capacity=16), dict()]
+    mix = [(16, 211), (14, 212)]
+    plots = [vx.Plot(K, plot_key(s), vx.make_opts(t2_placement=placement, **o)) for (K, s), o in zip(mix, opts)]
+    handles = [p.handle for p in plots]
+    r1, r2 = oracle_tables(*mix[0])
+    need, p = r2.shape[0], plots[0]
+    vx.vx_plot_batch(handles)
+    assert vx.vx_sync(p.handle, check=False) == vx.VX_ENOMEM
+    big = torch.zeros(16 * need + 256, dtype=torch.uint8, device="cuda")
+    t1 = torch.zeros_like(p._t1)
+    for table1 in (p._t1, t1):
+        vx.vx_plot_bind(p.handle, table1.data_ptr(), big.data_ptr(), p._scratch.data_ptr(), need)
+        p._t2.zero_()
+        big.zero_()
+        table1.zero_()
+        vx.vx_plot_batch(handles)
+        assert [vx.vx_sync(h, check=False) for h in handles] == [vx.VX_OK, vx.VX_OK]
+        assert vx.vx_table_info(p.handle, vx.VX_TABLE2)[1] == need
+        assert np.array_equal(big[: 16 * need].view(need, 16).cpu().numpy(), r2)
+        assert np.array_equal(table1[: r1.size].view(-1, 12).cpu().numpy(), r1)
+        assert int(p._t2.max()) == 0
+    for p in plots:
+        p.close()
