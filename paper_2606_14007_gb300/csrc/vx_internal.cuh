@@ -10,6 +10,8 @@
 
 #include <atomic>
 
+#include "smem_seen.h"
+
 namespace vx {
 
 // ---------------------------------------------------------------- limits
@@ -600,24 +602,17 @@ cudaError_t launch_on(On on, void (*fn)(P...), uint32_t grid, uint32_t block, si
     return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
 }
 
-// Allows a kernel `bytes` of dynamic shared memory on the current device.
-// The call is made when a device first needs that much (it costs as much
-// as a launch); `seen` is the kernel's own table, one entry per device.
-constexpr int kMaxDevices = 64;
-struct SmemSeen {
-    std::atomic<size_t> allowed[kMaxDevices] = {};
-};
+// Allows a kernel `bytes` of dynamic shared memory on the current device;
+// `seen` is the kernel's own table.
 template <class Fn>
 cudaError_t allow_smem(Fn fn, size_t bytes, SmemSeen &seen)
 {
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    const cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    const bool known = dev >= 0 && dev < kMaxDevices;
-    if (known && seen.allowed[dev].load(std::memory_order_acquire) >= bytes) return cudaSuccess;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess && known) seen.allowed[dev].store(bytes, std::memory_order_release);
-    return e;
+    return grow_allowed(seen, dev, bytes, [&](size_t b) {
+        return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b);
+    });
 }
 
 struct HashCfg {

@@ -44,3 +44,47 @@ int main()
 }
 """)
     assert out.strip() == "ok"
+
+
+def test_shared_memory_limits_of_two_threads(tmp_path):
+    # Two host threads launch the same kernel for the first time, one with
+    # much shared memory, one with little: whatever their order, the kernel is
+    # allowed as much as the table says.  The large thread's set is held open
+    # until the small one has finished (or, kept out meanwhile, for 200 ms).
+    out = run_cpp(tmp_path, r"""
+#include <chrono>
+#include <cstdio>
+#include <thread>
+#include "smem_seen.h"
+int main()
+{
+    static vx::SmemSeen seen;
+    std::atomic<size_t> attribute{0};
+    std::atomic<bool> large_set{false}, small_done{false};
+    std::thread large([&] {
+        vx::grow_allowed(seen, 0, 75000, [&](size_t b) {
+            attribute = b;
+            large_set = true;
+            for (int i = 0; i < 200 && !small_done; ++i) std::this_thread::sleep_for(std::chrono::milliseconds(1));
+            return 0;
+        });
+    });
+    std::thread small([&] {
+        while (!large_set) std::this_thread::yield();
+        vx::grow_allowed(seen, 0, 22000, [&](size_t b) { attribute = b; return 0; });
+        small_done = true;
+    });
+    large.join();
+    small.join();
+    printf("allowed %zu, attribute %zu\n", seen.allowed[0].load(), attribute.load());
+    if (seen.allowed[0] != 75000 || attribute != 75000) return 1;
+    // a refused size is not remembered, a smaller one needs no call, an
+    // unknown device makes the call each time
+    int calls = 0;
+    if (vx::grow_allowed(seen, 0, 90000, [&](size_t) { return ++calls; }) != 1 || seen.allowed[0] != 75000) return 2;
+    if (vx::grow_allowed(seen, 0, 75000, [&](size_t) { return ++calls; }) != 0 || calls != 1) return 3;
+    for (int i = 0; i < 2; ++i) vx::grow_allowed(seen, vx::kMaxDevices, 1, [&](size_t) { ++calls; return 0; });
+    return calls == 3 ? 0 : 4;
+}
+""")
+    assert out.strip() == "allowed 75000, attribute 75000"
