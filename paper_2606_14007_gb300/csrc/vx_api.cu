@@ -847,6 +847,8 @@ int vx_sort_table2(vx_plot *p, void *d_work, uint64_t work_bytes, void *stream)
         return VX_EINVAL;
     }
     if (p->t2_count == 0) return VX_OK;
+    uint64_t *result = nullptr;
+    VX_TRY(p, ensure_stage(p, &result));  // a plot that only ran in batches may have no pinned block yet
     cudaStream_t s = (cudaStream_t)stream;
     uint8_t *w = (uint8_t *)d_work;
     const vx::Plan &pl = p->plan;

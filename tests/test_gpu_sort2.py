@@ -88,3 +88,23 @@ def test_sort_table2_call_errors(vx):
     assert vx.lib().vx_sort_table2(p.handle, work.data_ptr(), wb - 256, None) == vx.VX_EINVAL
     assert vx.lib().vx_sort_table2(p.handle, work.data_ptr() + 8, wb - 256, None) == vx.VX_EINVAL
     p.close()
+
+
+@pytest.mark.parametrize("placement", [0, 1], ids=["slots", "lookback"])
+def test_sort_table2_of_plots_that_only_ran_in_a_batch(vx, placement):
+    # look-back batches leave no results in the plots' pinned blocks: a handle
+    # that never ran alone has none when its Table 2 is sorted
+    mix = [(16, 70), (14, 71)]
+    plots = [vx.Plot(K, plot_key(s), vx.make_opts(t2_placement=placement)) for K, s in mix]
+    vx.vx_plot_batch([p.handle for p in plots])
+    for (K, s), p in zip(mix, plots):
+        n2 = p.sync()
+        wb = vx.vx_sort_table2_work_bytes(p.handle)
+        work = torch.empty(max(wb, 256), dtype=torch.uint8, device="cuda")
+        vx.vx_sort_table2(p.handle, work.data_ptr(), wb)
+        assert vx.vx_sync(p.handle) == vx.VX_OK
+        assert vx.vx_table_info(p.handle, vx.VX_TABLE2)[1] == n2
+        key = plot_key(s)
+        ref = orc.sort_table2(orc.match(key, orc.table1(K, key), orc.default_distance(K)))
+        assert np.array_equal(p.t2.cpu().numpy(), ref)
+        p.close()
