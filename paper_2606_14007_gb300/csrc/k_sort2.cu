@@ -35,7 +35,7 @@ __global__ void k_s2_setup(Sort2Desc *dp)
     const uint64_t n2 = 1ull << d.p;
     const uint64_t nchunks = (n2 + kScanChunk - 1) / kScanChunk;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *d.ticket = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *d.ticket = *d.status = 0u;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += stride) {
         d.cnt2[i] = 0u;
         if (i < n1) d.cnt1[i] = 0u;
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kS2Threads, 3) k_s2_scatter(const Sort2Desc *_
     const uint4 *src;
     uint64_t left, bin0 = 0;  // records from the tile on; first bin of the CTA
     if (LEVEL == 1) {
-        const uint64_t n = *d.count, base = (uint64_t)blockIdx.x * kS2Tile;
+        const uint64_t n = d.count, base = (uint64_t)blockIdx.x * kS2Tile;
         if (base >= n) return;
         src = d.t2 + base;
         left = n - base;
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(256) k_s2_scan(const Sort2Desc *__restrict__ d
     if (c + 1 == nchunks && threadIdx.x == 0) {
         const uint64_t all = s_base + total;
         d.off[np] = all;
-        if (all != *d.count) atomicOr(d.status, kStSort2);
+        if (all != d.count) atomicOr(d.status, kStSort2);
     }
 }
 

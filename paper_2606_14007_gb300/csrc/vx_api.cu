@@ -854,7 +854,7 @@ int vx_sort_table2(vx_plot *p, void *d_work, uint64_t work_bytes, void *stream)
     const vx::Plan &pl = p->plan;
     vx::Sort2Desc d;
     memset(&d, 0, sizeof(d));
-    d.count = reinterpret_cast<const uint64_t *>(p->d_scratch + pl.o_t2off + 8 * (1ull << pl.p));
+    d.count = p->t2_count;
     d.p = sp.p;
     d.p1 = sp.p1;
     d.p2 = sp.p2;
@@ -871,7 +871,7 @@ int vx_sort_table2(vx_plot *p, void *d_work, uint64_t work_bytes, void *stream)
     d.off = reinterpret_cast<uint64_t *>(w + sp.o_off);
     d.lbs = reinterpret_cast<uint64_t *>(w + sp.o_lbs);
     d.ticket = reinterpret_cast<uint32_t *>(w + sp.o_ticket);
-    d.status = reinterpret_cast<uint32_t *>(p->d_scratch + pl.o_status);
+    d.status = reinterpret_cast<uint32_t *>(w + sp.o_status);
     vx::Sort2Desc *dd = reinterpret_cast<vx::Sort2Desc *>(w + sp.o_desc);
     VX_TRY(p, cudaMemcpyAsync(dd, &d, sizeof(d), cudaMemcpyHostToDevice, s));
     const vx::Sort2Launch g{sp.tiles1, sp.tiles2, sp.tiles_scan, sp.parts, sp.cap2,
@@ -881,7 +881,13 @@ int vx_sort_table2(vx_plot *p, void *d_work, uint64_t work_bytes, void *stream)
     p->last = s;
     p->have_last = true;
     p->res_pending = p->res_batch = false;
-    return record_result(p, s, false);  // vx_sync now waits for the sort and reads its status
+    // vx_sync now waits for the sort and reads its status, beside the counts
+    // already known; the scratch buffer may hold another plot's by now.
+    uint64_t *h = reinterpret_cast<uint64_t *>(reinterpret_cast<uint8_t *>(p->h_stage) + vx::kStageResultOffset);
+    h[1] = p->t2_count;
+    h[2] = p->t1_count;
+    VX_TRY(p, cudaMemcpyAsync(h, d.status, 4, cudaMemcpyDeviceToHost, s));
+    return record_result(p, s, true);
 }
 
 int vx_autotune(int K, const vx_opts *base, vx_opts *best, double *best_ms, void *stream)

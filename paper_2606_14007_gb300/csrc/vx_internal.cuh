@@ -103,7 +103,7 @@ struct Desc {
 // Table 2 sorted by hash2 (vx_sort_table2): one plot's second sorting pass
 // over 16-byte records, with its own slots in a caller-provided work buffer.
 struct Sort2Desc {
-    const uint64_t *count; // device word with the Table-2 record count
+    uint64_t count;        // Table-2 records
     int32_t p;             // partition bits (2^p partitions of ~2^11 records)
     int32_t p1, p2;        // first / second scatter level bits (p = p1 + p2)
     int32_t dbits;         // counting-sort digit bits inside a partition
@@ -117,7 +117,7 @@ struct Sort2Desc {
     uint64_t *off;         // [2^p + 1] partition offsets in the sorted table
     uint64_t *lbs;         // look-back words of the offset scan
     uint32_t *ticket;      // chunk ticket of the offset scan
-    uint32_t *status;      // the plot's status word
+    uint32_t *status;      // the sort's status word, in the work buffer like all else but t2
 };
 
 

@@ -411,7 +411,7 @@ struct Sort2Plan {
     int p, p1, p2, dbits;
     uint32_t cap1, cap2, chunks1;
     uint32_t tiles1, tiles2, tiles_scan, parts;
-    uint64_t o_desc, o_ticket, o_cnt1, o_cnt2, o_off, o_lbs, o_arecs, o_brecs;
+    uint64_t o_desc, o_ticket, o_status, o_cnt1, o_cnt2, o_off, o_lbs, o_arecs, o_brecs;
     uint64_t bytes;
 };
 
@@ -448,7 +448,8 @@ inline int make_sort2_plan(uint64_t n, Sort2Plan *out, size_t desc_bytes)
     const uint64_t np = S.parts, n1 = S.p2 > 0 ? (1ull << S.p1) : 0ull;
     uint64_t at = 0;
     S.o_desc = at; at = round_up(at + desc_bytes, 256);
-    S.o_ticket = at; at = round_up(at + 4, 256);
+    S.o_ticket = at;
+    S.o_status = at + 64; at = round_up(at + 68, 256);
     S.o_cnt1 = at; at = round_up(at + 4 * n1, 256);
     S.o_cnt2 = at; at = round_up(at + 4 * np, 256);
     S.o_off = at; at = round_up(at + 8 * (np + 1), 256);

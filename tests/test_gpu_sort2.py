@@ -108,3 +108,32 @@ def test_sort_table2_of_plots_that_only_ran_in_a_batch(vx, placement):
         ref = orc.sort_table2(orc.match(key, orc.table1(K, key), orc.default_distance(K)))
         assert np.array_equal(p.t2.cpu().numpy(), ref)
         p.close()
+
+
+def test_sort_table2_after_another_plot_took_the_scratch(vx):
+    # Plots A and B share Table 1 and scratch, each with its own Table 2: A's
+    # sort, issued after B ran, orders A's records and reports A's counts.
+    K = 18
+    t1b, t2b, scb = vx.vx_plot_required_bytes(K)
+    t1 = torch.empty(t1b, dtype=torch.uint8, device="cuda")
+    sc = torch.empty(scb, dtype=torch.uint8, device="cuda")
+    t2 = [torch.empty(t2b, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    keys = [plot_key(72), plot_key(73)]
+    refs = [orc.match(k, orc.table1(K, k), orc.default_distance(K)) for k in keys]
+    assert refs[0].shape[0] != refs[1].shape[0]
+    hs = []
+    for key, buf in zip(keys, t2):
+        hs.append(vx.vx_plot_create(K, key))
+        vx.vx_plot_bind(hs[-1], t1.data_ptr(), buf.data_ptr(), sc.data_ptr(), t2b // 16)
+        vx.vx_plot_run(hs[-1])
+        vx.vx_sync(hs[-1])
+    for h, buf, ref in zip(hs, t2, refs):
+        wb = vx.vx_sort_table2_work_bytes(h)
+        work = torch.empty(wb, dtype=torch.uint8, device="cuda")
+        vx.vx_sort_table2(h, work.data_ptr(), wb)
+        assert vx.vx_sync(h) == vx.VX_OK
+        n2 = vx.vx_table_info(h, vx.VX_TABLE2)[1]
+        assert n2 == ref.shape[0]
+        assert np.array_equal(buf[: 16 * n2].view(n2, 16).cpu().numpy(), orc.sort_table2(ref))
+    for h in hs:
+        vx.vx_plot_destroy(h)
