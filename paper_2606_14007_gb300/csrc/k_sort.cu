@@ -195,8 +195,14 @@ __global__ void __launch_bounds__(kScanCtaThreads) k_scan_counts(const Desc *__r
     __shared__ uint32_t s_c;
     __shared__ uint64_t s_base;
     __shared__ int s_ok;
-    pdl_go();
+    // The slot pair hash comes onto the SMs once the sort has ended (SRC 1
+    // waits for it), not onto those its CTAs leave first: at K <= 22 it has
+    // too few CTAs to fill the rest (cross-bucket match, K=21: 288 us a run
+    // with the CTAs let go at once, 192 so; K=22: 449 and 339, bucket match
+    // 235 and 221; K=23 and above the same).
+    if (SRC == 0) pdl_go();
     pdl_wait();
+    if (SRC == 1) pdl_go();
     const int plot = find_plot(tile_start, nplots, blockIdx.x);
     const Desc &d = descs[plot];
     uint32_t *ticket = SRC == 0 ? d.ticket_s : d.ticket;

@@ -576,3 +576,32 @@ def test_coarse_bits_past_ten_stay_refused(vx):
         with pytest.raises(vx.VxError) as e:
             vx.vx_plot_required_bytes(K, vx.make_opts(coarse_bits=11))
         assert e.value.code == vx.VX_EINVAL
+
+
+@pytest.mark.parametrize("K", [20, 21, 22])
+def test_cross_bucket_runs_take_no_longer_than_their_kernels(vx, K):
+    # Untraced runs chain their kernels, each starting while the one before
+    # ends: back to back they may not take longer than the same kernels traced
+    # one after the other (whose pair hash finds the whole device free).
+    p = vx.Plot(K, plot_key(650), vx.make_opts(match_scope=1))
+    n = 20
+    chained = []
+    for _ in range(5):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        for _ in range(n):
+            p.run()
+        b.record()
+        p.sync()
+        b.synchronize()
+        chained.append(a.elapsed_time(b) / n)
+    traced = []
+    for _ in range(5):
+        vx.vx_plot_profile(p.handle, n)
+        for _ in range(n):
+            p.run()
+        p.sync()
+        ms, runs = vx.vx_plot_profile_read(p.handle)
+        traced.append(sum(ms.values()) / runs)
+    p.close()
+    assert min(chained) <= 1.1 * min(traced)
