@@ -147,9 +147,9 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
     // 2^11 records: K=12 22.1 / 22.8 / 26.2 us, K=16 24.4 / 25.6 / 28.0,
     // K=18 39.5 / 34.6 / 37.0, K=19 55.7 / 49.6 / 46.5).  Options that the
     // partition count bears on keep the fixed size.
-    if (!opts.partition_log2 && K <= 18 && opts.coarse_bits < 0 && !opts.window_bits && !opts.match_scope &&
-        !opts.t2_placement)
-        P.s = K <= 16 ? 9 : 10;
+    const bool small = !opts.partition_log2 && K <= 18 && opts.coarse_bits < 0 && !opts.window_bits &&
+                       !opts.match_scope && !opts.t2_placement;
+    if (small) P.s = K <= 16 ? 9 : 10;
     if (P.s < 6 || P.s > 13) {
         *why = "partition_log2 must be in 6..13";
         return VX_EINVAL;
@@ -255,7 +255,11 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
     P.hchunks = (P.mode == kScatterStaged && P.p2 > 0) ? want : 1;
     while (P.hchunks > 1 && ((1ull << K) < (uint64_t)P.hchunks)) P.hchunks >>= 1;
     P.pchunks = P.fuse_pair_hash ? 1 : want;
-    while (P.pchunks > 1 && (1ull << P.p) < (uint64_t)P.pchunks) P.pchunks >>= 1;
+    // No more chunks than partitions of the fixed size: a chunk costs two
+    // launches (K=12 in 8 chunks of 2^9 records 119 us a run, in the 2 of
+    // 2^11 records 66; K=13 140 and, in 4, 91).
+    const int chunk_bits = small ? (K > kDefaultPartLog2 ? K - kDefaultPartLog2 : 0) : P.p;
+    while (P.pchunks > 1 && (1ull << chunk_bits) < (uint64_t)P.pchunks) P.pchunks >>= 1;
     // Records of the plot (of the window: Binomial(2^K, 2^-c), Poisson-like).
     const double wrec = std::ldexp((double)P.N, -(int)P.wbits);
     const double avg2 = std::ldexp((double)P.N, -P.pk);

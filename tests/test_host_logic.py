@@ -88,3 +88,40 @@ int main()
 }
 """)
     assert out.strip() == "allowed 75000, attribute 75000"
+
+
+PLANS = r"""
+#include <cstdio>
+#include "vx_plan.h"
+static vx::Plan plan(int K, uint32_t chunks, int part = 0, uint32_t npt = 0, int coarse = -1)
+{
+    vx_opts o;
+    memset(&o, 0, sizeof(o));
+    o.size = sizeof(o);
+    o.pipeline_chunks = chunks;
+    o.partition_log2 = part;
+    o.nonces_per_thread = npt;
+    o.coarse_bits = coarse;
+    vx::Plan p;
+    const char *why = nullptr;
+    if (vx::make_plan_sized(K, &o, &p, &why, 1024) != VX_OK) printf("K=%d: %s\n", K, why);
+    return p;
+}
+"""
+
+
+def test_small_partitions_do_not_raise_the_number_of_chunks(tmp_path):
+    # Small plots have 4 or 2 times the partitions that 2^11 records would
+    # give: a pipelined run still takes no more chunks than with those.
+    out = run_cpp(tmp_path, PLANS + r"""
+int main()
+{
+    for (int K = 1; K <= 24; ++K)
+        for (uint32_t c : {1u, 2u, 4u, 8u})
+            if (plan(K, c).pchunks != plan(K, c, 11).pchunks) return printf("K=%d, %u chunks\n", K, c), 1;
+    // where the partition size is the caller's, its partitions count
+    if (plan(12, 8, 9).pchunks != 8 || plan(12, 8, 11).pchunks != 2) return 2;
+    puts("ok");
+}
+""")
+    assert out.strip() == "ok"
