@@ -216,7 +216,7 @@ int build_tiles(vx_plot *const *plots, int n, uint32_t *h, const uint32_t *d, La
         const Plan &pl = plots[i]->plan;
         same_npt = same_npt && pl.npt == npt;
         auto_npt = auto_npt && pl.npt_auto;
-        nonces += pl.N;
+        nonces += pl.N / pl.hchunks;  // of one launch
         fuse = fuse && pl.fuse_pair_hash;
         slots = slots && pl.pair_slots;
         halo = halo || pl.scope != 0;

@@ -216,13 +216,18 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
         *why = "nonces_per_thread 4 or 16 needs the staged bucketing and a whole plot (no window)";
         return VX_EINVAL;
     }
-    if (P.npt == 0) {
+    // Nonce chunks, only where a second scatter level exists to overlap.
+    const int want = pc == 0 ? 1 : (int)pc;
+    const bool two_level = P.mode == kScatterStaged && (opts.coarse_bits >= 0 ? opts.coarse_bits < P.p : P.p > 10);
+    P.hchunks = two_level ? want : 1;
+    while (P.hchunks > 1 && ((1ull << K) < (uint64_t)P.hchunks)) P.hchunks >>= 1;
+    if (P.npt == 0) {  // a launch hashes one chunk (K=22 in 8 chunks 391 us with 4, 473 with the plot's 12)
         if (P.mode != kScatterStaged)
             P.npt = kPlanNoncesPerThread;
         else if (P.wbits)  // by the window's share of the nonces (2^24: 0.40 ms with 16, 0.47 with 8)
             P.npt = (P.N >> P.wbits) < (1ull << 22) ? kPlanNoncesPerThread : 16;
         else
-            P.npt = auto_nonces_per_thread(P.N);
+            P.npt = auto_nonces_per_thread(P.N / P.hchunks);
     }
     if (P.mode == kScatterDirect) {
         P.p1 = P.p;  // one level: the hash kernel claims final-partition slots
@@ -238,22 +243,19 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
         // tile's kernel also takes (K = 31: 10 + 10 bits 48.5 + 15.4 ms, 11 +
         // 9 bits 49.0 + 10.6; K = 30: 10 + 9 bits 24.27 + 5.38, 11 + 8 bits
         // 24.52 + 4.68; K = 29 not yet: 12.15 + 2.35 against 12.26 + 2.25).
-        P.p1 = P.p <= 10 ? P.p : P.p < 14 ? 8 : P.p == 14 ? 9 : P.p < 19 || P.wbits || P.npt != 16 ? 10 : 11;
+        P.p1 = !two_level ? P.p : P.p < 14 ? 8 : P.p == 14 ? 9 : P.p < 19 || P.wbits || P.npt != 16 ? 10 : 11;
     }
     P.p2 = P.p - P.p1;
     if (P.mode == kScatterStaged && (P.p1 > (opts.coarse_bits < 0 ? 11 : 10) || P.p2 > 11)) {
         *why = "coarse_bits leaves a scatter level wider than 10 (first) or 11 (second) bits";
         return VX_EINVAL;
     }
-    // Pipeline chunks, only where a second kernel exists to overlap (the
-    // second scatter level; the separate pair hash).  Off unless asked for:
+    // Partition chunks, only where a second kernel exists to overlap (the
+    // separate pair hash).  Both kinds of chunks are off unless asked for:
     // measured on GB300 at K=31 it does not pay, because each kernel of a
     // pair alone fills an SM's register file (the latency-bound sort needs
     // four resident CTAs, the ALU-bound hashes need ~24 warps), so the two
     // streams take turns instead of sharing SMs.
-    const int want = pc == 0 ? 1 : (int)pc;
-    P.hchunks = (P.mode == kScatterStaged && P.p2 > 0) ? want : 1;
-    while (P.hchunks > 1 && ((1ull << K) < (uint64_t)P.hchunks)) P.hchunks >>= 1;
     P.pchunks = P.fuse_pair_hash ? 1 : want;
     // No more chunks than partitions of the fixed size: a chunk costs two
     // launches (K=12 in 8 chunks of 2^9 records 119 us a run, in the 2 of

@@ -104,7 +104,7 @@ static vx::Plan plan(int K, uint32_t chunks, int part = 0, uint32_t npt = 0, int
     o.coarse_bits = coarse;
     vx::Plan p;
     const char *why = nullptr;
-    if (vx::make_plan_sized(K, &o, &p, &why, 1024) != VX_OK) printf("K=%d: %s\n", K, why);
+    if (vx::make_plan_sized(K, &o, &p, &why, 1024) != VX_OK) p.N = 0;  // refused
     return p;
 }
 """
@@ -121,6 +121,29 @@ int main()
             if (plan(K, c).pchunks != plan(K, c, 11).pchunks) return printf("K=%d, %u chunks\n", K, c), 1;
     // where the partition size is the caller's, its partitions count
     if (plan(12, 8, 9).pchunks != 8 || plan(12, 8, 11).pchunks != 2) return 2;
+    puts("ok");
+}
+""")
+    assert out.strip() == "ok"
+
+
+def test_automatic_hash_tiles_follow_the_chunk(tmp_path):
+    # A staged hash launch covers one nonce chunk: its automatic nonces per
+    # thread are those of the chunk's nonces, and an 11-bit first level comes
+    # only with the tile that has a kernel for it.
+    out = run_cpp(tmp_path, PLANS + r"""
+int main()
+{
+    for (int K = 1; K <= 32; ++K)
+        for (int part : {0, 6, 9, 11})
+            for (uint32_t c : {1u, 2u, 4u, 8u}) {
+                const vx::Plan p = plan(K, c, part);
+                if (p.N == 0) continue;  // refused
+                if (p.npt != vx::auto_nonces_per_thread(p.N / p.hchunks) || (p.p1 > 10 && p.npt != 16))
+                    return printf("K=%d part %d chunks %d: npt %d, p1 %d\n", K, part, p.hchunks, p.npt, p.p1), 1;
+                if (plan(K, c, part, 8).npt != 8 || plan(K, c, part, 16).npt != 16) return 2;
+            }
+    if (plan(24, 8, 0, 0, 4).npt != 8) return 3;  // two levels of the caller's own, 2^21 nonces a chunk
     puts("ok");
 }
 """)
