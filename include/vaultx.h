@@ -252,13 +252,13 @@ int vx_table_info(const vx_plot *plot, int which, const void **dptr, uint64_t *n
 
 /* Autotuner: times every distinct plan for K that the candidate options give
  * (partition size 2^9 .. 2^13 records, i.e. the physical partition count and
- * the sort tile; the staged bucketing with 4, 8 or 16 nonces per hash
- * thread, i.e. threads per nonce 1/4, 1/8, 1/16; the direct bucketing with
- * 8) on this device.  Each candidate runs one warm-up and three timed plots
- * with a fixed synthetic key in library-owned memory on stream (CUDA
- * events).  *best gets base (defaults if null) with the fastest candidate's
- * partition_log2, scatter_mode and nonces_per_thread, *best_ms its mean
- * plot time.
+ * the sort tile; the staged bucketing with 4, 8, 16 or the automatic number
+ * of nonces per hash thread; the direct bucketing with 8; the automatic
+ * choice of all three) on this device.  Each candidate runs one warm-up and
+ * three timed plots with a fixed synthetic key in library-owned memory on
+ * stream (CUDA events).  *best gets base (defaults if null) with the fastest
+ * candidate's partition_log2, scatter_mode and nonces_per_thread (0 where
+ * automatic), *best_ms its mean plot time.
  * Synchronous; a candidate that cannot be planned or allocated is skipped
  * (VX_ENOMEM if none ran).  The Python binding keeps an on-disk cache of the
  * result keyed by device and K.  The paper has no counterpart (its kernels

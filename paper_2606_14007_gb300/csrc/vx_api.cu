@@ -903,8 +903,7 @@ int vx_autotune(int K, const vx_opts *base, vx_opts *best, double *best_ms, void
     cudaStream_t s = (cudaStream_t)stream;
     uint8_t key[32];
     for (int i = 0; i < 32; ++i) key[i] = (uint8_t)(0xA5 ^ (i * 7));
-    struct Seen { int p, p1, p2, mode, npt; uint32_t cap2; int dbits; };
-    std::vector<Seen> seen;
+    std::vector<vx::Plan> seen;
     double best_t = 0;
     bool found = false;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -912,50 +911,36 @@ int vx_autotune(int K, const vx_opts *base, vx_opts *best, double *best_ms, void
         if (e0) cudaEventDestroy(e0);
         return VX_ECUDA;
     }
-    // candidates: partition size x bucketing strategy x nonces per hash
-    // thread (4, 8, 16 for the staged hash; the direct one takes 8)
-    for (int part = 9; part <= 13; ++part) {
-        for (int cand = 0; cand < 4; ++cand) {
-            const uint32_t mode = cand < 3 ? (uint32_t)vx::kScatterStaged : (uint32_t)vx::kScatterDirect;
-            vx_opts o = b0;
-            o.partition_log2 = part;
-            o.scatter_mode = mode;
-            o.nonces_per_thread = cand == 0 ? 4u : cand == 2 ? 16u : 8u;
-            vx::Plan pl;
-            const char *why = nullptr;
-            if (make_plan(K, &o, &pl, &why) != VX_OK) continue;
-            const Seen me{pl.p, pl.p1, pl.p2, pl.mode, pl.npt, pl.cap2, pl.dbits};
-            bool dup = false;
-            for (const Seen &x : seen)
-                dup = dup || (x.p == me.p && x.p1 == me.p1 && x.p2 == me.p2 && x.mode == me.mode &&
-                              x.npt == me.npt && x.cap2 == me.cap2 && x.dbits == me.dbits);
-            if (dup) continue;  // the planner clamped it to a plan already timed
-            seen.push_back(me);
-            vx_plot *p = nullptr;
-            if (vx_plot_create(K, key, &o, &p) != VX_OK) continue;
-            bool ok = vx_plot_alloc(p) == VX_OK && vx_plot_run(p, stream) == VX_OK &&
-                      vx_sync(p) == VX_OK;
-            float ms = 0;
-            if (ok) {
-                ok = cudaEventRecord(e0, s) == cudaSuccess;
-                for (int r = 0; ok && r < 3; ++r) ok = vx_plot_run(p, stream) == VX_OK;
-                ok = ok && cudaEventRecord(e1, s) == cudaSuccess && vx_sync(p) == VX_OK &&
-                     cudaEventSynchronize(e1) == cudaSuccess &&
-                     cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
-            }
-            vx_plot_destroy(p);
-            if (!ok) {
-                cudaGetLastError();  // a failed candidate (e.g. out of memory) is skipped
-                continue;
-            }
-            const double t = ms / 3.0;
-            if (!found || t < best_t) {
-                found = true;
-                best_t = t;
-                *best = o;
-                // report the partition size the planner actually used
-                if (pl.p > 0) best->partition_log2 = K - pl.p;
-            }
+    for (const vx_opts &o : vx::tune_candidates(b0)) {
+        vx::Plan pl;
+        const char *why = nullptr;
+        if (make_plan(K, &o, &pl, &why) != VX_OK) continue;
+        bool dup = false;  // the planner clamped it to a plan already timed
+        for (const vx::Plan &x : seen) dup = dup || vx::same_plan(x, pl);
+        if (dup) continue;
+        seen.push_back(pl);
+        vx_plot *p = nullptr;
+        if (vx_plot_create(K, key, &o, &p) != VX_OK) continue;
+        bool ok = vx_plot_alloc(p) == VX_OK && vx_plot_run(p, stream) == VX_OK && vx_sync(p) == VX_OK;
+        float ms = 0;
+        if (ok) {
+            ok = cudaEventRecord(e0, s) == cudaSuccess;
+            for (int r = 0; ok && r < 3; ++r) ok = vx_plot_run(p, stream) == VX_OK;
+            ok = ok && cudaEventRecord(e1, s) == cudaSuccess && vx_sync(p) == VX_OK &&
+                 cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
+        }
+        vx_plot_destroy(p);
+        if (!ok) {
+            cudaGetLastError();  // a failed candidate (e.g. out of memory) is skipped
+            continue;
+        }
+        const double t = ms / 3.0;
+        if (!found || t < best_t) {
+            found = true;
+            best_t = t;
+            *best = o;
+            // report the partition size the planner actually used
+            if (pl.p > 0 && o.partition_log2) best->partition_log2 = K - pl.p;
         }
     }
     cudaEventDestroy(e0);

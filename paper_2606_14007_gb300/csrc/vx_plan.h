@@ -12,6 +12,7 @@
 #include <cstdint>
 #include <cstring>
 #include <string>
+#include <vector>
 
 #include "../../include/vaultx.h"
 
@@ -407,6 +408,37 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
     P.scratch_bytes = at;
     *pl = P;
     return VX_OK;
+}
+
+// Whether two plans of the same K and base options run the same kernels on
+// the same slots (what the autotuner tells candidates apart by).
+inline bool same_plan(const Plan &a, const Plan &b)
+{
+    return a.p == b.p && a.p1 == b.p1 && a.p2 == b.p2 && a.mode == b.mode && a.npt == b.npt && a.cap2 == b.cap2 &&
+           a.dbits == b.dbits && a.hchunks == b.hchunks && a.pchunks == b.pchunks;
+}
+
+// What the autotuner times for `base`: partition size x bucketing strategy x
+// nonces per hash thread (4, 8, 16 and the planner's own, which may be 2 or
+// 12, for the staged hash, 8 for the direct one), and at last the planner's
+// choice of all three (pipeline chunks of small plots are clamped otherwise
+// there than at the same partition size asked for).
+inline std::vector<vx_opts> tune_candidates(const vx_opts &base)
+{
+    std::vector<vx_opts> c;
+    auto add = [&](int part, int mode, uint32_t npt) {
+        vx_opts o = base;
+        o.partition_log2 = part;
+        o.scatter_mode = (uint32_t)mode;
+        o.nonces_per_thread = npt;
+        c.push_back(o);
+    };
+    for (int part = 9; part <= 13; ++part) {
+        for (uint32_t npt : {4u, 8u, 16u, 0u}) add(part, kScatterStaged, npt);
+        add(part, kScatterDirect, 8u);
+    }
+    add(0, kScatterAuto, 0u);
+    return c;
 }
 
 // Table 2 sorted by hash2 (vx_sort_table2): partitions of ~2^11 of the n

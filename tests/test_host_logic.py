@@ -148,3 +148,38 @@ int main()
 }
 """)
     assert out.strip() == "ok"
+
+
+def test_the_untuned_plan_is_a_tuning_candidate(tmp_path):
+    # Whatever the planner picks by itself is among the plans the autotuner
+    # times, so a tuned plot is not slower than an untuned one.
+    out = run_cpp(tmp_path, PLANS + r"""
+int main()
+{
+    int plans = 0;
+    for (int K = 1; K <= 32; ++K)
+        for (uint32_t chunks : {0u, 2u, 8u})
+            for (uint32_t fuse : {0u, 1u})
+                for (uint32_t win : {0u, 2u})
+                    for (uint32_t place : {0u, 1u}) {
+                        vx_opts base;
+                        memset(&base, 0, sizeof(base));
+                        base.size = sizeof(base);
+                        base.coarse_bits = -1;
+                        base.pipeline_chunks = chunks;
+                        base.fuse_pair_hash = fuse;
+                        base.window_bits = win;
+                        base.t2_placement = place;
+                        vx::Plan own, p;
+                        const char *why = nullptr;
+                        if (vx::make_plan_sized(K, &base, &own, &why, 1024) != VX_OK) continue;
+                        bool found = false;
+                        for (const vx_opts &o : vx::tune_candidates(base))
+                            found = found || (vx::make_plan_sized(K, &o, &p, &why, 1024) == VX_OK && vx::same_plan(own, p));
+                        if (!found) return printf("K=%d chunks %u fuse %u window_bits %u\n", K, chunks, fuse, win), 1;
+                        ++plans;
+                    }
+    puts(plans > 300 ? "ok" : "few plans");
+}
+""")
+    assert out.strip() == "ok"
