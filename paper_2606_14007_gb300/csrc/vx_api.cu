@@ -940,7 +940,7 @@ int vx_autotune(int K, const vx_opts *base, vx_opts *best, double *best_ms, void
             best_t = t;
             *best = o;
             // report the partition size the planner actually used
-            if (pl.p > 0 && o.partition_log2) best->partition_log2 = K - pl.p;
+            if (pl.pk > 0 && o.partition_log2) best->partition_log2 = K - pl.pk;
         }
     }
     cudaEventDestroy(e0);

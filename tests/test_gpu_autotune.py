@@ -52,3 +52,12 @@ def test_autotune_plan_plots_correctly_and_caches(vx, tmp_path):
 def test_autotune_keeps_the_base_options(vx, tmp_path):
     o = vx.autotune(14, vx.make_opts(match_scope=1), cache_path=str(tmp_path / "t.json"))
     assert o.match_scope == 1
+
+
+def test_autotune_of_a_window_reports_its_partition_size(vx):
+    # 2^5 windows: the size asked for, not the one the window's share of the
+    # partitions would suggest (2^14 records and more, which are refused)
+    base = vx.make_opts(window_bits=5, window=3)
+    o, _ = vx.vx_autotune(20, base)
+    assert 9 <= o.partition_log2 <= 13 and o.window_bits == 5 and o.window == 3
+    vx.vx_plot_required_bytes(20, o)
