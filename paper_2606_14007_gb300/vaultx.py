@@ -250,13 +250,16 @@ def vx_autotune(K: int, opts: vx_opts | None = None, stream=None) -> tuple[vx_op
 
 
 _TUNED = ("partition_log2", "scatter_mode", "nonces_per_thread")
+# Counts up whenever the planner's own choices or the candidates change: a
+# stored choice holds only against the plans it was timed with.
+_TUNE_FORMAT = 2
 
 
 def autotune(K: int, opts: vx_opts | None = None, cache_path: str | None = None,
              stream=None) -> vx_opts:
-    """vx_autotune with an on-disk cache keyed by (device, K, base options):
-    the first call times the candidates, later calls (any process) reuse the
-    choice.  Cache file: cache_path, else $VX_TUNE_CACHE, else
+    """vx_autotune with an on-disk cache keyed by (device, K, base options,
+    format): the first call times the candidates, later calls (any process)
+    reuse the choice.  Cache file: cache_path, else $VX_TUNE_CACHE, else
     ~/.cache/vaultx/tune.json."""
     import json
     import os
@@ -267,7 +270,7 @@ def autotune(K: int, opts: vx_opts | None = None, cache_path: str | None = None,
     prop = torch.cuda.get_device_properties(torch.cuda.current_device())
     fields = {n: getattr(base, n) for n, _ in vx_opts._fields_
               if n not in ("size", "reserved") + _TUNED}
-    key = json.dumps([prop.name, prop.multi_processor_count, K, fields], sort_keys=True)
+    key = json.dumps([prop.name, prop.multi_processor_count, K, fields, _TUNE_FORMAT], sort_keys=True)
     try:
         with open(path) as f:
             cache = json.load(f)

@@ -353,3 +353,33 @@ def test_plot_file_that_cannot_be_opened_is_an_io_error(vx, tmp_path):
     assert rc == vx.VX_EIO
     rc, _, _, _ = vx.vx_plot_tiled_write(12, bytes(32), 40, path, check=False, stream=0)
     assert rc == vx.VX_EINVAL  # bad window bits are still refused first
+
+
+def test_tuning_cache_of_another_planner_is_not_used(vx, tmp_path, monkeypatch):
+    # Stored choices hold for the planner and candidates they were made with:
+    # an entry of another format is tuned again and stays in the file.
+    import json
+
+    import torch
+
+    class Prop:
+        name, multi_processor_count = "NVIDIA GB300", 152
+
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "get_device_properties", lambda d: Prop)
+    calls = []
+
+    def tune(K, opts=None, stream=None):
+        calls.append(K)
+        return vx.make_opts(partition_log2=10, scatter_mode=1, nonces_per_thread=4), 1.0
+
+    monkeypatch.setattr(vx, "vx_autotune", tune)
+    base = vx.vx_opts_default()
+    fields = {n: getattr(base, n) for n, _ in vx.vx_opts._fields_ if n not in ("size", "reserved") + vx._TUNED}
+    old = json.dumps([Prop.name, Prop.multi_processor_count, 30, fields], sort_keys=True)  # the first format
+    path = tmp_path / "tune.json"
+    path.write_text(json.dumps({old: {"partition_log2": 11, "scatter_mode": 1, "nonces_per_thread": 8, "ms": 1.0}}))
+    o = vx.autotune(30, cache_path=str(path))
+    assert calls == [30] and (o.partition_log2, o.nonces_per_thread) == (10, 4)
+    assert old in json.loads(path.read_text()) and len(json.loads(path.read_text())) == 2
+    assert vx.autotune(30, cache_path=str(path)).nonces_per_thread == 4 and calls == [30]
