@@ -123,8 +123,9 @@ typedef struct vx_opts {
                                    partitions; more pairs than the slot holds fail
                                    the plot with VX_EOVERFLOW: at K >= 26 with the
                                    default D a partition expects ~2040 +- 100 pairs
-                                   against 3910 places); 0 = automatic = 1 (the
-                                   faster on GB300 at K=31)                        */
+                                   against 3910 places); 0 = automatic = 2 where
+                                   the expected pairs fit the slots with a wide
+                                   margin (every default plot), else 1             */
     uint32_t match_scope;       /* 0 = (default) pairs inside one logical bucket
                                    (the fused Sort+Match kernel of Sec. III-A holds
                                    one bucket); 1 = cross-bucket: every pair i < j
@@ -237,8 +238,9 @@ int vx_plot_run(vx_plot *plot, void *stream);
  * block), so work queued later on the same
  * stream is not waited for, and the values are this run's even when a later
  * plot on the stream reuses the same Table-1 and scratch buffers.  After
- * vx_table1, vx_match or vx_plot_batch it synchronises the whole stream and
- * reads the scratch buffer.  The paper's host likewise waits for the device
+ * vx_plot_batch it synchronises the whole stream and reads the pinned block
+ * (where the batch's plots all place their pairs in slots) or the scratch
+ * buffer, after vx_table1 or vx_match the scratch buffer.  The paper's host likewise waits for the device
  * before Table 2 leaves it (Sec. III-A); the status codes (capacity
  * overflow, bounded-wait timeout) have no counterpart there. */
 int vx_sync(vx_plot *plot);
@@ -474,7 +476,7 @@ int vx_hash_nonces(const uint8_t key[32], uint64_t nonce0, uint64_t count, void 
 
 /* Measurement of the hash's ceiling, not a step of the path: keyed BLAKE3
  * of nonces nonce0 .. nonce0+count-1 in the Table-1 hash kernel's shape
- * (256 threads, 8 nonces per thread and step), with no record stores; each
+ * (256 threads, two nonces per thread and step), with no record stores; each
  * thread folds its hash words into one u32 of d_fold (device, 4-byte
  * aligned, fold_words words, a nonzero multiple of 256: the grid is
  * fold_words / 256 CTAs).  Timing it gives the integer-issue rate this

@@ -437,7 +437,6 @@ cudaError_t launch_hash_direct(const Desc *descs, int nplots, const uint32_t *ti
 // plot's CTAs stride over its range.  Skips plots whose Table 2 is invalid
 // (capacity exceeded, a wait timed out).
 constexpr int kT2HashThreads = 256;
-constexpr int kT2HashPer = 8;  // records per thread of the look-back pair hash's grid
 
 __global__ void __launch_bounds__(kT2HashThreads) k_t2_hash(const Desc *__restrict__ descs,
                                                             int nplots,

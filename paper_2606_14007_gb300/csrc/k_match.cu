@@ -231,17 +231,8 @@ cudaError_t launch_match_over(const Desc *descs, int nplots, On on, uint32_t max
     const size_t smem = match_smem_bytes(max_cap);
     const cudaError_t e = allow_smem(k_match_over, smem, seen);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(152, (unsigned)nplots);
-    cfg.blockDim = dim3(kMatchThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = on.s;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = on.pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_match_over, descs);
+    // One CTA per SM and plot: a look through the offsets next to always.
+    return launch_on(on, k_match_over, dim3(152, (unsigned)nplots), kMatchThreads, smem, descs);
 }
 
 }  // namespace vx

@@ -744,14 +744,19 @@ __global__ void __launch_bounds__(kGlThreads, MODE == kSortHash ? 2 : 3)
     if (threadIdx.x == 0) bulk_wait_all<false>();
 }
 
-// The planner's bound on a slot: 16 bytes a record (at least 4 * 2^dbits for
-// the last four) and 8 KB.  The layout above stays below it at every size it
-// admits (cap 14004: 225,272 of 232,448 bytes).
+// What the planner admits a slot by: the layout of k_sortmatch_gl, the smaller
+// front end, or 16 bytes a record (at least 4 * 2^dbits for the last four) and
+// 8 KB, the sort's need when the limits were set, whichever is more.  The
+// second decides near the limit (cap 14004, 13 bits: 232,424 bytes against
+// 224,888 of a CTA's 232,448), so what was refused stays refused; the first
+// is more in the middle (cap 9296, 13 bits: 161,016 against 157,096).
 size_t sortmatch_smem_bytes(uint32_t cap, int dbits)
 {
+    const size_t gl = SMLayout(cap, bitmap_words(dbits), false).bytes;
     cap = (cap + 3u) & ~3u;
     const size_t digits = (size_t)4 << dbits, recs = (size_t)cap * 4;
-    return (size_t)cap * 12 + (digits > recs ? digits : recs) + 8192 + 168;
+    const size_t limit = (size_t)cap * 12 + (digits > recs ? digits : recs) + 8192 + 168;
+    return gl > limit ? gl : limit;
 }
 
 uint32_t sortmatch_max_cap() { return 16384u; }

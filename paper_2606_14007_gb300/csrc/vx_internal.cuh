@@ -16,18 +16,14 @@ namespace vx {
 
 // ---------------------------------------------------------------- limits
 constexpr int kBucketBits = 24;          // 2^24 logical buckets (Sec. I-A, III-B)
-constexpr int kMaxK = 32;                // u32 nonces
 constexpr int kMaxCoarseBits = 10;       // first scatter level, <= 1024 bins
 constexpr int kMaxCoarseBitsWide = 11;   // ... up to 2048 (2^19 partitions and more)
 constexpr int kMaxFineBits = 10;         // second scatter level, <= 1024 bins
 constexpr int kMaxFineBitsWide = 11;     // ... up to 2048 (2^21 partitions, K = 32)
 constexpr int kScatterTile = 4096;       // records per CTA in the second scatter level
 constexpr int kScatterThreads = 512;
-constexpr int kSortThreads = 256;
 constexpr int kMatchThreads = 256;
-constexpr int kMaxSortDigitBits = 13;    // counting-sort digit of the partition sort
 constexpr int kMaxPartChunks = 8;         // partition chunks of a plot
-constexpr uint32_t kMaxPartition = 16384;  // records one partition may hold (smem)
 constexpr size_t kMaxSmemPerCta = 227 * 1024;  // opt-in dynamic shared memory per CTA
 
 // Status-word bits (device side; the host maps them to VX_E* codes).
@@ -53,7 +49,7 @@ struct Desc {
     int32_t p;           // partition bits (physical partitions = 2^p)
     int32_t p1;          // first scatter level bits (hash kernel)
     int32_t p2;          // second scatter level bits (p = p1 + p2)
-    int32_t dbits;       // counting-sort digit bits inside a partition
+    int32_t dbits;       // log2 of a partition's mean records (sizes the sort's bitmap)
     uint32_t cap1;       // records per level-1 slot (p2 > 0 only)
     uint32_t cap2;       // records per level-2 slot (final partitions)
     uint32_t chunks1;    // scatter-2 CTAs per level-1 slot = ceil(cap1 / tile)
@@ -106,7 +102,7 @@ struct Sort2Desc {
     uint64_t count;        // Table-2 records
     int32_t p;             // partition bits (2^p partitions of ~2^11 records)
     int32_t p1, p2;        // first / second scatter level bits (p = p1 + p2)
-    int32_t dbits;         // counting-sort digit bits inside a partition
+    int32_t dbits;         // log2 of a partition's mean records, rounded down (sizes the bitmap)
     uint32_t cap1, cap2;   // slot capacities (records) of the two levels
     uint32_t chunks1;      // second-level CTAs per first-level slot
     uint32_t spin_limit;   // polls before a bounded wait gives up
@@ -315,65 +311,6 @@ __device__ __forceinline__ uint32_t block_exclusive_scan_u32(uint32_t x, uint32_
     *total = ws[NT / 32];
     __syncthreads();
     return r;
-}
-
-// In-place exclusive scan of A[0..M) by a CTA of NT threads; returns the
-// total.  Warp w takes a contiguous run of A and walks it 32 entries at a
-// time (lane i on entry i: no bank conflicts); `ws` holds NT/32 words.
-// Ends with a __syncthreads.
-template <int NT>
-__device__ __forceinline__ uint32_t block_scan_inplace_u32(uint32_t *A, uint32_t M, uint32_t *ws)
-{
-    constexpr int NW = NT / 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t chunk = (M + NW - 1) / NW;
-    const uint32_t lo = min(M, (uint32_t)warp * chunk), hi = min(M, lo + chunk);
-    uint32_t sum = 0;
-    for (uint32_t i = lo + lane; i < hi; i += 32) sum += A[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) ws[warp] = sum;
-    __syncthreads();
-    uint32_t carry = 0, total = 0;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) {
-        const uint32_t t = ws[w];
-        carry += w < warp ? t : 0u;
-        total += t;
-    }
-    for (uint32_t base = lo; base < hi; base += 32) {
-        const uint32_t i = base + lane;
-        const uint32_t v = i < hi ? A[i] : 0u;
-        uint32_t incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (i < hi) A[i] = carry + incl - v;
-        carry += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    __syncthreads();
-    return total;
-}
-
-template <int NT>
-__device__ __forceinline__ uint64_t block_sum_u64(uint64_t x, uint64_t *ws)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    if (lane == 0) ws[warp] = x;
-    __syncthreads();
-    uint64_t s = 0;
-    if (threadIdx.x == 0) {
-        for (int w = 0; w < NT / 32; ++w) s += ws[w];
-        ws[NT / 32] = s;
-    }
-    __syncthreads();
-    s = ws[NT / 32];
-    __syncthreads();
-    return s;
 }
 
 // ------------------------------------------------ decoupled look-back
@@ -587,10 +524,10 @@ struct On {
 };
 
 template <class... P, class... A>
-cudaError_t launch_on(On on, void (*fn)(P...), uint32_t grid, uint32_t block, size_t smem, A... args)
+cudaError_t launch_on(On on, void (*fn)(P...), dim3 grid, uint32_t block, size_t smem, A... args)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = on.s;
@@ -692,7 +629,6 @@ cudaError_t launch_pair_hash(const uint32_t key[8], const uint32_t *pairs, uint6
 // fold[blocks * kHashThreads].
 cudaError_t launch_hash_peak(const uint32_t key[8], uint64_t nonce0, uint64_t count, uint32_t *fold,
                              uint32_t blocks, cudaStream_t s);
-size_t sort_smem_bytes(uint32_t cap, int dbits);
 size_t match_smem_bytes(uint32_t cap);
 constexpr int kHashThreads = 256;
 constexpr int kHashNoncesPerThread = 8;

@@ -254,9 +254,9 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
     // Partition chunks, only where a second kernel exists to overlap (the
     // separate pair hash).  Both kinds of chunks are off unless asked for:
     // measured on GB300 at K=31 it does not pay, because each kernel of a
-    // pair alone fills an SM's register file (the latency-bound sort needs
-    // four resident CTAs, the ALU-bound hashes need ~24 warps), so the two
-    // streams take turns instead of sharing SMs.
+    // pair alone fills an SM's register file (the sort's three CTAs and the
+    // ALU-bound hash's 24 to 32 warps take 60 k of the 64 k registers each),
+    // so the two streams take turns instead of sharing SMs.
     P.pchunks = P.fuse_pair_hash ? 1 : want;
     // No more chunks than partitions of the fixed size: a chunk costs two
     // launches (K=12 in 8 chunks of 2^9 records 119 us a run, in the 2 of

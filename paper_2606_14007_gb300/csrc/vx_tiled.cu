@@ -6,10 +6,10 @@
 // leaves a bucket, so each window's Table 1 and Table 2 are exactly the
 // whole plot's tables restricted to its buckets, and the windows in index
 // order concatenate to the whole plot's tables (Table 1 in (key64, nonce)
-// order, Table 2 in bucket order).  Each window hashes every nonce again and
-// keeps its own share: on GB300 hashing 2^31 nonces takes ~51 ms, less than
-// moving the 26 GB of unsorted records across the host link once, so
-// recomputing beats spilling the records and reading them back.
+// order, Table 2 in bucket order).  A window hashes its records again: on
+// GB300 hashing 2^31 nonces takes ~49 ms, less than moving the 26 GB of
+// unsorted records across the host link once, so recomputing beats spilling
+// the records and reading them back.
 //
 // The first window hashes every nonce, keeps its own records and stores each
 // nonce's window (one byte); every other window lists its own nonces from
