@@ -199,7 +199,10 @@ int vx_plot_alloc(vx_plot *plot);
 /* Table 1 (Sec. III-A hash stage; sort half of the fused Sort+Match kernel):
  * key setup, keyed BLAKE3 of every nonce, two-level bucketing scatter by
  * hash prefix, in-partition shared-memory sort.  Allocates (vx_plot_alloc)
- * if nothing is bound.  Asynchronous on stream. */
+ * if nothing is bound.  Asynchronous on stream.  Plans that place pairs in
+ * slots (t2_placement 2 and mostly 0) leave the pairs there for vx_match, 8
+ * bytes each: at K=31 83 ms, of which 5 a program that wants Table 1 alone
+ * saves with t2_placement 1 (pairs are then counted only). */
 int vx_table1(vx_plot *plot, void *stream);
 
 /* Table 2 (Sec. III-A match half of the fused Sort+Match kernel): pair
