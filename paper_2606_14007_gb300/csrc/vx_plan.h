@@ -238,13 +238,14 @@ inline int make_plan_sized(int K, const vx_opts *o, Plan *pl, const char **why, 
         // Two levels: the first takes most bits.  It claims inside the
         // ALU-bound hash, where more bins cost little, and the second then
         // writes longer runs (K = 28: 8 + 9 bits 6.04 + 1.34 ms, 9 + 8 bits
-        // 6.06 + 1.17, 10 + 7 bits 6.09 + 1.13); below 15 bits a few fewer
-        // (K = 25: 9 + 5 bits 2139 us per plot, 10 + 4 bits 2154, 7 + 7 bits
-        // 2142).  At 2^19 partitions and more 11 bits, which the largest
-        // tile's kernel also takes (K = 31: 10 + 10 bits 48.5 + 15.4 ms, 11 +
-        // 9 bits 49.0 + 10.6; K = 30: 10 + 9 bits 24.27 + 5.38, 11 + 8 bits
-        // 24.52 + 4.68; K = 29 not yet: 12.15 + 2.35 against 12.26 + 2.25).
-        P.p1 = !two_level ? P.p : P.p < 14 ? 8 : P.p == 14 ? 9 : P.p < 19 || P.wbits || P.npt != 16 ? 10 : 11;
+        // 6.06 + 1.17, 10 + 7 bits 6.09 + 1.13); below 15 bits, where 8 leave
+        // the second level few enough, no more than those (K = 25 a plot: 7 + 7
+        // bits 1921 us, 8 + 6 1916, 9 + 5 1915, 10 + 4 1922; K = 24: 8 + 5 bits
+        // 893, 10 + 3 904).  At 2^19 partitions and more 11 bits, which the
+        // largest tile's kernel also takes (K = 31: 10 + 10 bits 48.5 + 15.4
+        // ms, 11 + 9 bits 49.0 + 10.6; K = 30: 10 + 9 bits 24.27 + 5.38, 11 + 8
+        // bits 24.52 + 4.68; K = 29 not yet: 12.15 + 2.35 against 12.26 + 2.25).
+        P.p1 = !two_level ? P.p : P.p < 15 ? 8 : P.p < 19 || P.wbits || P.npt != 16 ? 10 : 11;
     }
     P.p2 = P.p - P.p1;
     if (P.mode == kScatterStaged && (P.p1 > (opts.coarse_bits < 0 ? 11 : 10) || P.p2 > 11)) {
