@@ -225,8 +225,9 @@ int vx_match(vx_plot *plot, void *stream);
  * status and the record counts in the handle's pinned host memory (left
  * there by the slot pair hash, copied otherwise) and an event that vx_sync
  * waits on.  Allocates if nothing is bound; a handle's first run also takes
- * 4 KB of device and 4 KB of pinned host memory, its own until
- * vx_plot_destroy.
+ * 1.5 KB of pinned host memory, its own until vx_plot_destroy, and as much
+ * device memory (of a static array for 256 handles at a time, then
+ * allocated).
  * Asynchronous.  One plot's runs must not overlap on the GPU (two runs of
  * the same plot on different streams race on its buffers): different plots
  * may run concurrently.  Plots that share Table-1 and scratch buffers may

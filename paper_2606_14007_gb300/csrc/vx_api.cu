@@ -313,6 +313,50 @@ cudaError_t ensure_stage(vx_plot *p, uint64_t **result)
     return e;
 }
 
+// Device copies of the handles' descriptors and tile prefixes: a slot of a
+// static array while there is one (each GPU that loads the library holds it),
+// else an allocation.  A program that makes a handle per plot would pay 130 us
+// a handle to allocate and free so little (K=14: 500 us from vx_plot_create to
+// vx_plot_destroy, 370 with the array).
+__device__ __align__(256) unsigned char g_desc_slots[vx::kStageSlots][vx::kStageBytes];
+std::mutex g_slot_mu;
+bool g_slot_used[vx::kMaxDevices][vx::kStageSlots];
+
+cudaError_t take_stage(vx_plot *p)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    void *base = nullptr;
+    if (dev >= 0 && dev < vx::kMaxDevices) {
+        if ((e = cudaGetSymbolAddress(&base, g_desc_slots)) != cudaSuccess) return e;
+        std::lock_guard<std::mutex> lk(g_slot_mu);
+        for (int i = 0; i < vx::kStageSlots; ++i) {
+            if (g_slot_used[dev][i]) continue;
+            g_slot_used[dev][i] = true;
+            p->stage_dev = dev;
+            p->stage_slot = i;
+            p->d_stage = static_cast<uint8_t *>(base) + (size_t)i * vx::kStageBytes;
+            return cudaSuccess;
+        }
+    }
+    if ((e = dev_alloc(&base, vx::kStageBytes)) == cudaSuccess) p->d_stage = static_cast<uint8_t *>(base);
+    return e;
+}
+
+// To be called once nothing queued reads it any more.
+void release_stage(vx_plot *p)
+{
+    if (p->stage_slot >= 0) {
+        std::lock_guard<std::mutex> lk(g_slot_mu);
+        g_slot_used[p->stage_dev][p->stage_slot] = false;
+    } else if (p->d_stage) {
+        cudaFree(p->d_stage);
+    }
+    p->d_stage = nullptr;
+    p->stage_slot = p->stage_dev = -1;
+}
+
 // Uploads the descriptor and the single-plot tile prefixes if they changed
 // and caches the single-plot launch set.  The device copy is the handle's
 // own: the scratch buffer may be shared with other plots, whose runs may
@@ -323,14 +367,12 @@ int upload_desc(vx_plot *p, cudaStream_t s)
     uint64_t *result = nullptr;
     VX_TRY(p, ensure_stage(p, &result));
     if (!p->d_stage) {
-        void *d = nullptr;
-        const cudaError_t e = dev_alloc(&d, vx::kStageResultOffset);
+        const cudaError_t e = take_stage(p);
         if (e != cudaSuccess) {
             cudaGetLastError();
             set_err(p, std::string("descriptor allocation failed: ") + cudaGetErrorName(e));
             return e == cudaErrorMemoryAllocation ? VX_ENOMEM : VX_ECUDA;
         }
-        p->d_stage = static_cast<uint8_t *>(d);
     }
     if (p->ev_pending) VX_TRY(p, cudaEventSynchronize(p->ev_stage));
     fill_desc(p, p->h_stage);
@@ -1008,8 +1050,8 @@ void vx_plot_destroy(vx_plot *p)
     if (p->ev_pending) cudaEventSynchronize(p->ev_stage);
     if (p->release) p->release(p->release_ctx, p);
     free_owned(p);
-    if (p->h_stage) cudaFreeHost(p->h_stage);
-    if (p->d_stage) cudaFree(p->d_stage);
+    if (p->h_stage) cudaFreeHost(p->h_stage);  // waits for the device, so nothing reads the descriptor either
+    release_stage(p);
     if (p->ev_stage) cudaEventDestroy(p->ev_stage);
     if (p->ev_done) cudaEventDestroy(p->ev_done);
     vx_plot_profile(p, 0);

@@ -83,6 +83,7 @@ struct vx_plot {
     bool desc_dirty = true;        // descriptor needs an upload
     vx::Desc *h_stage = nullptr;   // pinned block: Desc, tile prefixes, a run's result
     uint8_t *d_stage = nullptr;    // the first two on the device, at the same offsets
+    int stage_dev = -1, stage_slot = -1;  // its slot of the static array; -1: allocated
     cudaEvent_t ev_stage = nullptr;
     bool ev_pending = false;
     cudaStream_t last = nullptr;

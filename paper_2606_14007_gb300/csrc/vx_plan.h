@@ -23,9 +23,10 @@ constexpr int kSort2PartLog2 = 10;         // the same for the sort of Table 2 b
 constexpr uint32_t kDefaultSlackSigma = 12;
 constexpr int kMaxPartBits = 21;           // scatter levels of <= 10 and <= 11 bits
 constexpr int kAggMaxBits = 6;             // warp-aggregate ranks up to 64 bins
-constexpr size_t kStageBytes = 4096;       // a handle's pinned block: Desc, tile prefixes, result
-constexpr size_t kStageTilesOffset = 3584;
-constexpr size_t kStageResultOffset = 4064;  // status u32 at +0, Table-2 count u64 at +8
+constexpr size_t kStageBytes = 1536;       // a handle's pinned block: Desc, tile prefixes, result
+constexpr size_t kStageTilesOffset = 1024;
+constexpr size_t kStageResultOffset = 1472;  // status u32 at +0, Table-2 count u64 at +8
+constexpr int kStageSlots = 256;           // handles whose device copy needs no allocation
 constexpr uint64_t kWriteStageBytes = 256ull << 20;  // Sec. III-B: 256 MB pinned staging
 constexpr uint64_t kWriteChunkBytes = 4ull << 20;    // Sec. III-A: 4 MB sequential chunks
 constexpr int kPlanHashThreads = 256;      // threads per hash CTA

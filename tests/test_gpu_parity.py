@@ -605,3 +605,27 @@ def test_cross_bucket_runs_take_no_longer_than_their_kernels(vx, K):
         traced.append(sum(ms.values()) / runs)
     p.close()
     assert min(chained) <= 1.1 * min(traced)
+
+
+def test_many_handles_keep_their_own_descriptors(vx):
+    # more live handles than the static array has slots for their descriptors,
+    # then some given back and taken by new handles
+    K = 10
+    keys = [plot_key(1000 + i) for i in range(300)]
+    plots = [vx.Plot(K, k) for k in keys]
+    for p in plots:
+        p.run()
+    for p in plots[50:120]:
+        p.sync()
+        p.close()
+    keys[50:120] = [plot_key(2000 + i) for i in range(70)]
+    plots[50:120] = [vx.Plot(K, k).run() for k in keys[50:120]]
+    for p, k in zip(plots, keys):
+        p.run()
+    for i, (p, k) in enumerate(zip(plots, keys)):
+        n2 = p.sync()
+        if i % 5 == 0:
+            r1, r2 = oracle_plot(K, k)
+            assert np.array_equal(p.t1.cpu().numpy(), r1)
+            assert n2 == r2.shape[0] and np.array_equal(p.t2.cpu().numpy(), r2)
+        p.close()
