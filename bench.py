@@ -547,10 +547,10 @@ def main():
         for h in handles:
             vx.vx_plot_destroy(h)
         del t2_bufs
-        desc_bytes = 512
+        desc_bytes = 1360  # descriptor and tile prefixes, uploaded at a handle's first run
         e2e = {"value": N * args.e2e_steps * world / dt, "unit": UNIT,
                "h2d_bytes_per_step": desc_bytes,
-               "d2h_bytes_per_step": int(16 * sum(counts) / len(counts)) + 12,
+               "d2h_bytes_per_step": int(16 * sum(counts) / len(counts)) + 24,  # + status and counts
                "steps": args.e2e_steps, "d2h_gbs_measured": d2h_gbs,
                "note": "per step: vx_plot_create from a host key, vx_plot_bind, vx_plot_run, "
                        "vx_sync, Table 2 copied to pinned host memory with vx_table_copy "

@@ -27,8 +27,8 @@
 // offsets, and the pairs go through a 16-bit list in shared memory, so that
 // they are written one per lane, coalesced.
 //
-// Bound by instruction issue (59%) and the shared-memory data path (66%)
-// together at 24 warps per SM: 15.9 k warp instructions per 2048-record
+// Bound by instruction issue (59%) and the shared-memory data path (65%)
+// together at 24 warps per SM: 16.1 k warp instructions per 2048-record
 // partition, against 23 k for the counting sort with ranked digit runs, the
 // per-thread Table-1 stores and the record-wise pair stores before it: 31.0
 // -> 24.1 ms at K=31, 0.97 -> 0.75 ms at K=26, and with the items handed out
